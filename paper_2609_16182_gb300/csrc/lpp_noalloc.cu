@@ -9,14 +9,16 @@
 // lpp_presolve using only the arrays the caller passes plus one fixed
 // scratch array compiled into the library.
 //
-// Rows of up to kNaLong entries are reduced by one warp each (no scratch).
-// Longer rows are split by fixed 4096-entry windows of the entry array; a
-// window meets at most two long rows (one that started before it, one that
-// starts inside it), so each window stores at most two partial results in
-// the scratch array, and a third kernel adds a long row's partials in window
-// order.  Every slot a long row reads is written earlier in the same call, so
+// A warp takes 32 consecutive rows, with as many lanes per row as its length
+// asks for; rows of more than 512 entries are left to the whole block, and
+// rows of more than 4096 are split by fixed 4096-entry windows of the entry
+// array.  A window meets at most two such long rows (one that started before
+// it, one that starts inside it), so each window stores at most two partial
+// results in the scratch array, and a last kernel adds a long row's partials
+// in window order.  Every slot it reads is written earlier in the same call, so
 // nothing in the scratch array has to start at zero.
 #include <algorithm>
+#include <cstring>
 #include <mutex>
 
 #include "lpp_engine.h"
@@ -27,157 +29,229 @@ constexpr int kNaWindow = 4096;           // entries per window
 constexpr int kNaLong = 4096;             // longer rows use the windows
 constexpr int kNaMaxWindows = 1 << 16;    // => at most 268,435,456 nonzeros
 constexpr int kNaThreads = 256;
+constexpr int kNaWarps = kNaThreads / 32;
+// lanes per row by its length: one up to 4 entries, 4 up to 32, a warp up to
+// 512, the block beyond.  An FP64 warp instruction holds the pipe for 16
+// clocks however many lanes are active, so a warp must not wait for one long
+// row among short ones; lengths up to 4 are four fifths of a skewed LP's rows.
+constexpr int kNaOne = 4, kNaFour = 32, kNaWarp = 512;
 
 struct WindowPart {
-    double2 act[2];   // (min, max) finite parts for slot 0 / slot 1
-    int2 ninf[2];     // infinite-term counts
+    double2 act[2];   // (min, max) finite parts: [0] of the long row that started before the window,
+    int2 ninf[2];     // [1] of the one that starts in it; infinite-term counts
     int32_t row[2];   // which row each slot belongs to (-1: unused)
     int32_t pad[2];
 };
+static_assert(sizeof(WindowPart) == 64, "4 MiB of scratch");
 
 // The scratch of lpp_row_activity_noalloc: 4 MiB per device that loads the
 // library, held until the process exits; shared by every call.
 static __device__ __align__(256) WindowPart g_na_scratch[kNaMaxWindows];
-
-__device__ __forceinline__ bool na_fin(double x) {
-    return (__double_as_longlong(x) & 0x7ff0000000000000LL) != 0x7ff0000000000000LL;
-}
-__device__ __forceinline__ double na_norm(double x, double huge) {
-    if (x >= huge) return __longlong_as_double(0x7ff0000000000000LL);
-    if (x <= -huge) return __longlong_as_double((long long)0xfff0000000000000ULL);
-    return x;
-}
 
 struct NaArgs {
     int32_t m;
     int64_t nnz;
     const int32_t *rp, *ci;
     const double *val, *lb, *ub;
-    double huge;
+    long long huge_bits;  // |b| >= huge (or NaN) is infinite: one integer compare on the bits
     double *amin, *amax;
     int32_t *nmin, *nmax;
 };
 
-// accumulate entries [b, e) of a row
-__device__ __forceinline__ void na_accumulate(const NaArgs &a, int64_t b, int64_t e, int64_t stride, double &smin,
-                                              double &smax, int &cmin, int &cmax) {
-    for (int64_t k = b; k < e; k += stride) {
-        const double v = a.val[k];
-        const int32_t j = a.ci[k];
-        const double l = na_norm(a.lb[j], a.huge), u = na_norm(a.ub[j], a.huge);
-        const bool neg = __double_as_longlong(v) < 0;
-        const double bmin = neg ? u : l, bmax = neg ? l : u;
-        if (na_fin(bmin)) smin = fma(v, bmin, smin);
-        else cmin++;
-        if (na_fin(bmax)) smax = fma(v, bmax, smax);
-        else cmax++;
+struct NaSum {
+    double lo, hi;
+    int nlo, nhi;
+};
+
+// entries b + 0, b + W, .. below e of a row, U loads and gathers in flight:
+// the fused multiply-adds take them in order
+template <int W, int U>
+__device__ __forceinline__ void na_accumulate(const NaArgs &a, int32_t b, int32_t e, NaSum &s) {
+    for (int32_t k0 = b; k0 < e; k0 += U * W) {
+        int32_t j[U];
+        double v[U], l[U], u[U];
+#pragma unroll
+        for (int q = 0; q < U; q++) {
+            const bool in = k0 + q * W < e;
+            j[q] = in ? a.ci[k0 + q * W] : -1;
+            v[q] = in ? a.val[k0 + q * W] : 0.0;
+        }
+#pragma unroll
+        for (int q = 0; q < U; q++) {
+            l[q] = j[q] >= 0 ? a.lb[j[q]] : 0.0;
+            u[q] = j[q] >= 0 ? a.ub[j[q]] : 0.0;
+        }
+#pragma unroll
+        for (int q = 0; q < U; q++) {
+            if (k0 + q * W >= e) break;
+            const bool fl = (lpp::dbits(l[q]) & 0x7fffffffffffffffLL) < a.huge_bits;
+            const bool fu = (lpp::dbits(u[q]) & 0x7fffffffffffffffLL) < a.huge_bits;
+            const bool neg = lpp::is_neg(v[q]);
+            const double bl = neg ? u[q] : l[q], bh = neg ? l[q] : u[q];
+            if (neg ? fu : fl) s.lo = fma(v[q], bl, s.lo);
+            else s.nlo++;
+            if (neg ? fl : fu) s.hi = fma(v[q], bh, s.hi);
+            else s.nhi++;
+        }
     }
 }
 
-// one warp per row of at most kNaLong entries
-__global__ void __launch_bounds__(kNaThreads) k_na_short(NaArgs a) {
+template <int W>
+__device__ __forceinline__ void na_butterfly(NaSum &s) {
+    const unsigned mask = lpp::group_mask<W>();
+    s.lo = lpp::group_sum<W>(s.lo, mask);
+    s.hi = lpp::group_sum<W>(s.hi, mask);
+    s.nlo = lpp::group_sum<W>(s.nlo, mask);
+    s.nhi = lpp::group_sum<W>(s.nhi, mask);
+}
+
+__device__ __forceinline__ void na_row(const NaArgs &a, int32_t r, const NaSum &s) {
+    a.amin[r] = s.lo;
+    a.amax[r] = s.hi;
+    a.nmin[r] = s.nlo;
+    a.nmax[r] = s.nhi;
+}
+
+// the block's sum of entries [b, e): warp butterflies, then the warps'
+// (every thread must call it; thread 0 has the result)
+__device__ __forceinline__ NaSum na_block(const NaArgs &a, int32_t b, int32_t e, NaSum *s_w) {
+    NaSum s{0.0, 0.0, 0, 0};
+    na_accumulate<kNaThreads, 4>(a, b + threadIdx.x, e, s);
+    na_butterfly<32>(s);
+    if ((threadIdx.x & 31) == 0) s_w[threadIdx.x >> 5] = s;
+    __syncthreads();
+    NaSum w{0.0, 0.0, 0, 0};
+    if (threadIdx.x < 32) {
+        if (threadIdx.x < kNaWarps) w = s_w[threadIdx.x];
+        na_butterfly<32>(w);
+    }
+    __syncthreads();
+    return w;
+}
+
+// Row containing entry k, by a whole warp: the last row whose start is <= k
+// (skips empty rows).  Each step probes 32 rows of the interval, so 2 M rows
+// take five dependent loads instead of 21.
+__device__ __forceinline__ int32_t na_row_of(const int32_t *rp, int32_t m, int64_t k) {
     const int lane = threadIdx.x & 31;
-    const int64_t warps = (int64_t)gridDim.x * (kNaThreads / 32);
-    for (int64_t i = (int64_t)blockIdx.x * (kNaThreads / 32) + (threadIdx.x >> 5); i < a.m; i += warps) {
-        const int64_t b = a.rp[i], e = a.rp[i + 1];
-        if (e - b > kNaLong) continue;  // warp-uniform
-        double smin = 0.0, smax = 0.0;
-        int cmin = 0, cmax = 0;
-        na_accumulate(a, b + lane, e, 32, smin, smax, cmin, cmax);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            smin += __shfl_xor_sync(0xffffffffu, smin, o);
-            smax += __shfl_xor_sync(0xffffffffu, smax, o);
-            cmin += __shfl_xor_sync(0xffffffffu, cmin, o);
-            cmax += __shfl_xor_sync(0xffffffffu, cmax, o);
-        }
-        if (lane == 0) {
-            a.amin[i] = smin;
-            a.amax[i] = smax;
-            a.nmin[i] = cmin;
-            a.nmax[i] = cmax;
-        }
-    }
-}
-
-// row containing entry e: the last row whose start is <= e (skips empty rows)
-__device__ __forceinline__ int32_t na_row_of(const int32_t *rp, int32_t m, int64_t e) {
-    int32_t lo = 0, hi = m;  // rp[lo] <= e < rp[hi] holds for the answer lo
+    int64_t lo = 0, hi = m;  // rp[lo] <= k < rp[hi]
     while (hi - lo > 1) {
-        const int32_t mid = lo + (hi - lo) / 2;
-        if (rp[mid] <= e) lo = mid;
-        else hi = mid;
+        const int64_t p = lo + ((hi - lo) * (lane + 1)) / 33;
+        const int c = __popc(__ballot_sync(0xffffffffu, rp[p] <= k));
+        const int64_t l2 = c > 0 ? lo + ((hi - lo) * c) / 33 : lo;
+        hi = c < 32 ? lo + ((hi - lo) * (c + 1)) / 33 : hi;
+        lo = l2;
     }
-    return lo;
+    return (int32_t)lo;
 }
 
-template <typename T>
-__device__ __forceinline__ T na_block_sum(T v, T *s_w) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) s_w[threadIdx.x >> 5] = v;
+// window w of the entry array: the partials of the (at most two) long rows it meets
+__device__ __forceinline__ void na_window(const NaArgs &a, WindowPart &p, int32_t w, NaSum *s_w) {
+    __shared__ int32_t s_r[2];
+    const int64_t w0 = (int64_t)w * kNaWindow, w1 = min(a.nnz, w0 + kNaWindow);
+    if (threadIdx.x < 64) s_r[threadIdx.x >> 5] = na_row_of(a.rp, a.m, threadIdx.x < 32 ? w0 : w1 - 1);
     __syncthreads();
-    T t = T(0);
-    if (threadIdx.x == 0)
-        for (int w = 0; w < kNaThreads / 32; w++) t += s_w[w];
-    __syncthreads();
-    return t;
-}
-
-// one block per window: the partials of the (at most two) long rows it meets
-__global__ void __launch_bounds__(kNaThreads) k_na_windows(NaArgs a, WindowPart *scratch) {
-    __shared__ double s_d[kNaThreads / 32];
-    __shared__ int s_i[kNaThreads / 32];
-    const int64_t w0 = (int64_t)blockIdx.x * kNaWindow;
-    const int64_t w1 = min(a.nnz, w0 + kNaWindow);
-    const int32_t r0 = na_row_of(a.rp, a.m, w0);
-    const int32_t r1 = na_row_of(a.rp, a.m, w1 - 1);
     for (int slot = 0; slot < 2; slot++) {
-        const int32_t r = slot == 0 ? r0 : r1;
+        const int32_t r = s_r[slot];
         const int64_t rb = a.rp[r], re = a.rp[r + 1];
-        const bool use = re - rb > kNaLong && (slot == 0 || r1 != r0);
-        if (!use) {  // block-uniform
-            if (threadIdx.x == 0) scratch[blockIdx.x].row[slot] = -1;
-            continue;
-        }
-        const int64_t b = max(rb, w0), e = min(re, w1);
-        double smin = 0.0, smax = 0.0;
-        int cmin = 0, cmax = 0;
-        na_accumulate(a, b + threadIdx.x, e, kNaThreads, smin, smax, cmin, cmax);
-        smin = na_block_sum(smin, s_d);
-        smax = na_block_sum(smax, s_d);
-        cmin = na_block_sum(cmin, s_i);
-        cmax = na_block_sum(cmax, s_i);
+        const bool use = re - rb > kNaLong && (slot == 0 ? rb < w0 : rb >= w0);
+        if (threadIdx.x == 0) p.row[slot] = use ? r : -1;
+        if (!use) continue;  // block-uniform
+        const NaSum s = na_block(a, (int32_t)max(rb, w0), (int32_t)min(re, w1), s_w);
         if (threadIdx.x == 0) {
-            WindowPart &p = scratch[blockIdx.x];
-            p.act[slot] = make_double2(smin, smax);
-            p.ninf[slot] = make_int2(cmin, cmax);
-            p.row[slot] = r;
+            p.act[slot] = make_double2(s.lo, s.hi);
+            p.ninf[slot] = make_int2(s.nlo, s.nhi);
         }
     }
 }
 
-// one thread per long row: its window partials added in window order
-__global__ void k_na_long(NaArgs a, const WindowPart *scratch) {
-    const int64_t step = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.m; i += step) {
-        const int64_t rb = a.rp[i], re = a.rp[i + 1];
-        if (re - rb <= kNaLong) continue;
-        double smin = 0.0, smax = 0.0;
-        int cmin = 0, cmax = 0;
-        for (int64_t w = rb / kNaWindow; w <= (re - 1) / kNaWindow; w++) {
-            const int slot = rb <= w * kNaWindow ? 0 : 1;  // started before the window, or inside it
-            const WindowPart &p = scratch[w];
-            smin += p.act[slot].x;
-            smax += p.act[slot].y;
-            cmin += p.ninf[slot].x;
-            cmax += p.ninf[slot].y;
-        }
-        a.amin[i] = smin;
-        a.amax[i] = smax;
-        a.nmin[i] = cmin;
-        a.nmax[i] = cmax;
+// Blocks [0, windows): the long rows' windows, first so that they run beside
+// the rows; the other blocks: 256 rows each, those of at most 4096 entries.
+// Bound by the FP64 pipe (63% busy) and the latency of the two 8-byte bound
+// gathers per entry: 20 M entries in 2 M skewed rows take 244 us, 2660 us
+// with a warp per row (a median row of two entries used two of 32 lanes, and
+// infinities were tested by FP64 compares).  No shared memory for the entries:
+// a tile of them staged there, coalesced, took 510 us, because it leaves the
+// L1 too few lines for the gathers in flight (4% hits instead of 23%).
+__global__ void __launch_bounds__(kNaThreads, 5) k_na_rows(NaArgs a, WindowPart *scratch, int32_t windows) {
+    __shared__ int2 s_mid[kNaWarps][32];   // a warp's rows of 5 to 32 entries: (lane of the row, first entry)
+    __shared__ int32_t s_blk[kNaThreads];  // the block's rows of 513 to 4096 entries
+    __shared__ int32_t s_nblk;
+    __shared__ NaSum s_w[kNaWarps];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (blockIdx.x < (unsigned)windows) {
+        na_window(a, scratch[blockIdx.x], (int32_t)blockIdx.x, s_w);
+        return;
     }
+    const int64_t base = (int64_t)(blockIdx.x - windows) * kNaThreads;
+    if (tid == 0) s_nblk = 0;
+    __syncthreads();
+    const int64_t rl = base + tid;
+    const int32_t r = (int32_t)rl;
+    int32_t b = 0, e = 0;
+    if (rl < a.m) {
+        b = a.rp[r];
+        e = a.rp[r + 1];
+    }
+    const int32_t n = e - b;
+    if (rl < a.m && n <= kNaOne) {
+        NaSum s{0.0, 0.0, 0, 0};
+        na_accumulate<1, 4>(a, b, e, s);
+        na_row(a, r, s);
+    }
+    const unsigned mid = __ballot_sync(0xffffffffu, n > kNaOne && n <= kNaFour);
+    unsigned wide = __ballot_sync(0xffffffffu, n > kNaFour && n <= kNaWarp);
+    if (n > kNaOne && n <= kNaFour) s_mid[warp][__popc(mid & ((1u << lane) - 1u))] = make_int2(lane, b);
+    if (n > kNaWarp && n <= kNaLong) s_blk[atomicAdd(&s_nblk, 1)] = r;
+    __syncwarp();
+    const int nmid = __popc(mid);
+    for (int i0 = 0; i0 < nmid; i0 += 8) {
+        const int i = i0 + lane / 4;
+        const int2 it = i < nmid ? s_mid[warp][i] : make_int2(0, 0);
+        const int32_t eb = it.y, ee = eb + __shfl_sync(0xffffffffu, n, it.x);
+        NaSum s{0.0, 0.0, 0, 0};
+        if (i < nmid) na_accumulate<4, 4>(a, eb + (lane & 3), ee, s);
+        na_butterfly<4>(s);
+        if (i < nmid && (lane & 3) == 0) na_row(a, (int32_t)(rl - lane) + it.x, s);
+    }
+    while (wide) {
+        const int src = __ffs(wide) - 1;
+        wide &= wide - 1u;
+        const int32_t wb = __shfl_sync(0xffffffffu, b, src), we = __shfl_sync(0xffffffffu, e, src);
+        NaSum s{0.0, 0.0, 0, 0};
+        na_accumulate<32, 4>(a, wb + lane, we, s);
+        na_butterfly<32>(s);
+        if (lane == 0) na_row(a, (int32_t)(rl - lane) + src, s);
+    }
+    __syncthreads();
+    for (int i = 0; i < s_nblk; i++) {
+        const int32_t q = s_blk[i];
+        const NaSum s = na_block(a, a.rp[q], a.rp[q + 1], s_w);
+        if (tid == 0) na_row(a, q, s);
+    }
+}
+
+// one warp per window in which a long row starts: the row's partials, its
+// windows lane-strided, then a butterfly
+__global__ void __launch_bounds__(kNaThreads) k_na_long(NaArgs a, const WindowPart *scratch, int32_t windows) {
+    const int32_t w = (int32_t)((blockIdx.x * (unsigned)kNaThreads + threadIdx.x) >> 5);
+    const int lane = threadIdx.x & 31;
+    if (w >= windows) return;  // the same w in the whole warp
+    const int32_t r = scratch[w].row[1];
+    if (r < 0) return;
+    const int32_t last = (a.rp[r + 1] - 1) / kNaWindow;
+    NaSum s{0.0, 0.0, 0, 0};
+    for (int32_t q = w + lane; q <= last; q += 32) {
+        const int slot = q == w ? 1 : 0;
+        const double2 d = scratch[q].act[slot];
+        const int2 c = scratch[q].ninf[slot];
+        s.lo += d.x;
+        s.hi += d.y;
+        s.nlo += c.x;
+        s.nhi += c.y;
+    }
+    na_butterfly<32>(s);
+    if (lane == 0) na_row(a, r, s);
 }
 
 // device address of g_na_scratch, looked up once per device
@@ -207,14 +281,13 @@ extern "C" lpp_status lpp_row_activity_noalloc(int32_t m, int32_t n, int64_t nnz
         std::lock_guard<std::mutex> g(g_na_mu);
         if (!g_na_ptr[dev]) {
             // set-up, once per device, with that device current: the array's
-            // address, and all three kernels loaded now (with lazy module
+            // address, and both kernels loaded now (with lazy module
             // loading a kernel is otherwise loaded at its first launch, which
-            // for the window kernels is the first call with nnz > 4096)
+            // for the second is the first call with nnz > 4096)
             void *p = nullptr;
             e = cudaGetSymbolAddress(&p, g_na_scratch);
             cudaFuncAttributes fa;
-            if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_na_short);
-            if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_na_windows);
+            if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_na_rows);
             if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_na_long);
             if (e != cudaSuccess) return lpp_noalloc_fail(LPP_ERR_CUDA, cudaGetErrorString(e));
             g_na_ptr[dev] = p;
@@ -222,20 +295,15 @@ extern "C" lpp_status lpp_row_activity_noalloc(int32_t m, int32_t n, int64_t nnz
         scratch = g_na_ptr[dev];
     }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    NaArgs a{m, nnz, row_ptr, col_idx, val, lb, ub, huge, act_min, act_max, ninf_min, ninf_max};
-    int sms = 0;
-    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return lpp_noalloc_fail(LPP_ERR_CUDA, cudaGetErrorString(e));
-    const int sms_blocks = std::max(1, sms) * 8;
-    const int64_t warp_blocks = ((int64_t)m + kNaThreads / 32 - 1) / (kNaThreads / 32);
-    k_na_short<<<(unsigned)std::min<int64_t>(warp_blocks, sms_blocks), kNaThreads, 0, s>>>(a);
-    if (nnz > kNaLong) {
-        const unsigned windows = (unsigned)((nnz + kNaWindow - 1) / kNaWindow);
-        k_na_windows<<<windows, kNaThreads, 0, s>>>(a, static_cast<WindowPart *>(scratch));
-        const int64_t row_blocks = ((int64_t)m + 255) / 256;
-        k_na_long<<<(unsigned)std::min<int64_t>(row_blocks, sms_blocks), 256, 0, s>>>(
-            a, static_cast<const WindowPart *>(scratch));
-    }
+    long long hb;
+    std::memcpy(&hb, &huge, sizeof hb);
+    NaArgs a{m, nnz, row_ptr, col_idx, val, lb, ub, hb, act_min, act_max, ninf_min, ninf_max};
+    WindowPart *parts = static_cast<WindowPart *>(scratch);
+    const int32_t windows = nnz > kNaLong ? (int32_t)((nnz + kNaWindow - 1) / kNaWindow) : 0;
+    k_na_rows<<<(unsigned)(windows + (m + (int64_t)kNaThreads - 1) / kNaThreads), kNaThreads, 0, s>>>(a, parts,
+                                                                                                  windows);
+    if (windows)
+        k_na_long<<<(unsigned)((windows + kNaWarps - 1) / kNaWarps), kNaThreads, 0, s>>>(a, parts, windows);
     e = cudaGetLastError();
     if (e != cudaSuccess) return lpp_noalloc_fail(LPP_ERR_CUDA, cudaGetErrorString(e));
     return LPP_OK;
