@@ -159,19 +159,16 @@ __device__ void set_ctx(BlockState &S, const FusedArgs &F, const FusedLP &P) {
 
 // ------------------------------------------------------------- the kernel
 template <int NT>
-__global__ void __launch_bounds__(NT) k_batch_fused(FusedArgs F) {
+__global__ void __launch_bounds__(NT, NT == 256 ? 4 : (NT == 512 ? 2 : 8)) k_batch_fused(FusedArgs F) {
     extern __shared__ __align__(16) unsigned char s_dyn[];
     __shared__ BlockState S;
     constexpr int NW = NT / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    // per-warp candidate and test queues (the layout k_prop_groups uses)
+    // per-warp candidate queues
     double *qd = reinterpret_cast<double *>(s_dyn);
-    int32_t *qi = reinterpret_cast<int32_t *>(qd + 6 * NW * kQueueCap);
+    int32_t *qi = reinterpret_cast<int32_t *>(qd + 2 * NW * kQueueCap);
     CandQueue q{qd + (0 * NW + warp) * kQueueCap, qd + (1 * NW + warp) * kQueueCap,
                 qi + (0 * NW + warp) * kQueueCap, qi + (1 * NW + warp) * kQueueCap, 0};
-    TestQueue tq{qd + (2 * NW + warp) * kQueueCap, qd + (3 * NW + warp) * kQueueCap,
-                 qd + (4 * NW + warp) * kQueueCap, qd + (5 * NW + warp) * kQueueCap,
-                 qi + (2 * NW + warp) * kQueueCap, qi + (3 * NW + warp) * kQueueCap, 0};
     while (true) {
         if (tid == 0) {
             const int32_t t = atomicAdd(F.next, 1);
@@ -260,15 +257,10 @@ __global__ void __launch_bounds__(NT) k_batch_fused(FusedArgs F) {
                     const int32_t pos = p * per + lane / W;
                     const bool valid = pos < cnt;
                     const int32_t i = valid ? ord[b0 + pos] : 0;
-                    switch (W) {
-                        case 1: prop_group<1>(C, i, valid, rem, evaluated, tested, q, tq); break;
-                        case 8: prop_group<8>(C, i, valid, rem, evaluated, tested, q, tq); break;
-                        case 16: prop_group<16>(C, i, valid, rem, evaluated, tested, q, tq); break;
-                        default: prop_group<32>(C, i, valid, rem, evaluated, tested, q, tq); break;
-                    }
+                    if (c < 5) prop_row<false>(C, i, valid, W, rem, evaluated, tested, q);
+                    else prop_row<true>(C, i, valid, 32, rem, evaluated, tested, q);
                 }
             }
-            tq_flush(C, tq, q);
             cq_flush(C, q);
             int32_t removed = bsum<NT>(rem, S.w);
             rem = 0;
@@ -449,7 +441,7 @@ __global__ void __launch_bounds__(NT) k_batch_fused(FusedArgs F) {
                     // an unchanged row's S5 key is taken again when columns
                     // were dropped (it hashes the renumbered column indices)
                     const bool lost = K.r_len[i] != C.A.ptr[i + 1] - C.A.ptr[i];
-                    F.rdirty[nx][p] = (C.rdnext[i] | lost) ? 1 : (n2 != n ? 2 : 0);
+                    F.rdirty[nx][p] = (uint8_t)((C.rdnext[i] | lost ? kEval : 0) | (lost | (n2 != n) ? kRekey : 0));
                     F.act[nx][p] = C.act[i];
                     F.ninf[nx][p] = C.ninf[i];
                     F.hrow[nx][p] = C.hrow[i];
@@ -619,7 +611,7 @@ __global__ void __launch_bounds__(NT) k_batch_fused(FusedArgs F) {
 
 }  // namespace
 
-size_t batch_fused_smem(int threads) { return (size_t)(threads / 32) * kQueueCap * (6 * sizeof(double) + 4 * sizeof(int32_t)); }
+size_t batch_fused_smem(int threads) { return (size_t)(threads / 32) * kQueueCap * (2 * sizeof(double) + 2 * sizeof(int32_t)); }
 
 int batch_fused_blocks_per_sm(int threads) {
     int b = 0;

@@ -373,10 +373,11 @@ __global__ void __launch_bounds__(kBlock) k_rowvec(Ctx C, CompactCtx K) {
     if (C.lp_row) K.lp_row2[p] = C.lp_row[i];
     K.rp2[p] = K.r_off[i];
     // a row that lost entries (fixed columns) changed: evaluate it next round;
-    // an unchanged row's S5 key is taken again when columns were dropped (the
-    // key hashes column indices, which the compaction renumbers)
+    // its S5 key is taken again then, and an unchanged row's when columns were
+    // dropped (the key hashes column indices, which the compaction renumbers)
     const bool lost = K.r_len[i] != C.A.ptr[i + 1] - C.A.ptr[i];
-    K.rdirty2[p] = (C.rdnext[i] | lost) ? 1 : (!C.t_orig && K.c_pos[C.n] != C.n ? 2 : 0);
+    const bool renumbered = !C.t_orig && K.c_pos[C.n] != C.n;
+    K.rdirty2[p] = (uint8_t)((C.rdnext[i] | lost ? 1 : 0) | (lost | renumbered ? 2 : 0));  // kEval, kRekey
     K.act2[p] = C.act[i];
     K.ninf2[p] = C.ninf[i];
     K.hrow2[p] = C.hrow[i];

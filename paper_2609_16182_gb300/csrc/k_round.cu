@@ -28,36 +28,150 @@ namespace lpp {
 
 namespace {
 
-__global__ void __launch_bounds__(kBlock, 4) k_prop_groups(Ctx C, GroupGrid g) {
-    __shared__ double s_qx[kBlock / 32][kQueueCap], s_qa[kBlock / 32][kQueueCap];
-    __shared__ int32_t s_qj[kBlock / 32][kQueueCap], s_qk[kBlock / 32][kQueueCap];
-    __shared__ double s_ta[kBlock / 32][kQueueCap], s_ts[kBlock / 32][kQueueCap], s_tb[kBlock / 32][kQueueCap],
-        s_to[kBlock / 32][kQueueCap];
-    __shared__ int32_t s_tj[kBlock / 32][kQueueCap], s_tf[kBlock / 32][kQueueCap];
+// Rows of 257 to 4096 entries (kMidMin on), S1-S3 by the whole block with the
+// sums of prop_group<32>: 32 lane-strided chains, then the butterfly.  All
+// eight warps load the entries and their bounds, 512 at a time, into shared
+// memory (the candidate queues' space, emptied before); warp 0 then runs the
+// chains of the minimum and warp 1 those of the maximum while the next
+// entries are on their way.  A warp alone walked such a row four loads at a
+// time: 49 to 67 us a round for one row of 4000 entries among 20 k short ones.
+constexpr int32_t kMidMin = 257;
+constexpr int32_t kMidTile = 2 * kBlock;
+static_assert(kMidTile * 24 == (kBlock / 32) * kQueueCap * 24, "the tile fills the queues' space");
+struct MidShared {
+    double smin, smax;
+    unsigned long long h;
+    int nmin, nmax, kind;
+};
+
+__device__ __forceinline__ void prop_mid(const Ctx &C, int32_t i, MidShared &M, double *tile, int32_t &removed,
+                                         int32_t &evaluated, int32_t &tested, CandQueue &q) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    double *s_a = tile, *s_l = tile + kMidTile, *s_h = tile + 2 * kMidTile;
+    const int32_t beg = C.A.ptr[i], end = C.A.ptr[i + 1];
+    const bool rehash = C.rdirty[i] & kRekey;
+    cq_flush(C, q);
+    if (tid == 0) {
+        M.h = 0;
+        M.nmin = M.nmax = 0;
+    }
+    const bool neg0 = rehash ? is_neg(C.A.val[beg]) : false;
+    double sum = 0.0;  // warp 0: the lane's chain of the minimum, warp 1: of the maximum
+    int nmin = 0, nmax = 0;
+    unsigned long long h = 0;
+    int32_t j[2];
+    double a[2];
+    double2 b[2];
+    auto load = [&](int32_t t0) {
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+            const int32_t k = t0 + u * kBlock + tid;
+            j[u] = k < end ? C.A.idx[k] : -1;
+            a[u] = k < end ? C.A.val[k] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < 2; u++) b[u] = j[u] >= 0 ? C.lu[j[u]] : make_double2(0.0, 0.0);
+    };
+    load(beg);
+    for (int32_t t0 = beg; t0 < end; t0 += kMidTile) {
+        __syncthreads();  // the queues are empty, the chains of the tile before are done
+#pragma unroll
+        for (int u = 0; u < 2; u++) {
+            const bool neg = is_neg(a[u]);
+            double bmin = neg ? b[u].y : b[u].x, bmax = neg ? b[u].x : b[u].y;
+            // an infinite (or absent) term adds 0: a * 0 leaves the chain as it is
+            if (!is_fin(bmin)) {
+                nmin++;
+                bmin = 0.0;
+            }
+            if (!is_fin(bmax)) {
+                nmax++;
+                bmax = 0.0;
+            }
+            if (rehash && j[u] >= 0) h += entry_hash(j[u], neg != neg0);
+            s_a[u * kBlock + tid] = a[u];
+            s_l[u * kBlock + tid] = bmin;
+            s_h[u * kBlock + tid] = bmax;
+        }
+        __syncthreads();
+        const int32_t steps = (min(end - t0, kMidTile) + 31) / 32;
+        if (t0 + kMidTile < end) load(t0 + kMidTile);
+        if (warp < 2) {
+            const double *bb = warp == 0 ? s_l : s_h;
+#pragma unroll 4
+            for (int32_t t = 0; t < steps; t++) sum = fma(s_a[32 * t + lane], bb[32 * t + lane], sum);
+        }
+    }
+    nmin = __reduce_add_sync(0xffffffffu, nmin);
+    nmax = __reduce_add_sync(0xffffffffu, nmax);
+    if (rehash) h = group_sum<32>(h, 0xffffffffu);
+    if (warp < 2) sum = group_sum<32>(sum, 0xffffffffu);
+    if (lane == 0) {
+        if (nmin) atomicAdd(&M.nmin, nmin);
+        if (nmax) atomicAdd(&M.nmax, nmax);
+        if (rehash) atomicAdd(&M.h, h);
+        if (warp < 2) (warp == 0 ? M.smin : M.smax) = sum;
+    }
+    __syncthreads();
+    const double Lv = C.L[i], Uv = C.U[i];
+    if (tid == 0) {
+        uint8_t kind = RK_KEPT;
+        evaluated += end - beg;
+        removed += finish_row(C, i, beg, end - beg, Lv, Uv, M.smin, M.smax, M.nmin, M.nmax, rehash,
+                              M.h + len_hash(end - beg), kind);
+        M.kind = kind;
+    }
+    __syncthreads();
+    const double smin = M.smin, smax = M.smax;
+    const int rmin = M.nmin, rmax = M.nmax;
+    const bool kept = M.kind == RK_KEPT;
+    const bool up_row = kept && is_fin(Uv) && rmin <= 1, lo_row = kept && is_fin(Lv) && rmax <= 1;
+    if (up_row || lo_row)  // block-uniform
+        tighten_steps(C, q, (end - beg + kBlock - 1) / kBlock, beg + tid, kBlock, end, up_row, lo_row, Uv - smin,
+                      Lv - smax, slack_below(Uv, smin), slack_below(smax, Lv), rmin, rmax, tested);
+    __syncthreads();  // M is reused by the block's next row
+}
+
+// class of a block of k_prop_groups (its grid starts with class 5)
+__device__ __forceinline__ int prop_class(const GroupGrid &g, int b) { return 5 - grid_class(g, b); }
+
+__global__ void __launch_bounds__(kBlock, 4) k_prop_groups(Ctx C, GroupGrid g, int32_t per5) {
+    constexpr int kQ = (kBlock / 32) * kQueueCap;  // items of the warps' queues
+    __shared__ double s_q[3 * kQ];                 // coefficients, slacks, columns, flags
+    __shared__ MidShared s_m;
+    __shared__ int32_t s_mid[kBlock / 32];
+    __shared__ int32_t s_nmid;
     const int warp = threadIdx.x >> 5;
-    CandQueue q{s_qx[warp], s_qa[warp], s_qj[warp], s_qk[warp], 0};
-    TestQueue tq{s_ta[warp], s_ts[warp], s_tb[warp], s_to[warp], s_tj[warp], s_tf[warp], 0};
-    const int c = grid_class(g, blockIdx.x);
-    const int32_t lb = blockIdx.x - g.blk_start[c];
+    int32_t *s_qi = reinterpret_cast<int32_t *>(s_q + 2 * kQ);
+    CandQueue q{s_q + warp * kQueueCap, s_q + kQ + warp * kQueueCap, s_qi + warp * kQueueCap,
+                s_qi + kQ + warp * kQueueCap, 0};
+    const int c = prop_class(g, blockIdx.x);
+    const int32_t lb = blockIdx.x - g.blk_start[5 - c];
     int32_t removed = 0, evaluated = 0, tested = 0;
     const int W = prop_lanes(c);
-    const int32_t pos = C.A.cls_start[c] + lb * (kBlock / W) + threadIdx.x / W;
-    const bool valid = pos < C.A.cls_start[c + 1];
+    const int32_t per = c == 5 ? per5 : kBlock / W, at = threadIdx.x / W;
+    const int32_t pos = C.A.cls_start[c] + lb * per + at;
+    bool valid = at < per && pos < C.A.cls_start[c + 1];
     const int32_t i = valid ? C.A.order[pos] : 0;
-    switch (c) {
-        case 0:
-        case 1:
-        case 2: prop_group<1>(C, i, valid, removed, evaluated, tested, q, tq); break;
-        case 3: prop_group<8>(C, i, valid, removed, evaluated, tested, q, tq); break;
-        case 4: prop_group<16>(C, i, valid, removed, evaluated, tested, q, tq); break;
-        default: prop_group<32>(C, i, valid, removed, evaluated, tested, q, tq); break;
+    if (c < 5) {
+        prop_row<false>(C, i, valid, W, removed, evaluated, tested, q);
+    } else {
+        if (threadIdx.x == 0) s_nmid = 0;
+        __syncthreads();
+        if (valid && (C.rdirty[i] & kEval) && C.A.ptr[i + 1] - C.A.ptr[i] >= kMidMin) {
+            if ((threadIdx.x & 31) == 0) s_mid[atomicAdd(&s_nmid, 1)] = i;
+            valid = false;
+        }
+        prop_row<true>(C, i, valid, 32, removed, evaluated, tested, q);
+        __syncthreads();
+        const int32_t nmid = s_nmid;
+        for (int32_t t = 0; t < nmid; t++) prop_mid(C, s_mid[t], s_m, s_q, removed, evaluated, tested, q);
     }
-    tq_flush(C, tq, q);
     cq_flush(C, q);
-    block_add(removed, &C.st->rows_removed);
-    if (C.count_work) {  // statistics of a timed run only: each block_add is two block barriers
-        block_add(evaluated, &C.st->nnz_eval);
-        block_add(tested, &C.st->sides_tested);
+    warp_add(removed, &C.st->rows_removed);
+    if (C.count_work) {  // statistics of a timed run only
+        warp_add(evaluated, &C.st->nnz_eval);
+        warp_add(tested, &C.st->sides_tested);
     }
 }
 
@@ -81,8 +195,10 @@ __global__ void __launch_bounds__(kBlock) k_prop_long_partial(Ctx C, unsigned lo
     __shared__ int s_i[kBlock / 32];
     __shared__ unsigned long long s_h[kBlock / 32];
     const Chunk ch = C.A.chunks[blockIdx.x];
-    if (!C.rdirty[ch.seg]) return;  // block-uniform
-    const bool neg0 = is_neg(C.A.val[C.A.ptr[ch.seg]]);
+    const uint8_t flag = C.rdirty[ch.seg];
+    if (!flag) return;  // block-uniform
+    const bool rehash = flag & kRekey;
+    const bool neg0 = rehash ? is_neg(C.A.val[C.A.ptr[ch.seg]]) : false;
     double smin = 0.0, smax = 0.0;
     int nmin = 0, nmax = 0;
     unsigned long long h = 0;
@@ -97,13 +213,13 @@ __global__ void __launch_bounds__(kBlock) k_prop_long_partial(Ctx C, unsigned lo
         else nmin++;
         if (is_fin(bmax)) smax = fma(a, bmax, smax);
         else nmax++;
-        h += entry_hash(j, neg != neg0);
+        if (rehash) h += entry_hash(j, neg != neg0);
     }
     smin = block_reduce_ordered(smin, s_d);
     smax = block_reduce_ordered(smax, s_d);
     nmin = block_reduce_ordered(nmin, s_i);
     nmax = block_reduce_ordered(nmax, s_i);
-    h = block_reduce_ordered(h, s_h);
+    if (rehash) h = block_reduce_ordered(h, s_h);
     if (threadIdx.x == 0) {
         C.ch_act[blockIdx.x] = make_double2(smin, smax);
         C.ch_ninf[blockIdx.x] = make_int2(nmin, nmax);
@@ -119,7 +235,8 @@ __global__ void __launch_bounds__(kBlock) k_prop_long_combine(Ctx C, const unsig
     int32_t removed = 0, evaluated = 0;
     if (t < nlong) {  // the same t in the whole warp
         const int32_t i = C.A.order[C.A.cls_start[6] + t];
-        if (!C.rdirty[i]) {
+        const uint8_t flag = C.rdirty[i];
+        if (!flag) {
             if (lane == 0) {
                 C.rkind[i] = RK_KEPT;
                 C.lneed[t] = 0;
@@ -147,9 +264,7 @@ __global__ void __launch_bounds__(kBlock) k_prop_long_combine(Ctx C, const unsig
                 h += len_hash(len);
                 const double Lv = C.L[i], Uv = C.U[i];
                 uint8_t kind;
-                double sa = 0.0;
-                int32_t sj = -1;  // long rows are never singletons
-                removed = finish_row(C, i, beg, len, Lv, Uv, smin, smax, nmin, nmax, h, kind, sa, sj);
+                removed = finish_row(C, i, beg, len, Lv, Uv, smin, smax, nmin, nmax, flag & kRekey, h, kind);
                 evaluated = len;
                 C.lneed[t] = kind == RK_KEPT && ((is_fin(Uv) && nmin <= 1) || (is_fin(Lv) && nmax <= 1));
             }
@@ -168,9 +283,11 @@ __global__ void __launch_bounds__(kBlock) k_prop_long_tighten(Ctx C) {
     const int2 ni = C.ninf[i];
     const bool up_row = is_fin(Uv) && ni.x <= 1, lo_row = is_fin(Lv) && ni.y <= 1;
     const double dU = Uv - act.x, dL = Lv - act.y;
+    const float fU = slack_below(Uv, act.x), fL = slack_below(act.y, Lv);
     int32_t tested = 0;
+#pragma unroll 4
     for (int32_t k = ch.begin + threadIdx.x; k < ch.end; k += kBlock)
-        tighten_entry(C, C.A.idx[k], C.A.val[k], up_row, lo_row, dU, dL, ni.x, ni.y, tested);
+        tighten_entry(C, C.A.idx[k], C.A.val[k], up_row, lo_row, dU, dL, fU, fL, ni.x, ni.y, tested);
     block_add(tested, &C.st->sides_tested);  // the whole block returned above or reaches here
 }
 
@@ -595,15 +712,22 @@ inline unsigned blocks_for(int64_t cnt, int threads) {
 }  // namespace
 
 void launch_prop_short(const Ctx &C, cudaStream_t s) {
-    GroupGrid g;  // blocks per class at prop_lanes(c) lanes per row
+    // blocks per class at prop_lanes(c) lanes per row, the longest rows first
+    // (blk_start[k]: class 5 - k), so that their latency runs beside the short rows
+    GroupGrid g;
     int32_t acc = 0;
-    for (int c = 0; c < 6; c++) {
-        g.blk_start[c] = acc;
-        const int32_t per = kBlock / prop_lanes(c);
+    // rows of class 5 per block: a block takes its rows beyond 256 entries one
+    // after the other (about 6 us each), so as few as fill the chip
+    const int32_t cnt5 = C.A.cls_start[6] - C.A.cls_start[5];
+    const int32_t per5 = cnt5 <= 8 * 152 ? 1 : (cnt5 <= 32 * 152 ? 2 : 4);
+    for (int k = 0; k < 6; k++) {
+        const int c = 5 - k;
+        g.blk_start[k] = acc;
+        const int32_t per = c == 5 ? per5 : kBlock / prop_lanes(c);
         acc += (C.A.cls_start[c + 1] - C.A.cls_start[c] + per - 1) / per;
     }
     g.blk_start[6] = acc;
-    if (g.blk_start[6] > 0) (k_prop_groups<<<g.blk_start[6], kBlock, 0, s>>>(C, g), note_launch());
+    if (g.blk_start[6] > 0) (k_prop_groups<<<g.blk_start[6], kBlock, 0, s>>>(C, g, per5), note_launch());
 }
 
 bool prop_has_long(const Ctx &C) { return C.A.cls_start[7] > C.A.cls_start[6] && C.A.nchunks > 0; }

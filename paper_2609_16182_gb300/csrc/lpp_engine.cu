@@ -623,7 +623,7 @@ void Engine::prepare() {
     fill_u64(mL, m0, kEncNegInf, s);
     fill_u64(mU, m0, kEncPosInf, s);
     LPP_CUDA(cudaMemsetAsync(hasf, 0, (size_t)std::max(m0, 1), s));
-    LPP_CUDA(cudaMemsetAsync(rdirty[0], 1, (size_t)std::max(m0, 1), s));  // round 1 evaluates every row
+    LPP_CUDA(cudaMemsetAsync(rdirty[0], 3, (size_t)std::max(m0, 1), s));  // round 1 evaluates every row, keys and all
     LPP_CUDA(cudaMemsetAsync(rwork, 0, (size_t)std::max(m0, 1), s));
     fill_i32(verdict, (int64_t)nlp * V_SLOTS, kNone, s);
     LPP_CUDA(cudaMemsetAsync(rec_rk, 0, sizeof(int32_t) * (size_t)std::max(m0, 1), s));

@@ -61,7 +61,7 @@ __global__ void k_append(AppendArgs a) {
         if (i < a.m) {
             a.a_rmap[a.m0 + i] = a.rbase + (int32_t)i;
             a.a_lprow[a.m0 + i] = a.slot;
-            a.a_rdirty[a.m0 + i] = 1;
+            a.a_rdirty[a.m0 + i] = 3;  // kEval, kRekey
             a.rec_rk[a.rbase + i] = 0;
             a.rec_rr[a.rbase + i] = 0;
             a.rec_ra[a.rbase + i] = -1;

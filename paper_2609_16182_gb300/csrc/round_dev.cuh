@@ -45,6 +45,41 @@ __device__ __forceinline__ bool lt0(double s) {
 }
 __device__ __forceinline__ bool gt0(double s) { return dbits(s) > 0; }
 
+// ------------------------------------------------ S3 filter in single precision
+// An entry's implied bound can be accepted only if the row's slack is below
+// what the entry alone can span:  with x1 = dU + a bmin the sign tests of
+// pass_upper / pass_lower read  slack < |a| (u - l) - |a| bound_tol max(1, |old|)
+// in every case of sign and side (slack = U - smin or smax - L; an infinite
+// old bound or own term makes the span infinite).  The filter compares a lower
+// estimate of the slack with an upper estimate of |a| (u - l), taken from the
+// high words of the doubles in single precision, so it drops only entries
+// whose exact test fails: each estimate is off by at least 2^-21 of its
+// terms, the roundings of the exact test by at most a few 2^-53 of the same
+// terms.  It replaces, for nearly every entry, a queue trip with two FP64
+// instructions and two gathers by a few single-precision ones.
+// High words (sign bit cleared) to single precision: above / below |x|, by
+// at least 2^-21 |x|; then the same for signed values.
+__device__ __forceinline__ float f32_above(uint32_t hi) {
+    if (hi < (897u << 20)) return __uint_as_float(0x01000000u);  // |x| < 2^-126: 2^-125
+    if (hi >= (1151u << 20)) return __uint_as_float(0x7f800000u);
+    return __uint_as_float((hi << 3) - 0xc0000000u + 16u);
+}
+__device__ __forceinline__ float f32_below(uint32_t hi) {
+    if (hi < (898u << 20)) return 0.0f;
+    if (hi >= (1151u << 20)) return __uint_as_float(0x7f7fffffu);
+    return __uint_as_float((hi << 3) - 0xc0000000u - 16u);
+}
+__device__ __forceinline__ uint32_t hi_word(double x) { return (uint32_t)((unsigned long long)dbits(x) >> 32); }
+__device__ __forceinline__ float f32_hi(double x) {
+    const uint32_t h = hi_word(x), m = h & 0x7fffffffu;
+    return (int32_t)h < 0 ? -f32_below(m) : f32_above(m);
+}
+__device__ __forceinline__ float f32_lo(double x) {
+    const uint32_t h = hi_word(x), m = h & 0x7fffffffu;
+    return (int32_t)h < 0 ? -f32_above(m) : f32_below(m);
+}
+__device__ __forceinline__ float f32_mag(double x) { return f32_above(hi_word(x) & 0x7fffffffu); }
+
 // Implied upper bound x/a on column j (from a*x_j <= x with a > 0, or
 // a*x_j >= x with a < 0).  Accepted iff (uold = +inf or x/a < thr) and
 // |x/a| <= max_implied, thr = uold - bound_tol*max(1,|uold|) (one rounding).
@@ -52,12 +87,11 @@ __device__ __forceinline__ bool gt0(double s) { return dbits(s) > 0; }
 // fused multiply-add; the cap is tested only for candidates that pass.
 // A candidate that cannot lower the column's current minimum cur (x/a >= cur)
 // would not change the result: it is dropped by the same test, made against
-// min(cur, thr), and skips the divide.  pass_upper makes the sign test;
-// apply_cand the cap, the divide and the atomic.
-__device__ __forceinline__ bool pass_upper(const Ctx &C, int32_t j, double x, double a, double uold) {
+// min(cur, thr), and skips the divide.  pass_upper makes the sign test (e: cur,
+// encoded); apply_cand the cap, the divide and the atomic.
+__device__ __forceinline__ bool pass_upper(const Ctx &C, unsigned long long e, double x, double a, double uold) {
     // x/a must lie below both cur and thr: one test against min(cur, thr),
     // taken on the order-preserving encoding (integer pipes)
-    unsigned long long e = *((volatile unsigned long long *)&C.cand_u[j]);
     if (is_fin(uold)) {
         const unsigned long long et = enc_dbl(fma(-C.bound_tol, max1abs(uold), uold));
         e = et < e ? et : e;
@@ -69,8 +103,7 @@ __device__ __forceinline__ bool pass_upper(const Ctx &C, int32_t j, double x, do
 // Implied lower bound x/a: accepted iff (lold = -inf or x/a > thr) and
 // |x/a| <= max_implied, thr = lold + bound_tol*max(1,|lold|); a candidate
 // that cannot raise the current maximum is dropped with it.
-__device__ __forceinline__ bool pass_lower(const Ctx &C, int32_t j, double x, double a, double lold) {
-    unsigned long long e = *((volatile unsigned long long *)&C.cand_l[j]);
+__device__ __forceinline__ bool pass_lower(const Ctx &C, unsigned long long e, double x, double a, double lold) {
     if (is_fin(lold)) {
         const unsigned long long et = enc_dbl(fma(C.bound_tol, max1abs(lold), lold));
         e = et > e ? et : e;
@@ -81,174 +114,116 @@ __device__ __forceinline__ bool pass_lower(const Ctx &C, int32_t j, double x, do
 }
 
 // candidate kinds: implied bounds (capped) and singleton-row bounds (not)
-enum : int32_t { CQ_UPPER = 0, CQ_LOWER = 1, CQ_SING_UPPER = 2, CQ_SING_LOWER = 3 };
+enum : int32_t { CQ_UPPER = 0, CQ_LOWER = 1, CQ_SING_UPPER = 2, CQ_SING_LOWER = 3 };  // bit 0: a lower bound
 
-// the value x/a enters column j's candidates
-__device__ __forceinline__ void apply_cand(const Ctx &C, int32_t j, double x, double a, int32_t kind) {
-    if (kind < CQ_SING_UPPER && gt0(fma(-C.max_implied, fabs(a), fabs(x)))) return;
+// the value x/a enters column j's candidates; ec: the side's candidate as read
+// before (one that x/a does not improve on stands, whatever came since)
+__device__ __forceinline__ void apply_cand(const Ctx &C, int32_t j, double x, double a, int32_t kind,
+                                           unsigned long long ec) {
+    // |x / a| <= max_implied, exactly where single precision does not decide
+    if (kind < CQ_SING_UPPER) {
+        const float cap = __fmul_rd(f32_below(hi_word(C.max_implied)), f32_below(hi_word(a) & 0x7fffffffu));
+        if (!(f32_mag(x) <= cap) && gt0(fma(-C.max_implied, fabs(a), fabs(x)))) return;
+    }
     const double v = x / a;
     if (!is_fin(v)) return;
-    if (kind == CQ_UPPER || kind == CQ_SING_UPPER) atomic_min_dbl(&C.cand_u[j], v);
-    else atomic_max_dbl(&C.cand_l[j], v);
+    const unsigned long long e = enc_dbl(v);
+    if (kind == CQ_UPPER || kind == CQ_SING_UPPER) {
+        if (e < ec) atomicMin(&C.cand_u[j], e);
+    } else if (e > ec) {
+        atomicMax(&C.cand_l[j], e);
+    }
     touch_col(C, j);
 }
 
-// Sign tests of the two implied bounds of one entry (S3).  dU = U - smin and
-// dL = L - smax are the row's slacks: U - (min activity of the other
-// entries) = dU + a*bmin when every term is finite, = dU when this entry is
-// the one infinite term.  w1 / w2: a candidate x1/a (x2/a) of kind k1 (k2)
-// passed and still needs the cap and the divide.
-__device__ __forceinline__ void tighten_tests(const Ctx &C, int32_t j, double a, bool up_row, bool lo_row, double dU,
-                                              double dL, int nmin, int nmax, bool &w1, double &x1, int32_t &k1,
-                                              bool &w2, double &x2, int32_t &k2, int32_t &tested) {
+// above |a| (u - l)
+__device__ __forceinline__ float entry_span(double a, double2 b) {
+    const float w = __fsub_ru(f32_hi(b.y), f32_lo(b.x));
+    return __fmul_ru(f32_mag(a), w > 0.0f ? w : 0.0f);
+}
+// below the slack hi - lo of a row side
+__device__ __forceinline__ float slack_below(double hi, double lo) { return __fsub_rd(f32_lo(hi), f32_hi(lo)); }
+// may the exact test pass (a NaN span or slack passes)
+__device__ __forceinline__ bool span_passes(float slack, float span) { return !(slack >= span); }
+
+// one entry that passed the filter: the exact test of one of its sides.
+// flags: the candidate kind, | 4 if the entry's own term is finite (residual
+// = slack + a * bound, else the slack itself), | 8 for the lhs side
+enum : int32_t { CQ_OWN = 4, CQ_LHS = 8 };
+// First against the column's current candidate cur in single precision: x / a
+// improves on it only if  s + |a| (l - cur) < 0  (an upper bound; s the
+// positive slack, l the own term's bound, 0 if infinite) or  s + |a| (cur - u)
+// < 0  (a lower bound).  Most entries of a column that many rows hold fail
+// here, without an FP64 instruction.
+__device__ __forceinline__ void test_and_apply(const Ctx &C, double a, double slack, int32_t j, int32_t flags) {
+    const int32_t kind = flags & 3;
+    const bool upper = (kind & 1) == 0;
+    const unsigned long long ec = *((volatile unsigned long long *)(upper ? &C.cand_u[j] : &C.cand_l[j]));
+    double x = slack;
+    if (kind < CQ_SING_UPPER) {
+        const double2 b = C.lu[j];
+        const bool own = flags & CQ_OWN;
+        const double bnd = own ? (upper ? b.x : b.y) : 0.0;
+        if (ec != (upper ? kEncPosInf : kEncNegInf)) {
+            const double cur = dec_dbl(ec);
+            const float d = upper ? __fsub_rd(f32_lo(bnd), f32_hi(cur)) : __fsub_rd(f32_lo(cur), f32_hi(bnd));
+            const uint32_t ma = hi_word(a) & 0x7fffffffu;
+            const float s = (flags & CQ_LHS) ? -f32_hi(slack) : f32_lo(slack);
+            if (__fadd_rd(s, __fmul_rd(d >= 0.0f ? f32_below(ma) : f32_above(ma), d)) >= 0.0f) return;
+        }
+        if (own) x = fma(a, bnd, slack);
+        if (!(upper ? pass_upper(C, ec, x, a, b.y) : pass_lower(C, ec, x, a, b.x))) return;
+    }
+    apply_cand(C, j, x, a, kind, ec);
+}
+
+// flags of an entry side: the rhs side bounds x_j from above for a > 0, the
+// lhs side for a < 0
+__device__ __forceinline__ int32_t side_flags(bool neg, bool lhs, bool own_finite) {
+    return ((neg != lhs) ? CQ_LOWER : CQ_UPPER) | (own_finite ? CQ_OWN : 0) | (lhs ? CQ_LHS : 0);
+}
+
+// one entry, its candidates applied at once (long rows: few of them tighten)
+__device__ __forceinline__ void tighten_entry(const Ctx &C, int32_t j, double a, bool up_row, bool lo_row,
+                                              double dU, double dL, float fU, float fL, int nmin, int nmax,
+                                              int32_t &tested) {
     const double2 b = C.lu[j];
     const bool neg = is_neg(a);
-    const double bmin = neg ? b.y : b.x, bmax = neg ? b.x : b.y;
-    const bool fmn = is_fin(bmin), fmx = is_fin(bmax);
-    if (up_row && (fmn ? nmin == 0 : nmin == 1)) {
-        // a x_j <= U - (min activity of the other entries)
-        tested++;
-        x1 = fmn ? fma(a, bmin, dU) : dU;
-        if (!neg) {
-            k1 = CQ_UPPER;
-            w1 = pass_upper(C, j, x1, a, b.y);
-        } else {
-            k1 = CQ_LOWER;
-            w1 = pass_lower(C, j, x1, a, b.x);
-        }
-    }
-    if (lo_row && (fmx ? nmax == 0 : nmax == 1)) {
-        // a x_j >= L - (max activity of the other entries)
-        tested++;
-        x2 = fmx ? fma(a, bmax, dL) : dL;
-        if (!neg) {
-            k2 = CQ_LOWER;
-            w2 = pass_lower(C, j, x2, a, b.x);
-        } else {
-            k2 = CQ_UPPER;
-            w2 = pass_upper(C, j, x2, a, b.y);
-        }
-    }
+    const bool fmn = is_fin(neg ? b.y : b.x), fmx = is_fin(neg ? b.x : b.y);
+    const bool w1 = up_row && (fmn ? nmin == 0 : nmin == 1), w2 = lo_row && (fmx ? nmax == 0 : nmax == 1);
+    tested += (w1 ? 1 : 0) + (w2 ? 1 : 0);
+    const float span = entry_span(a, b);
+    if (w1 && span_passes(fU, span)) test_and_apply(C, a, dU, j, side_flags(neg, false, fmn));
+    if (w2 && span_passes(fL, span)) test_and_apply(C, a, dL, j, side_flags(neg, true, fmx));
 }
 
-// one entry, candidates applied at once (long rows: few of them tighten)
-__device__ __forceinline__ void tighten_entry(const Ctx &C, int32_t j, double a, bool up_row, bool lo_row,
-                                              double dU, double dL, int nmin, int nmax, int32_t &tested) {
-    bool w1 = false, w2 = false;
-    double x1 = 0.0, x2 = 0.0;
-    int32_t k1 = 0, k2 = 0;
-    tighten_tests(C, j, a, up_row, lo_row, dU, dL, nmin, nmax, w1, x1, k1, w2, x2, k2, tested);
-    if (w1) apply_cand(C, j, x1, a, k1);
-    if (w2) apply_cand(C, j, x2, a, k2);
-}
-
-// Per-warp queue of candidates that passed their sign tests.  The divide
-// (and the cap, the atomic) then runs 32 candidates at a time, one per lane,
-// instead of on the one or two lanes of a warp that produced a candidate in
-// a step: on GB300 an FP64 instruction costs the pipe the same however many
-// lanes are active.  Every lane of the warp must call cq_push / cq_flush.
+// Per-warp queue of the entry sides that passed the filter (and of the
+// singleton rows' bounds).  The exact test, the divide, the cap and the
+// atomic then run 32 at a time, one per lane, instead of on the one or two
+// lanes of a warp that have one in a step: on GB300 an FP64 instruction
+// costs the pipe the same however many lanes are active.  Every lane of the
+// warp must call cq_push / cq_flush.  1.5 KB per warp: shared memory is taken
+// from the L1, whose lines hold the bound gathers in flight.
 struct CandQueue {
-    double *x, *a;
-    int32_t *j, *kind;
+    double *a, *slack;
+    int32_t *j, *flags;
     int32_t n;  // items held, the same in every lane
 };
 constexpr int kQueueCap = 64;
 
-__device__ __forceinline__ void cq_push(const Ctx &C, CandQueue &q, bool want, double x, double a, int32_t j,
-                                        int32_t kind) {
-    const unsigned b = __ballot_sync(0xffffffffu, want);
-    if (b == 0u) return;
+// the first cnt <= 32 items, one per lane; the rest move up
+__device__ __forceinline__ void cq_run(const Ctx &C, CandQueue &q, int32_t cnt) {
     const int lane = threadIdx.x & 31;
-    if (want) {
-        const int32_t p = q.n + __popc(b & ((1u << lane) - 1u));
-        q.x[p] = x;
-        q.a[p] = a;
-        q.j[p] = j;
-        q.kind[p] = kind;
-    }
-    q.n += __popc(b);
-    if (q.n < 32) return;
     __syncwarp();
-    apply_cand(C, q.j[lane], q.x[lane], q.a[lane], q.kind[lane]);
-    const int32_t rest = q.n - 32;
-    double rx = 0.0, ra = 0.0;
-    int32_t rj = 0, rk = 0;
-    if (lane < rest) {
-        rx = q.x[32 + lane];
-        ra = q.a[32 + lane];
-        rj = q.j[32 + lane];
-        rk = q.kind[32 + lane];
-    }
-    __syncwarp();
-    if (lane < rest) {
-        q.x[lane] = rx;
-        q.a[lane] = ra;
-        q.j[lane] = rj;
-        q.kind[lane] = rk;
-    }
-    __syncwarp();
-    q.n = rest;
-}
-
-__device__ __forceinline__ void cq_flush(const Ctx &C, CandQueue &q) {
-    __syncwarp();
-    const int lane = threadIdx.x & 31;
-    if (lane < q.n) apply_cand(C, q.j[lane], q.x[lane], q.a[lane], q.kind[lane]);
-    q.n = 0;
-}
-
-// Per-warp queue of S3 tests: an entry side that qualifies (its row slack
-// finite, the other terms finite or it the one infinite term) is queued
-// with its coefficient a, the row slack, the bound of its own term and the
-// bound it would tighten; the residual, the threshold and the sign test (the
-// FP64 work) then run 32 tests at a time, and the passing candidates go on
-// to the candidate queue.  flags: the candidate kind, | 4 if the entry's own
-// term is finite (residual = slack + a * bnd, else the slack itself).
-struct TestQueue {
-    double *a, *slack, *bnd, *bold;
-    int32_t *j, *flags;
-    int32_t n;
-};
-
-__device__ __forceinline__ void tq_run(const Ctx &C, CandQueue &cq, bool have, double a, double slack, double bnd,
-                                       double bold, int32_t j, int32_t flags) {
-    bool w = false;
-    double x = 0.0;
-    const int32_t kind = flags & 3;
-    if (have) {
-        x = (flags & 4) ? fma(a, bnd, slack) : slack;
-        w = kind == CQ_UPPER ? pass_upper(C, j, x, a, bold) : pass_lower(C, j, x, a, bold);
-    }
-    cq_push(C, cq, w, x, a, j, kind);
-}
-
-__device__ __forceinline__ void tq_push(const Ctx &C, TestQueue &q, CandQueue &cq, bool want, double a, double slack,
-                                        double bnd, double bold, int32_t j, int32_t flags) {
-    const unsigned b = __ballot_sync(0xffffffffu, want);
-    if (b == 0u) return;
-    const int lane = threadIdx.x & 31;
-    if (want) {
-        const int32_t p = q.n + __popc(b & ((1u << lane) - 1u));
-        q.a[p] = a;
-        q.slack[p] = slack;
-        q.bnd[p] = bnd;
-        q.bold[p] = bold;
-        q.j[p] = j;
-        q.flags[p] = flags;
-    }
-    q.n += __popc(b);
-    if (q.n < 32) return;
-    __syncwarp();
-    const double ia = q.a[lane], isl = q.slack[lane], ibn = q.bnd[lane], ibo = q.bold[lane];
-    const int32_t ij = q.j[lane], ifl = q.flags[lane];
-    const int32_t rest = q.n - 32;
-    double ra = 0.0, rs = 0.0, rb = 0.0, ro = 0.0;
+    const bool have = lane < cnt;
+    const double ia = have ? q.a[lane] : 0.0, is = have ? q.slack[lane] : 0.0;
+    const int32_t ij = have ? q.j[lane] : 0, ifl = have ? q.flags[lane] : 0;
+    const int32_t rest = q.n - cnt;
+    double ra = 0.0, rs = 0.0;
     int32_t rj = 0, rf = 0;
     if (lane < rest) {
         ra = q.a[32 + lane];
         rs = q.slack[32 + lane];
-        rb = q.bnd[32 + lane];
-        ro = q.bold[32 + lane];
         rj = q.j[32 + lane];
         rf = q.flags[32 + lane];
     }
@@ -256,33 +231,33 @@ __device__ __forceinline__ void tq_push(const Ctx &C, TestQueue &q, CandQueue &c
     if (lane < rest) {
         q.a[lane] = ra;
         q.slack[lane] = rs;
-        q.bnd[lane] = rb;
-        q.bold[lane] = ro;
         q.j[lane] = rj;
         q.flags[lane] = rf;
     }
     __syncwarp();
     q.n = rest;
-    tq_run(C, cq, true, ia, isl, ibn, ibo, ij, ifl);
+    if (have) test_and_apply(C, ia, is, ij, ifl);
 }
 
-__device__ __forceinline__ void tq_flush(const Ctx &C, TestQueue &q, CandQueue &cq) {
-    __syncwarp();
+__device__ __forceinline__ void cq_push(const Ctx &C, CandQueue &q, bool want, double a, double slack, int32_t j,
+                                        int32_t flags) {
+    const unsigned b = __ballot_sync(0xffffffffu, want);
+    if (b == 0u) return;
     const int lane = threadIdx.x & 31;
-    const bool have = lane < q.n;
-    double ia = 0.0, isl = 0.0, ibn = 0.0, ibo = 0.0;
-    int32_t ij = 0, ifl = 0;
-    if (have) {
-        ia = q.a[lane];
-        isl = q.slack[lane];
-        ibn = q.bnd[lane];
-        ibo = q.bold[lane];
-        ij = q.j[lane];
-        ifl = q.flags[lane];
+    if (want) {
+        const int32_t p = q.n + __popc(b & ((1u << lane) - 1u));
+        q.a[p] = a;
+        q.slack[p] = slack;
+        q.j[p] = j;
+        q.flags[p] = flags;
     }
-    __syncwarp();
-    q.n = 0;
-    tq_run(C, cq, have, ia, isl, ibn, ibo, ij, ifl);
+    q.n += __popc(b);
+    if (q.n < 32) return;
+    cq_run(C, q, 32);
+}
+
+__device__ __forceinline__ void cq_flush(const Ctx &C, CandQueue &q) {
+    if (q.n > 0) cq_run(C, q, q.n);
 }
 
 // S2: class of a row from its activities, first match wins: infeasible
@@ -296,27 +271,43 @@ __device__ __forceinline__ long long dkey(double x) {
     return b >= 0 ? b : (b ^ 0x7fffffffffffffffLL);
 }
 
+// The FP64 sums U + delta(U), L - delta(L) (delta(x) = feas_tol max(1, |x|))
+// are formed only where the comparison with U or L itself, or their
+// single-precision estimates, does not decide: a row's classification then
+// costs no FP64 instruction in nearly every case.
 __device__ __forceinline__ bool classify(const Ctx &C, double Lv, double Uv, int32_t len, double smin, double smax,
                                          int nmin, int nmax, uint8_t &kind) {
     const double ft = C.feas_tol;
     const bool Lf = is_fin(Lv), Uf = is_fin(Uv);
     kind = RK_KEPT;
-    const double mL = max1abs(Lv), mU = max1abs(Uv);  // >= 1: their bits order like their values
-    if (Lf && Uf) {
-        const double d = ft * (dbits(mL) > dbits(mU) ? mL : mU);
-        if (dkey(Lv - Uv) > dkey(d)) return false;
+    const long long kL = dkey(Lv), kU = dkey(Uv), ksmin = dkey(smin), ksmax = dkey(smax);
+    if (Lf && Uf && kL > kU) {
+        const double mL = max1abs(Lv), mU = max1abs(Uv);  // >= 1: their bits order like their values
+        if (dkey(Lv - Uv) > dkey(ft * (dbits(mL) > dbits(mU) ? mL : mU))) return false;
     }
-    const double uhi = Uv + ft * mU, llo = Lv - ft * mL;  // U + delta(U), L - delta(L)
-    const long long ksmin = dkey(smin), ksmax = dkey(smax);
-    if (nmin == 0 && Uf && ksmin > dkey(uhi)) return false;
-    if (nmax == 0 && Lf && ksmax < dkey(llo)) return false;
+    if (nmin == 0 && Uf && ksmin > kU && ksmin > dkey(Uv + ft * max1abs(Uv))) return false;
+    if (nmax == 0 && Lf && ksmax < kL && ksmax < dkey(Lv - ft * max1abs(Lv))) return false;
     if (len == 0) {
         kind = RK_EMPTY;
         return true;
     }
-    const bool lo_ok = !Lf || (nmin == 0 && ksmin >= dkey(llo));
+    bool lo_ok = !Lf;
+    if (Lf && nmin == 0) {
+        lo_ok = ksmin >= kL;
+        if (!lo_ok) {
+            const float d = __fmul_ru(f32_mag(ft), f32_mag(max1abs(Lv)));
+            if (!(f32_hi(smin) < __fsub_rd(f32_lo(Lv), d))) lo_ok = ksmin >= dkey(Lv - ft * max1abs(Lv));
+        }
+    }
     if (lo_ok) {
-        const bool hi_ok = !Uf || (nmax == 0 && ksmax <= dkey(uhi));
+        bool hi_ok = !Uf;
+        if (Uf && nmax == 0) {
+            hi_ok = ksmax <= kU;
+            if (!hi_ok) {
+                const float d = __fmul_ru(f32_mag(ft), f32_mag(max1abs(Uv)));
+                if (!(f32_lo(smax) > __fadd_ru(f32_hi(Uv), d))) hi_ok = ksmax <= dkey(Uv + ft * max1abs(Uv));
+            }
+        }
         if (hi_ok) {
             kind = RK_REDUNDANT;
             return true;
@@ -327,15 +318,15 @@ __device__ __forceinline__ bool classify(const Ctx &C, double Lv, double Uv, int
 }
 
 
-// writes the row's S1/S2 results and records; a singleton row returns its
-// entry (sa, sj) for the caller to apply as bounds L/a, U/a
+// writes the row's S1/S2 results and records (a singleton row's bounds L/a,
+// U/a are the caller's to apply)
 __device__ __forceinline__ int32_t finish_row(const Ctx &C, int32_t i, int32_t beg, int32_t len, double Lv,
                                               double Uv, double smin, double smax, int nmin, int nmax,
-                                              unsigned long long h, uint8_t &kind, double &sa, int32_t &sj) {
+                                              bool rehash, unsigned long long h, uint8_t &kind) {
     const bool ok = classify(C, Lv, Uv, len, smin, smax, nmin, nmax, kind);
     C.act[i] = make_double2(smin, smax);
     C.ninf[i] = make_int2(nmin, nmax);
-    C.hrow[i] = h;
+    if (rehash) C.hrow[i] = h;  // else the key stands: the row's entries did not change
     const int32_t lp = lp_of_row(C, i);
     if (!ok) {
         atomicMin(&C.verdict[lp * V_SLOTS + V_S2_ROW], C.rmap[i]);
@@ -350,11 +341,8 @@ __device__ __forceinline__ int32_t finish_row(const Ctx &C, int32_t i, int32_t b
     C.rec_rr[o] = lp_round(C, lp);
     mark_lp_changed(C, lp);
     if (kind == RK_SINGLETON) {
-        // L <= a x_j <= U becomes a bound on x_j, always applied (no threshold)
-        sa = C.A.val[beg];
-        sj = C.A.idx[beg];
-        C.rec_ra[o] = C.cmap[sj];
-        C.rec_rv[o] = sa;
+        C.rec_ra[o] = C.cmap[C.A.idx[beg]];
+        C.rec_rv[o] = C.A.val[beg];
     } else {
         C.rec_ra[o] = -1;
         C.rec_rv[o] = 0.0;
@@ -362,127 +350,216 @@ __device__ __forceinline__ int32_t finish_row(const Ctx &C, int32_t i, int32_t b
     return 1;
 }
 
+// Queues the entry sides of a lane in todo: bit c the rhs side of entry k0 + c
+// stride, bit 16 + c its lhs side (the whole warp together).
+__device__ __forceinline__ void push_sides(const Ctx &C, CandQueue &q, unsigned todo, int32_t k0, int32_t stride,
+                                           double dU, double dL, unsigned imin, unsigned imax, bool sing) {
+    const int T = (int)__reduce_max_sync(0xffffffffu, (unsigned)__popc(todo));
+    for (int t = 0; t < T; t++) {
+        const bool want = todo != 0u;
+        const int bit = want ? __ffs(todo) - 1 : 0;
+        todo &= todo - 1u;
+        const bool lhs = bit >= 16;
+        int32_t j = 0;
+        double a = 0.0;
+        if (want) {
+            const int32_t k = k0 + (bit & 15) * stride;
+            j = C.A.idx[k];
+            a = C.A.val[k];
+        }
+        const bool own = !(((lhs ? imax : imin) >> (bit & 15)) & 1u);
+        int32_t f = side_flags(is_neg(a), lhs, own);
+        if (sing) f = (f & 1) | CQ_SING_UPPER;  // the row's side itself, untested
+        cq_push(C, q, want, a, lhs ? dL : dU, j, f);
+    }
+}
+
+// S3 over the entries k0, k0 + stride, .. below end of a lane (none if end <=
+// k0), T steps for the whole warp, four entries in flight: the entry sides
+// that pass the filter are queued.
+__device__ __forceinline__ void tighten_steps(const Ctx &C, CandQueue &q, int32_t T, int32_t k0, int32_t stride,
+                                              int32_t end, bool up_row, bool lo_row, double dU, double dL, float fU,
+                                              float fL, int nmin, int nmax, int32_t &tested) {
+    for (int32_t it = 0; it < T; it += 4, k0 += 4 * stride) {
+        int32_t j[4];
+        double a[4];
+        double2 b[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            const int32_t k = k0 + u * stride;
+            j[u] = k < end ? C.A.idx[k] : -1;
+            a[u] = k < end ? C.A.val[k] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; u++) b[u] = j[u] >= 0 ? C.lu[j[u]] : make_double2(0.0, 0.0);
+        unsigned todo = 0, imin = 0, imax = 0;
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            const bool neg = is_neg(a[u]), in = j[u] >= 0;
+            const bool fmn = is_fin(neg ? b[u].y : b[u].x), fmx = is_fin(neg ? b[u].x : b[u].y);
+            const bool w1 = in && up_row && (fmn ? nmin == 0 : nmin == 1);
+            const bool w2 = in && lo_row && (fmx ? nmax == 0 : nmax == 1);
+            tested += (w1 ? 1 : 0) + (w2 ? 1 : 0);
+            const float span = entry_span(a[u], b[u]);
+            imin |= (unsigned)!fmn << u;
+            imax |= (unsigned)!fmx << u;
+            todo |= (unsigned)(w1 && span_passes(fU, span)) << u | (unsigned)(w2 && span_passes(fL, span)) << (16 + u);
+        }
+        push_sides(C, q, todo, k0, stride, dU, dL, imin, imax, false);
+    }
+}
+
 // ------------------------------------------------------- S1 + S2 + S3 groups
-template <int W>
-__device__ __forceinline__ void prop_group(const Ctx &C, int32_t i, bool valid, int32_t &removed, int32_t &evaluated,
-                                           int32_t &tested, CandQueue &q, TestQueue &tq) {
-    const unsigned mask = group_mask<W>();
-    const int lane = threadIdx.x & (W - 1);
-    // A row none of whose bounds, entries or sides changed since its last
-    // evaluation has the same activities and class (kept) and yields the same
-    // implied bounds, which were then already applied or rejected: skip it
-    // (its lanes stay for the warp's queue steps).  Flag 2: such a row whose
-    // columns were renumbered by a compaction since; only its S5 key, which
-    // hashes the column indices, is taken again (no bound gathers).
+// Dirty flags of a row (rdirty): kEval, its activities must be taken again (a
+// bound in it, its entries or its sides changed), kRekey, its S5 key (its
+// entries changed, or the columns were renumbered).  A row without kEval has
+// the same activities and class (kept) and yields the same implied bounds,
+// which were then already applied or rejected.
+enum : uint8_t { kEval = 1, kRekey = 2 };
+
+// xor butterfly over W lanes, W at run time: every lane ends with the same bits
+template <typename T>
+__device__ __forceinline__ T lanes_sum(T v, int W, unsigned mask) {
+    for (int o = W / 2; o > 0; o >>= 1) v += __shfl_xor_sync(mask, v, o);
+    return v;
+}
+
+// S1-S3 of row i by W lanes.  LONG: a warp (W = 32) per row of any length, S3
+// walks the row again.  Else W = 1, 2 or 4 with at most 16 entries per lane,
+// whose spans stay in registers for S3, so that S3 reads only the entries that
+// pass the filter again.
+template <bool LONG>
+__device__ __forceinline__ void prop_row(const Ctx &C, int32_t i, bool valid, int W, int32_t &removed,
+                                         int32_t &evaluated, int32_t &tested, CandQueue &q) {
+    if constexpr (LONG) W = 32;
+    const int wl = threadIdx.x & 31, lane = wl & (W - 1);
+    const unsigned mask = LONG ? 0xffffffffu : ((1u << W) - 1u) << (wl & ~(W - 1));
     const uint8_t flag = valid ? C.rdirty[i] : 0;
-    const bool act = flag == 1, rehash = flag == 2;
+    const bool act = flag & kEval, rehash = flag & kRekey;
     if (valid && !act && lane == 0) C.rkind[i] = RK_KEPT;
     int32_t beg = 0, end = 0;
-    if (act || rehash) {
+    if (flag) {
         beg = C.A.ptr[i];
         end = C.A.ptr[i + 1];
     }
-    const bool neg0 = end > beg ? is_neg(C.A.val[beg]) : false;
+    const bool neg0 = rehash && end > beg ? is_neg(C.A.val[beg]) : false;
     double smin = 0.0, smax = 0.0;
     int nmin = 0, nmax = 0;
     unsigned long long h = 0;
+    float span[LONG ? 1 : 16];
+    unsigned imin = 0, imax = 0;  // entries with an infinite term
     // The lane's entries in steps of four, the tail of a step predicated: the
     // four bound gathers of a step overlap, and a warp whose lanes hold rows of
     // different lengths runs no separate remainder loop (which would issue
     // its FP64 work a second time for the lanes still in it).  The sums take
     // the entries in the same order as a plain loop.
-    for (int32_t k0 = beg + lane; k0 < end; k0 += 4 * W) {
+    auto step = [&](int32_t k0, int c4) {
         int32_t jq[4];
         double aq[4];
         double2 bq[4];
 #pragma unroll
-        for (int q = 0; q < 4; q++) {
-            const int32_t k = k0 + q * W;
-            jq[q] = k < end ? C.A.idx[k] : 0;
-            aq[q] = k < end ? C.A.val[k] : 0.0;
+        for (int e = 0; e < 4; e++) {
+            const int32_t k = k0 + e * W;
+            jq[e] = k < end ? C.A.idx[k] : 0;
+            aq[e] = k < end ? C.A.val[k] : 0.0;
         }
 #pragma unroll
-        for (int q = 0; q < 4; q++) bq[q] = act && k0 + q * W < end ? C.lu[jq[q]] : make_double2(0.0, 0.0);
+        for (int e = 0; e < 4; e++) bq[e] = act && k0 + e * W < end ? C.lu[jq[e]] : make_double2(0.0, 0.0);
 #pragma unroll
-        for (int q = 0; q < 4; q++) {
-            if (k0 + q * W >= end) break;
-            const double a = aq[q];
-            const double2 b = bq[q];
-            const bool neg = is_neg(a);
-            const double bmin = neg ? b.y : b.x, bmax = neg ? b.x : b.y;
-            if (is_fin(bmin)) smin = fma(a, bmin, smin);
-            else nmin++;
-            if (is_fin(bmax)) smax = fma(a, bmax, smax);
-            else nmax++;
-            h += entry_hash(jq[q], neg != neg0);
-        }
-    }
-    smin = group_sum<W>(smin, mask);
-    smax = group_sum<W>(smax, mask);
-    nmin = group_sum<W>(nmin, mask);
-    nmax = group_sum<W>(nmax, mask);
-    h = group_sum<W>(h, mask);
-    const int32_t len = end - beg;
-    if (rehash && lane == 0) C.hrow[i] = h + len_hash(len);
-    bool up_row = false, lo_row = false;
-    double dU = 0.0, dL = 0.0, Lv = 0.0, Uv = 0.0, sa = 0.0;
-    int32_t sj = -1;
-    if (act) {
-        h += len_hash(len);
-        if (lane == 0) evaluated += len;
-        Lv = C.L[i];
-        Uv = C.U[i];
-        uint8_t kind = RK_KEPT;
-        if (lane == 0) removed += finish_row(C, i, beg, len, Lv, Uv, smin, smax, nmin, nmax, h, kind, sa, sj);
-        kind = (uint8_t)__shfl_sync(mask, (int)kind, 0, W);
-        if (kind == RK_KEPT && len >= 2) {
-            up_row = is_fin(Uv) && nmin <= 1;
-            lo_row = is_fin(Lv) && nmax <= 1;
-            dU = Uv - smin;
-            dL = Lv - smax;
-        }
-    }
-    // a singleton row's bounds L/a and U/a (a < 0 swaps them)
-    const bool sing = sj >= 0, sneg = is_neg(sa);
-    cq_push(C, q, sing && is_fin(Lv), Lv, sa, sj, sneg ? CQ_SING_UPPER : CQ_SING_LOWER);
-    cq_push(C, q, sing && is_fin(Uv), Uv, sa, sj, sneg ? CQ_SING_LOWER : CQ_SING_UPPER);
-    // S3 over the row's entries, in steps the whole warp takes together
-    const int32_t trips = (up_row || lo_row) && lane < len ? (len - lane + W - 1) / W : 0;
-    const int32_t T = (int32_t)__reduce_max_sync(0xffffffffu, (unsigned)trips);
-    for (int32_t it = 0; it < T; it++) {
-        bool w1 = false, w2 = false;
-        double a = 0.0, bn1 = 0.0, bn2 = 0.0, bo1 = 0.0, bo2 = 0.0;
-        int32_t j = 0, f1 = 0, f2 = 0;
-        if (it < trips) {
-            const int32_t k = beg + lane + it * W;
-            j = C.A.idx[k];
-            a = C.A.val[k];
-            const double2 b = C.lu[j];
+        for (int e = 0; e < 4; e++) {
+            if (k0 + e * W >= end) break;
+            const double a = aq[e];
+            const double2 b = bq[e];
             const bool neg = is_neg(a);
             const double bmin = neg ? b.y : b.x, bmax = neg ? b.x : b.y;
             const bool fmn = is_fin(bmin), fmx = is_fin(bmax);
-            if (up_row && (fmn ? nmin == 0 : nmin == 1)) {  // a x_j <= U - (min activity of the others)
-                w1 = true;
-                bn1 = bmin;
-                bo1 = neg ? b.x : b.y;
-                f1 = (neg ? CQ_LOWER : CQ_UPPER) | (fmn ? 4 : 0);
+            if (fmn) smin = fma(a, bmin, smin);
+            else nmin++;
+            if (fmx) smax = fma(a, bmax, smax);
+            else nmax++;
+            if constexpr (!LONG) {
+                imin |= (unsigned)!fmn << (c4 + e);
+                imax |= (unsigned)!fmx << (c4 + e);
+                span[c4 + e] = entry_span(a, b);
             }
-            if (lo_row && (fmx ? nmax == 0 : nmax == 1)) {  // a x_j >= L - (max activity of the others)
-                w2 = true;
-                bn2 = bmax;
-                bo2 = neg ? b.y : b.x;
-                f2 = (neg ? CQ_UPPER : CQ_LOWER) | (fmx ? 4 : 0);
-            }
-            tested += (w1 ? 1 : 0) + (w2 ? 1 : 0);
+            if (rehash) h += entry_hash(jq[e], neg != neg0);
         }
-        tq_push(C, tq, q, w1, a, dU, bn1, bo1, j, f1);
-        tq_push(C, tq, q, w2, a, dL, bn2, bo2, j, f2);
+    };
+    if constexpr (LONG) {
+        for (int32_t k0 = beg + lane; k0 < end; k0 += 4 * W) step(k0, 0);
+    } else {
+#pragma unroll
+        for (int c = 0; c < 4; c++)
+            if (beg + lane + 4 * c * W < end) step(beg + lane + 4 * c * W, 4 * c);
+    }
+    if (W > 1) {  // the same W in the whole warp
+        smin = lanes_sum(smin, W, mask);
+        smax = lanes_sum(smax, W, mask);
+        nmin = lanes_sum(nmin, W, mask);
+        nmax = lanes_sum(nmax, W, mask);
+        if (__any_sync(0xffffffffu, rehash)) h = lanes_sum(h, W, mask);
+    }
+    const int32_t len = end - beg;
+    h += len_hash(len);
+    if (rehash && !act && lane == 0) C.hrow[i] = h;
+    bool up_row = false, lo_row = false;
+    double Lv = 0.0, Uv = 0.0;
+    int32_t kind = RK_KEPT;
+    bool sing = false;
+    if (act) {
+        if (lane == 0) evaluated += len;
+        Lv = C.L[i];
+        Uv = C.U[i];
+        if (lane == 0) {
+            uint8_t k = RK_KEPT;
+            removed += finish_row(C, i, beg, len, Lv, Uv, smin, smax, nmin, nmax, rehash, h, k);
+            kind = k;
+        }
+        if (W > 1) kind = __shfl_sync(mask, kind, wl & ~(W - 1));
+        if (kind == RK_KEPT && len >= 2) {
+            up_row = is_fin(Uv) && nmin <= 1;
+            lo_row = is_fin(Lv) && nmax <= 1;
+        }
+        sing = kind == RK_SINGLETON && lane == 0;
+    }
+    // S3 over the row's entries, in steps the whole warp takes together
+    const float fU = slack_below(Uv, smin), fL = slack_below(smax, Lv);
+    if constexpr (!LONG) {
+        // a x_j <= U - (min activity of the others): every entry when no term
+        // is infinite, the one infinite term alone when there is one
+        const int nq = lane < len ? (len - lane + W - 1) / W : 0;
+        const unsigned all = (1u << nq) - 1u;
+        const unsigned q1 = up_row ? (nmin == 0 ? all : imin) : 0u, q2 = lo_row ? (nmax == 0 ? all : imax) : 0u;
+        tested += __popc(q1) + __popc(q2);
+        unsigned todo = 0;
+        if (q1 | q2) {
+#pragma unroll
+            for (int c = 0; c < 4; c++) {
+                if (nq <= 4 * c) break;
+#pragma unroll
+                for (int e = 4 * c; e < 4 * c + 4; e++)
+                    todo |= (unsigned)span_passes(fU, span[e]) << e | (unsigned)span_passes(fL, span[e]) << (16 + e);
+            }
+            todo &= q1 | (q2 << 16);
+        }
+        // a singleton row L <= a x_j <= U becomes the bounds L/a and U/a, always
+        // applied (no threshold)
+        if (sing) todo = (is_fin(Uv) ? 1u : 0u) | (is_fin(Lv) ? 1u << 16 : 0u);
+        if (__any_sync(0xffffffffu, todo != 0u))  // the slacks are formed only when an entry needs them
+            push_sides(C, q, todo, beg + lane, W, sing ? Uv : Uv - smin, sing ? Lv : Lv - smax, imin, imax, sing);
+    } else {
+        const int32_t trips = (up_row || lo_row) && lane < len ? (len - lane + W - 1) / W : 0;
+        const int32_t T = (int32_t)__reduce_max_sync(0xffffffffu, (unsigned)trips);
+        tighten_steps(C, q, T, beg + lane, W, (up_row || lo_row) ? end : beg, up_row, lo_row, Uv - smin, Lv - smax, fU,
+                      fL, nmin, nmax, tested);
     }
 }
 
-// Lanes per row in S1-S3: one thread per row up to 16 entries (the row's
-// classification then runs on every lane of the warp), else the class width.
-__host__ __device__ __forceinline__ int prop_lanes(int c) { return c <= 2 ? 1 : 1 << c; }
+// Lanes per row in S1-S3: a lane holds up to 16 entries (rows up to 16, 32 and
+// 64 entries: 1, 2, 4 lanes), longer rows take a warp.  Fewer lanes per row
+// cost fewer butterfly steps, each two FP64 instructions: 8 lanes for 17 to
+// 32 entries cost 3.5 FP64 warp instructions a row, 2 lanes 2.1.
+__host__ __device__ __forceinline__ int prop_lanes(int c) { return c <= 2 ? 1 : (c == 5 ? 32 : 1 << (c - 2)); }
 
 // ------------------------------------------------- S3' finalise + S4 fixing
 // S3' + S4 on column j: apply the accepted candidates, check and snap the
