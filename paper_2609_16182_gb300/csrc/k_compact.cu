@@ -180,28 +180,180 @@ __global__ void __launch_bounds__(kBlock) k_locks_long(Ctx C, CompactCtx K) {
 }
 
 // ------------------------------------------------------- S6 + column keep
-// With the input CSC kept (Ctx::t_orig) the columns also stay in place: a
-// column that left in an earlier round (cinv < 0) is skipped, the others
-// keep their index (c_new = j), and one that leaves now gets cinv = -1.
 // (grid-stride over a grid of at most 8 blocks per SM: one block sum per block)
+// Columns in place (Ctx::in_place): a column that left in an earlier round
+// (cinv < 0) is skipped, a kept one with entries stays as it is (no S6 test
+// applies to it, its contribution is zero), and one that leaves now gets
+// cinv = -1.
 __global__ void __launch_bounds__(kBlock) k_colkeep(Ctx C, CompactCtx K) {
     int32_t fixed = 0;
     for (int32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < C.n; j += gridDim.x * blockDim.x) {
-        if (C.t_orig && (C.cinv[j] < 0 || (C.ckind[j] == CK_KEPT && K.c_len[j] > 0 && !K.lp_dead[lp_of_col(C, j)]))) {
-            // columns in place: one that left earlier keeps the flags it got
-            // then (its contribution was consumed by the objective sum), and a
-            // kept column with entries that S4 did not fix stays as it is
-            // (no S6 test applies to it, its contribution is zero)
+        if (C.in_place) {
+            const bool used = C.cchg[j] & CS_USED;
+            if (used && C.ckind[j] == CK_KEPT && !K.lp_dead[lp_of_col(C, j)]) continue;
+            if (C.cinv[j] < 0) continue;
+            K.c_len[j] = used;
+            fixed += colkeep_one(C, K, j);
+            if (!K.c_keep[j]) K.cinv[j] = -1;
         } else {
             fixed += colkeep_one(C, K, j);
-            if (C.t_orig) {
-                const bool kp = K.c_keep[j] != 0;
-                K.c_new[j] = kp ? j : -1;
-                if (!kp) K.cinv[j] = -1;
-            }
         }
     }
     block_add(fixed, &C.st->cols_fixed);
+}
+
+// ------------------------------------- columns in place: the rows' one pass
+// Over a kept row's entries with one byte gathered per entry (its column's
+// state): entries left and the side shift (as csr_count_row, the same order),
+// whether a column's bounds changed (the row is then evaluated next round),
+// and the columns still used, marked for S6.  It takes the place of an A^T
+// of the input kept through the rounds: the transpose at ingest, the marking
+// of the changed columns' rows through it, the counts per column and their
+// decrements.  COUNT false: a round that removed nothing, the marking alone.
+template <bool COUNT>
+__device__ __forceinline__ void inplace_entry(const Ctx &C, int32_t j, uint8_t st) {
+    if (COUNT && !(st & (CS_LEAVES | CS_USED))) C.cchg[j] = st | CS_USED;  // every writer stores the same byte
+}
+
+template <int W, bool COUNT>
+__device__ __forceinline__ void inplace_row(const Ctx &C, const CompactCtx &K, int32_t i, bool valid) {
+    const unsigned mask = group_mask<W>();
+    const int lane = threadIdx.x & (W - 1);
+    const bool keep = valid && C.rkind[i] == RK_KEPT && !K.lp_dead[lp_of_row(C, i)];
+    int32_t beg = 0, end = 0;
+    if (valid) {
+        beg = C.A.ptr[i];
+        end = C.A.ptr[i + 1];
+        if (COUNT && lane == 0) mark_tile(K.tile_a, beg, end, i);
+    }
+    int32_t cnt = 0, any = 0;
+    double sh = 0.0;
+    for (int32_t k0 = beg + lane; keep && k0 < end; k0 += 4 * W) {
+        int32_t jq[4];
+        uint8_t sq[4];
+#pragma unroll
+        for (int q = 0; q < 4; q++) jq[q] = k0 + q * W < end ? C.A.idx[k0 + q * W] : -1;
+#pragma unroll
+        for (int q = 0; q < 4; q++) sq[q] = jq[q] >= 0 ? C.cchg[jq[q]] : (uint8_t)0;
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            if (jq[q] < 0) break;
+            any |= sq[q] & CS_CHANGED;
+            if (!COUNT) continue;
+            if (sq[q] & CS_LEAVES) sh = fma(C.A.val[k0 + q * W], C.fixv[jq[q]], sh);
+            else cnt++;
+            inplace_entry<COUNT>(C, jq[q], sq[q]);
+        }
+    }
+    any = group_sum<W>(any, mask);
+    if (COUNT) {
+        cnt = group_sum<W>(cnt, mask);
+        sh = group_sum<W>(sh, mask);
+    }
+    if (valid && lane == 0) {
+        if (any) C.rdnext[i] = 1;
+        if (COUNT) {
+            K.r_keep[i] = keep;
+            K.r_len[i] = cnt;
+            K.shift[i] = sh;
+        }
+    }
+}
+
+// A row of 257 to 4096 entries by the whole block, 1024 entries in flight.
+// The shift's 32 lane-strided chains run in one warp, from shared memory, in
+// the tiles that hold a leaving column's entry.
+constexpr int32_t kMidRow = 257;
+constexpr int kMidStep = 4 * kBlock;
+template <bool COUNT>
+__device__ __forceinline__ void inplace_mid(const Ctx &C, const CompactCtx &K, int32_t i, double *s_a, double *s_v,
+                                            int32_t *s_sum) {
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int32_t beg = C.A.ptr[i], end = C.A.ptr[i + 1];
+    if (tid < 2) s_sum[tid] = 0;
+    int32_t cnt = 0, any = 0;
+    double sh = 0.0;
+    for (int32_t t0 = beg; t0 < end; t0 += kMidStep) {
+        int32_t jq[4];
+        uint8_t sq[4];
+#pragma unroll
+        for (int q = 0; q < 4; q++) jq[q] = t0 + q * kBlock + tid < end ? C.A.idx[t0 + q * kBlock + tid] : -1;
+#pragma unroll
+        for (int q = 0; q < 4; q++) sq[q] = jq[q] >= 0 ? C.cchg[jq[q]] : (uint8_t)0;
+        int32_t leaves = 0;
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            if (jq[q] < 0) continue;
+            any |= sq[q] & CS_CHANGED;
+            if (!COUNT) continue;
+            leaves |= sq[q] & CS_LEAVES;
+            cnt += !(sq[q] & CS_LEAVES);
+            inplace_entry<COUNT>(C, jq[q], sq[q]);
+        }
+        if (COUNT && __syncthreads_or(leaves)) {
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                const bool lv = jq[q] >= 0 && (sq[q] & CS_LEAVES);
+                s_a[q * kBlock + tid] = lv ? C.A.val[t0 + q * kBlock + tid] : 0.0;
+                s_v[q * kBlock + tid] = lv ? C.fixv[jq[q]] : 0.0;
+            }
+            __syncthreads();
+            if (tid < 32)
+                for (int32_t t = 0; t < kMidStep / 32; t++) sh = fma(s_a[32 * t + lane], s_v[32 * t + lane], sh);
+            __syncthreads();
+        }
+    }
+    __syncthreads();
+    any = __reduce_or_sync(0xffffffffu, (unsigned)any);
+    cnt = __reduce_add_sync(0xffffffffu, cnt);
+    if (lane == 0) {
+        if (any) s_sum[1] = 1;
+        if (cnt) atomicAdd(&s_sum[0], cnt);
+    }
+    if (COUNT && tid < 32) sh = group_sum<32>(sh, 0xffffffffu);
+    __syncthreads();
+    if (tid == 0) {
+        if (s_sum[1]) C.rdnext[i] = 1;
+        if (COUNT) {
+            mark_tile(K.tile_a, beg, end, i);
+            K.r_keep[i] = 1;
+            K.r_len[i] = s_sum[0];
+            K.shift[i] = sh;
+        }
+    }
+    __syncthreads();
+}
+
+// class of a block whose grid starts with the longest rows (class 5)
+template <bool COUNT>
+__global__ void __launch_bounds__(kBlock) k_inplace_rows(Ctx C, CompactCtx K, GroupGrid g, int32_t per5) {
+    __shared__ double s_a[COUNT ? kMidStep : 1], s_v[COUNT ? kMidStep : 1];
+    __shared__ int32_t s_mid[kBlock / 32], s_nmid, s_sum[2];
+    const int c = 5 - grid_class(g, blockIdx.x);
+    const int W = 1 << c, at = threadIdx.x / W;
+    const int32_t per = c == 5 ? per5 : kBlock / W;
+    const int32_t pos = C.A.cls_start[c] + (blockIdx.x - g.blk_start[5 - c]) * per + at;
+    bool valid = at < per && pos < C.A.cls_start[c + 1];
+    const int32_t i = valid ? C.A.order[pos] : 0;
+    switch (c) {
+        case 0: inplace_row<1, COUNT>(C, K, i, valid); break;
+        case 1: inplace_row<2, COUNT>(C, K, i, valid); break;
+        case 2: inplace_row<4, COUNT>(C, K, i, valid); break;
+        case 3: inplace_row<8, COUNT>(C, K, i, valid); break;
+        case 4: inplace_row<16, COUNT>(C, K, i, valid); break;
+        default: {
+            if (threadIdx.x == 0) s_nmid = 0;
+            __syncthreads();
+            if (valid && C.A.ptr[i + 1] - C.A.ptr[i] >= kMidRow && C.rkind[i] == RK_KEPT && !K.lp_dead[lp_of_row(C, i)]) {
+                if ((threadIdx.x & 31) == 0) s_mid[atomicAdd(&s_nmid, 1)] = i;
+                valid = false;
+            }
+            inplace_row<32, COUNT>(C, K, i, valid);
+            __syncthreads();
+            const int32_t nmid = s_nmid;
+            for (int32_t t = 0; t < nmid; t++) inplace_mid<COUNT>(C, K, s_mid[t], s_a, s_v, s_sum);
+        }
+    }
 }
 
 // --------------------------------------------------------------- CSR count
@@ -274,45 +426,49 @@ __global__ void __launch_bounds__(kBlock) k_csr_count_long(Ctx C, CompactCtx K) 
     }
 }
 
-// ------------------------------------- column counts with the input CSC kept
-// When T is the input's A^T (Ctx::t_orig) the entries per current column in
-// the kept rows are the previous counts less the entries of the rows this
-// round removed: their CSR entries, one atomic each (K.c_len holds the
-// previous counts on entry).
-template <int W>
-__device__ __forceinline__ void clen_dec_group(const Ctx &C, const CompactCtx &K, int32_t i, bool valid) {
-    const int lane = threadIdx.x & (W - 1);
-    int32_t beg = 0, end = 0;
-    if (valid && C.rkind[i] != RK_KEPT) {
-        beg = C.A.ptr[i];
-        end = C.A.ptr[i + 1];
-    }
-    for (int32_t k = beg + lane; k < end; k += W) atomicSub(&K.c_len[C.A.idx[k]], 1);
-}
-
-__global__ void __launch_bounds__(kBlock) k_clen_dec_groups(Ctx C, CompactCtx K, GroupGrid g) {
-    const int c = grid_class(g, blockIdx.x);
-    const int W = 1 << c;
-    const int32_t pos = C.A.cls_start[c] + (blockIdx.x - g.blk_start[c]) * (kBlock / W) + threadIdx.x / W;
-    const bool valid = pos < C.A.cls_start[c + 1];
-    const int32_t i = valid ? C.A.order[pos] : 0;
-    switch (c) {
-        case 0: clen_dec_group<1>(C, K, i, valid); break;
-        case 1: clen_dec_group<2>(C, K, i, valid); break;
-        case 2: clen_dec_group<4>(C, K, i, valid); break;
-        case 3: clen_dec_group<8>(C, K, i, valid); break;
-        case 4: clen_dec_group<16>(C, K, i, valid); break;
-        default: clen_dec_group<32>(C, K, i, valid); break;
-    }
-}
-
-__global__ void __launch_bounds__(kBlock) k_clen_dec_long(Ctx C, CompactCtx K) {
+// the chunks of the long rows, columns in place
+template <bool COUNT>
+__global__ void __launch_bounds__(kBlock) k_inplace_long(Ctx C, CompactCtx K) {
     const Chunk ch = C.A.chunks[blockIdx.x];
-    if (C.rkind[ch.seg] == RK_KEPT) return;  // block-uniform
-    for (int32_t k = ch.begin + threadIdx.x; k < ch.end; k += kBlock) atomicSub(&K.c_len[C.A.idx[k]], 1);
+    const int32_t i = ch.seg;
+    const bool keep = C.rkind[i] == RK_KEPT && !K.lp_dead[lp_of_row(C, i)];
+    int32_t cnt = 0, any = 0;
+    double sh = 0.0;
+    if (keep) {  // eight entries per thread and step in flight; the shift in entry order
+        for (int32_t k0 = ch.begin + threadIdx.x; k0 < ch.end; k0 += 8 * kBlock) {
+            int32_t jq[8];
+            uint8_t sq[8];
+#pragma unroll
+            for (int q = 0; q < 8; q++) jq[q] = k0 + q * kBlock < ch.end ? C.A.idx[k0 + q * kBlock] : -1;
+#pragma unroll
+            for (int q = 0; q < 8; q++) sq[q] = jq[q] >= 0 ? C.cchg[jq[q]] : (uint8_t)0;
+#pragma unroll
+            for (int q = 0; q < 8; q++) {
+                if (jq[q] < 0) break;
+                any |= sq[q] & CS_CHANGED;
+                if (!COUNT) continue;
+                if (sq[q] & CS_LEAVES) sh = fma(C.A.val[k0 + q * kBlock], C.fixv[jq[q]], sh);
+                else cnt++;
+                inplace_entry<COUNT>(C, jq[q], sq[q]);
+            }
+        }
+    }
+    if (__reduce_or_sync(0xffffffffu, (unsigned)any) && (threadIdx.x & 31) == 0) C.rdnext[i] = 1;
+    if (!COUNT) return;
+    cnt = block_sum_int(cnt);
+    sh = block_sum_dbl(sh);
+    if (threadIdx.x == 0) {
+        K.chr_cnt[blockIdx.x] = cnt;
+        K.chr_shift[blockIdx.x] = sh;
+        mark_tile(K.tile_a, ch.begin, ch.end, i);
+        if (ch.begin == C.A.ptr[i]) {  // the first chunk writes the flag
+            K.r_keep[i] = keep;
+            K.r_ch0[i] = blockIdx.x;
+        }
+    }
 }
 
-// ------------------------------------- the columns' one compaction (t_orig)
+// ------------------------------------- the columns' one compaction (in place until then)
 // keep flag of each column slot: still in the LP
 __global__ void k_cols_alive(const int32_t *cinv, int32_t n, int32_t *keep) {
     const int32_t j = blockIdx.x * blockDim.x + threadIdx.x;
@@ -337,33 +493,21 @@ __global__ void k_idx_renumber(int32_t *idx, int64_t nnz, const int32_t *pos) {
     if (k < nnz) idx[k] = pos[idx[k]];
 }
 
-// input rows / columns still in the LP, as a row kind (KEPT or not) and a
-// keep flag for the compaction of the input CSC into the result's
-__global__ void k_rows_left(const int32_t *rinv, int32_t m, uint8_t *rk) {
-    const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < m) rk[i] = rinv[i] >= 0 ? (uint8_t)RK_KEPT : (uint8_t)RK_EMPTY;
-}
-__global__ void k_cols_left(const int32_t *cinv, int32_t n, int32_t *keep, int32_t *len) {
-    const int32_t j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= n) return;
-    keep[j] = cinv[j] >= 0;
-    if (cinv[j] < 0) len[j] = 0;
-}
-// the result CSC's pointers from the kept input columns' offsets
-__global__ void k_cols_ptr(const CompactCtx K, int32_t n, int32_t *ptr) {
-    const int32_t j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j == 0) ptr[K.c_pos[n]] = K.c_off[n];
-    if (j < n && K.c_keep[j]) ptr[K.c_pos[j]] = K.c_off[j];
-}
-
 // ---------------------------------------------------------- vector gathers
 __global__ void __launch_bounds__(kBlock) k_rowvec(Ctx C, CompactCtx K) {
     const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= C.m) return;
-    if (i == C.m - 1) K.rp2[K.r_pos[C.m]] = K.r_off[C.m];
+    if (i == C.m - 1) {
+        K.rp2[K.r_pos[C.m]] = K.r_off[C.m];
+        C.st->m_new = K.r_pos[C.m];
+        C.st->nnz_new = K.r_off[C.m];
+        if (C.in_place) {  // the column slots stay, no A^T is compacted
+            C.st->n_new = C.n;
+            C.st->nnz_new_t = K.r_off[C.m];
+        }
+    }
     const int32_t p = K.r_pos[i];
-    K.r_new[i] = K.r_keep[i] ? p : -1;
-    if (K.rinv) K.rinv[C.rmap[i]] = K.r_keep[i] ? p : -1;
+    if (!C.in_place) K.r_new[i] = K.r_keep[i] ? p : -1;
     if (!K.r_keep[i]) return;
     const double sh = K.shift[i];
     const double Lv = C.L[i], Uv = C.U[i];
@@ -376,7 +520,7 @@ __global__ void __launch_bounds__(kBlock) k_rowvec(Ctx C, CompactCtx K) {
     // its S5 key is taken again then, and an unchanged row's when columns were
     // dropped (the key hashes column indices, which the compaction renumbers)
     const bool lost = K.r_len[i] != C.A.ptr[i + 1] - C.A.ptr[i];
-    const bool renumbered = !C.t_orig && K.c_pos[C.n] != C.n;
+    const bool renumbered = !C.in_place && K.c_pos[C.n] != C.n;
     K.rdirty2[p] = (uint8_t)((C.rdnext[i] | lost ? 1 : 0) | (lost | renumbered ? 2 : 0));  // kEval, kRekey
     K.act2[p] = C.act[i];
     K.ninf2[p] = C.ninf[i];
@@ -386,7 +530,11 @@ __global__ void __launch_bounds__(kBlock) k_rowvec(Ctx C, CompactCtx K) {
 __global__ void __launch_bounds__(kBlock) k_colvec(Ctx C, CompactCtx K) {
     const int32_t j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= C.n) return;
-    if (j == C.n - 1) K.cp2[K.c_pos[C.n]] = K.c_off[C.n];
+    if (j == C.n - 1) {
+        K.cp2[K.c_pos[C.n]] = K.c_off[C.n];
+        C.st->n_new = K.c_pos[C.n];
+        C.st->nnz_new_t = K.c_off[C.n];
+    }
     const int32_t p = K.c_pos[j];
     K.c_new[j] = K.c_keep[j] ? p : -1;
     if (!K.c_keep[j]) return;
@@ -397,8 +545,23 @@ __global__ void __launch_bounds__(kBlock) k_colvec(Ctx C, CompactCtx K) {
     K.cp2[p] = K.c_off[j];
 }
 
-// empty matrices still need ptr[0] = 0
-__global__ void k_zero_ptr(int32_t *p) { p[0] = 0; }
+// without rows or columns: ptr[0] = 0 and the sizes
+__global__ void k_empty(Ctx C, CompactCtx K) {
+    if (C.m == 0) {
+        K.rp2[0] = 0;
+        C.st->m_new = 0;
+        C.st->nnz_new = 0;
+        if (C.in_place) {
+            C.st->n_new = C.n;
+            C.st->nnz_new_t = 0;
+        }
+    }
+    if (C.n == 0 && !C.in_place) {
+        K.cp2[0] = 0;
+        C.st->n_new = 0;
+        C.st->nnz_new_t = 0;
+    }
+}
 
 // ---------------------------------------------------------------- scatter
 // Flat ordered compaction of all entries.  Segments of at most kFlatTile
@@ -425,6 +588,7 @@ struct FlatArgs {
     const int32_t *seg_ch0;                       // per long segment: its first chunk
     const int32_t *ch_off, *ch_cnt;               // per chunk: kept entries of its segment before it, its own
     const int32_t *oth_new;                       // per index of the other dimension: new index, -1 if dropped
+    const uint8_t *oth_state;                     // columns in place, instead: their states (they keep their index)
     const int32_t *tile_seg;                      // per tile: segment of its first entry
     int32_t *out_idx;
     double *out_val;
@@ -539,7 +703,10 @@ __global__ void __launch_bounds__(kBlock) k_scatter_flat(FlatArgs F) {
     }
 #pragma unroll
     for (int i = 0; i < kFlatPer; i++) {
-        if (jn[i] >= 0) jn[i] = F.oth_new[jn[i]];
+        if (jn[i] >= 0) {
+            if (F.oth_state) jn[i] = F.oth_state[jn[i]] & CS_LEAVES ? -1 : jn[i];
+            else jn[i] = F.oth_new[jn[i]];
+        }
         const unsigned bal = __ballot_sync(0xffffffffu, jn[i] >= 0);
         if (lane == 0) s_bal[i * (kBlock / 32) + warp] = bal;
     }
@@ -644,21 +811,71 @@ inline unsigned blocks_for(int64_t cnt, int threads) {
 
 }  // namespace
 
-void launch_compact_counts(const Ctx &C, const CompactCtx &K, cudaStream_t s, const SideStream *side) {
+void launch_inplace_rows(const Ctx &C, const CompactCtx &K, bool count, cudaStream_t s, const SideStream *side) {
+    GroupGrid g;  // the longest rows first (blk_start[k]: class 5 - k), few of them per block
+    int32_t acc = 0;
+    const int32_t cnt5 = C.A.cls_start[6] - C.A.cls_start[5];
+    const int32_t per5 = cnt5 <= 8 * 152 ? 1 : (cnt5 <= 32 * 152 ? 2 : 4);
+    for (int k = 0; k < 6; k++) {
+        const int c = 5 - k;
+        g.blk_start[k] = acc;
+        const int32_t per = c == 5 ? per5 : kBlock >> c;
+        acc += (C.A.cls_start[c + 1] - C.A.cls_start[c] + per - 1) / per;
+    }
+    g.blk_start[6] = acc;
+    // the long rows' chunks (and their prefix) on the side stream: disjoint
+    // rows, each tile start lies in one row, a column's state byte gets the
+    // same value from every writer
+    const int32_t along = C.A.cls_start[7] - C.A.cls_start[6];
+    const bool long_rows = along > 0 && C.A.nchunks > 0;
+    const bool fork = long_rows && side && side->s;
+    cudaStream_t sl = s;
+    if (fork) {
+        cudaEventRecord(side->fork, s);
+        cudaStreamWaitEvent(side->s, side->fork, 0);
+        sl = side->s;
+    }
+    if (long_rows) {
+        if (count) {
+            (k_inplace_long<true><<<C.A.nchunks, kBlock, 0, sl>>>(C, K), note_launch());
+            (k_long_prefix<<<blocks_for((int64_t)along * 32, 128), 128, 0, sl>>>(C.A, K.chr_cnt, K.chr_off, K.r_len,
+                                                                                  K.chr_shift, K.shift), note_launch());
+        } else {
+            (k_inplace_long<false><<<C.A.nchunks, kBlock, 0, sl>>>(C, K), note_launch());
+        }
+    }
+    if (acc > 0) {
+        if (count) (k_inplace_rows<true><<<acc, kBlock, 0, s>>>(C, K, g, per5), note_launch());
+        else (k_inplace_rows<false><<<acc, kBlock, 0, s>>>(C, K, g, per5), note_launch());
+    }
+    if (fork) {
+        cudaEventRecord(side->join, side->s);
+        cudaStreamWaitEvent(s, side->join, 0);
+    }
+}
+
+void launch_lp_dead(const Ctx &C, const CompactCtx &K, cudaStream_t s) {
     (k_lp_dead<<<blocks_for(C.nlp, 256), 256, 0, s>>>(C, K), note_launch());
+}
+
+static void launch_colkeep(const Ctx &C, const CompactCtx &K, cudaStream_t s) {
+    if (C.n > 0) (k_colkeep<<<std::min<unsigned>(blocks_for(C.n, kBlock), 8u * 152u), kBlock, 0, s>>>(C, K), note_launch());
+}
+
+void launch_compact_counts(const Ctx &C, const CompactCtx &K, cudaStream_t s, const SideStream *side) {
+    launch_lp_dead(C, K, s);
+    if (C.in_place) {  // the rows' one pass marks the columns in use, then S6
+        launch_inplace_rows(C, K, true, s, side);
+        launch_colkeep(C, K, s);
+        return;
+    }
     // 1. column counts over kept rows, then S6 and the column keep flags
     const GroupGrid ga = group_grid(C.A);
     const int32_t along = C.A.cls_start[7] - C.A.cls_start[6];
-    if (C.t_orig) {  // the previous counts less the removed rows' entries
-        if (C.n > 0 && K.c_len != C.clen)
-            cudaMemcpyAsync(K.c_len, C.clen, sizeof(int32_t) * (size_t)C.n, cudaMemcpyDeviceToDevice, s);
-        if (ga.blk_start[6] > 0) (k_clen_dec_groups<<<ga.blk_start[6], kBlock, 0, s>>>(C, K, ga), note_launch());
-        if (along > 0 && C.A.nchunks > 0) (k_clen_dec_long<<<C.A.nchunks, kBlock, 0, s>>>(C, K), note_launch());
-    }
     const GroupGrid gt = group_grid(C.T);
-    if (!C.t_orig && gt.blk_start[6] > 0) (k_csc_count_groups<<<gt.blk_start[6], kBlock, 0, s>>>(C, K, gt), note_launch());
+    if (gt.blk_start[6] > 0) (k_csc_count_groups<<<gt.blk_start[6], kBlock, 0, s>>>(C, K, gt), note_launch());
     const int32_t tlong = C.T.cls_start[7] - C.T.cls_start[6];
-    if (!C.t_orig && tlong > 0 && C.T.nchunks > 0) {
+    if (tlong > 0 && C.T.nchunks > 0) {
         (k_csc_count_long<<<C.T.nchunks, kBlock, 0, s>>>(C, K), note_launch());
         (k_long_prefix<<<blocks_for((int64_t)tlong * 32, 128), 128, 0, s>>>(C.T, K.cht_cnt, K.cht_off, K.c_len, nullptr,
                                                                              nullptr), note_launch());
@@ -668,7 +885,7 @@ void launch_compact_counts(const Ctx &C, const CompactCtx &K, cudaStream_t s, co
         if (gt.blk_start[6] > 0) (k_locks_groups<<<gt.blk_start[6], kBlock, 0, s>>>(C, K, gt), note_launch());
         if (tlong > 0 && C.T.nchunks > 0) (k_locks_long<<<C.T.nchunks, kBlock, 0, s>>>(C, K), note_launch());
     }
-    if (C.n > 0) (k_colkeep<<<std::min<unsigned>(blocks_for(C.n, kBlock), 8u * 152u), kBlock, 0, s>>>(C, K), note_launch());
+    launch_colkeep(C, K, s);
     // 2. row counts over kept columns and the side shifts; the long rows'
     // chunks (and their prefix) on the side stream when one is given: the
     // two touch disjoint rows, and each tile start lies in one row
@@ -693,49 +910,21 @@ void launch_compact_counts(const Ctx &C, const CompactCtx &K, cudaStream_t s, co
 }
 
 void launch_compact_scatter(const Ctx &C, const CompactCtx &K, int32_t nnz, cudaStream_t s) {
-    (k_zero_ptr<<<1, 1, 0, s>>>(K.rp2), note_launch());
-    if (!C.t_orig) (k_zero_ptr<<<1, 1, 0, s>>>(K.cp2), note_launch());
+    // k_rowvec and k_colvec write the pointers (entry 0 with the first kept
+    // segment or the total) and the new sizes; an empty dimension is left to k_empty
+    if (C.m == 0 || C.n == 0) (k_empty<<<1, 1, 0, s>>>(C, K), note_launch());
     if (C.m > 0) (k_rowvec<<<blocks_for(C.m, kBlock), kBlock, 0, s>>>(C, K), note_launch());
-    if (C.n > 0 && !C.t_orig) (k_colvec<<<blocks_for(C.n, kBlock), kBlock, 0, s>>>(C, K), note_launch());
+    if (C.n > 0 && !C.in_place) (k_colvec<<<blocks_for(C.n, kBlock), kBlock, 0, s>>>(C, K), note_launch());
     const int32_t ntiles = (int32_t)(((int64_t)nnz + kFlatTile - 1) / kFlatTile);
     if (ntiles > 0) {
         FlatArgs fa{C.A.ptr, C.A.idx, C.A.val, nnz, C.m, ntiles, K.r_keep, K.r_off, K.r_len, K.r_ch0,
-                    K.chr_off, K.chr_cnt, K.c_new, K.tile_a, K.ci2, K.rv2};
+                    K.chr_off, K.chr_cnt, K.c_new, C.in_place ? C.cchg : nullptr, K.tile_a, K.ci2, K.rv2};
         (k_scatter_flat<<<ntiles, kBlock, 0, s>>>(fa), note_launch());
-        if (!C.t_orig) {
+        if (!C.in_place) {
             FlatArgs ft{C.T.ptr, C.T.idx, C.T.val, nnz, C.n, ntiles, K.c_keep, K.c_off, K.c_len, K.c_ch0,
-                        K.cht_off, K.cht_cnt, K.r_new, K.tile_t, K.ri2, K.cv2};
+                        K.cht_off, K.cht_cnt, K.r_new, nullptr, K.tile_t, K.ri2, K.cv2};
             (k_scatter_flat<<<ntiles, kBlock, 0, s>>>(ft), note_launch());
         }
-    }
-}
-
-// The result's CSC from the input CSC C.T (input numbering, Ctx::t_orig):
-// C.rkind marks the input rows still in the LP, keep / len the input
-// columns still in it and their entries left; the one compaction of the
-// kept columns' kept entries, renumbered by rinv, into ptr / idx / val
-// (K.c_pos / c_off: the column scan, done by the caller between the two
-// calls).
-void launch_csc_from_input_counts(const Ctx &C, const CompactCtx &K, cudaStream_t s) {
-    const GroupGrid gt = group_grid(C.T);
-    if (gt.blk_start[6] > 0) (k_csc_count_groups<<<gt.blk_start[6], kBlock, 0, s>>>(C, K, gt), note_launch());
-    const int32_t tlong = C.T.cls_start[7] - C.T.cls_start[6];
-    if (tlong > 0 && C.T.nchunks > 0) {
-        (k_csc_count_long<<<C.T.nchunks, kBlock, 0, s>>>(C, K), note_launch());
-        (k_long_prefix<<<blocks_for((int64_t)tlong * 32, 128), 128, 0, s>>>(C.T, K.cht_cnt, K.cht_off, K.c_len, nullptr,
-                                                                             nullptr), note_launch());
-    }
-    if (C.n > 0) (k_cols_left<<<blocks_for(C.n, kBlock), kBlock, 0, s>>>(C.cinv, C.n, K.c_keep, K.c_len), note_launch());
-}
-
-void launch_csc_from_input_scatter(const Ctx &C, const CompactCtx &K, int64_t nnz, int32_t *ptr, int32_t *idx,
-                                   double *val, cudaStream_t s) {
-    (k_cols_ptr<<<blocks_for(std::max(C.n, 1), kBlock), kBlock, 0, s>>>(K, C.n, ptr), note_launch());
-    const int32_t ntiles = (int32_t)((nnz + kFlatTile - 1) / kFlatTile);
-    if (ntiles > 0) {
-        FlatArgs ft{C.T.ptr, C.T.idx, C.T.val, (int32_t)nnz, C.n, ntiles, K.c_keep, K.c_off, K.c_len, K.c_ch0,
-                    K.cht_off, K.cht_cnt, C.rinv, K.tile_t, idx, val};
-        (k_scatter_flat<<<ntiles, kBlock, 0, s>>>(ft), note_launch());
     }
 }
 
@@ -746,10 +935,6 @@ void launch_cols_final(const Ctx &C, const CompactCtx &K, int32_t n, int32_t *ci
                        cudaStream_t s) {
     if (n > 0) (k_cols_final<<<blocks_for(n, kBlock), kBlock, 0, s>>>(C, K, n, cinv), note_launch());
     if (nnz > 0) (k_idx_renumber<<<blocks_for(nnz, kBlock), kBlock, 0, s>>>(idx, nnz, K.c_pos), note_launch());
-}
-
-void launch_rows_left(const int32_t *rinv, int32_t m, uint8_t *rk, cudaStream_t s) {
-    if (m > 0) (k_rows_left<<<blocks_for(m, kBlock), kBlock, 0, s>>>(rinv, m, rk), note_launch());
 }
 
 void launch_offset(const Ctx &C, const CompactCtx &K, cudaStream_t s) {

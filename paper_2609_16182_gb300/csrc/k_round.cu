@@ -132,6 +132,37 @@ __device__ __forceinline__ void prop_mid(const Ctx &C, int32_t i, MidShared &M, 
     __syncthreads();  // M is reused by the block's next row
 }
 
+// The round's flags and counters to zero: the status counters, the per-LP
+// changed flags, the column lists' sizes, the next dirty flags and (outside a
+// first round, whose S3' writes every column's) the columns' kinds and states.
+__global__ void __launch_bounds__(kBlock) k_round_start(Ctx C, int32_t cols) {
+    const int64_t t = (int64_t)blockIdx.x * kBlock + threadIdx.x, step = (int64_t)gridDim.x * kBlock;
+    if (t < 8) reinterpret_cast<int32_t *>(C.st)[t] = 0;
+    if (t < 3) C.tl_cnt[t] = 0;
+    for (int64_t k = t; k < C.nlp; k += step) C.lp_changed[k] = 0;
+    // flag arrays start 256-byte aligned
+    auto zero = [&](uint8_t *p, int64_t cnt) {
+        for (int64_t k = t; k < cnt / 16; k += step) reinterpret_cast<uint4 *>(p)[k] = make_uint4(0, 0, 0, 0);
+        if (t < (cnt & 15)) p[cnt / 16 * 16 + t] = 0;
+    };
+    zero(C.rdnext, C.m);
+    if (cols) {
+        zero(C.ckind, C.n);
+        zero(C.cchg, C.n);
+    }
+}
+
+// an empty S5 table of cap slots; passes (if not 0): the pass sizes' array, zeroed
+__global__ void __launch_bounds__(kBlock) k_s5_init(unsigned long long *tkey, unsigned long long *tlead, int32_t cap,
+                                                    int32_t *cnt, int32_t passes) {
+    const int64_t t = (int64_t)blockIdx.x * kBlock + threadIdx.x, step = (int64_t)gridDim.x * kBlock;
+    for (int64_t k = t; k < cap / 2; k += step) {  // capacities are powers of two >= 2
+        reinterpret_cast<ulonglong2 *>(tkey)[k] = make_ulonglong2(0ULL, 0ULL);
+        reinterpret_cast<ulonglong2 *>(tlead)[k] = make_ulonglong2(~0ULL, ~0ULL);
+    }
+    for (int64_t k = t; k < passes; k += step) cnt[k] = 0;
+}
+
 // class of a block of k_prop_groups (its grid starts with class 5)
 __device__ __forceinline__ int prop_class(const GroupGrid &g, int b) { return 5 - grid_class(g, b); }
 
@@ -657,13 +688,6 @@ __global__ void __launch_bounds__(kBlock) k_s5_leader(Ctx C) {
     s5_leader_one(C, i);
 }
 
-// row r of a T entry (an input row when T is not compacted: its current
-// index, none once it left) is evaluated next round
-__device__ __forceinline__ void mark_row_of(const Ctx &C, int32_t r) {
-    if (C.t_orig) r = C.rinv[r];
-    if (r >= 0) C.rdnext[r] = 1;
-}
-
 // rows of the changed short columns need their activities next round: one
 // thread per listed column; columns longer than 32 entries are walked by the
 // whole warp in turn.  When the changed columns hold at least an eighth of the
@@ -682,27 +706,25 @@ __global__ void __launch_bounds__(kBlock) k_mark_list(Ctx C, int64_t nnz) {
         int32_t b = 0, e = 0;
         if (t < cnt) {
             const int32_t j = C.cl_list[t];
-            const int32_t jt = C.t_orig ? C.cmap[j] : j;
-            b = C.T.ptr[jt];
-            e = C.T.ptr[jt + 1];
+            b = C.T.ptr[j];
+            e = C.T.ptr[j + 1];
         }
         if (e - b <= 32)
-            for (int32_t k = b; k < e; k++) mark_row_of(C, C.T.idx[k]);
+            for (int32_t k = b; k < e; k++) C.rdnext[C.T.idx[k]] = 1;
         unsigned todo = __ballot_sync(0xffffffffu, e - b > 32);
         while (todo) {
             const int src = __ffs(todo) - 1;
             todo &= todo - 1u;
             const int32_t sb = __shfl_sync(0xffffffffu, b, src), se = __shfl_sync(0xffffffffu, e, src);
-            for (int32_t k = sb + lane; k < se; k += 32) mark_row_of(C, C.T.idx[k]);
+            for (int32_t k = sb + lane; k < se; k += 32) C.rdnext[C.T.idx[k]] = 1;
         }
     }
 }
 
 __global__ void __launch_bounds__(kBlock) k_mark_long(Ctx C, int64_t nnz) {
     const Chunk ch = C.T.chunks[blockIdx.x];
-    const int32_t j = C.t_orig ? C.cinv[ch.seg] : ch.seg;
-    if (j < 0 || !C.cchg[j] || 8 * (int64_t)*C.cl_nnz >= nnz) return;
-    for (int32_t k = ch.begin + threadIdx.x; k < ch.end; k += kBlock) mark_row_of(C, C.T.idx[k]);
+    if (!C.cchg[ch.seg] || 8 * (int64_t)*C.cl_nnz >= nnz) return;
+    for (int32_t k = ch.begin + threadIdx.x; k < ch.end; k += kBlock) C.rdnext[C.T.idx[k]] = 1;
 }
 
 inline unsigned blocks_for(int64_t cnt, int threads) {
@@ -710,6 +732,18 @@ inline unsigned blocks_for(int64_t cnt, int threads) {
 }
 
 }  // namespace
+
+void launch_round_start(const Ctx &C, bool cols, cudaStream_t s) {
+    const int64_t most = std::max<int64_t>({(int64_t)C.m / 16, (int64_t)C.n / 16, (int64_t)C.nlp, 64});
+    (k_round_start<<<std::min<unsigned>(blocks_for(most, kBlock), 4u * 152u), kBlock, 0, s>>>(C, cols ? 1 : 0),
+     note_launch());
+}
+
+void launch_s5_init(const Ctx &C, int32_t cap, int32_t *cnt, int32_t passes, cudaStream_t s) {
+    (k_s5_init<<<std::min<unsigned>(blocks_for(std::max(cap / 2, passes), kBlock), 8u * 152u), kBlock, 0, s>>>(
+         C.tkey, C.tlead, cap, cnt, passes),
+     note_launch());
+}
 
 void launch_prop_short(const Ctx &C, cudaStream_t s) {
     // blocks per class at prop_lanes(c) lanes per row, the longest rows first

@@ -325,6 +325,8 @@ __device__ __forceinline__ int32_t row_search(const int32_t *ptr, int32_t m, int
     return lo;
 }
 
+// (CHECK false: the rows alone; row_of NULL: the checks alone)
+template <bool CHECK>
 __global__ void __launch_bounds__(kScanThreads) k_rows_check(const int32_t *ptr, const int32_t *idx, const double *val,
                                                              int32_t m, int32_t n, int64_t nnz, int32_t *row_of,
                                                              int32_t *err) {
@@ -375,14 +377,15 @@ __global__ void __launch_bounds__(kScanThreads) k_rows_check(const int32_t *ptr,
     for (int x = tid; x < len; x += kScanThreads) {
         const int64_t k = k0 + x;
         const int32_t r = s_row[x];
-        row_of[k] = r;
+        if (row_of) row_of[k] = r;
+        if (!CHECK) continue;
         const int32_t j = idx[k];
         const double a = val[k];
         if (j < 0 || j >= n) e |= ERR_COL;
         if (!is_fin(a) || a == 0.0) e |= ERR_VAL;
         if (k > 0 && (int64_t)ptr[r] < k && idx[k - 1] >= j) e |= ERR_ORDER;  // k - 1 in the same row
     }
-    if (e) atomicOr(err, e);
+    if (CHECK && e) atomicOr(err, e);
 }
 
 __device__ __forceinline__ double norm_inf(double x, double huge) {
@@ -638,8 +641,15 @@ void check_csr(const int32_t *ptr, const int32_t *idx, const double *val, int32_
     (k_check_ptr<<<blocks_for((int64_t)m + 1, 256), 256, 0, s>>>(ptr, m, nnz, err), note_launch());
     // row_of[0] is unused (callers read row_of + 1)
     if (nnz > 0 && m > 0)
-        (k_rows_check<<<(unsigned)((nnz + kRowTile - 1) / kRowTile), kScanThreads, 0, s>>>(ptr, idx, val, m, n, nnz,
-                                                                                           row_of + 1, err),
+        (k_rows_check<true><<<(unsigned)((nnz + kRowTile - 1) / kRowTile), kScanThreads, 0, s>>>(
+             ptr, idx, val, m, n, nnz, row_of ? row_of + 1 : nullptr, err),
+         note_launch());
+}
+
+void rows_of(const int32_t *ptr, int32_t m, int64_t nnz, int32_t *row_of, cudaStream_t s) {
+    if (nnz > 0 && m > 0)
+        (k_rows_check<false><<<(unsigned)((nnz + kRowTile - 1) / kRowTile), kScanThreads, 0, s>>>(
+             ptr, nullptr, nullptr, m, 0, nnz, row_of, nullptr),
          note_launch());
 }
 

@@ -435,6 +435,12 @@ uint64_t tuner_key(int32_t count, int64_t nnz, int32_t dualfix) {
     return ((uint64_t)a << 32) | ((uint64_t)b << 1) | (uint64_t)(dualfix != 0);
 }
 
+// the options the persistent kernel carries
+bool fused_options(const lpp_opts &o) {
+    return o.batch_persistent && !o.parallel_cols && !o.col_singletons && !o.doubletons && !o.dual_records && !o.timing &&
+           o.max_rounds > 0;
+}
+
 // Runs the batch in the persistent kernel when every LP qualifies (no row or
 // column beyond 4096 entries, none of the steps it does not carry); returns
 // false, with nothing done, otherwise.  E is prepared (ingested, checked,
@@ -442,9 +448,7 @@ uint64_t tuner_key(int32_t count, int64_t nnz, int32_t dualfix) {
 bool batch_fused(Engine &E, const std::vector<Member> &mem, int32_t count, lpp_reduced **outs, lpp_postsolve **recs,
                  lpp_status *per_lp) {
     const lpp_opts &o = E.o;
-    if (!o.batch_persistent || o.parallel_cols || o.col_singletons || o.doubletons || o.dual_records || o.timing ||
-        o.max_rounds <= 0)
-        return false;
+    if (!fused_options(o)) return false;
     if (E.A.cls_start[7] != E.A.cls_start[6] || E.T.cls_start[7] != E.T.cls_start[6]) return false;
     cudaStream_t s = E.s;
     const int32_t m0 = E.m0, n0 = E.n0;
@@ -469,10 +473,10 @@ bool batch_fused(Engine &E, const std::vector<Member> &mem, int32_t count, lpp_r
     FusedArgs F;
     std::memset(&F, 0, sizeof F);
     F.base = E.ctx(1);
-    F.base.t_orig = 0;  // each block compacts its LP's CSC itself
-    F.base.rinv = F.base.cinv = F.base.clen = nullptr;
+    F.base.in_place = 0;  // each block compacts its LP's columns and CSC itself
+    F.base.cinv = nullptr;
     F.K = E.K;
-    F.K.rinv = F.K.cinv = nullptr;
+    F.K.cinv = nullptr;
     for (int b = 0; b < 2; b++) {
         F.frp[b] = P.alloc<int32_t>((size_t)m0 + count + 1);
         F.ftp[b] = P.alloc<int32_t>((size_t)n0 + count + 1);
@@ -699,7 +703,7 @@ lpp_status lpp_presolve(const lpp_lp *in, const lpp_opts *opts, lpp_reduced **ou
         const lpp_opts o = resolve_opts(opts);
         auto E = std::make_unique<Engine>();
         Member mm{in->m, in->n, in->nnz, 0, 0, 0, in->obj_offset};
-        E->lazy_req = true;  // the CSC is compacted once, at the end, when no step reads it
+        E->lazy_req = true;  // no A^T during the rounds when no step reads it
         E->setup(o, 1, {mm});
         // ingest: checks, copies, CSC, schedules (bytes: the input once, the CSC written)
         E->tbegin(F_INGEST, 24.0 * in->nnz + 48.0 * in->m + 40.0 * in->n);
@@ -775,7 +779,8 @@ lpp_status lpp_presolve_batch(const lpp_lp *ins, int32_t count, const lpp_opts *
                 throw StatusError(LPP_ERR_INVALID, "batch too large for int32 indices");
         }
         auto E = std::make_unique<Engine>();
-        E->lazy_req = true;  // the CSC is compacted once, at the end, when no step reads it
+        E->lazy_req = true;  // no A^T during the rounds when no step reads it
+        E->need_t = fused_options(o);  // the persistent kernel starts from it
         E->setup(o, count, mem);
         E->ingest_batch(ins, count);
         E->prepare();

@@ -48,6 +48,8 @@ enum : uint8_t {
 // CK_DOUBLETON: eliminated through a doubleton equation, S5e)
 enum : uint8_t { CK_KEPT = 0, CK_FIXED = 1, CK_EMPTY = 2, CK_PARALLEL = 3, CK_SUBST = 4, CK_DOUBLETON = 5 };
 // verdict slots per LP, in step order
+// column states of a round with the columns in place (Ctx::cchg)
+enum : uint8_t { CS_CHANGED = 1, CS_LEAVES = 2, CS_USED = 4 };
 enum { V_S2_ROW = 0, V_S3_COL = 1, V_S5_ROW = 2, V_S5E_COL = 3, V_S6_COL = 4, V_SLOTS = 5 };
 
 // Global counters of a round (block-aggregated atomics).
@@ -92,13 +94,13 @@ struct Ctx {
     double2 *lu;
     double *c;                      // written only by S5d (one product per column and round)
     const int32_t *cmap, *lp_col;
-    // t_orig: the CSC T is the input's A^T, never compacted, and the columns
-    // stay in their input slots (no step that reads columns' entries is on).
-    // rinv maps an input row to its current index, cinv an input column to
-    // its slot (-1 once either left); clen: entries per column in the
-    // current rows.
-    const int32_t *rinv, *cinv, *clen;
-    int32_t t_orig;
+    // in_place: the columns stay in their input slots and no A^T is kept
+    // during the rounds (no step that reads columns' entries is on).  cinv
+    // maps an input column to its slot (-1 once it left); cchg then holds, per
+    // slot, CS_CHANGED and CS_LEAVES of this round and CS_USED, set by the
+    // pass over the kept rows' entries.
+    const int32_t *cinv;
+    int32_t in_place;
     // rows whose activities must be recomputed this round (1) and the flags
     // being gathered for the next round; columns whose bounds changed
     const uint8_t *rdirty;
@@ -204,9 +206,7 @@ struct CompactCtx {
     double2 *act2;                             // carried results of clean rows
     int2 *ninf2;
     unsigned long long *hrow2;
-    // CSC kept in the input's numbering and columns kept in place
-    // (Ctx::t_orig): the input-to-current maps, updated in place
-    int32_t *rinv, *cinv;
+    int32_t *cinv;  // columns in place (Ctx::in_place): updated in place
 };
 
 // ------------------------------------------------------------------ helpers

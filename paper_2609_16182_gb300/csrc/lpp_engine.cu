@@ -192,18 +192,60 @@ __global__ void k_gather_lps(const SrcDesc *d, int32_t *rp, int32_t *ci, double 
 }
 
 __global__ void k_set_i32(int32_t *p, int32_t v) { *p = v; }
-__global__ void k_csc_sizes(const CompactCtx K, int32_t n, DevStatus *st) {
-    st->n_new = K.c_pos[n];
-    st->nnz_new_t = K.c_off[n];
+// everything that starts at a fixed value, one pass over rows and columns
+struct InitArgs {
+    int32_t m, n, nlp;
+    int32_t *rmap;
+    unsigned long long *mL, *mU;
+    uint8_t *hasf, *rdirty, *rwork;
+    int32_t *rk, *rr, *ra;
+    double *rv;
+    int32_t *cmap, *cinv;
+    double *contrib;
+    unsigned long long *cand_l, *cand_u;
+    uint32_t *ctouch;
+    int32_t *ck, *cr;
+    double *cv;
+    int32_t *verdict;
+    uint8_t *dead;
+    DevStatus *st;
+};
+__global__ void __launch_bounds__(256) k_init_work(InitArgs I) {
+    const int32_t t = blockIdx.x * 256 + threadIdx.x, step = gridDim.x * 256;
+    for (int32_t i = t; i < I.m; i += step) {
+        I.rmap[i] = i;
+        I.mL[i] = kEncNegInf;
+        I.mU[i] = kEncPosInf;
+        I.hasf[i] = 0;
+        I.rdirty[i] = 3;  // round 1 evaluates every row, keys and all
+        I.rwork[i] = 0;
+        I.rk[i] = 0;
+        I.rr[i] = 0;
+        I.ra[i] = -1;
+        I.rv[i] = 0.0;
+    }
+    for (int32_t j = t; j < I.n; j += step) {
+        I.cmap[j] = j;
+        if (I.cinv) I.cinv[j] = j;
+        if (I.contrib) I.contrib[j] = 0.0;
+        I.cand_l[j] = kEncNegInf;
+        I.cand_u[j] = kEncPosInf;
+        I.ctouch[j] = 0u;
+        I.ck[j] = 0;
+        I.cr[j] = 0;
+        I.cv[j] = 0.0;
+    }
+    for (int32_t k = t; k < I.nlp * V_SLOTS; k += step) I.verdict[k] = kNone;
+    for (int32_t k = t; k < I.nlp; k += step) I.dead[k] = 0;
+    if (t == 0) {
+        const bool ok = I.st->err == 0;
+        I.st->m_new = ok ? I.m : 0;
+        I.st->n_new = ok ? I.n : 0;
+    }
 }
 
-// cols_in_place: the column slots stay (n), the CSC is not compacted
-__global__ void k_sizes(const CompactCtx K, int32_t m, int32_t n, int32_t cols_in_place, DevStatus *st) {
-    st->m_new = K.r_pos[m];
-    st->nnz_new = K.r_off[m];
-    st->n_new = cols_in_place ? n : K.c_pos[n];
-    st->nnz_new_t = cols_in_place ? K.r_off[m] : K.c_off[n];
-}
+// the columns left, after the scan of their keep flags
+__global__ void k_cols_left(const int32_t *pos, int32_t n, DevStatus *st) { st->n_new = pos[n]; }
 
 const char *kFamNames[F_NUM] = {"prop",     "colfin",   "s5",     "compact_count", "scan", "compact_scatter",
                                 "schedule", "ingest",   "finish", "s5c", "s5d", "s5e"};
@@ -228,8 +270,6 @@ Engine::~Engine() {
     pool.release();
     if (s) cudaStreamSynchronize(s);
     pinned_put(st_h);
-    pinned_put(verdict_h);
-    pinned_put(changed_h);
     pinned_put(s5_left_h);
     pinned_put(de_cnt_h);
     if (own_stream && s) cudaStreamDestroy(s);
@@ -276,9 +316,14 @@ void Engine::setup(const lpp_opts &opts, int32_t nlp_, const std::vector<Member>
     }
     pool.s = s;
     keep_pool_memory(o.device);
-    st_h = static_cast<DevStatus *>(pinned_get_sized(sizeof(DevStatus)));
-    verdict_h = static_cast<int32_t *>(pinned_get_sized(sizeof(int32_t) * (size_t)nlp * V_SLOTS));
-    changed_h = static_cast<uint8_t *>(pinned_get_sized((size_t)nlp));
+    // status, verdicts and changed flags in one block: one copy reads them
+    st_bytes = sizeof(DevStatus) + sizeof(int32_t) * (size_t)nlp * V_SLOTS + (size_t)nlp;
+    st_h = static_cast<DevStatus *>(pinned_get_sized(st_bytes));
+    verdict_h = reinterpret_cast<int32_t *>(st_h + 1);
+    changed_h = reinterpret_cast<uint8_t *>(verdict_h + (size_t)nlp * V_SLOTS);
+    st = reinterpret_cast<DevStatus *>(pool.alloc<unsigned char>(st_bytes));
+    verdict = reinterpret_cast<int32_t *>(st + 1);
+    lp_changed = reinterpret_cast<uint8_t *>(verdict + (size_t)nlp * V_SLOTS);
     s5_left_h = static_cast<int32_t *>(pinned_get_sized(sizeof(int32_t)));
     const bool arena = nlp > 1;
     for (int b = 0; b < 2; b++) {
@@ -322,14 +367,8 @@ void Engine::setup(const lpp_opts &opts, int32_t nlp_, const std::vector<Member>
     }
     rdnext = pool.alloc<uint8_t>(m0);
     cchg = pool.alloc<uint8_t>(n0);
-    t_orig = lazy_req && !o.parallel_cols && !o.col_singletons && !o.dual_fixing && !o.doubletons;
-    t_fixed = false;
-    if (t_orig) {
-        rinv = pool.alloc<int32_t>(m0);
-        cinv = pool.alloc<int32_t>(n0);
-        clive = pool.alloc<int32_t>(n0);
-        rleft = pool.alloc<uint8_t>(m0);
-    }
+    in_place = lazy_req && !o.parallel_cols && !o.col_singletons && !o.dual_fixing && !o.doubletons;
+    if (in_place) cinv = pool.alloc<int32_t>(n0);
     rkind = pool.alloc<uint8_t>(m0);
     rwork = pool.alloc<uint8_t>(m0);
     hasf = pool.alloc<uint8_t>(m0);
@@ -356,8 +395,6 @@ void Engine::setup(const lpp_opts &opts, int32_t nlp_, const std::vector<Member>
     ch_ninf = pool.alloc<int2>(cap_chunk);
     ch_hash = pool.alloc<unsigned long long>(cap_chunk);
     lneed = pool.alloc<uint8_t>(cap_long_a + 1);
-    verdict = pool.alloc<int32_t>((size_t)nlp * V_SLOTS);
-    lp_changed = pool.alloc<uint8_t>(nlp);
     lp_dead = pool.alloc<uint8_t>(nlp);
     std::memset(&K, 0, sizeof K);
     K.r_keep = pool.alloc<int32_t>(m0 + 1);
@@ -463,11 +500,20 @@ void Engine::setup(const lpp_opts &opts, int32_t nlp_, const std::vector<Member>
         rec_sval = pool.alloc<double>(nnz0);
         sub_used = pool.alloc<unsigned long long>(1);
     }
-    st = pool.alloc<DevStatus>(1);
     LPP_CUDA(cudaMemsetAsync(st, 0, sizeof(DevStatus), s));
 }
 
 void Engine::ingest_plain(const lpp_lp &in) {
+    set_matrix();
+    if (in.on_device && in_place && o.max_rounds > 0) {
+        // read where they lie: the first round always compacts, into the
+        // library's buffers
+        m_rp = in.row_ptr;
+        m_ci = in.col_idx;
+        m_rv = in.val;
+        ingest_vectors(in.lhs, in.rhs, in.lb, in.ub, in.c, m0, n0, o.huge, L[0], U[0], lu[0], c[0], &st->err, s);
+        return;
+    }
     const cudaMemcpyKind kind = in.on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     LPP_CUDA(cudaMemcpyAsync(rp[0], in.row_ptr, sizeof(int32_t) * (size_t)(in.m + 1), kind, s));
     if (in.nnz > 0) {
@@ -508,6 +554,7 @@ void Engine::ingest_plain(const lpp_lp &in) {
 }
 
 void Engine::ingest_batch(const lpp_lp *ins, int32_t count) {
+    set_matrix();
     double *slhs = L[1], *srhs = U[1], *slb = reinterpret_cast<double *>(lu[1]), *sub = slb + n0, *sc = c[1];
     const bool dev = ins[0].on_device != 0;
     for (int32_t k = 0; k < count; k++)
@@ -577,62 +624,60 @@ void Engine::ingest_batch(const lpp_lp *ins, int32_t count) {
 }
 
 void Engine::prepare() {
-    // S0: checks, then A^T by a stable transpose
-    int32_t *row_of = pool.alloc<int32_t>(nnz0 + 1);
-    check_csr(rp[0], ci[0], rv[0], m0, n0, nnz0, row_of, scan_tmp, &st->err, s);
+    // S0: checks, then A^T by a stable transpose where it is needed
+    const bool want_t = !in_place || need_t;
+    int32_t *row_of = want_t ? pool.alloc<int32_t>(nnz0 + 1) : nullptr;
+    check_csr(m_rp, m_ci, m_rv, m0, n0, nnz0, row_of, scan_tmp, &st->err, s);
+    t_hist = pool.alloc<int32_t>(transpose_hist_elems(nnz0));  // S5e and the result's A^T transpose with it too
     LPP_CUDA(cudaGetLastError());
-    read_status();
-    if (st_h->err) {
-        char buf[160];
-        std::snprintf(buf, sizeof buf,
-                      "invalid LP (checks failed: %s%s%s%s%s)", (st_h->err & 1) ? "row_ptr " : "",
-                      (st_h->err & 2) ? "col_idx-range " : "", (st_h->err & 4) ? "val-not-finite-or-zero " : "",
-                      (st_h->err & 8) ? "col_idx-not-increasing " : "", (st_h->err & 16) ? "vectors" : "");
-        throw StatusError(LPP_ERR_INVALID, buf);
+    if (want_t) {
+        read_status();
+        check_status();
+        TransposeBufs tb;
+        tb.k0 = reinterpret_cast<uint32_t *>(ci[1]);
+        tb.k1 = reinterpret_cast<uint32_t *>(ti[1]);
+        tb.v0 = reinterpret_cast<int32_t *>(rv[1]);
+        tb.v1 = reinterpret_cast<int32_t *>(rv[1]) + nnz0;
+        tb.hist = t_hist;
+        tb.tmp = scan_tmp;
+        transpose(rp[0], ci[0], rv[0], row_of + 1, m0, n0, nnz0, tb, tp[0], ti[0], tv[0], s);
+        LPP_CUDA(cudaGetLastError());
     }
-    TransposeBufs tb;
-    tb.k0 = reinterpret_cast<uint32_t *>(ci[1]);
-    tb.k1 = reinterpret_cast<uint32_t *>(ti[1]);
-    tb.v0 = reinterpret_cast<int32_t *>(rv[1]);
-    tb.v1 = reinterpret_cast<int32_t *>(rv[1]) + nnz0;
-    tb.hist = pool.alloc<int32_t>(transpose_hist_elems(nnz0));
-    tb.tmp = scan_tmp;
-    t_hist = tb.hist;  // S5e transposes its rewritten matrices with it
-    transpose(rp[0], ci[0], rv[0], row_of + 1, m0, n0, nnz0, tb, tp[0], ti[0], tv[0], s);
-    LPP_CUDA(cudaGetLastError());
     if (vec_pending) {  // the vectors' copies overlapped the checks and the transpose
         vec_pending = false;
         LPP_CUDA(cudaStreamWaitEvent(s, ev_vec, 0));
         double *slb = reinterpret_cast<double *>(lu[1]);
         ingest_vectors(L[1], U[1], slb, slb + n0, c[1], m0, n0, o.huge, L[0], U[0], lu[0], c[0], &st->err, s);
     }
-    iota(rmap[0], m0, 0, s);
-    iota(cmap[0], n0, 0, s);
-    if (t_orig) {
-        iota(rinv, m0, 0, s);
-        iota(cinv, n0, 0, s);
-        ptr_diff(tp[0], n0, clive, s);
-        // every column starts kept at its own slot, with no contribution
-        fill_i32(K.c_keep, n0, 1, s);
-        iota(K.c_new, n0, 0, s);
-        LPP_CUDA(cudaMemsetAsync(K.contrib, 0, sizeof(double) * (size_t)std::max(n0, 1), s));
-    }
-    fill_u64(cand_l, n0, kEncNegInf, s);
-    fill_u64(cand_u, n0, kEncPosInf, s);
-    LPP_CUDA(cudaMemsetAsync(ctouch, 0, sizeof(uint32_t) * (size_t)std::max(n0, 1), s));
-    fill_u64(mL, m0, kEncNegInf, s);
-    fill_u64(mU, m0, kEncPosInf, s);
-    LPP_CUDA(cudaMemsetAsync(hasf, 0, (size_t)std::max(m0, 1), s));
-    LPP_CUDA(cudaMemsetAsync(rdirty[0], 3, (size_t)std::max(m0, 1), s));  // round 1 evaluates every row, keys and all
-    LPP_CUDA(cudaMemsetAsync(rwork, 0, (size_t)std::max(m0, 1), s));
-    fill_i32(verdict, (int64_t)nlp * V_SLOTS, kNone, s);
-    LPP_CUDA(cudaMemsetAsync(rec_rk, 0, sizeof(int32_t) * (size_t)std::max(m0, 1), s));
-    LPP_CUDA(cudaMemsetAsync(rec_rr, 0, sizeof(int32_t) * (size_t)std::max(m0, 1), s));
-    fill_i32(rec_ra, m0, -1, s);
-    LPP_CUDA(cudaMemsetAsync(rec_rv, 0, sizeof(double) * (size_t)std::max(m0, 1), s));
-    LPP_CUDA(cudaMemsetAsync(rec_ck, 0, sizeof(int32_t) * (size_t)std::max(n0, 1), s));
-    LPP_CUDA(cudaMemsetAsync(rec_cr, 0, sizeof(int32_t) * (size_t)std::max(n0, 1), s));
-    LPP_CUDA(cudaMemsetAsync(rec_cv, 0, sizeof(double) * (size_t)std::max(n0, 1), s));
+    InitArgs I;
+    std::memset(&I, 0, sizeof I);
+    I.m = m0;
+    I.n = n0;
+    I.nlp = nlp;
+    I.rmap = rmap[0];
+    I.mL = mL;
+    I.mU = mU;
+    I.hasf = hasf;
+    I.rdirty = rdirty[0];
+    I.rwork = rwork;
+    I.rk = rec_rk;
+    I.rr = rec_rr;
+    I.ra = rec_ra;
+    I.rv = rec_rv;
+    I.cmap = cmap[0];
+    I.cinv = cinv;
+    I.contrib = in_place ? K.contrib : nullptr;
+    I.cand_l = cand_l;
+    I.cand_u = cand_u;
+    I.ctouch = ctouch;
+    I.ck = rec_ck;
+    I.cr = rec_cr;
+    I.cv = rec_cv;
+    I.verdict = verdict;
+    I.dead = lp_dead;
+    I.st = st;
+    (k_init_work<<<(unsigned)std::min<int64_t>(std::max<int64_t>((std::max(m0, n0) + 255) / 256, 1), 8 * 152), 256, 0,
+                   s>>>(I), note_launch());
     if (o.dual_records) {  // no source (-1, round -1: read as 0); no candidate row yet
         fill_i32(reinterpret_cast<int32_t *>(rec_bs), 4 * (int64_t)n0, -1, s);
         fill_i32(reinterpret_cast<int32_t *>(bsrc), 2 * (int64_t)n0, INT32_MAX, s);
@@ -663,35 +708,43 @@ void Engine::prepare() {
     n = n0;
     nnz = nnz0;
     cur = 0;
-    (k_set_i32<<<1, 1, 0, s>>>(&st->m_new, m0), note_launch());
-    (k_set_i32<<<1, 1, 0, s>>>(&st->n_new, n0), note_launch());
-    schedule_current();
+    // sizes for the schedules: k_init_work (none if a check failed, so that
+    // they read no unchecked pointer)
+    schedule_current(want_t);
     read_status();  // also keeps offs alive until its copy is done
-    if (st_h->err) throw StatusError(LPP_ERR_INVALID, "invalid LP (checks failed: vectors)");
-    adopt_schedule();
-    t_fixed = t_orig;  // from here on T and its schedule stay the input's
+    check_status();
+    adopt_schedule(want_t);
 }
 
-// Launches the schedule builds of the current CSR and CSC (not of a CSC kept
-// as the input's); the segment counts are read from st->m_new / st->n_new on
-// the device (m, n bound them).
-void Engine::schedule_current() {
-    build_schedule(rp[cur], &st->m_new, m, nnz, sa, st->cls_r, &st->nchunk_r, s);
-    if (!t_fixed) build_schedule(tp[cur], &st->n_new, n, nnz, sb, st->cls_c, &st->nchunk_c, s);
+void Engine::check_status() {
+    if (!st_h->err) return;
+    char buf[160];
+    std::snprintf(buf, sizeof buf,
+                  "invalid LP (checks failed: %s%s%s%s%s)", (st_h->err & 1) ? "row_ptr " : "",
+                  (st_h->err & 2) ? "col_idx-range " : "", (st_h->err & 4) ? "val-not-finite-or-zero " : "",
+                  (st_h->err & 8) ? "col_idx-not-increasing " : "", (st_h->err & 16) ? "vectors" : "");
+    throw StatusError(LPP_ERR_INVALID, buf);
+}
+
+// Launches the schedule builds of the current CSR and (cols) CSC; the segment
+// counts are read from st->m_new / st->n_new on the device (m, n bound them).
+void Engine::schedule_current(bool cols) {
+    build_schedule(m_rp, &st->m_new, m, nnz, sa, st->cls_r, &st->nchunk_r, s);
+    if (cols) build_schedule(tp[cur], &st->n_new, n, nnz, sb, st->cls_c, &st->nchunk_c, s);
     LPP_CUDA(cudaGetLastError());
 }
 
 // After read_status(): the host copies of the current schedules.
-void Engine::adopt_schedule() {
-    A.ptr = rp[cur];
-    A.idx = ci[cur];
-    A.val = rv[cur];
+void Engine::adopt_schedule(bool cols) {
+    A.ptr = m_rp;
+    A.idx = m_ci;
+    A.val = m_rv;
     A.order = sa.order;
     A.chunks = sa.chunks;
     A.lfirst = sa.lfirst;
     A.cnt = m;
     segmat_from_counts(A, st_h->cls_r, st_h->nchunk_r);
-    if (t_fixed) {
+    if (!cols) {
         if (A.cls_start[kNumClass] != m) throw StatusError(LPP_ERR_CUDA, "internal: schedule does not cover every segment");
         return;
     }
@@ -708,9 +761,7 @@ void Engine::adopt_schedule() {
 }
 
 void Engine::read_status() {
-    LPP_CUDA(cudaMemcpyAsync(st_h, st, sizeof(DevStatus), cudaMemcpyDeviceToHost, s));
-    LPP_CUDA(cudaMemcpyAsync(verdict_h, verdict, sizeof(int32_t) * (size_t)nlp * V_SLOTS, cudaMemcpyDeviceToHost, s));
-    LPP_CUDA(cudaMemcpyAsync(changed_h, lp_changed, (size_t)nlp, cudaMemcpyDeviceToHost, s));
+    LPP_CUDA(cudaMemcpyAsync(st_h, st, st_bytes, cudaMemcpyDeviceToHost, s));
     LPP_CUDA(cudaStreamSynchronize(s));
 }
 
@@ -731,10 +782,8 @@ Ctx Engine::ctx(int32_t round) const {
     C.c = c[cur];
     C.cmap = cmap[cur];
     C.lp_col = lpcol[cur];
-    C.t_orig = t_orig ? 1 : 0;
-    C.rinv = rinv;
+    C.in_place = in_place ? 1 : 0;
     C.cinv = cinv;
-    C.clen = t_orig ? clive : nullptr;
     C.act = act[cur];
     C.ninf = ninf[cur];
     C.rdirty = rdirty[cur];
@@ -811,11 +860,10 @@ void Engine::compact(int32_t round) {
     K.rp2 = rp[nx];
     K.ci2 = ci[nx];
     K.rv2 = rv[nx];
-    K.cp2 = t_orig ? nullptr : tp[nx];
-    K.ri2 = t_orig ? nullptr : ti[nx];
-    K.cv2 = t_orig ? nullptr : tv[nx];
-    K.rinv = t_orig ? rinv : nullptr;
-    K.cinv = t_orig ? cinv : nullptr;
+    K.cp2 = in_place ? nullptr : tp[nx];
+    K.ri2 = in_place ? nullptr : ti[nx];
+    K.cv2 = in_place ? nullptr : tv[nx];
+    K.cinv = cinv;
     K.L2 = L[nx];
     K.U2 = U[nx];
     K.rmap2 = rmap[nx];
@@ -829,40 +877,36 @@ void Engine::compact(int32_t round) {
     K.ninf2 = ninf[nx];
     K.hrow2 = hrow[nx];
     const Ctx C = ctx(round);
-    // columns kept in place (t_orig): their counts are updated in place, no
-    // column scan, no column vectors moved; the slots of the columns that
-    // leave are marked (cinv) and dropped once, at the end
-    int32_t *own_clen = K.c_len;
-    if (t_orig) K.c_len = clive;
     tbegin(F_COUNT, 4.0 * nnz * 2 + 8.0 * nnz + 24.0 * m + 40.0 * n);
     ensure_side_stream();
     const SideStream side{s_long, ev_fork, ev_join};
     launch_compact_counts(C, K, s, &side);
     tend();
-    tbegin(F_SCAN, 16.0 * (m + (t_orig ? 0 : n)) * 2);
+    // columns in place: no column scan, no column vectors moved; the slots of
+    // the columns that leave are marked (cinv) and dropped once, at the end
+    tbegin(F_SCAN, 16.0 * (m + (in_place ? 0 : n)) * 2);
     scan_excl2(K.r_keep, K.r_len, K.r_pos, K.r_off, m, scan_tmp, s);
-    if (!t_orig) scan_excl2(K.c_keep, K.c_len, K.c_pos, K.c_off, n, scan_tmp, s);
+    if (!in_place) scan_excl2(K.c_keep, K.c_len, K.c_pos, K.c_off, n, scan_tmp, s);
     tend();
     // the objective constant of the columns that left: with the columns in
-    // place (t_orig) each slot's contribution stays until one sum at the end
-    if (!t_orig) launch_offset(C, K, s);
-    (k_sizes<<<1, 1, 0, s>>>(K, m, n, t_orig ? 1 : 0, st), note_launch());
+    // place each slot's contribution stays until one sum at the end
+    if (!in_place) launch_offset(C, K, s);
     tbegin(F_SCATTER, 24.0 * nnz * 2 + 48.0 * (m + n));
     launch_compact_scatter(C, K, (int32_t)nnz, s);
     tend();
     LPP_CUDA(cudaGetLastError());
-    K.c_len = own_clen;
     // the next buffers become current; sizes and schedules are read back at
     // the end of the round (one host sync per round)
-    if (t_orig) {  // the column vectors stay where they are: they move with cur
+    if (in_place) {  // the column vectors stay where they are: they move with cur
         std::swap(lu[cur], lu[nx]);
         std::swap(c[cur], c[nx]);
         std::swap(cmap[cur], cmap[nx]);
         std::swap(lpcol[cur], lpcol[nx]);
     }
     cur = nx;
+    set_matrix();
     tbegin(F_SCHED, 8.0 * (m + n));
-    schedule_current();
+    schedule_current(!in_place);
     tend();
 }
 
@@ -888,18 +932,11 @@ Engine::StepOut Engine::step(int32_t r, bool first_round, bool force) {
     r_nnz.push_back(nnz);
     nnz_processed += nnz;
     LPP_CUDA(cudaEventRecord(ev_round[0], s));
-    LPP_CUDA(cudaMemsetAsync(st, 0, 8 * sizeof(int32_t), s));
-    LPP_CUDA(cudaMemsetAsync(lp_changed, 0, (size_t)nlp, s));
-    if (m > 0) LPP_CUDA(cudaMemsetAsync(rdnext, 0, (size_t)m, s));
-    // the column lists of S3' start empty; outside a first round only listed
-    // columns are finalised, the others keep kind KEPT and no change flag
-    LPP_CUDA(cudaMemsetAsync(col_cnt, 0, 3 * sizeof(int32_t), s));
-    if (!first_round && n > 0) {
-        LPP_CUDA(cudaMemsetAsync(ckind, 0, (size_t)n, s));
-        LPP_CUDA(cudaMemsetAsync(cchg, 0, (size_t)n, s));
-    }
     Ctx C = ctx(r);
     C.list_touched = first_round ? 0 : 1;  // a first round's S3' checks every column
+    // outside a first round only listed columns are finalised, the others keep
+    // kind KEPT and no change flag
+    launch_round_start(C, !first_round, s);
     tbegin(F_PROP, 0.0);  // bytes and ops set once the evaluated nonzeros are known
     const size_t prop_mark = marks.size();
     // the long rows' chunk kernels on a second stream, beside the short
@@ -918,7 +955,7 @@ Engine::StepOut Engine::step(int32_t r, bool first_round, bool force) {
     tbegin(F_COLFIN, 33.0 * n);
     if (o.dual_records) launch_bound_src(C, s);
     launch_colfin(C, first_round, s);
-    launch_mark_dirty(C, nnz, s);
+    if (!in_place) launch_mark_dirty(C, nnz, s);
     tend();
     LPP_CUDA(cudaGetLastError());
     // S5: leader passes.  Skipped when the last S5 resolved every key group
@@ -928,10 +965,8 @@ Engine::StepOut Engine::step(int32_t r, bool first_round, bool force) {
     int32_t tcap = std::min(tcap_max, pow2_at_least(2 * (int64_t)std::max(m, 1)));
     tbegin(F_S5, run_s5 ? 16.0 * tcap + 12.0 * m : 0.0);
     if (run_s5) {
-        LPP_CUDA(cudaMemsetAsync(tkey, 0, sizeof(unsigned long long) * tcap, s));
-        LPP_CUDA(cudaMemsetAsync(tlead, 0xff, sizeof(unsigned long long) * tcap, s));
+        launch_s5_init(C, tcap, s5_cnt, o.par_max_iter + 2, s);
         C.tcap = tcap;
-        LPP_CUDA(cudaMemsetAsync(s5_cnt, 0, sizeof(int32_t) * (size_t)(o.par_max_iter + 2), s));
         C.s5_out = s5_list[0];
         C.s5_out_cnt = s5_cnt + 1;
         launch_s5_pass(C, s);
@@ -958,8 +993,7 @@ Engine::StepOut Engine::step(int32_t r, bool first_round, bool force) {
     if (n1 > 0 && o.par_max_iter > 1) {
         tbegin(F_S5, 0.0);
         tcap = std::min(tcap_max, pow2_at_least(2 * (int64_t)n1));
-        LPP_CUDA(cudaMemsetAsync(tkey, 0, sizeof(unsigned long long) * tcap, s));
-        LPP_CUDA(cudaMemsetAsync(tlead, 0xff, sizeof(unsigned long long) * tcap, s));
+        launch_s5_init(C, tcap, nullptr, 0, s);
         C.tcap = tcap;
         int32_t chunk = 2, left = n1;
         for (int32_t pass = 1; pass < o.par_max_iter;) {
@@ -1028,8 +1062,18 @@ Engine::StepOut Engine::step(int32_t r, bool first_round, bool force) {
     }
     out.structural = first_round || force || st_h->rows_removed > 0 || st_h->cols_fixed > 0 || newly_dead;
     const int32_t rows_removed = st_h->rows_removed, bounds = st_h->bounds_changed;
-    if (out.structural) compact(r);
-    else std::swap(rdirty[cur], rdnext);  // same numbering: next round's flags
+    if (out.structural) {
+        compact(r);
+    } else {  // same numbering: next round's flags
+        if (in_place && bounds > 0) {
+            tbegin(F_COLFIN, 5.0 * nnz);
+            ensure_side_stream();
+            const SideStream side{s_long, ev_fork, ev_join};
+            launch_inplace_rows(C, K, false, s, &side);
+            tend();
+        }
+        std::swap(rdirty[cur], rdnext);
+    }
     LPP_CUDA(cudaEventRecord(ev_round[1], s));
     read_status();
     if (st_h->err) throw StatusError(LPP_ERR_CUDA, "internal: S5 hash table overflow");
@@ -1042,7 +1086,7 @@ Engine::StepOut Engine::step(int32_t r, bool first_round, bool force) {
         m = m_new;
         n = n_new;
         nnz = nnz_new;
-        adopt_schedule();
+        adopt_schedule(!in_place);
     }
     LPP_CUDA(cudaEventElapsedTime(&out.ms, ev_round[0], ev_round[1]));
     r_ms.push_back(out.ms);
@@ -1152,11 +1196,12 @@ void Engine::run_s5e(const Ctx &C) {
         std::swap(tp[0], tp[1]);
         std::swap(ti[0], ti[1]);
         std::swap(tv[0], tv[1]);
+        set_matrix();
         nnz = nnz2;
-        schedule_current();
+        schedule_current(true);
         read_status();
         if (st_h->err) throw StatusError(LPP_ERR_CUDA, "internal: S5e rewrite placed an entry outside its row");
-        adopt_schedule();
+        adopt_schedule(true);
         launch_s5e_mark(ctx(C.round), de, nj, s);
         LPP_CUDA(cudaGetLastError());
     }
@@ -1211,10 +1256,13 @@ void Engine::run() {
         }
     }
     if (o.dep_rows && nlp == 1 && lp_status[0] == LPP_OK) remove_dependent();
-    if (t_orig) {
+    if (in_place) {
         launch_offset(ctx(rounds), K, s);  // every slot's contribution, once, in column order
         finish_cols();
         finish_csc();
+        read_status();
+        if (st_h->n_new < 0 || st_h->n_new > n) throw StatusError(LPP_ERR_CUDA, "internal: column compaction size");
+        n = st_h->n_new;
     }
     float lms = 0.f;
     LPP_CUDA(cudaEventRecord(eend, s));
@@ -1297,7 +1345,7 @@ void Engine::remove_dependent() {
     m = m_new;
     n = n_new;
     nnz = nnz_new;
-    adopt_schedule();
+    adopt_schedule(!in_place);
     for (int v = 0; v < V_SLOTS; v++)
         if (verdict_h[v] != kNone) {  // S6 found an unbounded column
             lp_status[0] = v == V_S6_COL ? LPP_UNBOUNDED : LPP_INFEASIBLE;
@@ -1323,45 +1371,35 @@ void Engine::finish_cols() {
     K.lp_col2 = lpcol[nx];
     const Ctx C = ctx(rounds);
     launch_cols_final(C, K, n, cinv, ci[cur], nnz, s);
-    (k_csc_sizes<<<1, 1, 0, s>>>(K, n, st), note_launch());  // n_new: the columns left
+    (k_cols_left<<<1, 1, 0, s>>>(K.c_pos, n, st), note_launch());
     LPP_CUDA(cudaGetLastError());
     tend();
-    read_status();
-    const int32_t n_new = st_h->n_new;
-    if (n_new < 0 || n_new > n) throw StatusError(LPP_ERR_CUDA, "internal: column compaction size");
     std::swap(lu[cur], lu[nx]);
     std::swap(c[cur], c[nx]);
     std::swap(cmap[cur], cmap[nx]);
     std::swap(lpcol[cur], lpcol[nx]);
-    n = n_new;
 }
 
-// The result's CSC when the rounds kept the input's: one compaction of the
-// input CSC (slot 0) to the rows and columns still in the LP, renumbered,
-// into the other slot, which then becomes the current one.  Its sizes must
-// be the current CSR's.
+// The result's A^T when the rounds kept the columns in place: the transpose of
+// the reduced CSR (fewer entries than the input's, and once instead of the
+// input's at ingest and its compaction here).  The other buffers, dead by now,
+// are its scratch.  n bounds the columns left (their count is still on the
+// device; pointers past it are not used).
 void Engine::finish_csc() {
-    tbegin(F_SCATTER, 24.0 * nnz0 + 12.0 * nnz + 16.0 * (m0 + n0));
-    launch_rows_left(rinv, m0, rleft, s);
-    Ctx C0 = ctx(rounds);
-    C0.rkind = rleft;
-    C0.m = m0;
-    C0.n = n0;
-    launch_csc_from_input_counts(C0, K, s);
-    scan_excl2(K.c_keep, K.c_len, K.c_pos, K.c_off, n0, scan_tmp, s);
-    const int o = 1;  // the slot not holding the input CSC
-    launch_csc_from_input_scatter(C0, K, nnz0, tp[o], ti[o], tv[o], s);
-    (k_csc_sizes<<<1, 1, 0, s>>>(K, n0, st), note_launch());
+    tbegin(F_SCATTER, 24.0 * nnz + 12.0 * nnz + 16.0 * (m + n));
+    const int nx = cur ^ 1;
+    int32_t *row_of = reinterpret_cast<int32_t *>(tv[nx]);
+    rows_of(rp[cur], m, nnz, row_of, s);
+    TransposeBufs tb;
+    tb.k0 = reinterpret_cast<uint32_t *>(ci[nx]);
+    tb.k1 = reinterpret_cast<uint32_t *>(ti[nx]);
+    tb.v0 = reinterpret_cast<int32_t *>(rv[nx]);
+    tb.v1 = reinterpret_cast<int32_t *>(rv[nx]) + nnz0;
+    tb.hist = t_hist;
+    tb.tmp = scan_tmp;
+    transpose(rp[cur], ci[cur], rv[cur], row_of, m, n, nnz, tb, tp[cur], ti[cur], tv[cur], s);
     LPP_CUDA(cudaGetLastError());
     tend();
-    read_status();
-    if (st_h->n_new != n || st_h->nnz_new_t != nnz)
-        throw StatusError(LPP_ERR_CUDA, "internal: result CSC sizes disagree with the CSR");
-    if (cur != o) {
-        std::swap(tp[0], tp[1]);
-        std::swap(ti[0], ti[1]);
-        std::swap(tv[0], tv[1]);
-    }
     T.ptr = tp[cur];
     T.idx = ti[cur];
     T.val = tv[cur];

@@ -138,16 +138,24 @@ struct Engine {
     double2 *ch_act;
     int2 *ch_ninf;
     int32_t tcap_max;
-    // The CSC kept as the input's A^T and the columns kept in place instead
-    // of compacted each round (set by setup when lazy_req and no step that
-    // reads columns' entries is on): input-to-current row map, column map
-    // (the slot itself while the column is in the LP, -1 once it left),
-    // entries per column in the current rows, and at the end the input rows
-    // still in the LP (columns and CSC are compacted once, at the end).
-    bool lazy_req = false, t_orig = false, t_fixed = false;
-    int32_t *rinv = nullptr, *cinv = nullptr, *clive = nullptr;
-    uint8_t *rleft = nullptr;
-    void finish_cols();  // the columns' one compaction (t_orig)
+    // The columns kept in place and no A^T during the rounds instead of both
+    // compacted each round (set by setup when lazy_req and no step that reads
+    // columns' entries is on): column map (the slot itself while the column is
+    // in the LP, -1 once it left); at the end the columns are compacted once
+    // and the result's A^T is the transpose of its CSR.  need_t: A^T of the
+    // input is built all the same (the persistent batch kernel starts from it).
+    bool lazy_req = false, in_place = false, need_t = false;
+    int32_t *cinv = nullptr;
+    // The first round reads a device input where it lies (no compaction has
+    // written the buffers yet): the current matrix's arrays.
+    const int32_t *m_rp = nullptr, *m_ci = nullptr;
+    const double *m_rv = nullptr;
+    void set_matrix() {
+        m_rp = rp[cur];
+        m_ci = ci[cur];
+        m_rv = rv[cur];
+    }
+    void finish_cols();  // the columns' one compaction (in place until then)
     // opts.dep_rows: the equality rows' dependencies found on the host and
     // the rows removed by one more compaction (single LP)
     void remove_dependent();
@@ -156,7 +164,7 @@ struct Engine {
     int32_t *rmap_rec = nullptr;
     int64_t dep_pivots = 0, dep_peeled = 0;
     int32_t dep_found = 0, dep_stopped = 0;
-    void finish_csc();   // the result's CSC from the input's (t_orig)
+    void finish_csc();   // the result's A^T (columns in place)
     // compaction work
     CompactCtx K;
     int32_t *scan_tmp;
@@ -173,11 +181,12 @@ struct Engine {
     int4 *rec_bs = nullptr;                         // bound sources (NULL unless opts.dual_records):
     int2 *bsrc = nullptr;                           // per original column, and this round's per column
     DevStatus *st;
-    DevStatus *st_h = nullptr;  // pinned mirror
+    DevStatus *st_h = nullptr;  // pinned mirror of st, the verdicts and the changed flags, one block
+    size_t st_bytes = 0;
     int32_t *verdict_h = nullptr;
     uint8_t *changed_h = nullptr;
     int32_t *s5_left_h = nullptr;  // rows still unmatched after a chunk of S5 passes
-    SegMat A, T;
+    SegMat A{}, T{};
     // per-LP results
     std::vector<int32_t> lp_rounds, lp_status, lp_where, lp_index, lp_round;
     std::vector<uint8_t> lp_done;
@@ -225,8 +234,9 @@ struct Engine {
     std::vector<uint8_t> lp_dropped;
     Ctx ctx(int32_t round) const;
     void read_status();
-    void schedule_current();
-    void adopt_schedule();
+    void schedule_current(bool cols);
+    void adopt_schedule(bool cols);
+    void check_status();  // throws if the input checks failed
     void compact(int32_t round);
     void run_s5c(const Ctx &C0);  // S5c: keys, the changed groups, their leader passes
     void run_s5d(const Ctx &C);   // S5d: column singletons, then a status read

@@ -40,7 +40,8 @@ void build_schedule(const int32_t *ptr, const int32_t *cnt_dev, int32_t cnt_max,
 void segmat_from_counts(SegMat &M, const int32_t cls[kNumClass], int32_t nchunks);
 GroupGrid group_grid(const SegMat &M);
 
-// Input checks: returns error bits in *err (device).  row_of[nnz] is filled.
+// Input checks: returns error bits in *err (device).  row_of (unless NULL)
+// gets the row of each entry from row_of[1] on.
 void check_csr(const int32_t *ptr, const int32_t *idx, const double *val, int32_t m, int32_t n, int64_t nnz,
                int32_t *row_of, int32_t *tmp, int32_t *err, cudaStream_t s);
 // Vectors: normalise |v| >= huge to +-inf, check NaN / wrong-signed infinity,
@@ -48,6 +49,8 @@ void check_csr(const int32_t *ptr, const int32_t *idx, const double *val, int32_
 void ingest_vectors(const double *lhs, const double *rhs, const double *lb, const double *ub, const double *c,
                     int32_t m, int32_t n, double huge, double *L, double *U, double2 *lu, double *cc, int32_t *err,
                     cudaStream_t s);
+// the row of each entry, row_of[0 .. nnz)
+void rows_of(const int32_t *ptr, int32_t m, int64_t nnz, int32_t *row_of, cudaStream_t s);
 // A^T in CSR form (stable: rows increasing inside each column).
 struct TransposeBufs {
     uint32_t *k0, *k1;  // keys [nnz]
@@ -72,6 +75,10 @@ void fill_i32(int32_t *a, int64_t cnt, int32_t v, cudaStream_t s);
 void split_lu(const double2 *lu, int32_t n, double *lb, double *ub, cudaStream_t s);
 
 // ---------------------------------------------------------------- k_round.cu
+// the round's flags and counters to zero (cols: the columns' too)
+void launch_round_start(const Ctx &C, bool cols, cudaStream_t s);
+// an empty S5 table of cap slots, cnt[0 .. passes) zero
+void launch_s5_init(const Ctx &C, int32_t cap, int32_t *cnt, int32_t passes, cudaStream_t s);
 // S1-S3: the rows of classes 0-5 (launch_prop_short) and the chunked long
 // rows (launch_prop_long) touch disjoint rows and meet only in atomics, so
 // they may run on two streams at once
@@ -217,19 +224,17 @@ struct SideStream {
     cudaEvent_t fork, join;
 };
 void launch_compact_counts(const Ctx &C, const CompactCtx &K, cudaStream_t s, const SideStream *side = nullptr);
+// columns in place: the rows of changed columns marked for the next round (a round that removed nothing)
+void launch_inplace_rows(const Ctx &C, const CompactCtx &K, bool count, cudaStream_t s,
+                         const SideStream *side = nullptr);
+void launch_lp_dead(const Ctx &C, const CompactCtx &K, cudaStream_t s);
 void launch_compact_scatter(const Ctx &C, const CompactCtx &K, int32_t nnz, cudaStream_t s);
-// the result's CSC from the input CSC when it was not compacted (Ctx::t_orig):
-// counts and keep flags, then (after the caller's column scan) the scatter
-void launch_rows_left(const int32_t *rinv, int32_t m, uint8_t *rk, cudaStream_t s);
-// columns kept in place (Ctx::t_orig): their keep flags, then (after the
+// columns kept in place (Ctx::in_place): their keep flags, then (after the
 // caller's scan of them into K.c_pos) their vectors to K.lu2 / c2 / cmap2 /
 // lp_col2, cinv to final indices and the CSR's column indices renumbered
 void launch_cols_alive(const int32_t *cinv, int32_t n, int32_t *keep, cudaStream_t s);
 void launch_cols_final(const Ctx &C, const CompactCtx &K, int32_t n, int32_t *cinv, int32_t *idx, int64_t nnz,
                        cudaStream_t s);
-void launch_csc_from_input_counts(const Ctx &C, const CompactCtx &K, cudaStream_t s);
-void launch_csc_from_input_scatter(const Ctx &C, const CompactCtx &K, int64_t nnz, int32_t *ptr, int32_t *idx,
-                                   double *val, cudaStream_t s);
 void launch_offset(const Ctx &C, const CompactCtx &K, cudaStream_t s);
 
 }  // namespace lpp

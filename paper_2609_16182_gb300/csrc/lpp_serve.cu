@@ -190,12 +190,13 @@ void Engine::init_empty() {
     m = n = 0;
     nnz = 0;
     cur = 0;
+    set_matrix();
     LPP_CUDA(cudaMemsetAsync(rp[0], 0, sizeof(int32_t), s));
     LPP_CUDA(cudaMemsetAsync(tp[0], 0, sizeof(int32_t), s));
     LPP_CUDA(cudaMemsetAsync(&st->m_new, 0, sizeof(int32_t) * 2, s));  // m_new, n_new
-    schedule_current();
+    schedule_current(true);
     read_status();
-    adopt_schedule();
+    adopt_schedule(true);
 }
 
 void Engine::append(int32_t slot, const lpp_lp &in, int32_t rbase, int32_t cbase, int32_t round0) {
@@ -297,9 +298,9 @@ void Engine::append(int32_t slot, const lpp_lp &in, int32_t rbase, int32_t cbase
 
 void Engine::reschedule() {
     k_sizes_set(m, n);
-    schedule_current();
+    schedule_current(true);
     read_status();
-    adopt_schedule();
+    adopt_schedule(true);
 }
 
 }  // namespace lpp
