@@ -15,8 +15,8 @@
 // then writes its entries from its own offset.
 #include <algorithm>
 
-#include "compact_dev.cuh"
 #include "lpp_launch.h"
+#include "phase_dev.cuh"
 
 namespace lpp {
 
@@ -37,14 +37,6 @@ __device__ __forceinline__ int32_t group_count(const int32_t *idx, int32_t beg, 
     int32_t c = 0;
     for (int32_t k = beg + lane; k < end; k += W) c += keep(idx[k]) ? 1 : 0;
     return group_sum<W>(c, group_mask<W>());
-}
-
-// The flat scatter's tile t starts at entry t * kFlatTile; the segment (or
-// chunk) [b, e) that holds that entry records itself.  Segments and chunks
-// are at most kFlatTile long, so each holds at most one tile start.
-__device__ __forceinline__ void mark_tile(int32_t *tile, int32_t b, int32_t e, int32_t seg) {
-    const int64_t t = ((int64_t)b + kFlatTile - 1) / kFlatTile;
-    if (t * kFlatTile < e) tile[t] = seg;
 }
 
 // ---------------------------------------------------------------- CSC count
@@ -79,19 +71,6 @@ __global__ void __launch_bounds__(kBlock) k_csc_count_groups(Ctx C, CompactCtx K
     }
 }
 
-__device__ __forceinline__ int32_t block_sum_int(int32_t v) {
-    __shared__ int32_t s_w[kBlock / 32];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) s_w[threadIdx.x >> 5] = v;
-    __syncthreads();
-    int32_t t = 0;
-    if (threadIdx.x == 0)
-        for (int w = 0; w < kBlock / 32; w++) t += s_w[w];
-    __syncthreads();
-    return t;
-}
-
 __global__ void __launch_bounds__(kBlock) k_csc_count_long(Ctx C, CompactCtx K) {
     const Chunk ch = C.T.chunks[blockIdx.x];
     int32_t c = 0;
@@ -104,39 +83,10 @@ __global__ void __launch_bounds__(kBlock) k_csc_count_long(Ctx C, CompactCtx K) 
     }
 }
 
-// per long segment (one warp): chunk offsets (prefix in chunk order), the
-// total, and the sum of the chunks' side shifts (lane-strided, then a butterfly)
 __global__ void k_long_prefix(const SegMat M, const int32_t *ch_cnt, int32_t *ch_off, int32_t *len_out,
                               const double *ch_shift, double *shift_out) {
-    const int32_t t = (int32_t)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
-    const int lane = threadIdx.x & 31;
-    const int32_t nlong = M.cls_start[7] - M.cls_start[6];
-    if (t >= nlong) return;  // the same t in the whole warp
-    const int32_t q1 = M.lfirst[t + 1];
-    int32_t carry = 0;
-    double sh = 0.0;
-    for (int32_t q0 = M.lfirst[t]; q0 < q1; q0 += 32) {
-        const int32_t q = q0 + lane;
-        const int32_t c = q < q1 ? ch_cnt[q] : 0;
-        int32_t inc = c;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int32_t y = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o) inc += y;
-        }
-        if (q < q1) {
-            ch_off[q] = carry + inc - c;
-            if (ch_shift) sh += ch_shift[q];
-        }
-        carry += __shfl_sync(0xffffffffu, inc, 31);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) sh += __shfl_xor_sync(0xffffffffu, sh, o);
-    if (lane == 0) {
-        const int32_t seg = M.order[M.cls_start[6] + t];
-        len_out[seg] = carry;
-        if (shift_out) shift_out[seg] = sh;
-    }
+    long_prefix(M, (int32_t)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5), ch_cnt, ch_off, len_out, ch_shift,
+                shift_out);
 }
 
 template <int W>
@@ -181,179 +131,25 @@ __global__ void __launch_bounds__(kBlock) k_locks_long(Ctx C, CompactCtx K) {
 
 // ------------------------------------------------------- S6 + column keep
 // (grid-stride over a grid of at most 8 blocks per SM: one block sum per block)
-// Columns in place (Ctx::in_place): a column that left in an earlier round
-// (cinv < 0) is skipped, a kept one with entries stays as it is (no S6 test
-// applies to it, its contribution is zero), and one that leaves now gets
-// cinv = -1.
 __global__ void __launch_bounds__(kBlock) k_colkeep(Ctx C, CompactCtx K) {
     int32_t fixed = 0;
     for (int32_t j = blockIdx.x * blockDim.x + threadIdx.x; j < C.n; j += gridDim.x * blockDim.x) {
-        if (C.in_place) {
-            const bool used = C.cchg[j] & CS_USED;
-            if (used && C.ckind[j] == CK_KEPT && !K.lp_dead[lp_of_col(C, j)]) continue;
-            if (C.cinv[j] < 0) continue;
-            K.c_len[j] = used;
-            fixed += colkeep_one(C, K, j);
-            if (!K.c_keep[j]) K.cinv[j] = -1;
-        } else {
-            fixed += colkeep_one(C, K, j);
-        }
+        fixed += C.in_place ? colkeep_in_place(C, K, j) : colkeep_one(C, K, j);
     }
     block_add(fixed, &C.st->cols_fixed);
 }
 
-// ------------------------------------- columns in place: the rows' one pass
-// Over a kept row's entries with one byte gathered per entry (its column's
-// state): entries left and the side shift (as csr_count_row, the same order),
-// whether a column's bounds changed (the row is then evaluated next round),
-// and the columns still used, marked for S6.  It takes the place of an A^T
-// of the input kept through the rounds: the transpose at ingest, the marking
-// of the changed columns' rows through it, the counts per column and their
-// decrements.  COUNT false: a round that removed nothing, the marking alone.
-template <bool COUNT>
-__device__ __forceinline__ void inplace_entry(const Ctx &C, int32_t j, uint8_t st) {
-    if (COUNT && !(st & (CS_LEAVES | CS_USED))) C.cchg[j] = st | CS_USED;  // every writer stores the same byte
-}
+__global__ void __launch_bounds__(kBlock) k_suspect_rows(Ctx C, RowGrid R) { suspect_block(C, R, blockIdx.x); }
+__global__ void __launch_bounds__(kBlock) k_suspect_long(Ctx C) { suspect_chunk(C, blockIdx.x); }
 
-template <int W, bool COUNT>
-__device__ __forceinline__ void inplace_row(const Ctx &C, const CompactCtx &K, int32_t i, bool valid) {
-    const unsigned mask = group_mask<W>();
-    const int lane = threadIdx.x & (W - 1);
-    const bool keep = valid && C.rkind[i] == RK_KEPT && !K.lp_dead[lp_of_row(C, i)];
-    int32_t beg = 0, end = 0;
-    if (valid) {
-        beg = C.A.ptr[i];
-        end = C.A.ptr[i + 1];
-        if (COUNT && lane == 0) mark_tile(K.tile_a, beg, end, i);
-    }
-    int32_t cnt = 0, any = 0;
-    double sh = 0.0;
-    for (int32_t k0 = beg + lane; keep && k0 < end; k0 += 4 * W) {
-        int32_t jq[4];
-        uint8_t sq[4];
-#pragma unroll
-        for (int q = 0; q < 4; q++) jq[q] = k0 + q * W < end ? C.A.idx[k0 + q * W] : -1;
-#pragma unroll
-        for (int q = 0; q < 4; q++) sq[q] = jq[q] >= 0 ? C.cchg[jq[q]] : (uint8_t)0;
-#pragma unroll
-        for (int q = 0; q < 4; q++) {
-            if (jq[q] < 0) break;
-            any |= sq[q] & CS_CHANGED;
-            if (!COUNT) continue;
-            if (sq[q] & CS_LEAVES) sh = fma(C.A.val[k0 + q * W], C.fixv[jq[q]], sh);
-            else cnt++;
-            inplace_entry<COUNT>(C, jq[q], sq[q]);
-        }
-    }
-    any = group_sum<W>(any, mask);
-    if (COUNT) {
-        cnt = group_sum<W>(cnt, mask);
-        sh = group_sum<W>(sh, mask);
-    }
-    if (valid && lane == 0) {
-        if (any) C.rdnext[i] = 1;
-        if (COUNT) {
-            K.r_keep[i] = keep;
-            K.r_len[i] = cnt;
-            K.shift[i] = sh;
-        }
-    }
-}
-
-// A row of 257 to 4096 entries by the whole block, 1024 entries in flight.
-// The shift's 32 lane-strided chains run in one warp, from shared memory, in
-// the tiles that hold a leaving column's entry.
-constexpr int32_t kMidRow = 257;
-constexpr int kMidStep = 4 * kBlock;
 template <bool COUNT>
-__device__ __forceinline__ void inplace_mid(const Ctx &C, const CompactCtx &K, int32_t i, double *s_a, double *s_v,
-                                            int32_t *s_sum) {
-    const int tid = threadIdx.x, lane = tid & 31;
-    const int32_t beg = C.A.ptr[i], end = C.A.ptr[i + 1];
-    if (tid < 2) s_sum[tid] = 0;
-    int32_t cnt = 0, any = 0;
-    double sh = 0.0;
-    for (int32_t t0 = beg; t0 < end; t0 += kMidStep) {
-        int32_t jq[4];
-        uint8_t sq[4];
-#pragma unroll
-        for (int q = 0; q < 4; q++) jq[q] = t0 + q * kBlock + tid < end ? C.A.idx[t0 + q * kBlock + tid] : -1;
-#pragma unroll
-        for (int q = 0; q < 4; q++) sq[q] = jq[q] >= 0 ? C.cchg[jq[q]] : (uint8_t)0;
-        int32_t leaves = 0;
-#pragma unroll
-        for (int q = 0; q < 4; q++) {
-            if (jq[q] < 0) continue;
-            any |= sq[q] & CS_CHANGED;
-            if (!COUNT) continue;
-            leaves |= sq[q] & CS_LEAVES;
-            cnt += !(sq[q] & CS_LEAVES);
-            inplace_entry<COUNT>(C, jq[q], sq[q]);
-        }
-        if (COUNT && __syncthreads_or(leaves)) {
-#pragma unroll
-            for (int q = 0; q < 4; q++) {
-                const bool lv = jq[q] >= 0 && (sq[q] & CS_LEAVES);
-                s_a[q * kBlock + tid] = lv ? C.A.val[t0 + q * kBlock + tid] : 0.0;
-                s_v[q * kBlock + tid] = lv ? C.fixv[jq[q]] : 0.0;
-            }
-            __syncthreads();
-            if (tid < 32)
-                for (int32_t t = 0; t < kMidStep / 32; t++) sh = fma(s_a[32 * t + lane], s_v[32 * t + lane], sh);
-            __syncthreads();
-        }
-    }
-    __syncthreads();
-    any = __reduce_or_sync(0xffffffffu, (unsigned)any);
-    cnt = __reduce_add_sync(0xffffffffu, cnt);
-    if (lane == 0) {
-        if (any) s_sum[1] = 1;
-        if (cnt) atomicAdd(&s_sum[0], cnt);
-    }
-    if (COUNT && tid < 32) sh = group_sum<32>(sh, 0xffffffffu);
-    __syncthreads();
-    if (tid == 0) {
-        if (s_sum[1]) C.rdnext[i] = 1;
-        if (COUNT) {
-            mark_tile(K.tile_a, beg, end, i);
-            K.r_keep[i] = 1;
-            K.r_len[i] = s_sum[0];
-            K.shift[i] = sh;
-        }
-    }
-    __syncthreads();
+__global__ void __launch_bounds__(kBlock) k_inplace_rows(Ctx C, CompactCtx K, RowGrid R) {
+    __shared__ InplaceShared S;
+    inplace_block<COUNT>(C, K, R, blockIdx.x, S);
 }
-
-// class of a block whose grid starts with the longest rows (class 5)
 template <bool COUNT>
-__global__ void __launch_bounds__(kBlock) k_inplace_rows(Ctx C, CompactCtx K, GroupGrid g, int32_t per5) {
-    __shared__ double s_a[COUNT ? kMidStep : 1], s_v[COUNT ? kMidStep : 1];
-    __shared__ int32_t s_mid[kBlock / 32], s_nmid, s_sum[2];
-    const int c = 5 - grid_class(g, blockIdx.x);
-    const int W = 1 << c, at = threadIdx.x / W;
-    const int32_t per = c == 5 ? per5 : kBlock / W;
-    const int32_t pos = C.A.cls_start[c] + (blockIdx.x - g.blk_start[5 - c]) * per + at;
-    bool valid = at < per && pos < C.A.cls_start[c + 1];
-    const int32_t i = valid ? C.A.order[pos] : 0;
-    switch (c) {
-        case 0: inplace_row<1, COUNT>(C, K, i, valid); break;
-        case 1: inplace_row<2, COUNT>(C, K, i, valid); break;
-        case 2: inplace_row<4, COUNT>(C, K, i, valid); break;
-        case 3: inplace_row<8, COUNT>(C, K, i, valid); break;
-        case 4: inplace_row<16, COUNT>(C, K, i, valid); break;
-        default: {
-            if (threadIdx.x == 0) s_nmid = 0;
-            __syncthreads();
-            if (valid && C.A.ptr[i + 1] - C.A.ptr[i] >= kMidRow && C.rkind[i] == RK_KEPT && !K.lp_dead[lp_of_row(C, i)]) {
-                if ((threadIdx.x & 31) == 0) s_mid[atomicAdd(&s_nmid, 1)] = i;
-                valid = false;
-            }
-            inplace_row<32, COUNT>(C, K, i, valid);
-            __syncthreads();
-            const int32_t nmid = s_nmid;
-            for (int32_t t = 0; t < nmid; t++) inplace_mid<COUNT>(C, K, s_mid[t], s_a, s_v, s_sum);
-        }
-    }
+__global__ void __launch_bounds__(kBlock) k_inplace_long(Ctx C, CompactCtx K) {
+    inplace_chunk<COUNT>(C, K, blockIdx.x);
 }
 
 // --------------------------------------------------------------- CSR count
@@ -379,19 +175,6 @@ __global__ void __launch_bounds__(kBlock) k_csr_count_groups(Ctx C, CompactCtx K
     }
 }
 
-__device__ __forceinline__ double block_sum_dbl(double v) {
-    __shared__ double s_w[kBlock / 32];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) s_w[threadIdx.x >> 5] = v;
-    __syncthreads();
-    double t = 0.0;
-    if (threadIdx.x == 0)
-        for (int w = 0; w < kBlock / 32; w++) t += s_w[w];
-    __syncthreads();
-    return t;
-}
-
 __global__ void __launch_bounds__(kBlock) k_csr_count_long(Ctx C, CompactCtx K) {
     const Chunk ch = C.A.chunks[blockIdx.x];
     const int32_t i = ch.seg;
@@ -413,48 +196,6 @@ __global__ void __launch_bounds__(kBlock) k_csr_count_long(Ctx C, CompactCtx K) 
             }
         }
     }
-    cnt = block_sum_int(cnt);
-    sh = block_sum_dbl(sh);
-    if (threadIdx.x == 0) {
-        K.chr_cnt[blockIdx.x] = cnt;
-        K.chr_shift[blockIdx.x] = sh;
-        mark_tile(K.tile_a, ch.begin, ch.end, i);
-        if (ch.begin == C.A.ptr[i]) {  // the first chunk writes the flag
-            K.r_keep[i] = keep;
-            K.r_ch0[i] = blockIdx.x;
-        }
-    }
-}
-
-// the chunks of the long rows, columns in place
-template <bool COUNT>
-__global__ void __launch_bounds__(kBlock) k_inplace_long(Ctx C, CompactCtx K) {
-    const Chunk ch = C.A.chunks[blockIdx.x];
-    const int32_t i = ch.seg;
-    const bool keep = C.rkind[i] == RK_KEPT && !K.lp_dead[lp_of_row(C, i)];
-    int32_t cnt = 0, any = 0;
-    double sh = 0.0;
-    if (keep) {  // eight entries per thread and step in flight; the shift in entry order
-        for (int32_t k0 = ch.begin + threadIdx.x; k0 < ch.end; k0 += 8 * kBlock) {
-            int32_t jq[8];
-            uint8_t sq[8];
-#pragma unroll
-            for (int q = 0; q < 8; q++) jq[q] = k0 + q * kBlock < ch.end ? C.A.idx[k0 + q * kBlock] : -1;
-#pragma unroll
-            for (int q = 0; q < 8; q++) sq[q] = jq[q] >= 0 ? C.cchg[jq[q]] : (uint8_t)0;
-#pragma unroll
-            for (int q = 0; q < 8; q++) {
-                if (jq[q] < 0) break;
-                any |= sq[q] & CS_CHANGED;
-                if (!COUNT) continue;
-                if (sq[q] & CS_LEAVES) sh = fma(C.A.val[k0 + q * kBlock], C.fixv[jq[q]], sh);
-                else cnt++;
-                inplace_entry<COUNT>(C, jq[q], sq[q]);
-            }
-        }
-    }
-    if (__reduce_or_sync(0xffffffffu, (unsigned)any) && (threadIdx.x & 31) == 0) C.rdnext[i] = 1;
-    if (!COUNT) return;
     cnt = block_sum_int(cnt);
     sh = block_sum_dbl(sh);
     if (threadIdx.x == 0) {
@@ -508,23 +249,7 @@ __global__ void __launch_bounds__(kBlock) k_rowvec(Ctx C, CompactCtx K) {
     }
     const int32_t p = K.r_pos[i];
     if (!C.in_place) K.r_new[i] = K.r_keep[i] ? p : -1;
-    if (!K.r_keep[i]) return;
-    const double sh = K.shift[i];
-    const double Lv = C.L[i], Uv = C.U[i];
-    K.L2[p] = is_fin(Lv) ? Lv - sh : Lv;
-    K.U2[p] = is_fin(Uv) ? Uv - sh : Uv;
-    K.rmap2[p] = C.rmap[i];
-    if (C.lp_row) K.lp_row2[p] = C.lp_row[i];
-    K.rp2[p] = K.r_off[i];
-    // a row that lost entries (fixed columns) changed: evaluate it next round;
-    // its S5 key is taken again then, and an unchanged row's when columns were
-    // dropped (the key hashes column indices, which the compaction renumbers)
-    const bool lost = K.r_len[i] != C.A.ptr[i + 1] - C.A.ptr[i];
-    const bool renumbered = !C.in_place && K.c_pos[C.n] != C.n;
-    K.rdirty2[p] = (uint8_t)((C.rdnext[i] | lost ? 1 : 0) | (lost | renumbered ? 2 : 0));  // kEval, kRekey
-    K.act2[p] = C.act[i];
-    K.ninf2[p] = C.ninf[i];
-    K.hrow2[p] = C.hrow[i];
+    if (K.r_keep[i]) rowvec_one(C, K, i, p, K.r_off[i], !C.in_place && K.c_pos[C.n] != C.n);
 }
 
 __global__ void __launch_bounds__(kBlock) k_colvec(Ctx C, CompactCtx K) {
@@ -563,197 +288,9 @@ __global__ void k_empty(Ctx C, CompactCtx K) {
     }
 }
 
-// ---------------------------------------------------------------- scatter
-// Flat ordered compaction of all entries.  Segments of at most kFlatTile
-// entries, and the chunks of kChunk entries of the long ones, are the units.
-// Block t takes the entries [t T, t T + T) of the matrix, T = kFlatTile:
-//   1. one thread per segment between the segments of the entries t T and
-//      (t + 1) T (coalesced, independent loads) marks the first in-tile entry
-//      of each of its units in the tile, with a keep bit and the unit's base;
-//      a block max-scan of the marks gives every entry the first in-tile
-//      entry of its unit, or -1 if its segment is dropped;
-//   2. striped (coalesced): keep = unit kept and the other index kept (one
-//      gather of its new index, -1 if dropped); one ballot per warp and
-//      step, exclusive scan of the counts;
-//   3. striped: a kept entry x of unit s goes to
-//         off[s] + (kept entries of s before x),
-//      where the second term is scan(x) - scan(first in-tile entry of s) plus,
-//      for a unit that started in an earlier tile, len[s] minus its kept
-//      entries in this tile (it ends in this tile: it has at most T entries).
-struct FlatArgs {
-    const int32_t *ptr, *idx;
-    const double *val;
-    int32_t nnz, cnt, ntiles;
-    const int32_t *seg_keep, *seg_off, *seg_len;  // per segment: kept, new offset, kept entries
-    const int32_t *seg_ch0;                       // per long segment: its first chunk
-    const int32_t *ch_off, *ch_cnt;               // per chunk: kept entries of its segment before it, its own
-    const int32_t *oth_new;                       // per index of the other dimension: new index, -1 if dropped
-    const uint8_t *oth_state;                     // columns in place, instead: their states (they keep their index)
-    const int32_t *tile_seg;                      // per tile: segment of its first entry
-    int32_t *out_idx;
-    double *out_val;
-};
-
-constexpr int kFlatPer = kFlatTile / kBlock;  // entries per thread
-constexpr int kFlatWords = kFlatTile / 32;    // ballot words per tile
-
 __global__ void __launch_bounds__(kBlock) k_scatter_flat(FlatArgs F) {
-    __shared__ __align__(16) int16_t s_start[kFlatTile];
-    __shared__ int32_t s_raw[kFlatTile];
-    __shared__ unsigned s_bal[kFlatWords + 1];
-    __shared__ int32_t s_cb[kFlatWords + 1];
-    __shared__ int32_t s_wmax[kBlock / 32];
-    __shared__ int32_t s_re;
-    __shared__ int32_t s_fp;
-    const int t = blockIdx.x;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int32_t k0 = (int32_t)((int64_t)t * kFlatTile);
-    const int32_t len = F.nnz - k0 < kFlatTile ? F.nnz - k0 : kFlatTile;
-
-    // 1a. no marks; 1b. one thread per segment marks its units
-    {
-        int4 *w = reinterpret_cast<int4 *>(s_start);
-        for (int q = tid; q < kFlatTile / 8; q += kBlock) w[q] = make_int4(-1, -1, -1, -1);
-    }
-    if (tid == 0) s_fp = 0;
-    __syncthreads();
-    const int32_t lo = F.tile_seg[t];
-    const int32_t hi = t + 1 < F.ntiles ? F.tile_seg[t + 1] : F.cnt - 1;
-    const int32_t k1 = k0 + len;
-    for (int32_t r = lo + tid; r <= hi; r += kBlock) {
-        const int32_t pb = __ldg(F.ptr + r), pe = __ldg(F.ptr + r + 1);
-        if (pe <= pb || pb >= k1) continue;  // empty, or after the tile
-        const bool emit = F.seg_keep[r] != 0;
-        // units of r that meet the tile: the segment, or chunks q0..q1
-        int32_t q0 = 0, q1 = 0;
-        const bool lng = pe - pb >= kLongMin;
-        if (lng) {
-            q0 = ((pb > k0 ? pb : k0) - pb) / kChunk;
-            q1 = ((pe < k1 ? pe : k1) - 1 - pb) / kChunk;
-        }
-        for (int32_t q = q0; q <= q1; q++) {
-            const int32_t vb = pb + q * kChunk;
-            const int32_t ve = lng ? min(vb + kChunk, pe) : pe;
-            const int32_t xs = vb > k0 ? vb - k0 : 0;
-            s_start[xs] = (int16_t)(2 * xs + (emit ? 1 : 0));
-            if (emit) {
-                int32_t raw, ln;
-                if (lng) {
-                    const int32_t ch = F.seg_ch0[r] + q;
-                    raw = F.seg_off[r] + F.ch_off[ch];
-                    ln = F.ch_cnt[ch];
-                } else {
-                    raw = F.seg_off[r];
-                    ln = F.seg_len[r];
-                }
-                if (vb < k0) {  // the unit holding entry k0
-                    raw += ln;
-                    s_re = ve - k0;
-                    s_fp = 1;
-                }
-                s_raw[xs] = raw;
-            }
-        }
-    }
-    __syncthreads();
-    // 1c. inclusive max-scan of the marks (blocked, 16 per thread)
-    {
-        const int x0 = tid * kFlatPer;
-        int4 *w = reinterpret_cast<int4 *>(s_start + x0);
-        int4 a = w[0], b = w[1];
-        int16_t v[kFlatPer];
-        memcpy(v, &a, 16);
-        memcpy(v + 8, &b, 16);
-        int32_t run = -1;
-#pragma unroll
-        for (int e = 0; e < kFlatPer; e++) {
-            run = v[e] > run ? v[e] : run;
-        }
-        int32_t inc = run;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int32_t y = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o && y > inc) inc = y;
-        }
-        if (lane == 31) s_wmax[warp] = inc;
-        int32_t prev = __shfl_up_sync(0xffffffffu, inc, 1);
-        if (lane == 0) prev = -1;
-        __syncthreads();
-        for (int q = 0; q < warp; q++) prev = s_wmax[q] > prev ? s_wmax[q] : prev;
-        run = prev;
-#pragma unroll
-        for (int e = 0; e < kFlatPer; e++) {
-            run = v[e] > run ? v[e] : run;
-            v[e] = (x0 + e < len && (run & 1)) ? (int16_t)(run >> 1) : (int16_t)-1;
-        }
-        memcpy(&a, v, 16);
-        memcpy(&b, v + 8, 16);
-        w[0] = a;
-        w[1] = b;
-    }
-    __syncthreads();
-
-    // 2. keep flags, striped
-    int32_t jn[kFlatPer];
-#pragma unroll
-    for (int i = 0; i < kFlatPer; i++) {
-        const int x = i * kBlock + tid;
-        jn[i] = -1;
-        if (x < len && s_start[x] >= 0) jn[i] = F.idx[k0 + x];
-    }
-#pragma unroll
-    for (int i = 0; i < kFlatPer; i++) {
-        if (jn[i] >= 0) {
-            if (F.oth_state) jn[i] = F.oth_state[jn[i]] & CS_LEAVES ? -1 : jn[i];
-            else jn[i] = F.oth_new[jn[i]];
-        }
-        const unsigned bal = __ballot_sync(0xffffffffu, jn[i] >= 0);
-        if (lane == 0) s_bal[i * (kBlock / 32) + warp] = bal;
-    }
-    __syncthreads();
-    if (warp == 0) {  // exclusive scan of the ballot counts
-        constexpr int per = kFlatWords / 32;
-        int32_t c[per], tot = 0;
-#pragma unroll
-        for (int q = 0; q < per; q++) {
-            c[q] = __popc(s_bal[lane * per + q]);
-            tot += c[q];
-        }
-        int32_t inc = tot;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int32_t y = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o) inc += y;
-        }
-        int32_t acc = inc - tot;
-#pragma unroll
-        for (int q = 0; q < per; q++) {
-            s_cb[lane * per + q] = acc;
-            acc += c[q];
-        }
-        if (lane == 31) {
-            s_cb[kFlatWords] = inc;
-            s_bal[kFlatWords] = 0u;
-        }
-    }
-    __syncthreads();
-
-    // 3. positions and copies, striped
-    auto scan_at = [&](int y) {  // kept entries of the tile before position y (0 <= y <= T)
-        const int q = y >> 5;
-        return s_cb[q] + __popc(s_bal[q] & ((1u << (y & 31)) - 1u));
-    };
-    const int32_t fix = s_fp ? scan_at(s_re) : 0;
-#pragma unroll
-    for (int i = 0; i < kFlatPer; i++) {
-        if (jn[i] < 0) continue;
-        const int x = i * kBlock + tid;
-        const int xs = s_start[x];
-        int32_t p = s_raw[xs] - scan_at(xs) + scan_at(x);
-        if (xs == 0) p -= fix;
-        F.out_idx[p] = jn[i];
-        F.out_val[p] = F.val[k0 + x];
-    }
+    __shared__ FlatShared S;
+    flat_tile(F, blockIdx.x, S);
 }
 
 // ---------------------------------------------------------- objective constant
@@ -812,17 +349,8 @@ inline unsigned blocks_for(int64_t cnt, int threads) {
 }  // namespace
 
 void launch_inplace_rows(const Ctx &C, const CompactCtx &K, bool count, cudaStream_t s, const SideStream *side) {
-    GroupGrid g;  // the longest rows first (blk_start[k]: class 5 - k), few of them per block
-    int32_t acc = 0;
-    const int32_t cnt5 = C.A.cls_start[6] - C.A.cls_start[5];
-    const int32_t per5 = cnt5 <= 8 * 152 ? 1 : (cnt5 <= 32 * 152 ? 2 : 4);
-    for (int k = 0; k < 6; k++) {
-        const int c = 5 - k;
-        g.blk_start[k] = acc;
-        const int32_t per = c == 5 ? per5 : kBlock >> c;
-        acc += (C.A.cls_start[c + 1] - C.A.cls_start[c] + per - 1) / per;
-    }
-    g.blk_start[6] = acc;
+    const RowGrid R = class_grid(C.A);
+    const int32_t acc = R.g.blk_start[6];
     // the long rows' chunks (and their prefix) on the side stream: disjoint
     // rows, each tile start lies in one row, a column's state byte gets the
     // same value from every writer
@@ -845,8 +373,8 @@ void launch_inplace_rows(const Ctx &C, const CompactCtx &K, bool count, cudaStre
         }
     }
     if (acc > 0) {
-        if (count) (k_inplace_rows<true><<<acc, kBlock, 0, s>>>(C, K, g, per5), note_launch());
-        else (k_inplace_rows<false><<<acc, kBlock, 0, s>>>(C, K, g, per5), note_launch());
+        if (count) (k_inplace_rows<true><<<acc, kBlock, 0, s>>>(C, K, R), note_launch());
+        else (k_inplace_rows<false><<<acc, kBlock, 0, s>>>(C, K, R), note_launch());
     }
     if (fork) {
         cudaEventRecord(side->join, side->s);
@@ -865,6 +393,12 @@ static void launch_colkeep(const Ctx &C, const CompactCtx &K, cudaStream_t s) {
 void launch_compact_counts(const Ctx &C, const CompactCtx &K, cudaStream_t s, const SideStream *side) {
     launch_lp_dead(C, K, s);
     if (C.in_place) {  // the rows' one pass marks the columns in use, then S6
+        if (C.round > 1) {
+            const RowGrid R = class_grid(C.A);
+            if (R.g.blk_start[6] > 0) (k_suspect_rows<<<R.g.blk_start[6], kBlock, 0, s>>>(C, R), note_launch());
+            if (C.A.cls_start[7] > C.A.cls_start[6] && C.A.nchunks > 0)
+                (k_suspect_long<<<C.A.nchunks, kBlock, 0, s>>>(C), note_launch());
+        }
         launch_inplace_rows(C, K, true, s, side);
         launch_colkeep(C, K, s);
         return;

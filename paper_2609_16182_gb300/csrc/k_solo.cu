@@ -1,0 +1,626 @@
+// k_solo.cu -- all rounds of one LP in one cooperative kernel.
+//
+// A round of the launched path is some twenty kernels and two host reads; on
+// an LP of up to a few hundred thousand entries each of them is latency (5 to
+// 10 us), whatever the LP's size.  Here every round runs on the device: the
+// blocks stay resident and the steps of a round, the bodies the round's kernels
+// launch (phase_dev.cuh), are separated by grid barriers.  The control
+// decisions (which steps run, whether to compact, whether to stop) are taken
+// by every block alike from counters read after a barrier, as the host takes
+// them in Engine::step, so an LP gets the bits of the launched path.  A call on
+// 20 k rows (0.18 M entries, 13 rounds) takes 1.6 ms, 2.3 ms launched; on 200
+// rows (one block, its barriers block barriers) 0.83 ms, 1.16 ms launched.
+//
+// The columns stay in place (Ctx::in_place); row vectors and matrix alternate
+// between two buffers as there.  Counters exist twice, by the round's parity:
+// the next round's are cleared after the first barrier of a round, when no
+// block reads the previous round's any more.
+#include <algorithm>
+
+#include "../../include/lpp.h"
+#include "lpp_launch.h"
+#include "phase_dev.cuh"
+
+namespace lpp {
+
+namespace {
+
+union PhaseShared {
+    PropShared prop;
+    InplaceShared rows;
+    FlatShared flat;
+};
+
+struct SoloShared {
+    Ctx C;
+    CompactCtx K;
+    int32_t cls[kNumClass];
+    int32_t base[kNumClass], fill[kNumClass];  // the block's places per class
+    int32_t w[2 * (kBlock / 32)], tot[2], before[2];
+    int32_t pbase, kept;
+    int32_t n2;
+};
+
+// sums of two ints over the block, to every thread
+__device__ __forceinline__ int2 block_sum2(int32_t a, int32_t b, int32_t *s_w) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    a = __reduce_add_sync(0xffffffffu, a);
+    b = __reduce_add_sync(0xffffffffu, b);
+    __syncthreads();
+    if (lane == 0) {
+        s_w[warp] = a;
+        s_w[kBlock / 32 + warp] = b;
+    }
+    __syncthreads();
+    int2 t = make_int2(0, 0);
+#pragma unroll
+    for (int w = 0; w < kBlock / 32; w++) {
+        t.x += s_w[w];
+        t.y += s_w[kBlock / 32 + w];
+    }
+    return t;
+}
+
+// exclusive scan of two ints over the block; returns the totals
+__device__ __forceinline__ int2 block_scan2(int32_t a, int32_t b, int32_t &ea, int32_t &eb, int32_t *s_w) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int32_t xa = a, xb = b;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int32_t ya = __shfl_up_sync(0xffffffffu, xa, o), yb = __shfl_up_sync(0xffffffffu, xb, o);
+        if (lane >= o) {
+            xa += ya;
+            xb += yb;
+        }
+    }
+    __syncthreads();
+    if (lane == 31) {
+        s_w[warp] = xa;
+        s_w[kBlock / 32 + warp] = xb;
+    }
+    __syncthreads();
+    int2 t = make_int2(0, 0), p = make_int2(0, 0);
+#pragma unroll
+    for (int w = 0; w < kBlock / 32; w++) {
+        if (w == warp) p = t;
+        t.x += s_w[w];
+        t.y += s_w[kBlock / 32 + w];
+    }
+    ea = p.x + xa - a;
+    eb = p.y + xb - b;
+    return t;
+}
+
+__device__ __forceinline__ unsigned long long now_ns() {
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+    return t;
+}
+
+// rows [lo, hi) of a contiguous split of m rows over the grid, whole tiles of kBlock rows
+__device__ __forceinline__ void row_range(int32_t m, int32_t &lo, int32_t &hi) {
+    const int32_t tiles = (m + kBlock - 1) / kBlock, per = (tiles + gridDim.x - 1) / gridDim.x;
+    const int64_t a = (int64_t)blockIdx.x * per * kBlock;
+    lo = (int32_t)min((int64_t)m, a);
+    hi = (int32_t)min((int64_t)m, a + (int64_t)per * kBlock);
+}
+
+// The block's count of new rows per class is in S.cls: reserves its places
+// per class (S.base) among all blocks' in cls.  Every thread calls it.
+__device__ __forceinline__ void reserve_classes(SoloShared &S, int32_t *cls) {
+    __syncthreads();
+    if (threadIdx.x < kNumClass) {
+        const int32_t v = S.cls[threadIdx.x];
+        S.base[threadIdx.x] = v ? atomicAdd(cls + threadIdx.x, v) : 0;
+        S.fill[threadIdx.x] = 0;
+    }
+    __syncthreads();
+}
+
+// the rows [pb, pb + cnt) of ptr into order, by class (after a grid barrier on cls)
+__device__ __forceinline__ void fill_order(SoloShared &S, const int32_t *cls, const int32_t *ptr, int32_t pb,
+                                           int32_t cnt, int32_t *order) {
+    const int lane = threadIdx.x & 31;
+    int32_t start = 0;
+    for (int32_t t0 = 0; t0 < cnt; t0 += kBlock) {
+        const int32_t t = t0 + threadIdx.x;
+        const bool in = t < cnt;
+        const int c = in ? seg_class(ptr[pb + t + 1] - ptr[pb + t]) : kNumClass;
+        const unsigned peers = __match_any_sync(0xffffffffu, c);
+        const int first = __ffs(peers) - 1;
+        int32_t at = 0;
+        if (in && lane == first) at = atomicAdd(&S.fill[c], __popc(peers));
+        at = __shfl_sync(0xffffffffu, at, first);
+        if (in) {
+            start = 0;
+            for (int k = 0; k < c; k++) start += cls[k];
+            order[start + S.base[c] + at + __popc(peers & ((1u << lane) - 1u))] = pb + t;
+        }
+    }
+}
+
+// block 0: the chunks of the long rows (class 6, in schedule order)
+__device__ __forceinline__ void build_chunks(SoloShared &S, const int32_t *cls, const int32_t *ptr,
+                                             const int32_t *order, Chunk *chunks, int32_t *lfirst, int32_t *nchunk) {
+    int32_t start = 0;
+    for (int k = 0; k < 6; k++) start += cls[k];
+    const int32_t nlong = cls[6];
+    int32_t carry = 0;
+    for (int32_t t0 = 0; t0 < nlong; t0 += kBlock) {
+        const int32_t t = t0 + threadIdx.x;
+        int32_t sg = 0, pb = 0, pe = 0, v = 0, q, dummy;
+        if (t < nlong) {
+            sg = order[start + t];
+            pb = ptr[sg];
+            pe = ptr[sg + 1];
+            v = (pe - pb + kChunk - 1) / kChunk;
+        }
+        const int2 tot = block_scan2(v, 0, q, dummy, S.w);
+        if (t < nlong) {
+            q += carry;
+            lfirst[t] = q;
+            for (int32_t k = pb; k < pe; k += kChunk, q++) chunks[q] = Chunk{sg, k, min(pe, k + kChunk), t};
+        }
+        carry += tot.x;
+    }
+    if (threadIdx.x == 0) {
+        lfirst[nlong] = carry;
+        *nchunk = carry;
+    }
+}
+
+template <class F>
+__device__ __forceinline__ void each_block(int32_t total, F &&f) {
+    for (int32_t b = blockIdx.x; b < total; b += gridDim.x) {
+        f(b);
+        __syncthreads();  // the body's shared memory is reused
+    }
+}
+
+__global__ void __launch_bounds__(kBlock, 2) k_solo(const __grid_constant__ SoloArgs F) {
+    __shared__ SoloShared S;
+    __shared__ PhaseShared P;
+    const int tid = threadIdx.x;
+    const int32_t gt = blockIdx.x * kBlock + tid, gstep = gridDim.x * kBlock;
+    SoloCtl *ctl = F.ctl;
+    if (*F.err_in) return;  // the input checks failed (the same for every block)
+    int32_t m = F.m, nnz = F.nnz, cur = 0, nchunk = 0, rounds = 0, act_buf = 0, act_m = F.m;
+    const int32_t n = F.n;
+    uint8_t *rd = F.rdirty[0], *rd2 = F.rdirty[1], *rdnext = F.rdnext;
+    const int32_t *rp = F.in_rp, *ci = F.in_ci;
+    const double *rv = F.in_rv;
+    bool s5_clean = false;
+    long long s5_left = 0;
+    int32_t status = LPP_OK, where = LPP_WHERE_NONE, vindex = -1, vround = 0;
+    // every block takes the same branches, so each passes the same barriers
+#define GRID_SYNC()                                        \
+    do {                                                   \
+        if (!grid_barrier(ctl->bar, &ctl->err)) goto out;  \
+    } while (0)
+
+    // the input's rows by class
+    {
+        int32_t lo, hi;
+        row_range(m, lo, hi);
+        if (tid < kNumClass) S.cls[tid] = 0;
+        __syncthreads();
+        for (int32_t i = lo + tid; i < hi; i += kBlock) atomicAdd(&S.cls[seg_class(rp[i + 1] - rp[i])], 1);
+        reserve_classes(S, ctl->c[1].cls);
+        GRID_SYNC();
+        fill_order(S, ctl->c[1].cls, rp, lo, hi - lo, F.order);
+        GRID_SYNC();
+        if (ctl->c[1].cls[6] > 0) {
+            if (blockIdx.x == 0) build_chunks(S, ctl->c[1].cls, rp, F.order, F.chunks, F.lfirst, &ctl->c[1].nchunk);
+            GRID_SYNC();
+        }
+        nchunk = ctl->c[1].nchunk;
+        __syncthreads();
+        if (tid < kNumClass) S.cls[tid] = ctl->c[1].cls[tid];
+        __syncthreads();
+    }
+
+    for (int32_t r = 1; r <= F.max_rounds; r++) {
+        SoloCnt &N = ctl->c[r & 1], &X = ctl->c[(r & 1) ^ 1];
+        const unsigned long long t0 = now_ns();
+        const bool first = r == 1;
+        const int nx = cur ^ 1;
+        int32_t tcap = 2;
+        while (tcap < 2 * (int64_t)m && tcap < F.tcap_max) tcap <<= 1;
+        if (tid == 0) {
+            Ctx &C = S.C;
+            C = F.base;
+            C.A.ptr = rp;
+            C.A.idx = ci;
+            C.A.val = rv;
+            C.A.order = F.order;
+            C.A.chunks = F.chunks;
+            C.A.lfirst = F.lfirst;
+            C.A.cnt = m;
+            C.A.nchunks = nchunk;
+            C.A.cls_start[0] = 0;
+            for (int k = 0; k < kNumClass; k++) C.A.cls_start[k + 1] = C.A.cls_start[k] + S.cls[k];
+            C.m = m;
+            C.n = n;
+            C.round = r;
+            C.L = F.L[cur];
+            C.U = F.U[cur];
+            C.rmap = F.rmap[cur];
+            C.act = F.act[cur];
+            C.ninf = F.ninf[cur];
+            C.hrow = F.hrow[cur];
+            C.rdirty = rd;
+            C.rdnext = rdnext;
+            C.st = &N.st;
+            C.tl_cnt = &N.tl_cnt;
+            C.cl_cnt = &N.cl_cnt;
+            C.cl_nnz = &N.cl_nnz;
+            C.lp_changed = reinterpret_cast<uint8_t *>(&N.changed);
+            C.tcap = tcap;
+            C.s5_out = F.s5l[0];
+            C.s5_out_cnt = &N.n1;
+            C.list_touched = first ? 0 : 1;
+            CompactCtx &K = S.K;
+            K = F.K;
+            K.rp2 = F.rp[nx];
+            K.ci2 = F.ci[nx];
+            K.rv2 = F.rv[nx];
+            K.L2 = F.L[nx];
+            K.U2 = F.U[nx];
+            K.rmap2 = F.rmap[nx];
+            K.act2 = F.act[nx];
+            K.ninf2 = F.ninf[nx];
+            K.hrow2 = F.hrow[nx];
+            K.rdirty2 = rd2;
+        }
+        __syncthreads();
+        const Ctx &C = S.C;
+        const CompactCtx &K = S.K;
+        rounds = r;
+        act_buf = cur;
+        act_m = m;
+        const int32_t nlong = S.cls[6];
+        const bool run_s5 = first || !s5_clean;
+
+        // flags and the S5 table, beside S1-S3 (which touch neither)
+        for (int32_t i = gt; i < m; i += gstep) rdnext[i] = 0;
+        if (!first)
+            for (int32_t j = gt; j < n; j += gstep) {
+                C.ckind[j] = CK_KEPT;
+                C.cchg[j] = 0;
+            }
+        if (run_s5)
+            for (int32_t k = gt; k < tcap; k += gstep) {
+                C.tkey[k] = 0ULL;
+                C.tlead[k] = ~0ULL;
+            }
+        // S1-S3
+        int32_t removed = 0, u0 = 0, u1 = 0;
+        if (nlong > 0) each_block(nchunk, [&](int32_t b) { prop_long_chunk(C, b); });
+        {
+            const RowGrid R = prop_grid(C.A);
+            each_block(R.g.blk_start[6], [&](int32_t b) { prop_block(C, R, b, P.prop, removed, u0, u1); });
+        }
+        GRID_SYNC();
+        if (blockIdx.x == 0 && tid < (int)(sizeof(SoloCnt) / 4)) reinterpret_cast<int32_t *>(&X)[tid] = 0;
+        if (nlong > 0) {
+            for (int32_t t = gt >> 5; t < nlong; t += gstep >> 5) prop_long_row(C, t, removed, u0);
+            GRID_SYNC();
+            each_block(nchunk, [&](int32_t b) { prop_long_tighten(C, b, u1); });
+            GRID_SYNC();
+        }
+        warp_add(removed, &N.st.rows_removed);
+        removed = 0;
+        if (C.dual_rec) {
+            const RowGrid R = class_grid(C.A);
+            each_block(R.g.blk_start[6], [&](int32_t b) { bsrc_block(C, R, b); });
+            if (nlong > 0)
+                each_block(nchunk, [&](int32_t b) {
+                    const Chunk ch = C.A.chunks[b];
+                    if (C.rdirty[ch.seg]) bsrc_row(C, ch.seg, ch.begin + tid, ch.end, kBlock);
+                });
+            GRID_SYNC();
+        }
+        // S3' + S4 on the columns, S5's insertion on the rows (independent)
+        {
+            int32_t changed = 0, fixed = 0, z = 0;
+            if (first) {
+                for (int32_t j = gt; j < n; j += gstep) colfin_one(C, j, true, changed, fixed, z);
+            } else {
+                const int32_t cnt = N.tl_cnt;
+                for (int32_t t = gt; t < cnt; t += gstep) colfin_one(C, C.tl_list[t], false, changed, fixed, z);
+            }
+            __syncwarp();
+            warp_add(changed, &N.st.bounds_changed);
+            warp_add(fixed, &N.st.cols_fixed);
+            if (run_s5)
+                for (int32_t i = gt; i < m; i += gstep) {
+                    int32_t slot = -1;
+                    if (C.rkind[i] == RK_KEPT && rp[i + 1] - rp[i] >= 2) slot = s5_insert_row(C, i, (uint32_t)tcap);
+                    C.rslot[i] = slot;
+                    C.rwork[i] = slot >= 0 ? 1 : 0;
+                }
+        }
+        GRID_SYNC();
+        if (run_s5) {
+            // first pass: every row against its leader
+            int32_t um = 0;
+            const RowGrid R = class_grid(C.A);
+            each_block(R.g.blk_start[6], [&](int32_t b) {
+                int c;
+                bool valid;
+                const int32_t i = class_row(C.A, R, b, c, valid);
+                const bool left = match_class(C, c, i, valid, removed, um);
+                const unsigned want = __ballot_sync(0xffffffffu, left);
+                int32_t at = 0;
+                if ((tid & 31) == 0 && want) at = atomicAdd(&N.n1, __popc(want));
+                at = __shfl_sync(0xffffffffu, at, 0);
+                if (left) F.s5l[0][at + __popc(want & ((1u << (tid & 31)) - 1u))] = i;
+            });
+            each_block(nlong, [&](int32_t t) { match_long(C, t, F.s5l[0], &N.n1, removed, um); });
+            __syncwarp();
+            warp_add(removed, &N.merged);
+            removed = 0;
+            GRID_SYNC();
+            const int32_t n1 = N.n1;
+            int32_t left = n1;
+            if (n1 > 0 && F.par_max_iter > 1) {
+                // the table empty again, then the later passes: in one block for a
+                // short list, else over the grid
+                for (int32_t i = gt; i < m; i += gstep) {
+                    const int32_t sl = C.rslot[i];
+                    if (sl >= 0) {
+                        C.tkey[sl] = 0ULL;
+                        C.tlead[sl] = ~0ULL;
+                    }
+                }
+                GRID_SYNC();
+                const bool alone = n1 <= 8 * kBlock;
+                if (!alone || blockIdx.x == 0) {
+                    const int32_t ft = alone ? tid : gt, fs = alone ? kBlock : gstep;
+                    int32_t from = 0;
+                    int32_t *cnt = F.s5_cnt;  // [par_max_iter + 2], zero
+                    for (int32_t p = 1; p < F.par_max_iter && left > 0; p++) {
+                        const int32_t *lst = F.s5l[from];
+                        int32_t *nxt = F.s5l[from ^ 1];
+                        const uint32_t cap = s5_tail_cap(C, left);
+                        for (int32_t t = ft; t < left; t += fs) {
+                            const int32_t i = __ldcg(lst + t);
+                            C.rslot[i] = s5_insert_row(C, i, cap);
+                        }
+                        if (alone) __syncthreads();
+                        else GRID_SYNC();
+                        for (int32_t tb = ft & ~31; tb < left; tb += fs) {
+                            int32_t rm, i;
+                            bool lf;
+                            s5_tail_match_one(C, lst, left, tb + (tid & 31), rm, lf, i);
+                            removed += rm;
+                            const unsigned want = __ballot_sync(0xffffffffu, lf);
+                            int32_t at = 0;
+                            if ((tid & 31) == 0 && want) at = atomicAdd(cnt + p, __popc(want));
+                            at = __shfl_sync(0xffffffffu, at, 0);
+                            if (lf) nxt[at + __popc(want & ((1u << (tid & 31)) - 1u))] = i;
+                        }
+                        if (alone) __syncthreads();
+                        else GRID_SYNC();
+                        for (int32_t t = ft; t < left; t += fs) {
+                            const int32_t sl = __ldcg(C.rslot + __ldcg(lst + t));
+                            if (sl >= 0) {
+                                C.tkey[sl] = 0ULL;
+                                C.tlead[sl] = ~0ULL;
+                            }
+                        }
+                        const int32_t next = __ldcg(cnt + p);
+                        if (alone) __syncthreads();
+                        else GRID_SYNC();
+                        if (ft == 0) cnt[p] = 0;  // for the next round's passes (read by all above)
+                        left = next;
+                        from ^= 1;
+                    }
+                    __syncwarp();
+                    warp_add(removed, &N.merged);
+                    removed = 0;
+                    if (ft == 0) N.n2 = left;
+                }
+                GRID_SYNC();
+                left = N.n2;
+            }
+            s5_clean = left == 0;
+            s5_left += left;
+            if (N.merged > 0)
+                for (int32_t i = gt; i < m; i += gstep)
+                    if (C.hasf[i]) s5_leader_one(C, i);
+        }
+        if (N.st.rows_removed + N.merged > 0) {
+            if (!first) {  // the columns that may have become empty
+                const RowGrid R = class_grid(C.A);
+                each_block(R.g.blk_start[6], [&](int32_t b) { suspect_block(C, R, b); });
+                if (nlong > 0) each_block(nchunk, [&](int32_t b) { suspect_chunk(C, b); });
+            }
+            GRID_SYNC();
+        }
+        {
+            // the round's decisions, the same in every block
+            // (verdicts are read here and after S6's barrier, not at the round's
+            // end: another block may by then be in the next round's S2)
+            int v = 0;
+            while (v < V_SLOTS && C.verdict[v] == kNone) v++;
+            const bool dead = v < V_SLOTS;
+            const int32_t rows_removed = N.st.rows_removed + N.merged;
+            const bool structural = first || rows_removed > 0 || N.st.cols_fixed > 0 || dead;
+            const int32_t nnz0 = nnz;
+            if (dead) {
+                // the LP leaves empty: no rows, no columns, no contribution of the columns still in it
+                for (int32_t j = gt; j < n; j += gstep)
+                    if (C.cinv[j] >= 0) {
+                        K.contrib[j] = 0.0;
+                        K.cinv[j] = -1;
+                    }
+                if (blockIdx.x == 0 && tid == 0) K.rp2[0] = 0;
+                m = 0;
+                nnz = 0;
+                cur = nx;
+            } else if (structural) {
+                const RowGrid R = class_grid(C.A);
+                each_block(R.g.blk_start[6], [&](int32_t b) { inplace_block<true>(C, K, R, b, P.rows); });
+                if (nlong > 0) each_block(nchunk, [&](int32_t b) { inplace_chunk<true>(C, K, b); });
+                GRID_SYNC();
+                if (nlong > 0)
+                    for (int32_t t = gt >> 5; t < nlong; t += gstep >> 5)
+                        long_prefix(C.A, t, K.chr_cnt, K.chr_off, K.r_len, K.chr_shift, K.shift);
+                int32_t fixed = 0;
+                for (int32_t j = gt; j < n; j += gstep) fixed += colkeep_in_place(C, K, j);
+                __syncwarp();
+                warp_add(fixed, &N.st.cols_fixed);
+                if (nlong > 0) GRID_SYNC();
+                // new rows and offsets: the blocks' sums, then each block's own scan
+                int32_t lo, hi;
+                row_range(m, lo, hi);
+                int32_t ka = 0, la = 0;
+                for (int32_t i = lo + tid; i < hi; i += kBlock) {
+                    ka += K.r_keep[i];
+                    la += K.r_keep[i] ? K.r_len[i] : 0;
+                }
+                int2 bt = block_sum2(ka, la, S.w);
+                if (tid == 0) {
+                    F.btot[2 * blockIdx.x] = bt.x;
+                    F.btot[2 * blockIdx.x + 1] = bt.y;
+                }
+                GRID_SYNC();
+                while (v > 0 && C.verdict[v - 1] != kNone) v--;  // S6's slot is the last
+                ka = la = 0;
+                int32_t ta = 0, tb = 0;
+                for (int32_t b = tid; b < (int32_t)gridDim.x; b += kBlock) {
+                    const int32_t x = F.btot[2 * b], y = F.btot[2 * b + 1];
+                    ta += x;
+                    tb += y;
+                    if (b < (int32_t)blockIdx.x) {
+                        ka += x;
+                        la += y;
+                    }
+                }
+                const int2 all = block_sum2(ta, tb, S.w), pre = block_sum2(ka, la, S.w);
+                __syncthreads();
+                if (tid < kNumClass) S.cls[tid] = 0;
+                __syncthreads();
+                int32_t pos = pre.x, off = pre.y;
+                for (int32_t t0 = lo; t0 < hi; t0 += kBlock) {
+                    const int32_t i = t0 + tid;
+                    const bool kp = i < hi && K.r_keep[i];
+                    const int32_t ln = kp ? K.r_len[i] : 0;
+                    int32_t ea, eb;
+                    const int2 tt = block_scan2(kp ? 1 : 0, ln, ea, eb, S.w);
+                    if (i < hi) K.r_off[i] = off + eb;
+                    if (kp) {
+                        rowvec_one(C, K, i, pos + ea, off + eb, false);
+                        atomicAdd(&S.cls[seg_class(ln)], 1);
+                    }
+                    pos += tt.x;
+                    off += tt.y;
+                }
+                if (blockIdx.x == 0 && tid == 0) K.rp2[all.x] = all.y;
+                reserve_classes(S, X.cls);
+                GRID_SYNC();
+                // the kept entries, and the new rows by class
+                {
+                    const int32_t ntiles = (int32_t)(((int64_t)nnz + kFlatTile - 1) / kFlatTile);
+                    const FlatArgs fa{rp, ci, rv, nnz, m, ntiles, K.r_keep, K.r_off, K.r_len, K.r_ch0,
+                                      K.chr_off, K.chr_cnt, K.c_new, C.cchg, K.tile_a, K.ci2, K.rv2};
+                    each_block(ntiles, [&](int32_t b) { flat_tile(fa, b, P.flat); });
+                }
+                fill_order(S, X.cls, K.rp2, pre.x, pos - pre.x, F.order);
+                GRID_SYNC();
+                if (X.cls[6] > 0) {
+                    if (blockIdx.x == 0) build_chunks(S, X.cls, K.rp2, F.order, F.chunks, F.lfirst, &X.nchunk);
+                    GRID_SYNC();
+                }
+                nchunk = X.nchunk;
+                __syncthreads();
+                if (tid < kNumClass) S.cls[tid] = X.cls[tid];
+                m = all.x;
+                nnz = all.y;
+                cur = nx;
+                rp = F.rp[nx];
+                ci = F.ci[nx];
+                rv = F.rv[nx];
+                uint8_t *t = rd;
+                rd = rd2;
+                rd2 = t;
+            } else {
+                if (N.st.bounds_changed > 0) {
+                    const RowGrid R = class_grid(C.A);
+                    each_block(R.g.blk_start[6], [&](int32_t b) { inplace_block<false>(C, K, R, b, P.rows); });
+                    if (nlong > 0) each_block(nchunk, [&](int32_t b) { inplace_chunk<false>(C, K, b); });
+                }
+                GRID_SYNC();
+                uint8_t *t = rd;
+                rd = rdnext;
+                rdnext = t;
+            }
+            if (N.st.cols_fixed > 0) s5_clean = false;  // rows lost entries
+            if (blockIdx.x == 0 && tid == 0) {
+                int32_t *q = F.rstat + 6 * (int64_t)(r - 1);
+                q[0] = nnz0;
+                q[1] = rows_removed;
+                q[2] = N.st.cols_fixed;
+                q[3] = N.st.bounds_changed;
+                q[4] = (int32_t)(now_ns() - t0);
+                if (N.st.err) atomicOr(&ctl->err, N.st.err);
+            }
+            if (v < V_SLOTS) {
+                status = v == V_S6_COL ? LPP_UNBOUNDED : LPP_INFEASIBLE;
+                where = (v == V_S2_ROW || v == V_S5_ROW) ? LPP_WHERE_ROW : LPP_WHERE_COL;
+                vindex = C.verdict[v];
+                vround = r;
+                break;
+            }
+        }
+        if (!N.changed) break;
+        __syncthreads();  // every thread has read S before the next round rewrites it
+    }
+out:
+    if (blockIdx.x == 0 && tid == 0) {
+        SoloOut &o = ctl->out;
+        o.status = status;
+        o.where = where;
+        o.index = vindex;
+        o.round = vround;
+        o.rounds = rounds;
+        o.m = m;
+        o.nnz = nnz;
+        o.cur = cur;
+        o.act_buf = act_buf;
+        o.act_m = act_m;
+        o.s5_left = s5_left;
+    }
+#undef GRID_SYNC
+}
+
+}  // namespace
+
+// blocks of a cooperative launch of k_solo for an LP of these sizes, 0 if the
+// device cannot take one
+int solo_blocks(int32_t m, int32_t n, int64_t nnz) {
+    static int per_sm = -1, sms = 0;
+    if (per_sm < 0) {
+        int dev = 0, coop = 0, nb = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (coop) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_solo, kBlock, 0);
+        per_sm = coop ? nb : 0;
+    }
+    if (per_sm <= 0 || sms <= 0) return 0;
+    const int64_t want = std::max<int64_t>({1, ((int64_t)m + kBlock - 1) / kBlock, ((int64_t)n + 2 * kBlock - 1) / (2 * kBlock),
+                                            (nnz + 8 * kBlock - 1) / (8 * kBlock)});
+    return (int)std::min<int64_t>(want, (int64_t)per_sm * sms);
+}
+
+bool launch_solo(const SoloArgs &F, int blocks, cudaStream_t s) {
+    SoloArgs Fv = F;
+    void *args[] = {&Fv};
+    if (cudaLaunchCooperativeKernel((const void *)k_solo, dim3(blocks), dim3(kBlock), args, 0, s) != cudaSuccess) return false;
+    note_launch();
+    return true;
+}
+
+}  // namespace lpp

@@ -156,6 +156,36 @@ __global__ void __launch_bounds__(1024) k_scan_top(T *tsum, int32_t ntiles, Out 
     }
 }
 
+// A short array (at most kScanSmall elements) by one block, a launch instead of
+// three: eight values per thread and step (at the limit four steps, 12 us,
+// about what the three launches take).
+constexpr int64_t kScanSmall = 32768;
+template <class T, class In, class Out>
+__global__ void __launch_bounds__(1024) k_scan_one(In in, Out out, int64_t cnt) {
+    __shared__ T s_w[33];
+    T carry = zero_of<T>();
+    for (int64_t base = 0; base < cnt; base += 1024 * kPerThread) {
+        const int64_t k = base + (int64_t)threadIdx.x * kPerThread;
+        T v[kPerThread];
+        in.get8(k, cnt, v);
+        T s = zero_of<T>();
+#pragma unroll
+        for (int q = 0; q < kPerThread; q++) s = s + v[q];
+        T ex;
+        const T tot = block_excl_scan(s, ex, s_w);
+        T run = carry + ex;
+        T o[kPerThread];
+#pragma unroll
+        for (int q = 0; q < kPerThread; q++) {
+            o[q] = run;
+            run = run + v[q];
+        }
+        out.put8(k, cnt, o);
+        carry = carry + tot;
+    }
+    if (threadIdx.x == 0) out(cnt, carry);
+}
+
 template <class T, class In, class Out>
 __global__ void __launch_bounds__(kScanThreads) k_scan_down(In in, Out out, int64_t cnt, const T *tsum) {
     __shared__ T s_w[33];
@@ -544,15 +574,15 @@ __global__ void k_gather_t(const int32_t *perm, const int32_t *row_of, const dou
 }
 
 // A^T row pointers from the sorted column keys: key[p] starts column j's
-// run at p for every j in (key[p-1], key[p]]; columns after the last key end at nnz
+// run at p for every j in (key[p-1], key[p]]; columns after the last key end at
+// nnz, a thread each (n may be a bound far above it)
 __global__ void k_colptr_from_keys(const uint32_t *key, int64_t nnz, int32_t n, int32_t *tptr) {
     const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p <= n && p > (int64_t)key[nnz - 1]) tptr[p] = (int32_t)nnz;
     if (p >= nnz) return;
     const int32_t kp = (int32_t)key[p];
     const int32_t kq = p == 0 ? -1 : (int32_t)key[p - 1];
     for (int32_t j = kq + 1; j <= kp; j++) tptr[j] = (int32_t)p;
-    if (p == nnz - 1)
-        for (int32_t j = kp + 1; j <= n; j++) tptr[j] = (int32_t)nnz;
 }
 
 // segment lengths from a pointer array
@@ -582,6 +612,10 @@ inline unsigned blocks_for(int64_t cnt, int threads) {
 size_t scan_tmp_elems(int64_t cnt) { return 2 * ((size_t)((cnt + kScanTile - 1) / kScanTile) + 1); }
 
 void scan_excl(const int32_t *in, int32_t *out, int64_t cnt, int32_t *tmp, cudaStream_t s) {
+    if (cnt <= kScanSmall) {
+        (k_scan_one<int32_t><<<1, 1024, 0, s>>>(In1{in}, Out1{out}, cnt), note_launch());
+        return;
+    }
     const int32_t ntiles = (int32_t)((cnt + kScanTile - 1) / kScanTile);
     if (ntiles > 0) (k_scan_reduce<int32_t><<<ntiles, kScanThreads, 0, s>>>(In1{in}, cnt, tmp), note_launch());
     (k_scan_top<int32_t><<<1, 1024, 0, s>>>(tmp, ntiles, Out1{out}, cnt), note_launch());
@@ -590,6 +624,10 @@ void scan_excl(const int32_t *in, int32_t *out, int64_t cnt, int32_t *tmp, cudaS
 
 void scan_excl2(const int32_t *a, const int32_t *b, int32_t *oa, int32_t *ob, int64_t cnt, int32_t *tmp,
                 cudaStream_t s) {
+    if (cnt <= kScanSmall) {
+        (k_scan_one<Pair><<<1, 1024, 0, s>>>(In2{a, b}, Out2{oa, ob}, cnt), note_launch());
+        return;
+    }
     const int32_t ntiles = (int32_t)((cnt + kScanTile - 1) / kScanTile);
     Pair *t = reinterpret_cast<Pair *>(tmp);
     if (ntiles > 0) (k_scan_reduce<Pair><<<ntiles, kScanThreads, 0, s>>>(In2{a, b}, cnt, t), note_launch());
@@ -690,7 +728,8 @@ void transpose(const int32_t *ptr, const int32_t *idx, const double *val, const 
         vin = vbuf[p & 1];
     }
     (k_gather_t<<<blocks_for(nnz, 256), 256, 0, s>>>(vin, row_of, val, nnz, tidx, tval), note_launch());
-    (k_colptr_from_keys<<<blocks_for(nnz, 256), 256, 0, s>>>(kin, nnz, n, tptr), note_launch());
+    (k_colptr_from_keys<<<blocks_for(std::max<int64_t>(nnz, (int64_t)n + 1), 256), 256, 0, s>>>(kin, nnz, n, tptr),
+     note_launch());
 }
 
 void sort_pairs(const uint32_t *keys, const int32_t *vals, int64_t cnt, int bits, const TransposeBufs &b,

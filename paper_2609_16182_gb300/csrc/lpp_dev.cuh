@@ -49,7 +49,8 @@ enum : uint8_t {
 enum : uint8_t { CK_KEPT = 0, CK_FIXED = 1, CK_EMPTY = 2, CK_PARALLEL = 3, CK_SUBST = 4, CK_DOUBLETON = 5 };
 // verdict slots per LP, in step order
 // column states of a round with the columns in place (Ctx::cchg)
-enum : uint8_t { CS_CHANGED = 1, CS_LEAVES = 2, CS_USED = 4 };
+// (CS_SUSPECT: a row that left held it, so it may be empty now; CS_USED: a kept row holds it)
+enum : uint8_t { CS_CHANGED = 1, CS_LEAVES = 2, CS_USED = 4, CS_SUSPECT = 8 };
 enum { V_S2_ROW = 0, V_S3_COL = 1, V_S5_ROW = 2, V_S5E_COL = 3, V_S6_COL = 4, V_SLOTS = 5 };
 
 // Global counters of a round (block-aggregated atomics).
@@ -97,8 +98,7 @@ struct Ctx {
     // in_place: the columns stay in their input slots and no A^T is kept
     // during the rounds (no step that reads columns' entries is on).  cinv
     // maps an input column to its slot (-1 once it left); cchg then holds, per
-    // slot, CS_CHANGED and CS_LEAVES of this round and CS_USED, set by the
-    // pass over the kept rows' entries.
+    // slot, the CS_ bits of this round.
     const int32_t *cinv;
     int32_t in_place;
     // rows whose activities must be recomputed this round (1) and the flags

@@ -209,6 +209,7 @@ struct InitArgs {
     int32_t *verdict;
     uint8_t *dead;
     DevStatus *st;
+    double *offset, off0;  // one LP: its objective constant
 };
 __global__ void __launch_bounds__(256) k_init_work(InitArgs I) {
     const int32_t t = blockIdx.x * 256 + threadIdx.x, step = gridDim.x * 256;
@@ -238,6 +239,7 @@ __global__ void __launch_bounds__(256) k_init_work(InitArgs I) {
     for (int32_t k = t; k < I.nlp * V_SLOTS; k += step) I.verdict[k] = kNone;
     for (int32_t k = t; k < I.nlp; k += step) I.dead[k] = 0;
     if (t == 0) {
+        if (I.offset) I.offset[0] = I.off0;
         const bool ok = I.st->err == 0;
         I.st->m_new = ok ? I.m : 0;
         I.st->n_new = ok ? I.n : 0;
@@ -270,6 +272,7 @@ Engine::~Engine() {
     pool.release();
     if (s) cudaStreamSynchronize(s);
     pinned_put(st_h);
+    pinned_put(solo_h);
     pinned_put(s5_left_h);
     pinned_put(de_cnt_h);
     if (own_stream && s) cudaStreamDestroy(s);
@@ -369,6 +372,8 @@ void Engine::setup(const lpp_opts &opts, int32_t nlp_, const std::vector<Member>
     cchg = pool.alloc<uint8_t>(n0);
     in_place = lazy_req && !o.parallel_cols && !o.col_singletons && !o.dual_fixing && !o.doubletons;
     if (in_place) cinv = pool.alloc<int32_t>(n0);
+    solo = in_place && nlp == 1 && nnz0 <= kSoloNnz && !o.timing && !o.dep_rows && o.max_rounds > 0 &&
+           o.max_rounds <= 1024 && solo_blocks(m0, n0, nnz0) > 0;
     rkind = pool.alloc<uint8_t>(m0);
     rwork = pool.alloc<uint8_t>(m0);
     hasf = pool.alloc<uint8_t>(m0);
@@ -676,6 +681,8 @@ void Engine::prepare() {
     I.verdict = verdict;
     I.dead = lp_dead;
     I.st = st;
+    I.offset = nlp == 1 ? K.offset : nullptr;
+    I.off0 = mem[0].obj_offset;
     (k_init_work<<<(unsigned)std::min<int64_t>(std::max<int64_t>((std::max(m0, n0) + 255) / 256, 1), 8 * 152), 256, 0,
                    s>>>(I), note_launch());
     if (o.dual_records) {  // no source (-1, round -1: read as 0); no candidate row yet
@@ -701,13 +708,19 @@ void Engine::prepare() {
         LPP_CUDA(cudaMemsetAsync(rec_srhs, 0, sizeof(double) * (size_t)std::max(m0, 1), s));
         LPP_CUDA(cudaMemsetAsync(sub_used, 0, sizeof(unsigned long long), s));
     }
-    std::vector<double> offs(nlp);
-    for (int32_t k = 0; k < nlp; k++) offs[k] = mem[k].obj_offset;
-    LPP_CUDA(cudaMemcpyAsync(K.offset, offs.data(), sizeof(double) * nlp, cudaMemcpyHostToDevice, s));
     m = m0;
     n = n0;
     nnz = nnz0;
     cur = 0;
+    if (solo) {  // the kernel of the rounds checks the error bits and bins the rows itself
+        LPP_CUDA(cudaGetLastError());
+        return;
+    }
+    std::vector<double> offs(nlp);
+    if (nlp > 1) {
+        for (int32_t k = 0; k < nlp; k++) offs[k] = mem[k].obj_offset;
+        LPP_CUDA(cudaMemcpyAsync(K.offset, offs.data(), sizeof(double) * nlp, cudaMemcpyHostToDevice, s));
+    }
     // sizes for the schedules: k_init_work (none if a check failed, so that
     // they read no unchecked pointer)
     schedule_current(want_t);
@@ -1209,24 +1222,8 @@ void Engine::run_s5e(const Ctx &C) {
     read_status();
 }
 
-void Engine::run() {
+void Engine::run_rounds() {
     const int32_t R = std::max(0, o.max_rounds);
-    s5_clean = false;
-    s5c_dirty = true;
-    s5_left = 0;
-    lp_rounds.assign(nlp, 0);
-    lp_status.assign(nlp, LPP_OK);
-    lp_where.assign(nlp, LPP_WHERE_NONE);
-    lp_index.assign(nlp, -1);
-    lp_round.assign(nlp, 0);
-    lp_done.assign(nlp, 0);
-    lp_dropped.assign(nlp, 0);
-    cudaEvent_t eloop, eend;
-    LPP_CUDA(cudaEventCreate(&eloop));
-    LPP_CUDA(cudaEventCreate(&eend));
-    spare_events.push_back(eloop);
-    spare_events.push_back(eend);
-    LPP_CUDA(cudaEventRecord(eloop, s));
     int32_t live = nlp;
     for (int32_t r = 1; r <= R && live > 0; r++) {
         const StepOut so = step(r, r == 1, false);
@@ -1255,6 +1252,115 @@ void Engine::run() {
             }
         }
     }
+}
+
+// The rounds in one cooperative kernel: one launch, one read of its results.
+void Engine::run_solo() {
+    const int32_t R = o.max_rounds;
+    const int blocks = solo_blocks(m0, n0, nnz0);
+    const size_t ctl_bytes = sizeof(SoloCtl) + 6 * sizeof(int32_t) * (size_t)R;
+    SoloArgs F;
+    std::memset(&F, 0, sizeof F);
+    unsigned char *blk = pool.alloc<unsigned char>(ctl_bytes);
+    LPP_CUDA(cudaMemsetAsync(blk, 0, sizeof(SoloCtl), s));
+    LPP_CUDA(cudaMemsetAsync(s5_cnt, 0, sizeof(int32_t) * (size_t)(o.par_max_iter + 2), s));
+    F.base = ctx(1);
+    F.K = K;
+    F.K.cinv = cinv;
+    F.K.lp_dead = lp_dead;
+    F.in_rp = m_rp;
+    F.in_ci = m_ci;
+    F.in_rv = m_rv;
+    for (int b = 0; b < 2; b++) {
+        F.rp[b] = rp[b];
+        F.ci[b] = ci[b];
+        F.rv[b] = rv[b];
+        F.L[b] = L[b];
+        F.U[b] = U[b];
+        F.rmap[b] = rmap[b];
+        F.act[b] = act[b];
+        F.ninf[b] = ninf[b];
+        F.hrow[b] = hrow[b];
+        F.rdirty[b] = rdirty[b];
+        F.s5l[b] = s5_list[b];
+    }
+    F.rdnext = rdnext;
+    F.order = sa.order;
+    F.lfirst = sa.lfirst;
+    F.chunks = sa.chunks;
+    F.s5_cnt = s5_cnt;
+    F.btot = pool.alloc<int32_t>(2 * (size_t)blocks);
+    F.ctl = reinterpret_cast<SoloCtl *>(blk);
+    F.rstat = reinterpret_cast<int32_t *>(blk + sizeof(SoloCtl));
+    F.err_in = &st->err;
+    F.m = m0;
+    F.n = n0;
+    F.nnz = (int32_t)nnz0;
+    F.tcap_max = tcap_max;
+    F.max_rounds = R;
+    F.par_max_iter = o.par_max_iter;
+    if (!launch_solo(F, blocks, s)) {
+        cudaGetLastError();
+        throw StatusError(LPP_ERR_CUDA, "internal: cooperative launch refused");
+    }
+    solo_h = static_cast<unsigned char *>(pinned_get_sized(ctl_bytes));
+    LPP_CUDA(cudaMemcpyAsync(solo_h, blk, ctl_bytes, cudaMemcpyDeviceToHost, s));
+    read_status();
+    check_status();
+    const SoloCtl &c = *reinterpret_cast<const SoloCtl *>(solo_h);
+    const int32_t *q = reinterpret_cast<const int32_t *>(solo_h + sizeof(SoloCtl));
+    if (c.err & 4) throw StatusError(LPP_ERR_CUDA, "internal: round barrier timed out");
+    if (c.err) throw StatusError(LPP_ERR_CUDA, "internal: S5 hash table overflow");
+    const SoloOut &u = c.out;
+    if (u.rounds < 1 || u.rounds > R || u.m < 0 || u.m > m0 || u.nnz < 0 || u.nnz > nnz0)
+        throw StatusError(LPP_ERR_CUDA, "internal: sizes of the rounds' kernel");
+    for (int32_t r = 0; r < u.rounds; r++, q += 6) {
+        r_nnz.push_back(q[0]);
+        nnz_processed += q[0];
+        r_rows.push_back(q[1]);
+        r_cols.push_back(q[2]);
+        r_bounds.push_back(q[3]);
+        r_ms.push_back(1e-6f * (float)(uint32_t)q[4]);
+    }
+    rounds = u.rounds;
+    lp_rounds[0] = u.rounds;
+    lp_status[0] = u.status;
+    lp_where[0] = u.where;
+    lp_index[0] = u.index;
+    lp_round[0] = u.round;
+    s5_left = u.s5_left;
+    act_m = u.act_m;
+    act_buf = u.act_buf;
+    m = u.m;
+    nnz = u.nnz;
+    cur = u.cur;
+    if (cur == 1) {  // the columns stayed in buffer 0: they move with cur
+        std::swap(lu[0], lu[1]);
+        std::swap(this->c[0], this->c[1]);
+        std::swap(cmap[0], cmap[1]);
+    }
+    set_matrix();
+}
+
+void Engine::run() {
+    s5_clean = false;
+    s5c_dirty = true;
+    s5_left = 0;
+    lp_rounds.assign(nlp, 0);
+    lp_status.assign(nlp, LPP_OK);
+    lp_where.assign(nlp, LPP_WHERE_NONE);
+    lp_index.assign(nlp, -1);
+    lp_round.assign(nlp, 0);
+    lp_done.assign(nlp, 0);
+    lp_dropped.assign(nlp, 0);
+    cudaEvent_t eloop, eend;
+    LPP_CUDA(cudaEventCreate(&eloop));
+    LPP_CUDA(cudaEventCreate(&eend));
+    spare_events.push_back(eloop);
+    spare_events.push_back(eend);
+    LPP_CUDA(cudaEventRecord(eloop, s));
+    if (solo) run_solo();
+    else run_rounds();
     if (o.dep_rows && nlp == 1 && lp_status[0] == LPP_OK) remove_dependent();
     if (in_place) {
         launch_offset(ctx(rounds), K, s);  // every slot's contribution, once, in column order

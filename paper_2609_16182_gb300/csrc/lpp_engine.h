@@ -59,6 +59,12 @@ struct DevPool {
     ~DevPool() { release(); }
 };
 
+// Most entries of an LP whose rounds run in one kernel (Engine::solo).
+// Measured, the rounds launched / in one kernel: 1.5 k entries 597 / 380 us,
+// 0.18 M 2088 / 1380, 1.8 M 2343 / 2053; 7.8 M 5126 / 6964 (two blocks per SM
+// at 128 registers hold fewer gathers in flight than the launched kernels).
+constexpr int64_t kSoloNnz = 2 << 20;
+
 // per-LP description of an arena member
 struct Member {
     int32_t m, n;
@@ -183,6 +189,7 @@ struct Engine {
     DevStatus *st;
     DevStatus *st_h = nullptr;  // pinned mirror of st, the verdicts and the changed flags, one block
     size_t st_bytes = 0;
+    unsigned char *solo_h = nullptr;  // pinned copy of the rounds' kernel's results
     int32_t *verdict_h = nullptr;
     uint8_t *changed_h = nullptr;
     int32_t *s5_left_h = nullptr;  // rows still unmatched after a chunk of S5 passes
@@ -218,6 +225,9 @@ struct Engine {
     void ingest_batch(const lpp_lp *ins, int32_t count);
     void prepare();  // after ingest: transpose, schedules, work init
     void run();      // the round loop
+    bool solo = false;  // all rounds in one kernel (one LP of at most kSoloNnz entries, columns in place)
+    void run_solo();
+    void run_rounds();
     struct StepOut {
         bool structural = false;
         float ms = 0.f;

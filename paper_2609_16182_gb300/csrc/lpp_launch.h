@@ -159,6 +159,52 @@ void launch_s5e_scatter(const Ctx &C, const S5eBufs &D, const int32_t *rp2, int3
 // on the rewritten matrices: the rows of the cnt columns in jlist are dirty
 void launch_s5e_mark(const Ctx &C, const S5eBufs &D, int32_t cnt, cudaStream_t s);
 
+// ----------------------------------------------------------------- k_solo.cu
+// All rounds of one LP in one cooperative kernel (columns in place).
+struct SoloCnt {  // counters of a round
+    DevStatus st;
+    int32_t tl_cnt, cl_cnt, cl_nnz;
+    int32_t merged;     // rows S5 removed
+    int32_t n1, n2;     // rows unmatched after S5's first and last pass
+    int32_t cls[kNumClass], nchunk;  // the rows' classes at the round's start
+    int32_t changed;
+};
+struct SoloOut {
+    int32_t status, where, index, round, rounds;
+    int32_t m, nnz, cur;      // reduced rows and entries, in buffer cur
+    int32_t act_buf, act_m;   // the last round's row results
+    long long s5_left;
+};
+struct SoloCtl {  // zero before the launch
+    SoloOut out;
+    unsigned bar[2];
+    int32_t err, pad;
+    SoloCnt c[2];  // by the round's parity
+};
+struct SoloArgs {
+    Ctx base;
+    CompactCtx K;
+    const int32_t *in_rp, *in_ci;  // the first round's matrix
+    const double *in_rv;
+    int32_t *rp[2], *ci[2];
+    double *rv[2], *L[2], *U[2];
+    int32_t *rmap[2];
+    double2 *act[2];
+    int2 *ninf[2];
+    unsigned long long *hrow[2];
+    uint8_t *rdirty[2], *rdnext;
+    int32_t *order, *lfirst;
+    Chunk *chunks;
+    int32_t *s5l[2], *s5_cnt;  // S5: lists of unmatched rows, sizes per pass (zero before)
+    int32_t *btot;             // two per block
+    SoloCtl *ctl;
+    const int32_t *err_in;     // the input checks' error bits
+    int32_t *rstat;            // six per round: nonzeros, rows removed, columns fixed, bounds changed, ns
+    int32_t m, n, nnz, tcap_max, max_rounds, par_max_iter;
+};
+int solo_blocks(int32_t m, int32_t n, int64_t nnz);
+bool launch_solo(const SoloArgs &F, int blocks, cudaStream_t s);
+
 // ---------------------------------------------------------------- k_batch.cu
 // The persistent batch kernel: one thread block per LP at a time, every round
 // of the LP on the device (LPs whose rows and columns all have at most 4096
