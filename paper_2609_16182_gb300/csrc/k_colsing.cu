@@ -84,15 +84,60 @@ __device__ __forceinline__ bool s5d_eligible(const Ctx &C, int32_t j, double a, 
     return true;
 }
 
-// a column's term in the rest activities
-__device__ __forceinline__ void s5d_term(const Ctx &C, int32_t k, double a, double &mnr, double &mxr, int32_t &nmn,
-                                         int32_t &nmx) {
-    const double2 bk = C.lu[k];
-    const double bmn = a > 0.0 ? bk.x : bk.y, bmx = a > 0.0 ? bk.y : bk.x;
-    if (is_fin(bmn)) mnr = mnr + a * bmn;
-    else nmn++;
-    if (is_fin(bmx)) mxr = mxr + a * bmx;
-    else nmx++;
+// Which rest activities the test of column j (coefficient a) reads: one with
+// an infinite term fails it at once, and a free column reads neither (it is
+// eligible whatever the row holds).  The walks below stop at the first such
+// term and skip the sum that is not read; walking every candidate row to its
+// end cost 1.9 ms of 8.4 ms on an LP of 500 k rows.
+struct S5dNeed {
+    bool mn, mx;
+};
+__device__ __forceinline__ S5dNeed s5d_need(const Ctx &C, int32_t j, double a) {
+    const double2 b = C.lu[j];
+    const bool fl = is_fin(b.x), fu = is_fin(b.y);
+    return is_neg(a) ? S5dNeed{fl, fu} : S5dNeed{fu, fl};
+}
+// the coefficient of singleton column j
+__device__ __forceinline__ double s5d_coef(const Ctx &C, int32_t j) { return C.T.val[C.T.ptr[j]]; }
+
+// Entries q0, q0 + W, .. below end of row i's rest: the sums that are read (in
+// order) and the counts of infinite terms; four entries in flight, stops once
+// the test has failed.
+template <int W>
+__device__ __forceinline__ bool s5d_walk(const Ctx &C, int32_t j, S5dNeed need, int32_t q0, int32_t end, double &mnr,
+                                         double &mxr, int32_t &nmn, int32_t &nmx) {
+    for (; q0 < end; q0 += 4 * W) {
+        int32_t k[4];
+        double a[4];
+        double2 b[4];
+        uint8_t ck[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            k[u] = q0 + u * W < end ? C.A.idx[q0 + u * W] : -1;
+            a[u] = k[u] >= 0 ? C.A.val[q0 + u * W] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            ck[u] = k[u] >= 0 ? C.ckind[k[u]] : (uint8_t)CK_PARALLEL;
+            b[u] = k[u] >= 0 ? C.lu[k[u]] : make_double2(0.0, 0.0);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            if (k[u] < 0 || k[u] == j || ck[u] == CK_PARALLEL) continue;
+            const bool neg = is_neg(a[u]);
+            const double bmn = neg ? b[u].y : b[u].x, bmx = neg ? b[u].x : b[u].y;
+            if (need.mn) {
+                if (is_fin(bmn)) mnr = mnr + a[u] * bmn;
+                else nmn++;
+            }
+            if (need.mx) {
+                if (is_fin(bmx)) mxr = mxr + a[u] * bmx;
+                else nmx++;
+            }
+        }
+        if (nmn | nmx) return false;
+    }
+    return true;
 }
 
 // Short candidate rows, one per thread (row order: the same sums as a
@@ -109,14 +154,11 @@ __global__ void __launch_bounds__(kBlock) k_s5d_check(Ctx C, const int32_t *rcan
         tasks[atomicAdd(ntask, 1)] = i;
         return;
     }
-    double a = 0.0, mnr = 0.0, mxr = 0.0;
+    const double a = s5d_coef(C, j);
+    const S5dNeed need = s5d_need(C, j, a);
+    double mnr = 0.0, mxr = 0.0;
     int32_t nmn = 0, nmx = 0;
-    for (int32_t q = beg; q < end; q++) {
-        const int32_t k = C.A.idx[q];
-        if (k == j) a = C.A.val[q];
-        if (s5d_skip(C, k, j)) continue;
-        s5d_term(C, k, C.A.val[q], mnr, mxr, nmn, nmx);
-    }
+    if ((need.mn || need.mx) && !s5d_walk<1>(C, j, need, beg, end, mnr, mxr, nmn, nmx)) return;
     if (!s5d_eligible(C, j, a, s5d_side(C, i, j, a), mnr, mxr, nmn, nmx)) return;
     relig[i] = 1;
     if (C.c[j] == 0.0) return;  // changes no cost: no bid
@@ -162,25 +204,29 @@ __global__ void __launch_bounds__(kTaskThreads) k_s5d_check_long(Ctx C, const in
                                                                 int32_t *cmin, const int32_t *tasks,
                                                                 const int32_t *ntask) {
     __shared__ double s_d[kTaskThreads / 32];
-    __shared__ int32_t s_i[kTaskThreads / 32];
-    __shared__ double s_a;
     const int32_t nt = *ntask;
     for (int32_t t = blockIdx.x; t < nt; t += gridDim.x) {
         const int32_t i = tasks[t], j = rcand[i];
         const int32_t beg = C.A.ptr[i], end = C.A.ptr[i + 1];
+        const double a = s5d_coef(C, j);
+        const S5dNeed need = s5d_need(C, j, a);
         double mnr = 0.0, mxr = 0.0;
         int32_t nmn = 0, nmx = 0;
-        for (int32_t q = beg + threadIdx.x; q < end; q += kTaskThreads) {
-            const int32_t k = C.A.idx[q];
-            if (k == j) s_a = C.A.val[q];
-            if (s5d_skip(C, k, j)) continue;
-            s5d_term(C, k, C.A.val[q], mnr, mxr, nmn, nmx);
+        bool ok = true;
+        if (need.mn || need.mx) {  // block-uniform
+            // the threads' sums are their entries in order, 1024 entries of the
+            // row between two looks at whether the test has failed
+            for (int32_t q0 = beg; ok && q0 < end; q0 += 4 * kTaskThreads) {
+                const bool fine = s5d_walk<kTaskThreads>(C, j, need, q0 + (int32_t)threadIdx.x,
+                                                         min(end, q0 + 4 * kTaskThreads), mnr, mxr, nmn, nmx);
+                ok = __syncthreads_and(fine) != 0;
+            }
+            if (ok) {
+                mnr = block_sum_ordered(mnr, s_d);
+                mxr = block_sum_ordered(mxr, s_d);
+            }
         }
-        mnr = block_sum_ordered(mnr, s_d);
-        mxr = block_sum_ordered(mxr, s_d);
-        nmn = block_sum_ordered(nmn, s_i);
-        nmx = block_sum_ordered(nmx, s_i);
-        const bool ok = s5d_eligible(C, j, s_a, s5d_side(C, i, j, s_a), mnr, mxr, nmn, nmx);  // block-uniform
+        ok = ok && s5d_eligible(C, j, a, s5d_side(C, i, j, a), mnr, mxr, nmn, nmx);  // block-uniform
         if (ok) {
             if (threadIdx.x == 0) relig[i] = 1;
             if (C.c[j] != 0.0) {  // changes a cost: bid
@@ -322,14 +368,13 @@ __global__ void __launch_bounds__(kTaskThreads) k_s5d_chunk_sums(Ctx C, const in
     const Chunk ch = C.A.chunks[blockIdx.x];
     const int32_t i = ch.seg, j = rcand[i];
     if (j == kNone) return;  // block-uniform
+    const double a = s5d_coef(C, j);
+    const S5dNeed need = s5d_need(C, j, a);
     double mnr = 0.0, mxr = 0.0;
     int32_t nmn = 0, nmx = 0;
-    for (int32_t q = ch.begin + threadIdx.x; q < ch.end; q += kTaskThreads) {
-        const int32_t k = C.A.idx[q];
-        if (k == j) cs_a[i] = C.A.val[q];
-        if (s5d_skip(C, k, j)) continue;
-        s5d_term(C, k, C.A.val[q], mnr, mxr, nmn, nmx);
-    }
+    if (threadIdx.x == 0) cs_a[i] = a;  // every chunk of the row the same
+    if (need.mn || need.mx)  // an infinite term found ends the row's test: the sums are then not read
+        s5d_walk<kTaskThreads>(C, j, need, ch.begin + threadIdx.x, ch.end, mnr, mxr, nmn, nmx);
     mnr = block_sum_ordered(mnr, s_d);
     mxr = block_sum_ordered(mxr, s_d);
     nmn = block_sum_ordered(nmn, s_i);

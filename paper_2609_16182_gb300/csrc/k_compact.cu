@@ -104,19 +104,29 @@ __device__ __forceinline__ void lock_group(const Ctx &C, const CompactCtx &K, in
     if (valid && lane == 0) K.c_lock[j] = lk;
 }
 
-__global__ void __launch_bounds__(kBlock) k_locks_groups(Ctx C, CompactCtx K, GroupGrid g) {
-    const int c = grid_class(g, blockIdx.x);
-    const int W = 1 << c;
-    const int32_t pos = C.T.cls_start[c] + (blockIdx.x - g.blk_start[c]) * (kBlock / W) + threadIdx.x / W;
-    const bool valid = pos < C.T.cls_start[c + 1];
-    const int32_t j = valid ? C.T.order[pos] : 0;
+__global__ void __launch_bounds__(kBlock) k_locks_groups(Ctx C, CompactCtx K, RowGrid R) {
+    int c;
+    bool valid;
+    const int32_t j = class_row(C.T, R, blockIdx.x, c, valid);
+    if (c == 5) {  // columns of 65 to 4096 entries: the whole block (c_lock is zero before)
+        for (int32_t q = 0; q < R.per5; q++) {
+            const int32_t pos = C.T.cls_start[5] + (int32_t)(blockIdx.x - R.g.blk_start[0]) * R.per5 + q;
+            if (pos >= C.T.cls_start[6]) break;
+            const int32_t k = C.T.order[pos], e = C.T.ptr[k + 1];
+            int32_t lk = 0;
+#pragma unroll 4
+            for (int32_t t = C.T.ptr[k] + (int32_t)threadIdx.x; t < e; t += kBlock) lk |= entry_locks(C, C.T.idx[t], C.T.val[t]);
+            lk = __reduce_or_sync(0xffffffffu, (unsigned)lk);
+            if ((threadIdx.x & 31) == 0 && lk) atomicOr(&K.c_lock[k], lk);
+        }
+        return;
+    }
     switch (c) {
         case 0: lock_group<1>(C, K, j, valid); break;
         case 1: lock_group<2>(C, K, j, valid); break;
         case 2: lock_group<4>(C, K, j, valid); break;
         case 3: lock_group<8>(C, K, j, valid); break;
-        case 4: lock_group<16>(C, K, j, valid); break;
-        default: lock_group<32>(C, K, j, valid); break;
+        default: lock_group<16>(C, K, j, valid); break;
     }
 }
 
@@ -159,19 +169,30 @@ __device__ __forceinline__ void csr_count_group(const Ctx &C, const CompactCtx &
     csr_count_row<W>(C, K, i, valid, valid && C.rkind[i] == RK_KEPT && !K.lp_dead[lp_of_row(C, i)]);
 }
 
-__global__ void __launch_bounds__(kBlock) k_csr_count_groups(Ctx C, CompactCtx K, GroupGrid g) {
-    const int c = grid_class(g, blockIdx.x);
-    const int W = 1 << c;
-    const int32_t pos = C.A.cls_start[c] + (blockIdx.x - g.blk_start[c]) * (kBlock / W) + threadIdx.x / W;
-    const bool valid = pos < C.A.cls_start[c + 1];
-    const int32_t i = valid ? C.A.order[pos] : 0;
+__global__ void __launch_bounds__(kBlock) k_csr_count_groups(Ctx C, CompactCtx K, RowGrid R) {
+    __shared__ double s_a[kMidStep], s_v[kMidStep];
+    __shared__ int32_t s_mid[kBlock / 32], s_nmid, s_sum[1];
+    int c;
+    bool valid;
+    const int32_t i = class_row(C.A, R, blockIdx.x, c, valid);
     switch (c) {
         case 0: csr_count_group<1>(C, K, i, valid); break;
         case 1: csr_count_group<2>(C, K, i, valid); break;
         case 2: csr_count_group<4>(C, K, i, valid); break;
         case 3: csr_count_group<8>(C, K, i, valid); break;
         case 4: csr_count_group<16>(C, K, i, valid); break;
-        default: csr_count_group<32>(C, K, i, valid); break;
+        default: {
+            if (threadIdx.x == 0) s_nmid = 0;
+            __syncthreads();
+            if (valid && C.A.ptr[i + 1] - C.A.ptr[i] >= kMidRow && C.rkind[i] == RK_KEPT && !K.lp_dead[lp_of_row(C, i)]) {
+                if ((threadIdx.x & 31) == 0) s_mid[atomicAdd(&s_nmid, 1)] = i;
+                valid = false;
+            }
+            csr_count_group<32>(C, K, i, valid);
+            __syncthreads();
+            const int32_t nmid = s_nmid;
+            for (int32_t t = 0; t < nmid; t++) count_mid(C, K, s_mid[t], s_a, s_v, s_sum);
+        }
     }
 }
 
@@ -404,7 +425,7 @@ void launch_compact_counts(const Ctx &C, const CompactCtx &K, cudaStream_t s, co
         return;
     }
     // 1. column counts over kept rows, then S6 and the column keep flags
-    const GroupGrid ga = group_grid(C.A);
+    const RowGrid ga = class_grid(C.A);
     const int32_t along = C.A.cls_start[7] - C.A.cls_start[6];
     const GroupGrid gt = group_grid(C.T);
     if (gt.blk_start[6] > 0) (k_csc_count_groups<<<gt.blk_start[6], kBlock, 0, s>>>(C, K, gt), note_launch());
@@ -416,7 +437,8 @@ void launch_compact_counts(const Ctx &C, const CompactCtx &K, cudaStream_t s, co
     }
     if (C.dualfix && C.n > 0) {
         cudaMemsetAsync(K.c_lock, 0, sizeof(int32_t) * (size_t)C.n, s);
-        if (gt.blk_start[6] > 0) (k_locks_groups<<<gt.blk_start[6], kBlock, 0, s>>>(C, K, gt), note_launch());
+        const RowGrid rt = class_grid(C.T);
+        if (rt.g.blk_start[6] > 0) (k_locks_groups<<<rt.g.blk_start[6], kBlock, 0, s>>>(C, K, rt), note_launch());
         if (tlong > 0 && C.T.nchunks > 0) (k_locks_long<<<C.T.nchunks, kBlock, 0, s>>>(C, K), note_launch());
     }
     launch_colkeep(C, K, s);
@@ -436,7 +458,7 @@ void launch_compact_counts(const Ctx &C, const CompactCtx &K, cudaStream_t s, co
         (k_long_prefix<<<blocks_for((int64_t)along * 32, 128), 128, 0, sl>>>(C.A, K.chr_cnt, K.chr_off, K.r_len,
                                                                               K.chr_shift, K.shift), note_launch());
     }
-    if (ga.blk_start[6] > 0) (k_csr_count_groups<<<ga.blk_start[6], kBlock, 0, s>>>(C, K, ga), note_launch());
+    if (ga.g.blk_start[6] > 0) (k_csr_count_groups<<<ga.g.blk_start[6], kBlock, 0, s>>>(C, K, ga), note_launch());
     if (fork) {
         cudaEventRecord(side->join, side->s);
         cudaStreamWaitEvent(s, side->join, 0);

@@ -717,6 +717,49 @@ __device__ __forceinline__ void inplace_mid(const Ctx &C, const CompactCtx &K, i
     __syncthreads();
 }
 
+// The same row by the keep flags (the columns compacted each round): entries
+// left and the side shift.
+__device__ __forceinline__ void count_mid(const Ctx &C, const CompactCtx &K, int32_t i, double *s_a, double *s_v,
+                                          int32_t *s_sum) {
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int32_t beg = C.A.ptr[i], end = C.A.ptr[i + 1];
+    if (tid == 0) s_sum[0] = 0;
+    int32_t cnt = 0;
+    double sh = 0.0;
+    for (int32_t t0 = beg; t0 < end; t0 += kMidStep) {
+        int32_t jq[2];
+        bool kq[2];
+#pragma unroll
+        for (int q = 0; q < 2; q++) jq[q] = t0 + q * kBlock + tid < end ? C.A.idx[t0 + q * kBlock + tid] : -1;
+#pragma unroll
+        for (int q = 0; q < 2; q++) kq[q] = jq[q] < 0 || K.c_keep[jq[q]];
+        cnt += (jq[0] >= 0 && kq[0]) + (jq[1] >= 0 && kq[1]);
+        if (__syncthreads_or(!kq[0] || !kq[1])) {
+#pragma unroll
+            for (int q = 0; q < 2; q++) {
+                s_a[q * kBlock + tid] = kq[q] ? 0.0 : C.A.val[t0 + q * kBlock + tid];
+                s_v[q * kBlock + tid] = kq[q] ? 0.0 : C.fixv[jq[q]];
+            }
+            __syncthreads();
+            if (tid < 32)
+                for (int32_t t = 0; t < kMidStep / 32; t++) sh = fma(s_a[32 * t + lane], s_v[32 * t + lane], sh);
+            __syncthreads();
+        }
+    }
+    __syncthreads();
+    cnt = __reduce_add_sync(0xffffffffu, cnt);
+    if (lane == 0 && cnt) atomicAdd(&s_sum[0], cnt);
+    if (tid < 32) sh = group_sum<32>(sh, 0xffffffffu);
+    __syncthreads();
+    if (tid == 0) {
+        mark_tile(K.tile_a, beg, end, i);
+        K.r_keep[i] = 1;
+        K.r_len[i] = s_sum[0];
+        K.shift[i] = sh;
+    }
+    __syncthreads();
+}
+
 // the rows of block b of class_grid
 struct InplaceShared {
     double a[kMidStep], v[kMidStep];
