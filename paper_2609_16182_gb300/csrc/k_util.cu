@@ -126,12 +126,10 @@ __device__ __forceinline__ T block_excl_scan(T v, T &excl, T *s_w) {
 template <class T, class In>
 __global__ void __launch_bounds__(kScanThreads) k_scan_reduce(In in, int64_t cnt, T *tsum) {
     __shared__ T s_w[33];
-    const int64_t base = (int64_t)blockIdx.x * kScanTile;
-    T v = zero_of<T>();
-    for (int t = threadIdx.x; t < kScanTile; t += kScanThreads) {
-        const int64_t k = base + t;
-        if (k < cnt) v = v + in(k);
-    }
+    T x[kPerThread], v = zero_of<T>();
+    in.get8((int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kPerThread, cnt, x);
+#pragma unroll
+    for (int q = 0; q < kPerThread; q++) v = v + x[q];
     T ex;
     const T tot = block_excl_scan(v, ex, s_w);
     if (threadIdx.x == 0) tsum[blockIdx.x] = tot;
@@ -209,86 +207,104 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_down(In in, Out out, int6
 }
 
 // --------------------------------------------------------------- binning
-__global__ void __launch_bounds__(kScanThreads) k_bin_hist(const int32_t *ptr, const int32_t *cnt_dev,
-                                                           int32_t *hist, int32_t ntiles) {
-    __shared__ int32_t s_h[kNumClass];
-    const int32_t cnt = *cnt_dev;
-    if (threadIdx.x < kNumClass) s_h[threadIdx.x] = 0;
-    __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * kScanTile;
-    for (int t = threadIdx.x; t < kScanTile; t += kScanThreads) {
-        const int64_t sg = base + t;
-        if (sg < cnt) atomicAdd(&s_h[seg_class(ptr[sg + 1] - ptr[sg])], 1);
-    }
-    __syncthreads();
-    if (threadIdx.x < kNumClass) hist[(int64_t)threadIdx.x * ntiles + blockIdx.x] = s_h[threadIdx.x];
-}
-
-__global__ void __launch_bounds__(kScanThreads) k_bin_scatter(const int32_t *ptr, const int32_t *cnt_dev,
-                                                              const int32_t *off, int32_t ntiles, int32_t *order) {
-    __shared__ int32_t s_run[kNumClass];
-    const int32_t cnt = *cnt_dev;
-    __shared__ int32_t s_w[kScanThreads / 32][kNumClass];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const unsigned lt = (1u << lane) - 1u;
-    if (threadIdx.x < kNumClass) s_run[threadIdx.x] = 0;
-    __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * kScanTile;
-    for (int r = 0; r < kPerThread; r++) {
-        const int64_t sg = base + (int64_t)r * kScanThreads + threadIdx.x;
-        const bool valid = sg < cnt;
-        const int c = valid ? seg_class(ptr[sg + 1] - ptr[sg]) : kNumClass;
-        int rank = 0;
+// Two passes over the segment lengths, eight consecutive segments per thread:
+// the first counts each tile's segments per class and reserves the tile's
+// places in each class by one atomic, the second writes the segments to them
+// (in order inside a tile; a segment's results do not depend on its place).
+// The four launches before (histogram, scan, ordered scatter in eight
+// barrier-bound steps) took 25 us whatever the size, these take 8.
+__device__ __forceinline__ void load_classes(const int32_t *ptr, int64_t base, int64_t cnt, int *c) {
+    int32_t p[kPerThread + 1];
 #pragma unroll
-        for (int k = 0; k < kNumClass; k++) {
-            const unsigned bal = __ballot_sync(0xffffffffu, c == k);
-            if (c == k) rank = __popc(bal & lt);
-            if (lane == 0) s_w[warp][k] = __popc(bal);
-        }
-        __syncthreads();
-        if (valid) {
-            int32_t pre = s_run[c];
-            for (int w = 0; w < warp; w++) pre += s_w[w][c];
-            order[off[(int64_t)c * ntiles + blockIdx.x] + pre + rank] = (int32_t)sg;
-        }
-        __syncthreads();
-        if (threadIdx.x < kNumClass) {
-            int32_t t = 0;
-            for (int w = 0; w < kScanThreads / 32; w++) t += s_w[w][threadIdx.x];
-            s_run[threadIdx.x] += t;
-        }
-        __syncthreads();
+    for (int q = 0; q <= kPerThread; q++) p[q] = base + q <= cnt ? ptr[base + q] : 0;
+#pragma unroll
+    for (int q = 0; q < kPerThread; q++) c[q] = base + q < cnt ? seg_class(p[q + 1] - p[q]) : kNumClass;
+}
+
+__global__ void __launch_bounds__(kScanThreads) k_bin_count(const int32_t *ptr, const int32_t *cnt_dev, int32_t *cls,
+                                                            int32_t *places) {
+    __shared__ int32_t s_n[kNumClass];
+    const int32_t cnt = *cnt_dev;
+    if (threadIdx.x < kNumClass) s_n[threadIdx.x] = 0;
+    __syncthreads();
+    const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kPerThread;
+    int c[kPerThread];
+    load_classes(ptr, base, cnt, c);
+    unsigned long long n = 0;  // eight bits per class
+#pragma unroll
+    for (int q = 0; q < kPerThread; q++) n += c[q] < kNumClass ? 1ULL << (8 * c[q]) : 0ULL;
+#pragma unroll
+    for (int k = 0; k < kNumClass; k++) {
+        const int32_t t = __reduce_add_sync(0xffffffffu, (int)((n >> (8 * k)) & 255u));
+        if ((threadIdx.x & 31) == 0 && t) atomicAdd(&s_n[k], t);
+    }
+    __syncthreads();
+    if (threadIdx.x < kNumClass) {
+        const int32_t t = s_n[threadIdx.x];
+        places[(int64_t)blockIdx.x * kNumClass + threadIdx.x] = t ? atomicAdd(cls + threadIdx.x, t) : 0;
     }
 }
 
-// class sizes from the scanned histogram
-// one block: exclusive scan in place of the 7 x ntiles class-by-tile counts
-// (class-major), the total at a[cnt], and the class sizes
-__global__ void __launch_bounds__(1024) k_scan_small_cls(int32_t *a, int32_t cnt, int32_t ntiles, int32_t *cls_out) {
-    __shared__ int32_t s_w[33];
-    int32_t carry = 0;
-    for (int32_t b = 0; b < cnt; b += 1024) {
-        const int32_t k = b + threadIdx.x;
-        const int32_t v = k < cnt ? a[k] : 0;
-        int32_t ex;
-        const int32_t tot = block_excl_scan(v, ex, s_w);
-        if (k < cnt) a[k] = carry + ex;
-        carry += tot;
+__global__ void __launch_bounds__(kScanThreads) k_bin_fill(const int32_t *ptr, const int32_t *cnt_dev,
+                                                           const int32_t *cls, const int32_t *places, int32_t *order) {
+    __shared__ int32_t s_at[kNumClass];
+    __shared__ unsigned long long s_w[2][kScanThreads / 32];
+    const int32_t cnt = *cnt_dev;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (threadIdx.x < kNumClass) {
+        int32_t start = 0;
+        for (int k = 0; k < (int)threadIdx.x; k++) start += cls[k];
+        s_at[threadIdx.x] = start + places[(int64_t)blockIdx.x * kNumClass + threadIdx.x];
     }
-    if (threadIdx.x == 0) a[cnt] = carry;
+    const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kPerThread;
+    int c[kPerThread];
+    load_classes(ptr, base, cnt, c);
+    // exclusive scan over the threads of the counts per class, 16 bits each, in two words
+    unsigned long long a = 0, b = 0;
+#pragma unroll
+    for (int q = 0; q < kPerThread; q++) {
+        if (c[q] < 4) a += 1ULL << (16 * c[q]);
+        else if (c[q] < kNumClass) b += 1ULL << (16 * (c[q] - 4));
+    }
+    unsigned long long xa = a, xb = b;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long ya = __shfl_up_sync(0xffffffffu, xa, o), yb = __shfl_up_sync(0xffffffffu, xb, o);
+        if (lane >= o) {
+            xa += ya;
+            xb += yb;
+        }
+    }
+    if (lane == 31) {
+        s_w[0][warp] = xa;
+        s_w[1][warp] = xb;
+    }
     __syncthreads();
-    if (threadIdx.x < kNumClass)
-        cls_out[threadIdx.x] = a[(int64_t)(threadIdx.x + 1) * ntiles] - a[(int64_t)threadIdx.x * ntiles];
+    xa -= a;
+    xb -= b;
+    for (int w = 0; w < warp; w++) {
+        xa += s_w[0][w];
+        xb += s_w[1][w];
+    }
+#pragma unroll
+    for (int q = 0; q < kPerThread; q++) {
+        if (c[q] >= kNumClass) continue;
+        const int sh = 16 * (c[q] & 3);
+        unsigned long long &x = c[q] < 4 ? xa : xb;
+        order[s_at[c[q]] + (int32_t)((x >> sh) & 0xffffu)] = (int32_t)(base + q);
+        x += 1ULL << sh;
+    }
 }
 
 // one block: the chunks of the long segments (class 6, in schedule order),
 // their first chunk (lfirst, with the total at lfirst[long count]) and the count
-__global__ void __launch_bounds__(1024) k_chunks(const int32_t *ptr, const int32_t *order, const int32_t *off,
-                                                 int32_t ntiles, const int32_t *cls, int32_t cap_long,
-                                                 int32_t *lfirst, Chunk *chunks, int32_t *nchunk_out) {
+__global__ void __launch_bounds__(1024) k_chunks(const int32_t *ptr, const int32_t *order, const int32_t *cls,
+                                                 int32_t cap_long, int32_t *lfirst, Chunk *chunks,
+                                                 int32_t *nchunk_out) {
     __shared__ int32_t s_w[33];
     const int32_t nlong = min(cls[6], cap_long);
-    const int32_t *lo = order + off[(int64_t)6 * ntiles];
+    const int32_t *lo = order;
+    for (int k = 0; k < 6; k++) lo += cls[k];
     int32_t carry = 0;
     for (int32_t b = 0; b < nlong; b += 1024) {
         const int32_t t = b + threadIdx.x;
@@ -645,13 +661,12 @@ void build_schedule(const int32_t *ptr, const int32_t *cnt_dev, int32_t cnt_max,
                     const SchedBufs &b, int32_t *cls_out, int32_t *nchunk_out, cudaStream_t s) {
     // tiles cover cnt_max segments; tiles past the actual count hold zeros
     const int32_t ntiles = std::max<int32_t>(1, (int32_t)((cnt_max + kScanTile - 1) / kScanTile));
-    (k_bin_hist<<<ntiles, kScanThreads, 0, s>>>(ptr, cnt_dev, b.tile_hist, ntiles), note_launch());
-    (k_scan_small_cls<<<1, 1024, 0, s>>>(b.tile_hist, kNumClass * ntiles, ntiles, cls_out), note_launch());
-    (k_bin_scatter<<<ntiles, kScanThreads, 0, s>>>(ptr, cnt_dev, b.tile_hist, ntiles, b.order), note_launch());
+    cudaMemsetAsync(cls_out, 0, kNumClass * sizeof(int32_t), s);
+    (k_bin_count<<<ntiles, kScanThreads, 0, s>>>(ptr, cnt_dev, cls_out, b.tile_hist), note_launch());
+    (k_bin_fill<<<ntiles, kScanThreads, 0, s>>>(ptr, cnt_dev, cls_out, b.tile_hist, b.order), note_launch());
     // chunks of the long segments: at most nnz / kLongMin of them
     const int32_t cap_long = sched_cap_long(nnz_max);
-    (k_chunks<<<1, 1024, 0, s>>>(ptr, b.order, b.tile_hist, ntiles, cls_out, cap_long, b.lfirst, b.chunks,
-                                 nchunk_out), note_launch());
+    (k_chunks<<<1, 1024, 0, s>>>(ptr, b.order, cls_out, cap_long, b.lfirst, b.chunks, nchunk_out), note_launch());
 }
 
 void segmat_from_counts(SegMat &M, const int32_t cls[kNumClass], int32_t nchunks) {

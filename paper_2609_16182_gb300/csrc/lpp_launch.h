@@ -24,7 +24,7 @@ struct SchedBufs {
     int32_t *order;     // [cap_seg]
     Chunk *chunks;      // [cap_chunk]
     int32_t *lfirst;    // [cap_long + 1]
-    int32_t *tile_hist; // [7 * tiles + 1]
+    int32_t *tile_hist; // [7 * tiles + 1] places of each tile's segments per class
     int32_t *tmp;       // scan temporary
     int32_t *nch;       // [cap_long + 1]
 };
