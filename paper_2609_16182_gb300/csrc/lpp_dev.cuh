@@ -309,13 +309,6 @@ __device__ __forceinline__ void block_add(int32_t v, int32_t *dst) {
     if (threadIdx.x == 0 && s_acc) atomicAdd(dst, s_acc);
 }
 
-// warp-aggregated counter: one atomic per warp with something to add, no
-// barrier (the warps of a block end on their own); the whole warp must call it
-__device__ __forceinline__ void warp_add(int32_t v, int32_t *dst) {
-    v = __reduce_add_sync(0xffffffffu, v);
-    if ((threadIdx.x & 31) == 0 && v) atomicAdd(dst, v);
-}
-
 // Appends `value` to list[*cnt ...] for each thread with `want`: one shared
 // atomic per thread, one global atomic per block.  Every thread of the block
 // must call it.  The order within the list is unspecified.

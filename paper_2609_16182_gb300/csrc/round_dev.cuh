@@ -16,6 +16,13 @@ namespace {
 
 namespace cg = cooperative_groups;
 
+// warp-aggregated counter: one atomic per warp with something to add, no
+// barrier (the warps of a block end on their own); the whole warp must call it
+__device__ __forceinline__ void warp_add(int32_t v, int32_t *dst) {
+    v = __reduce_add_sync(0xffffffffu, v);
+    if ((threadIdx.x & 31) == 0 && v) atomicAdd(dst, v);
+}
+
 // appends v to list[*cnt ...] with one atomic per group of converged threads
 __device__ __forceinline__ void coalesced_append(int32_t v, int32_t *cnt, int32_t *list) {
     cg::coalesced_group g = cg::coalesced_threads();
