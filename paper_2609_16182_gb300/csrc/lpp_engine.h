@@ -304,6 +304,7 @@ namespace lpp {
 // postsolve records; the host copies are made on first access.
 struct DeviceRecords {
     int32_t m0 = 0, n0 = 0, n_final = 0, act_m = 0;
+    int device = 0;
     int32_t *rk = nullptr, *rr = nullptr, *ra = nullptr, *ck = nullptr, *cr = nullptr;
     double *rv = nullptr, *cv = nullptr;
     int32_t *ca = nullptr, *cp = nullptr;  // S5c merges: leader, pass (NULL without parallel_cols)
@@ -335,7 +336,7 @@ struct lpp_postsolve {
     int32_t r0 = 0, c0 = 0;          // first original row / column of this LP in the arena
     int32_t cstart = 0;              // first kept column of this LP in the final arena
     int32_t astart = 0, acnt = 0;    // this LP's rows in the last round's numbering
-    bool host_ready = false;
+    int host_have = 0;               // record groups copied to the host (REC_* in lpp_api.cu)
     std::vector<int32_t> row_kind, row_round, row_aux, col_kind, col_round, col_map, col_aux, col_pass;
     std::vector<double> row_val, col_val, col_lb, col_ub, act_min, act_max, col_mrg;
     std::vector<int64_t> sub_beg;                 // substitutions: per row, into sub_col / sub_val

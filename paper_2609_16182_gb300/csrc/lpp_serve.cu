@@ -374,6 +374,7 @@ void finish_slot(lpp_server *S, int32_t k, const std::vector<int32_t> &rng, cons
     const int32_t mr = r1 - r0, nc = c1 - c0, nz = z1 - z0, na = a1 - a0;
     auto *R = new lpp_reduced();
     auto D = std::make_shared<DeviceRecords>();
+    D->device = E.o.device;
     auto own = [&](size_t bytes, std::vector<void *> &into) {
         void *p = nullptr;
         LPP_CUDA(cudaMallocAsync(&p, bytes ? bytes : 1, E.s));
