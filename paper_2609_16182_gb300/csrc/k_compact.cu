@@ -316,28 +316,11 @@ __global__ void __launch_bounds__(kBlock) k_scatter_flat(FlatArgs F) {
 
 // ---------------------------------------------------------- objective constant
 // one LP: tiles of kScanTile columns summed in a fixed order, then the tiles
-// the contributions are consumed: reset to zero once read (a column whose
-// flags are not recomputed in a later round then contributes nothing)
 __global__ void __launch_bounds__(kBlock) k_offset_tiles(double *contrib, int32_t n, double *part) {
-    const int64_t base = (int64_t)blockIdx.x * kScanTile;
-    double s = 0.0;
-    for (int t = threadIdx.x; t < kScanTile; t += kBlock) {
-        const int64_t j = base + t;
-        if (j < n) {
-            const double v = contrib[j];
-            s += v;
-            if (v != 0.0) contrib[j] = 0.0;
-        }
-    }
-    s = block_sum_dbl(s);
-    if (threadIdx.x == 0) part[blockIdx.x] = s;
+    offset_tile(contrib, n, part, blockIdx.x);
 }
-// one block: thread t adds tiles t, t+256, ... in order, then the fixed-order block sum
 __global__ void __launch_bounds__(kBlock) k_offset_final(const double *part, int32_t ntiles, double *offset) {
-    double s = 0.0;
-    for (int32_t t = threadIdx.x; t < ntiles; t += kBlock) s += part[t];
-    s = block_sum_dbl(s);
-    if (threadIdx.x == 0) offset[0] += s;
+    offset_final(part, ntiles, offset);
 }
 // many LPs: column range of each LP, then one warp per LP
 __global__ void k_lp_ranges(const int32_t *lp_col, int32_t n, int32_t *first, int32_t *last) {

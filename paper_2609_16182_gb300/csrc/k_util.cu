@@ -474,18 +474,6 @@ constexpr int kRadixWarps = kScanThreads / 32;
 constexpr int kRadixChunk = kRadixTile / kRadixWarps;  // 512 keys per warp
 constexpr int kRadixSteps = kRadixChunk / 32;          // 16
 
-// lanes of the warp holding the same 8-bit digit d (d = 256: none), from 9
-// independent full-warp ballots; every lane of the warp must call it
-__device__ __forceinline__ unsigned digit_peers(int d) {
-    unsigned m = __ballot_sync(0xffffffffu, d < 256);
-#pragma unroll
-    for (int b = 0; b < 8; b++) {
-        const unsigned bb = __ballot_sync(0xffffffffu, (d >> b) & 1);
-        m &= ((d >> b) & 1) ? bb : ~bb;
-    }
-    return d < 256 ? m : 0u;
-}
-
 __global__ void __launch_bounds__(kScanThreads) k_radix_hist(const uint32_t *keys, int64_t cnt, int shift,
                                                              int32_t *hist, int32_t ntiles) {
     __shared__ int32_t s_h[256];

@@ -790,8 +790,8 @@ lpp_status lpp_presolve(const lpp_lp *in, const lpp_opts *opts, lpp_reduced **ou
         E->tend();
         E->run();
         E->tbegin(F_FINISH, 0.0);  // records and the reduced LP handed over
-        double offset = 0.0;
-        LPP_CUDA(cudaMemcpyAsync(&offset, E->K.offset, sizeof(double), cudaMemcpyDeviceToHost, E->s));
+        double offset = E->solo_offset;
+        if (!E->solo) LPP_CUDA(cudaMemcpyAsync(&offset, E->K.offset, sizeof(double), cudaMemcpyDeviceToHost, E->s));
         auto D = take_records(*E);
         // the reduced LP takes the current buffers
         auto *R = new lpp_reduced();

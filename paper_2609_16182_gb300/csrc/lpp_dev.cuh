@@ -347,4 +347,16 @@ __device__ __forceinline__ int grid_class(const GroupGrid &g, int b) {
     return c;
 }
 
+// lanes of the warp holding the same 8-bit digit d (d = 256: none), from 9
+// independent full-warp ballots; every lane of the warp must call it
+__device__ __forceinline__ unsigned digit_peers(int d) {
+    unsigned m = __ballot_sync(0xffffffffu, d < 256);
+#pragma unroll
+    for (int b = 0; b < 8; b++) {
+        const unsigned bb = __ballot_sync(0xffffffffu, (d >> b) & 1);
+        m &= ((d >> b) & 1) ? bb : ~bb;
+    }
+    return d < 256 ? m : 0u;
+}
+
 }  // namespace lpp

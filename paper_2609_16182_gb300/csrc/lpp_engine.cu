@@ -1299,7 +1299,35 @@ void Engine::run_solo() {
     F.tcap_max = tcap_max;
     F.max_rounds = R;
     F.par_max_iter = o.par_max_iter;
-    if (!launch_solo(F, blocks, s)) {
+    SoloFinish G;
+    std::memset(&G, 0, sizeof G);
+    const int fblocks = solo_finish_blocks(n0, nnz0);
+    G.ctl = F.ctl;
+    G.err_in = F.err_in;
+    G.n = n0;
+    for (int b = 0; b < 2; b++) {
+        G.rp[b] = rp[b];
+        G.ci[b] = ci[b];
+        G.rv[b] = rv[b];
+        G.tp[b] = tp[b];
+        G.ti[b] = ti[b];
+        G.tv[b] = tv[b];
+    }
+    G.half = nnz0;
+    G.lu = lu[0];
+    G.c = this->c[0];
+    G.cmap = cmap[0];
+    G.lu2 = lu[1];
+    G.c2 = this->c[1];
+    G.cmap2 = cmap[1];
+    G.cinv = cinv;
+    G.pos = K.c_pos;
+    G.contrib = K.contrib;
+    G.part = K.offset_part;
+    G.offset = K.offset;
+    G.btot = pool.alloc<int32_t>((size_t)fblocks);
+    G.hist = pool.alloc<int32_t>((size_t)fblocks * 256);
+    if (!launch_solo(F, blocks, s) || !launch_solo_finish(G, fblocks, s)) {
         cudaGetLastError();
         throw StatusError(LPP_ERR_CUDA, "internal: cooperative launch refused");
     }
@@ -1312,7 +1340,8 @@ void Engine::run_solo() {
     if (c.err & 4) throw StatusError(LPP_ERR_CUDA, "internal: round barrier timed out");
     if (c.err) throw StatusError(LPP_ERR_CUDA, "internal: S5 hash table overflow");
     const SoloOut &u = c.out;
-    if (u.rounds < 1 || u.rounds > R || u.m < 0 || u.m > m0 || u.nnz < 0 || u.nnz > nnz0)
+    if (u.rounds < 1 || u.rounds > R || u.m < 0 || u.m > m0 || u.nnz < 0 || u.nnz > nnz0 || u.n < 0 ||
+        u.n > n0)
         throw StatusError(LPP_ERR_CUDA, "internal: sizes of the rounds' kernel");
     for (int32_t r = 0; r < u.rounds; r++, q += 6) {
         r_nnz.push_back(q[0]);
@@ -1334,12 +1363,17 @@ void Engine::run_solo() {
     m = u.m;
     nnz = u.nnz;
     cur = u.cur;
-    if (cur == 1) {  // the columns stayed in buffer 0: they move with cur
+    n = u.n;
+    solo_offset = u.offset;
+    if (cur == 0) {  // the columns were compacted into buffer 1: they move with cur
         std::swap(lu[0], lu[1]);
         std::swap(this->c[0], this->c[1]);
         std::swap(cmap[0], cmap[1]);
     }
     set_matrix();
+    T.ptr = tp[cur];
+    T.idx = ti[cur];
+    T.val = tv[cur];
 }
 
 void Engine::run() {
@@ -1362,7 +1396,7 @@ void Engine::run() {
     if (solo) run_solo();
     else run_rounds();
     if (o.dep_rows && nlp == 1 && lp_status[0] == LPP_OK) remove_dependent();
-    if (in_place) {
+    if (in_place && !solo) {
         launch_offset(ctx(rounds), K, s);  // every slot's contribution, once, in column order
         finish_cols();
         finish_csc();

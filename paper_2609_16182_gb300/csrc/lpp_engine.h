@@ -190,6 +190,7 @@ struct Engine {
     DevStatus *st_h = nullptr;  // pinned mirror of st, the verdicts and the changed flags, one block
     size_t st_bytes = 0;
     unsigned char *solo_h = nullptr;  // pinned copy of the rounds' kernel's results
+    double solo_offset = 0.0;         // objective constant of the reduced LP, with it
     int32_t *verdict_h = nullptr;
     uint8_t *changed_h = nullptr;
     int32_t *s5_left_h = nullptr;  // rows still unmatched after a chunk of S5 passes

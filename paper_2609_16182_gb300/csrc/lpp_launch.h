@@ -174,6 +174,8 @@ struct SoloOut {
     int32_t m, nnz, cur;      // reduced rows and entries, in buffer cur
     int32_t act_buf, act_m;   // the last round's row results
     long long s5_left;
+    double offset;            // of the reduced LP, by launch_solo_finish, as is n
+    int32_t n, pad;
 };
 struct SoloCtl {  // zero before the launch
     SoloOut out;
@@ -204,6 +206,29 @@ struct SoloArgs {
 };
 int solo_blocks(int32_t m, int32_t n, int64_t nnz);
 bool launch_solo(const SoloArgs &F, int blocks, cudaStream_t s);
+// The end of such a run: objective constant, the columns' one compaction and
+// the reduced LP's A^T.  Reads the sizes launch_solo left in ctl.
+struct SoloFinish {
+    SoloCtl *ctl;
+    const int32_t *err_in;
+    int32_t n;                       // column slots
+    const int32_t *rp[2];            // the reduced CSR is in [ctl->out.cur]; the other buffers are scratch
+    int32_t *ci[2];
+    double *rv[2];
+    int32_t *tp[2], *ti[2];          // A^T, to [ctl->out.cur]
+    double *tv[2];
+    int64_t half;                    // entries of rv's first half (the payload's second buffer begins there)
+    const double2 *lu;
+    const double *c;
+    const int32_t *cmap;
+    double2 *lu2;
+    double *c2;
+    int32_t *cmap2, *cinv, *pos;
+    double *contrib, *part, *offset;
+    int32_t *btot, *hist;            // one / 256 per block
+};
+int solo_finish_blocks(int32_t n, int64_t nnz);
+bool launch_solo_finish(const SoloFinish &F, int blocks, cudaStream_t s);
 
 // ---------------------------------------------------------------- k_batch.cu
 // The persistent batch kernel: one thread block per LP at a time, every round

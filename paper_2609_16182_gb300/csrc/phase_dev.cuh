@@ -1058,6 +1058,32 @@ __device__ __forceinline__ void rowvec_one(const Ctx &C, const CompactCtx &K, in
     K.hrow2[p] = C.hrow[i];
 }
 
+// ---------------------------------------------------------- objective constant
+// The contributions of tile t's columns, summed in a fixed order, and consumed:
+// reset to zero once read (a column whose flags are not recomputed in a later
+// round then contributes nothing).
+__device__ __forceinline__ void offset_tile(double *contrib, int32_t n, double *part, int32_t t) {
+    const int64_t base = (int64_t)t * kScanTile;
+    double s = 0.0;
+    for (int q = threadIdx.x; q < kScanTile; q += kBlock) {
+        const int64_t j = base + q;
+        if (j < n) {
+            const double v = contrib[j];
+            s += v;
+            if (v != 0.0) contrib[j] = 0.0;
+        }
+    }
+    s = block_sum_dbl(s);
+    if (threadIdx.x == 0) part[t] = s;
+}
+// one block: thread t adds tiles t, t+256, ... in order, then the fixed-order block sum
+__device__ __forceinline__ void offset_final(const double *part, int32_t ntiles, double *offset) {
+    double s = 0.0;
+    for (int32_t t = threadIdx.x; t < ntiles; t += kBlock) s += part[t];
+    s = block_sum_dbl(s);
+    if (threadIdx.x == 0) offset[0] += s;
+}
+
 }  // namespace
 
 }  // namespace lpp
