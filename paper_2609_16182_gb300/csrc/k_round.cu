@@ -250,51 +250,13 @@ __global__ void __launch_bounds__(kTailBlock) k_s5_tail_block(Ctx C, int32_t *l0
 }
 
 // All remaining later passes of a long list in one cooperative launch (every
-// block resident): the passes of the launched form, separated by grid
-// barriers.  Mutable data (lists, slots, leaders, counts) is read at L2.  A
-// barrier that waits too long (it cannot, with every block resident) sets
-// st->err bit 4 and the kernel returns.  Same starting point and result
-// slot as k_s5_tail_block.
+// block resident; s5_later_passes).  Same starting point and result slot as
+// k_s5_tail_block.
 __global__ void __launch_bounds__(kBlock) k_s5_tail_grid(Ctx C, int32_t *l0, int32_t *l1, int32_t *cnt, int32_t p0,
                                                         int32_t max_iter, unsigned *bar) {
-    const int lane = threadIdx.x & 31;
-    const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, gstride = (int64_t)gridDim.x * blockDim.x;
-    const int64_t gwarp = gtid >> 5;
-    int32_t n = __ldcg(cnt + p0), from = (p0 - 1) & 1, rem = 0;
-    bool ok = true;
-    int32_t p = p0;
-    for (; p < max_iter && n > 0 && ok; p++) {
-        const int32_t *lst = from ? l1 : l0;
-        int32_t *nxt = from ? l0 : l1;
-        const uint32_t cap = s5_tail_cap(C, n);
-        for (int64_t t = gtid; t < n; t += gstride) {
-            const int32_t i = __ldcg(lst + t);
-            C.rslot[i] = s5_insert_row(C, i, cap);
-        }
-        if (!(ok = grid_barrier(bar, &C.st->err))) break;
-        for (int64_t tb = gwarp * 32; tb < n; tb += gstride) {  // warp-uniform: every lane calls the match
-            int32_t rm, i;
-            bool left;
-            s5_tail_match_one(C, lst, n, (int32_t)(tb + lane), rm, left, i);
-            rem += rm;
-            const unsigned want = __ballot_sync(0xffffffffu, left);
-            int32_t base = 0;
-            if (lane == 0 && want) base = atomicAdd(cnt + p + 1, __popc(want));
-            base = __shfl_sync(0xffffffffu, base, 0);
-            if (left) nxt[base + __popc(want & ((1u << lane) - 1u))] = i;
-        }
-        if (!(ok = grid_barrier(bar, &C.st->err))) break;
-        for (int64_t t = gtid; t < n; t += gstride) {
-            const int32_t sl = __ldcg(C.rslot + __ldcg(lst + t));
-            if (sl >= 0) {
-                C.tkey[sl] = 0ULL;
-                C.tlead[sl] = ~0ULL;
-            }
-        }
-        if (!(ok = grid_barrier(bar, &C.st->err))) break;
-        n = __ldcg(cnt + p + 1);
-        from ^= 1;
-    }
+    int32_t n = __ldcg(cnt + p0), rem = 0;
+    unsigned gen = 0;
+    const bool ok = s5_later_passes(C, l0, l1, cnt + 1, p0, max_iter, n, rem, bar, &C.st->err, gen);
     block_add(rem, &C.st->rows_removed);
     if (blockIdx.x == 0 && threadIdx.x == 0 && ok) cnt[max_iter] = n;
 }

@@ -193,9 +193,10 @@ __global__ void __launch_bounds__(kBlock, 2) k_solo(const __grid_constant__ Solo
     long long s5_left = 0;
     int32_t status = LPP_OK, where = LPP_WHERE_NONE, vindex = -1, vround = 0;
     // every block takes the same branches, so each passes the same barriers
-#define GRID_SYNC()                                        \
-    do {                                                   \
-        if (!grid_barrier(ctl->bar, &ctl->err)) goto out;  \
+    unsigned gen = 0;
+#define GRID_SYNC()                                            \
+    do {                                                       \
+        if (!grid_barrier(ctl->bar, &ctl->err, gen)) goto out; \
     } while (0)
 
     // the input's rows by class
@@ -364,8 +365,7 @@ __global__ void __launch_bounds__(kBlock, 2) k_solo(const __grid_constant__ Solo
             const int32_t n1 = N.n1;
             int32_t left = n1;
             if (n1 > 0 && F.par_max_iter > 1) {
-                // the table empty again, then the later passes: in one block for a
-                // short list, else over the grid
+                // the table empty again, then the later passes
                 for (int32_t i = gt; i < m; i += gstep) {
                     const int32_t sl = C.rslot[i];
                     if (sl >= 0) {
@@ -374,55 +374,16 @@ __global__ void __launch_bounds__(kBlock, 2) k_solo(const __grid_constant__ Solo
                     }
                 }
                 GRID_SYNC();
-                const bool alone = n1 <= 8 * kBlock;
-                if (!alone || blockIdx.x == 0) {
-                    const int32_t ft = alone ? tid : gt, fs = alone ? kBlock : gstep;
-                    int32_t from = 0;
-                    int32_t *cnt = F.s5_cnt;  // [par_max_iter + 2], zero
-                    for (int32_t p = 1; p < F.par_max_iter && left > 0; p++) {
-                        const int32_t *lst = F.s5l[from];
-                        int32_t *nxt = F.s5l[from ^ 1];
-                        const uint32_t cap = s5_tail_cap(C, left);
-                        for (int32_t t = ft; t < left; t += fs) {
-                            const int32_t i = __ldcg(lst + t);
-                            C.rslot[i] = s5_insert_row(C, i, cap);
-                        }
-                        if (alone) __syncthreads();
-                        else GRID_SYNC();
-                        for (int32_t tb = ft & ~31; tb < left; tb += fs) {
-                            int32_t rm, i;
-                            bool lf;
-                            s5_tail_match_one(C, lst, left, tb + (tid & 31), rm, lf, i);
-                            removed += rm;
-                            const unsigned want = __ballot_sync(0xffffffffu, lf);
-                            int32_t at = 0;
-                            if ((tid & 31) == 0 && want) at = atomicAdd(cnt + p, __popc(want));
-                            at = __shfl_sync(0xffffffffu, at, 0);
-                            if (lf) nxt[at + __popc(want & ((1u << (tid & 31)) - 1u))] = i;
-                        }
-                        if (alone) __syncthreads();
-                        else GRID_SYNC();
-                        for (int32_t t = ft; t < left; t += fs) {
-                            const int32_t sl = __ldcg(C.rslot + __ldcg(lst + t));
-                            if (sl >= 0) {
-                                C.tkey[sl] = 0ULL;
-                                C.tlead[sl] = ~0ULL;
-                            }
-                        }
-                        const int32_t next = __ldcg(cnt + p);
-                        if (alone) __syncthreads();
-                        else GRID_SYNC();
-                        if (ft == 0) cnt[p] = 0;  // for the next round's passes (read by all above)
-                        left = next;
-                        from ^= 1;
-                    }
-                    __syncwarp();
-                    warp_add(removed, &N.merged);
-                    removed = 0;
-                    if (ft == 0) N.n2 = left;
-                }
+                if (!s5_later_passes(C, F.s5l[0], F.s5l[1], F.s5_cnt, 1, F.par_max_iter, left, removed, ctl->bar,
+                                     &ctl->err, gen))
+                    goto out;
+                __syncwarp();
+                warp_add(removed, &N.merged);
+                removed = 0;
+                if (gt == 0) N.n2 = left;
                 GRID_SYNC();
                 left = N.n2;
+                for (int32_t q = gt; q < F.par_max_iter; q += gstep) F.s5_cnt[q] = 0;  // for the next round's passes
             }
             s5_clean = left == 0;
             s5_left += left;
@@ -761,9 +722,10 @@ __global__ void __launch_bounds__(kBlock) k_solo_finish(const __grid_constant__ 
     row_range(n, lo, hi);
     int passes = 1;
     while (passes < 4 && (int64_t)n > (int64_t)1 << (8 * passes)) passes++;
-#define GRID_SYNC()                                    \
-    do {                                               \
-        if (!grid_barrier(ctl->bar, &ctl->err)) return; \
+    unsigned gen = 0;
+#define GRID_SYNC()                                             \
+    do {                                                        \
+        if (!grid_barrier(ctl->bar + 1, &ctl->err, gen)) return; \
     } while (0)
     each_block(ctiles, [&](int32_t b) { offset_tile(F.contrib, n, F.part, b); });
     {

@@ -393,9 +393,8 @@ void Engine::setup(const lpp_opts &opts, int32_t nlp_, const std::vector<Member>
     tlead = pool.alloc<unsigned long long>(tcap_max);
     s5_list[0] = pool.alloc<int32_t>(m0);
     s5_list[1] = pool.alloc<int32_t>(m0);
-    s5_cnt = pool.alloc<int32_t>((size_t)o.par_max_iter + 2);
-    s5_bar = pool.alloc<unsigned>(2);
-    LPP_CUDA(cudaMemsetAsync(s5_bar, 0, 2 * sizeof(unsigned), s));
+    s5_cnt = pool.alloc<int32_t>((size_t)o.par_max_iter + 3);
+    s5_bar = reinterpret_cast<unsigned *>(s5_cnt + o.par_max_iter + 2);  // zero with the counts
     ch_act = pool.alloc<double2>(cap_chunk);
     ch_ninf = pool.alloc<int2>(cap_chunk);
     ch_hash = pool.alloc<unsigned long long>(cap_chunk);
@@ -978,7 +977,7 @@ Engine::StepOut Engine::step(int32_t r, bool first_round, bool force) {
     int32_t tcap = std::min(tcap_max, pow2_at_least(2 * (int64_t)std::max(m, 1)));
     tbegin(F_S5, run_s5 ? 16.0 * tcap + 12.0 * m : 0.0);
     if (run_s5) {
-        launch_s5_init(C, tcap, s5_cnt, o.par_max_iter + 2, s);
+        launch_s5_init(C, tcap, s5_cnt, o.par_max_iter + 3, s);
         C.tcap = tcap;
         C.s5_out = s5_list[0];
         C.s5_out_cnt = s5_cnt + 1;
@@ -1005,7 +1004,7 @@ Engine::StepOut Engine::step(int32_t r, bool first_round, bool force) {
     bool resolved = n1 == 0;
     if (n1 > 0 && o.par_max_iter > 1) {
         tbegin(F_S5, 0.0);
-        tcap = std::min(tcap_max, pow2_at_least(2 * (int64_t)n1));
+        tcap = std::min(tcap_max, pow2_at_least(4 * (int64_t)n1));  // two halves for the passes in turn
         launch_s5_init(C, tcap, nullptr, 0, s);
         C.tcap = tcap;
         int32_t chunk = 2, left = n1;

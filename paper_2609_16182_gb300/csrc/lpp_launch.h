@@ -179,7 +179,7 @@ struct SoloOut {
 };
 struct SoloCtl {  // zero before the launch
     SoloOut out;
-    unsigned bar[2];
+    unsigned bar[2];  // arrivals at the barriers of the rounds, of the finish
     int32_t err, pad;
     SoloCnt c[2];  // by the round's parity
 };

@@ -660,18 +660,18 @@ __device__ __forceinline__ void colfin_one(const Ctx &C, int32_t j, bool full, i
 // elects the leader of its key: the first equality row, else the first row
 // (Sec. 3.2), by atomicMin on (is_ineq, row).  Returns the slot, -1 if the
 // table is full (an internal error: the capacity is at least twice the rows).
-__device__ __forceinline__ int32_t s5_insert_row(const Ctx &C, int32_t i, uint32_t cap) {
+__device__ __forceinline__ int32_t s5_insert_row(const Ctx &C, int32_t i, uint32_t cap, uint32_t off = 0) {
     unsigned long long key = C.hrow[i];
     if (key == 0) key = 1;
     uint32_t sl = (uint32_t)(key ^ (key >> 32)) & (cap - 1u);
     for (uint32_t probe = 0; probe < cap; probe++) {
-        const unsigned long long prev = atomicCAS(&C.tkey[sl], 0ULL, key);
+        const unsigned long long prev = atomicCAS(&C.tkey[off + sl], 0ULL, key);
         if (prev == 0ULL || prev == key) {
             const double Lv = C.L[i], Uv = C.U[i];
             const bool eq = is_fin(Lv) && Lv == Uv;
             const unsigned long long code = ((unsigned long long)(eq ? 0u : 1u) << 32) | (uint32_t)i;
-            atomicMin(&C.tlead[sl], code);
-            return (int32_t)sl;
+            atomicMin(&C.tlead[off + sl], code);
+            return (int32_t)(off + sl);
         }
         sl = (sl + 1u) & (cap - 1u);
     }
