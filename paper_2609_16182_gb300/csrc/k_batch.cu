@@ -399,10 +399,18 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : (NT == 512 ? 2 : 8)) k_bat
                 // S6 inputs: entries of each column in kept rows, locks
                 for (int32_t j = c0 + tid; j < c0 + n; j += NT) {
                     int32_t cnt = 0, lk = 0;
-                    for (int32_t e = C.T.ptr[j]; e < C.T.ptr[j + 1]; e++) {
-                        const int32_t i = C.T.idx[e];
-                        cnt += C.rkind[i] == RK_KEPT;
-                        if (C.dualfix) lk |= entry_locks(C, i, C.T.val[e]);
+                    const int32_t e1 = C.T.ptr[j + 1];
+                    for (int32_t e = C.T.ptr[j]; e < e1; e += 4) {  // four entries' loads in flight
+                        int32_t i[4], kd[4];
+#pragma unroll
+                        for (int u = 0; u < 4; u++) i[u] = e + u < e1 ? C.T.idx[e + u] : -1;
+#pragma unroll
+                        for (int u = 0; u < 4; u++) kd[u] = i[u] >= 0 ? C.rkind[i[u]] : (int32_t)RK_EMPTY;
+#pragma unroll
+                        for (int u = 0; u < 4; u++) {
+                            cnt += kd[u] == RK_KEPT;
+                            if (C.dualfix && i[u] >= 0) lk |= entry_locks(C, i[u], C.T.val[e + u]);
+                        }
                     }
                     K.c_len[j] = cnt;
                     if (C.dualfix) K.c_lock[j] = lk;
@@ -505,13 +513,24 @@ __global__ void __launch_bounds__(NT, NT == 256 ? 4 : (NT == 512 ? 2 : 8)) k_bat
                             o = z0 + off[sg];
                         }
                         if (own && e - b <= 32)
-                            for (int32_t x = b; x < e; x++) {
-                                const int32_t ni = nw[idx[x]];
-                                if (ni >= 0) {
-                                    oi[o] = ni;
-                                    ov[o] = val[x];
-                                    o++;
+                            for (int32_t x = b; x < e; x += 4) {  // four entries' loads in flight
+                                int32_t ni[4];
+                                double v[4];
+#pragma unroll
+                                for (int u = 0; u < 4; u++) {
+                                    ni[u] = x + u < e ? idx[x + u] : -1;
+                                    v[u] = x + u < e ? val[x + u] : 0.0;
                                 }
+#pragma unroll
+                                for (int u = 0; u < 4; u++)
+                                    if (ni[u] >= 0) ni[u] = nw[ni[u]];
+#pragma unroll
+                                for (int u = 0; u < 4; u++)
+                                    if (ni[u] >= 0) {
+                                        oi[o] = ni[u];
+                                        ov[o] = v[u];
+                                        o++;
+                                    }
                             }
                         unsigned todo = __ballot_sync(0xffffffffu, own && e - b > 32);
                         while (todo) {
