@@ -778,6 +778,17 @@ __global__ void k_fill_i32(int32_t *a, int64_t cnt, int32_t v) {
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (k < cnt) a[k] = v;
 }
+__global__ void __launch_bounds__(256) k_publish(FetchArgs a) {
+    for (int k = 0; k < a.n; k++)
+        for (int32_t t = threadIdx.x; t < a.words[k]; t += 256) a.dst[k][t] = a.src[k][t];
+    __threadfence_system();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence_system();
+        *(volatile uint32_t *)a.flag = a.seq;
+    }
+}
+
 __global__ void k_split_lu(const double2 *lu, int32_t n, double *lb, double *ub) {
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= n) return;
@@ -789,6 +800,8 @@ __global__ void k_split_lu(const double2 *lu, int32_t n, double *lb, double *ub)
 void fill_i32(int32_t *a, int64_t cnt, int32_t v, cudaStream_t s) {
     if (cnt > 0) (k_fill_i32<<<(unsigned)((cnt + 255) / 256), 256, 0, s>>>(a, cnt, v), note_launch());
 }
+void launch_publish(const FetchArgs &a, cudaStream_t s) { (k_publish<<<1, 256, 0, s>>>(a), note_launch()); }
+
 void split_lu(const double2 *lu, int32_t n, double *lb, double *ub, cudaStream_t s) {
     if (n > 0) (k_split_lu<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(lu, n, lb, ub), note_launch());
 }

@@ -8,6 +8,7 @@
 // arena equals its result alone.
 #pragma once
 #include <cstdint>
+#include <initializer_list>
 #include <memory>
 #include <mutex>
 #include <stdexcept>
@@ -193,6 +194,8 @@ struct Engine {
     double solo_offset = 0.0;         // objective constant of the reduced LP, with it
     int32_t *verdict_h = nullptr;
     uint8_t *changed_h = nullptr;
+    uint32_t *fetch_flag = nullptr;  // pinned: the number of the last fetch the device has stored
+    uint32_t fetch_seq = 0;
     int32_t *s5_left_h = nullptr;  // rows still unmatched after a chunk of S5 passes
     SegMat A{}, T{};
     // per-LP results
@@ -244,6 +247,12 @@ struct Engine {
     cudaEvent_t ev_round[2] = {nullptr, nullptr};
     std::vector<uint8_t> lp_dropped;
     Ctx ctx(int32_t round) const;
+    struct FetchItem {
+        void *dst;  // pinned
+        const void *src;
+        size_t bytes;  // whole words of 4
+    };
+    void fetch(std::initializer_list<FetchItem> items);
     void read_status();
     void schedule_current(bool cols);
     void adopt_schedule(bool cols);

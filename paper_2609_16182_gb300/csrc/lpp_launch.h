@@ -72,6 +72,15 @@ void iota(int32_t *a, int32_t cnt, int32_t base, cudaStream_t s);
 void ptr_diff(const int32_t *ptr, int32_t cnt, int32_t *out, cudaStream_t s);  // out[i] = ptr[i+1] - ptr[i]
 void fill_u64(unsigned long long *a, int64_t cnt, unsigned long long v, cudaStream_t s);
 void fill_i32(int32_t *a, int64_t cnt, int32_t v, cudaStream_t s);
+// device words to pinned host memory, then seq to *flag (pinned)
+constexpr int kFetchMax = 2;
+struct FetchArgs {
+    uint32_t *dst[kFetchMax];
+    const uint32_t *src[kFetchMax];
+    int32_t words[kFetchMax], n;
+    uint32_t *flag, seq;
+};
+void launch_publish(const FetchArgs &a, cudaStream_t s);
 void split_lu(const double2 *lu, int32_t n, double *lb, double *ub, cudaStream_t s);
 
 // ---------------------------------------------------------------- k_round.cu
