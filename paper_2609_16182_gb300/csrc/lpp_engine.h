@@ -61,10 +61,11 @@ struct DevPool {
 };
 
 // Most entries of an LP whose rounds run in one kernel (Engine::solo).
-// Measured, the rounds launched / in one kernel: 1.5 k entries 597 / 380 us,
-// 0.18 M 2088 / 1380, 1.8 M 2343 / 2053; 7.8 M 5126 / 6964 (two blocks per SM
-// at 128 registers hold fewer gathers in flight than the launched kernels).
-constexpr int64_t kSoloNnz = 2 << 20;
+// Measured, the rounds launched / in one kernel, us: 1.5 k entries 597 / 353,
+// 0.18 M 2088 / 1163, 2.4 M 2433 / 2230; 3.1 M 3469 / 3907, 4.7 M 2743 / 3367 (two
+// blocks per SM at 128 registers hold fewer gathers in flight than the launched
+// kernels).
+constexpr int64_t kSoloNnz = 5 << 19;
 
 // per-LP description of an arena member
 struct Member {
