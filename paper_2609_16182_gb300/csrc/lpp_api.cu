@@ -1146,7 +1146,18 @@ lpp_status lpp_postsolve_primal(const lpp_postsolve *Pc, const double *x_red, do
     lpp_postsolve *P = const_cast<lpp_postsolve *>(Pc);
     if (!P->dev->ca && !P->dev->sb) {
         if (!x_red && P->info.n_red > 0) return set_err(LPP_ERR_INVALID, "NULL argument");
-        return guarded([&]() -> lpp_status { return primal_on_device(P, x_red, x_orig); });
+        bool room = true;
+        const lpp_status st = guarded([&]() -> lpp_status {
+            try {
+                return primal_on_device(P, x_red, x_orig);
+            } catch (const CudaError &e) {
+                if (e.code != cudaErrorMemoryAllocation) throw;
+                cudaGetLastError();
+                room = false;  // the host form below needs none
+                return LPP_OK;
+            }
+        });
+        if (room) return st;
     }
     const lpp_status st = guarded([&]() -> lpp_status { materialize(P, REC_ROWS | REC_COLS | REC_MERGES | REC_SUBST); return LPP_OK; });
     if (st != LPP_OK) return st;
