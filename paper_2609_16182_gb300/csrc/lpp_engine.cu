@@ -804,7 +804,10 @@ void Engine::fetch(std::initializer_list<FetchItem> items) {
         if (k % 256) continue;
         // an error on the stream ends the wait; a finished stream has published
         const cudaError_t e = cudaStreamQuery(s);
-        if (e == cudaErrorNotReady) continue;
+        if (e == cudaErrorNotReady) {
+            cudaGetLastError();  // not an error of the launches that follow
+            continue;
+        }
         LPP_CUDA(e);
         LPP_CUDA(cudaStreamSynchronize(s));
         if (!seen()) throw StatusError(LPP_ERR_CUDA, "internal: status not published");
