@@ -256,8 +256,7 @@ __global__ void k_idx_renumber(int32_t *idx, int64_t nnz, const int32_t *pos) {
 }
 
 // ---------------------------------------------------------- vector gathers
-__global__ void __launch_bounds__(kBlock) k_rowvec(Ctx C, CompactCtx K) {
-    const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void rowvec_at(const Ctx &C, const CompactCtx &K, int32_t i) {
     if (i >= C.m) return;
     if (i == C.m - 1) {
         K.rp2[K.r_pos[C.m]] = K.r_off[C.m];
@@ -273,8 +272,7 @@ __global__ void __launch_bounds__(kBlock) k_rowvec(Ctx C, CompactCtx K) {
     if (K.r_keep[i]) rowvec_one(C, K, i, p, K.r_off[i], !C.in_place && K.c_pos[C.n] != C.n);
 }
 
-__global__ void __launch_bounds__(kBlock) k_colvec(Ctx C, CompactCtx K) {
-    const int32_t j = blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void colvec_at(const Ctx &C, const CompactCtx &K, int32_t j) {
     if (j >= C.n) return;
     if (j == C.n - 1) {
         K.cp2[K.c_pos[C.n]] = K.c_off[C.n];
@@ -289,6 +287,16 @@ __global__ void __launch_bounds__(kBlock) k_colvec(Ctx C, CompactCtx K) {
     K.cmap2[p] = C.cmap[j];
     if (C.lp_col) K.lp_col2[p] = C.lp_col[j];
     K.cp2[p] = K.c_off[j];
+}
+
+__global__ void __launch_bounds__(kBlock) k_rowvec(Ctx C, CompactCtx K) {
+    rowvec_at(C, K, blockIdx.x * kBlock + threadIdx.x);
+}
+// rows, then columns from block rb on (the columns compacted each round)
+__global__ void __launch_bounds__(kBlock) k_vecs(Ctx C, CompactCtx K, int32_t rb) {
+    const int32_t b = blockIdx.x;
+    if (b < rb) rowvec_at(C, K, b * kBlock + threadIdx.x);
+    else colvec_at(C, K, (b - rb) * kBlock + threadIdx.x);
 }
 
 // without rows or columns: ptr[0] = 0 and the sizes
@@ -312,6 +320,12 @@ __global__ void k_empty(Ctx C, CompactCtx K) {
 __global__ void __launch_bounds__(kBlock) k_scatter_flat(FlatArgs F) {
     __shared__ FlatShared S;
     flat_tile(F, blockIdx.x, S);
+}
+
+__global__ void __launch_bounds__(kBlock) k_scatter_both(FlatArgs A, FlatArgs T) {
+    __shared__ FlatShared S;
+    const bool second = (int32_t)blockIdx.x >= A.ntiles;
+    flat_tile(second ? T : A, blockIdx.x - (second ? A.ntiles : 0), S);
 }
 
 // ---------------------------------------------------------- objective constant
@@ -452,17 +466,22 @@ void launch_compact_scatter(const Ctx &C, const CompactCtx &K, int32_t nnz, cuda
     // k_rowvec and k_colvec write the pointers (entry 0 with the first kept
     // segment or the total) and the new sizes; an empty dimension is left to k_empty
     if (C.m == 0 || C.n == 0) (k_empty<<<1, 1, 0, s>>>(C, K), note_launch());
-    if (C.m > 0) (k_rowvec<<<blocks_for(C.m, kBlock), kBlock, 0, s>>>(C, K), note_launch());
-    if (C.n > 0 && !C.in_place) (k_colvec<<<blocks_for(C.n, kBlock), kBlock, 0, s>>>(C, K), note_launch());
+    const int32_t rb = C.m > 0 ? (int32_t)blocks_for(C.m, kBlock) : 0;
+    if (C.in_place) {
+        if (rb > 0) (k_rowvec<<<rb, kBlock, 0, s>>>(C, K), note_launch());
+    } else if (C.m > 0 || C.n > 0) {
+        (k_vecs<<<rb + (C.n > 0 ? (int32_t)blocks_for(C.n, kBlock) : 0), kBlock, 0, s>>>(C, K, rb), note_launch());
+    }
     const int32_t ntiles = (int32_t)(((int64_t)nnz + kFlatTile - 1) / kFlatTile);
     if (ntiles > 0) {
         FlatArgs fa{C.A.ptr, C.A.idx, C.A.val, nnz, C.m, ntiles, K.r_keep, K.r_off, K.r_len, K.r_ch0,
                     K.chr_off, K.chr_cnt, K.c_new, C.in_place ? C.cchg : nullptr, K.tile_a, K.ci2, K.rv2};
-        (k_scatter_flat<<<ntiles, kBlock, 0, s>>>(fa), note_launch());
-        if (!C.in_place) {
+        if (C.in_place) {
+            (k_scatter_flat<<<ntiles, kBlock, 0, s>>>(fa), note_launch());
+        } else {
             FlatArgs ft{C.T.ptr, C.T.idx, C.T.val, nnz, C.n, ntiles, K.c_keep, K.c_off, K.c_len, K.c_ch0,
                         K.cht_off, K.cht_cnt, K.r_new, nullptr, K.tile_t, K.ri2, K.cv2};
-            (k_scatter_flat<<<ntiles, kBlock, 0, s>>>(ft), note_launch());
+            (k_scatter_both<<<2 * ntiles, kBlock, 0, s>>>(fa, ft), note_launch());
         }
     }
 }

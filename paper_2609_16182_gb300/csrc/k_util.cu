@@ -18,6 +18,14 @@ namespace {
 constexpr int kScanThreads = 256;
 constexpr int kPerThread = kScanTile / kScanThreads;  // 8
 
+// a schedule's build: segments ptr[0, *cnt_dev], buffers, class sizes and chunk count
+struct SchedJob {
+    const int32_t *ptr, *cnt_dev;
+    SchedBufs b;
+    int32_t *cls, *nchunk;
+    int32_t tiles, cap_long;
+};
+
 struct Pair {
     int32_t a, b;
 };
@@ -124,21 +132,19 @@ __device__ __forceinline__ T block_excl_scan(T v, T &excl, T *s_w) {
 }
 
 template <class T, class In>
-__global__ void __launch_bounds__(kScanThreads) k_scan_reduce(In in, int64_t cnt, T *tsum) {
-    __shared__ T s_w[33];
+__device__ __forceinline__ void scan_reduce_tile(In in, int64_t cnt, T *tsum, int32_t tile, T *s_w) {
     T x[kPerThread], v = zero_of<T>();
-    in.get8((int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kPerThread, cnt, x);
+    in.get8((int64_t)tile * kScanTile + (int64_t)threadIdx.x * kPerThread, cnt, x);
 #pragma unroll
     for (int q = 0; q < kPerThread; q++) v = v + x[q];
     T ex;
     const T tot = block_excl_scan(v, ex, s_w);
-    if (threadIdx.x == 0) tsum[blockIdx.x] = tot;
+    if (threadIdx.x == 0) tsum[tile] = tot;
 }
 
 // one block: exclusive scan of tsum[0..ntiles) in place, tsum[ntiles] = out[cnt] = total
 template <class T, class Out>
-__global__ void __launch_bounds__(1024) k_scan_top(T *tsum, int32_t ntiles, Out out, int64_t cnt) {
-    __shared__ T s_w[33];
+__device__ __forceinline__ void scan_top_block(T *tsum, int32_t ntiles, Out out, int64_t cnt, T *s_w) {
     T carry = zero_of<T>();
     for (int32_t b = 0; b < ntiles; b += 1024) {
         const int32_t k = b + threadIdx.x;
@@ -159,8 +165,7 @@ __global__ void __launch_bounds__(1024) k_scan_top(T *tsum, int32_t ntiles, Out 
 // about what the three launches take).
 constexpr int64_t kScanSmall = 32768;
 template <class T, class In, class Out>
-__global__ void __launch_bounds__(1024) k_scan_one(In in, Out out, int64_t cnt) {
-    __shared__ T s_w[33];
+__device__ __forceinline__ void scan_one_block(In in, Out out, int64_t cnt, T *s_w) {
     T carry = zero_of<T>();
     for (int64_t base = 0; base < cnt; base += 1024 * kPerThread) {
         const int64_t k = base + (int64_t)threadIdx.x * kPerThread;
@@ -185,10 +190,9 @@ __global__ void __launch_bounds__(1024) k_scan_one(In in, Out out, int64_t cnt) 
 }
 
 template <class T, class In, class Out>
-__global__ void __launch_bounds__(kScanThreads) k_scan_down(In in, Out out, int64_t cnt, const T *tsum) {
-    __shared__ T s_w[33];
+__device__ __forceinline__ void scan_down_tile(In in, Out out, int64_t cnt, const T *tsum, int32_t tile, T *s_w) {
     static_assert(kPerThread == 8, "the scan's thread step is eight values");
-    const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kPerThread;
+    const int64_t base = (int64_t)tile * kScanTile + (int64_t)threadIdx.x * kPerThread;
     T v[kPerThread];
     in.get8(base, cnt, v);
     T s = zero_of<T>();
@@ -196,7 +200,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_down(In in, Out out, int6
     for (int q = 0; q < kPerThread; q++) s = s + v[q];
     T ex;
     block_excl_scan(s, ex, s_w);
-    T run = tsum[blockIdx.x] + ex;
+    T run = tsum[tile] + ex;
     T o[kPerThread];
 #pragma unroll
     for (int q = 0; q < kPerThread; q++) {
@@ -204,6 +208,55 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_down(In in, Out out, int6
         run = run + v[q];
     }
     out.put8(base, cnt, o);
+}
+
+__global__ void __launch_bounds__(kScanThreads) k_scan_reduce(In1 in, int64_t cnt, int32_t *tsum) {
+    __shared__ int32_t s_w[33];
+    scan_reduce_tile(in, cnt, tsum, blockIdx.x, s_w);
+}
+__global__ void __launch_bounds__(1024) k_scan_top(int32_t *tsum, int32_t ntiles, Out1 out, int64_t cnt) {
+    __shared__ int32_t s_w[33];
+    scan_top_block(tsum, ntiles, out, cnt, s_w);
+}
+__global__ void __launch_bounds__(kScanThreads) k_scan_down(In1 in, Out1 out, int64_t cnt, const int32_t *tsum) {
+    __shared__ int32_t s_w[33];
+    scan_down_tile(in, out, cnt, tsum, blockIdx.x, s_w);
+}
+__global__ void __launch_bounds__(1024) k_scan_one(In1 in, Out1 out, int64_t cnt) {
+    __shared__ int32_t s_w[33];
+    scan_one_block(in, out, cnt, s_w);
+}
+
+// The pair scans of one or two matrices (rows of A, rows of A^T) in one launch
+// each: the blocks past the first job's take the second (tiles 0: no such job).
+struct PairJob {
+    In2 in;
+    Out2 out;
+    int64_t cnt;
+    Pair *tsum;
+    int32_t tiles;
+};
+__global__ void __launch_bounds__(kScanThreads) k_pairs_reduce(PairJob a, PairJob b) {
+    __shared__ Pair s_w[33];
+    const bool second = (int32_t)blockIdx.x >= a.tiles;
+    scan_reduce_tile(second ? b.in : a.in, second ? b.cnt : a.cnt, second ? b.tsum : a.tsum,
+                     blockIdx.x - (second ? a.tiles : 0), s_w);
+}
+__global__ void __launch_bounds__(1024) k_pairs_top(PairJob a, PairJob b) {
+    __shared__ Pair s_w[33];
+    const PairJob &J = blockIdx.x ? b : a;
+    scan_top_block(J.tsum, J.tiles, J.out, J.cnt, s_w);
+}
+__global__ void __launch_bounds__(kScanThreads) k_pairs_down(PairJob a, PairJob b) {
+    __shared__ Pair s_w[33];
+    const bool second = (int32_t)blockIdx.x >= a.tiles;
+    scan_down_tile(second ? b.in : a.in, second ? b.out : a.out, second ? b.cnt : a.cnt, second ? b.tsum : a.tsum,
+                   blockIdx.x - (second ? a.tiles : 0), s_w);
+}
+__global__ void __launch_bounds__(1024) k_pairs_one(PairJob a, PairJob b) {
+    __shared__ Pair s_w[33];
+    const PairJob &J = blockIdx.x ? b : a;
+    scan_one_block(J.in, J.out, J.cnt, s_w);
 }
 
 // --------------------------------------------------------------- binning
@@ -221,13 +274,21 @@ __device__ __forceinline__ void load_classes(const int32_t *ptr, int64_t base, i
     for (int q = 0; q < kPerThread; q++) c[q] = base + q < cnt ? seg_class(p[q + 1] - p[q]) : kNumClass;
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_bin_count(const int32_t *ptr, const int32_t *cnt_dev, int32_t *cls,
-                                                            int32_t *places) {
+// One or two matrices per launch: the blocks past the first one's tiles take
+// the second.  With the schedules, scans, vectors and scatters of A and A^T launched
+// one after the other, a presolve of 500 k rows with col_singletons and dual_fixing
+// (eight compactions) took 6.16 ms, now 5.75, with parallel_cols 7.24, now 6.84.
+__global__ void __launch_bounds__(kScanThreads) k_bin_count(SchedJob ja, SchedJob jb) {
     __shared__ int32_t s_n[kNumClass];
-    const int32_t cnt = *cnt_dev;
+    const bool second = (int32_t)blockIdx.x >= ja.tiles;
+    const SchedJob &J = second ? jb : ja;
+    const int32_t tile = blockIdx.x - (second ? ja.tiles : 0);
+    const int32_t *ptr = J.ptr;
+    int32_t *cls = J.cls, *places = J.b.tile_hist;
+    const int32_t cnt = *J.cnt_dev;
     if (threadIdx.x < kNumClass) s_n[threadIdx.x] = 0;
     __syncthreads();
-    const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kPerThread;
+    const int64_t base = (int64_t)tile * kScanTile + (int64_t)threadIdx.x * kPerThread;
     int c[kPerThread];
     load_classes(ptr, base, cnt, c);
     unsigned long long n = 0;  // eight bits per class
@@ -241,22 +302,26 @@ __global__ void __launch_bounds__(kScanThreads) k_bin_count(const int32_t *ptr, 
     __syncthreads();
     if (threadIdx.x < kNumClass) {
         const int32_t t = s_n[threadIdx.x];
-        places[(int64_t)blockIdx.x * kNumClass + threadIdx.x] = t ? atomicAdd(cls + threadIdx.x, t) : 0;
+        places[(int64_t)tile * kNumClass + threadIdx.x] = t ? atomicAdd(cls + threadIdx.x, t) : 0;
     }
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_bin_fill(const int32_t *ptr, const int32_t *cnt_dev,
-                                                           const int32_t *cls, const int32_t *places, int32_t *order) {
+__global__ void __launch_bounds__(kScanThreads) k_bin_fill(SchedJob ja, SchedJob jb) {
     __shared__ int32_t s_at[kNumClass];
     __shared__ unsigned long long s_w[2][kScanThreads / 32];
-    const int32_t cnt = *cnt_dev;
+    const bool second = (int32_t)blockIdx.x >= ja.tiles;
+    const SchedJob &J = second ? jb : ja;
+    const int32_t tile = blockIdx.x - (second ? ja.tiles : 0);
+    const int32_t *ptr = J.ptr, *cls = J.cls, *places = J.b.tile_hist;
+    int32_t *order = J.b.order;
+    const int32_t cnt = *J.cnt_dev;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (threadIdx.x < kNumClass) {
         int32_t start = 0;
         for (int k = 0; k < (int)threadIdx.x; k++) start += cls[k];
-        s_at[threadIdx.x] = start + places[(int64_t)blockIdx.x * kNumClass + threadIdx.x];
+        s_at[threadIdx.x] = start + places[(int64_t)tile * kNumClass + threadIdx.x];
     }
-    const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kPerThread;
+    const int64_t base = (int64_t)tile * kScanTile + (int64_t)threadIdx.x * kPerThread;
     int c[kPerThread];
     load_classes(ptr, base, cnt, c);
     // exclusive scan over the threads of the counts per class, 16 bits each, in two words
@@ -296,14 +361,16 @@ __global__ void __launch_bounds__(kScanThreads) k_bin_fill(const int32_t *ptr, c
     }
 }
 
-// one block: the chunks of the long segments (class 6, in schedule order),
+// one block per matrix: the chunks of the long segments (class 6, in schedule order),
 // their first chunk (lfirst, with the total at lfirst[long count]) and the count
-__global__ void __launch_bounds__(1024) k_chunks(const int32_t *ptr, const int32_t *order, const int32_t *cls,
-                                                 int32_t cap_long, int32_t *lfirst, Chunk *chunks,
-                                                 int32_t *nchunk_out) {
+__global__ void __launch_bounds__(1024) k_chunks(SchedJob ja, SchedJob jb) {
     __shared__ int32_t s_w[33];
-    const int32_t nlong = min(cls[6], cap_long);
-    const int32_t *lo = order;
+    const SchedJob &J = blockIdx.x ? jb : ja;
+    const int32_t *ptr = J.ptr, *cls = J.cls;
+    int32_t *lfirst = J.b.lfirst, *nchunk_out = J.nchunk;
+    Chunk *chunks = J.b.chunks;
+    const int32_t nlong = min(cls[6], J.cap_long);
+    const int32_t *lo = J.b.order;
     for (int k = 0; k < 6; k++) lo += cls[k];
     int32_t carry = 0;
     for (int32_t b = 0; b < nlong; b += 1024) {
@@ -617,26 +684,33 @@ size_t scan_tmp_elems(int64_t cnt) { return 2 * ((size_t)((cnt + kScanTile - 1) 
 
 void scan_excl(const int32_t *in, int32_t *out, int64_t cnt, int32_t *tmp, cudaStream_t s) {
     if (cnt <= kScanSmall) {
-        (k_scan_one<int32_t><<<1, 1024, 0, s>>>(In1{in}, Out1{out}, cnt), note_launch());
+        (k_scan_one<<<1, 1024, 0, s>>>(In1{in}, Out1{out}, cnt), note_launch());
         return;
     }
     const int32_t ntiles = (int32_t)((cnt + kScanTile - 1) / kScanTile);
-    if (ntiles > 0) (k_scan_reduce<int32_t><<<ntiles, kScanThreads, 0, s>>>(In1{in}, cnt, tmp), note_launch());
-    (k_scan_top<int32_t><<<1, 1024, 0, s>>>(tmp, ntiles, Out1{out}, cnt), note_launch());
-    if (ntiles > 0) (k_scan_down<int32_t><<<ntiles, kScanThreads, 0, s>>>(In1{in}, Out1{out}, cnt, tmp), note_launch());
+    if (ntiles > 0) (k_scan_reduce<<<ntiles, kScanThreads, 0, s>>>(In1{in}, cnt, tmp), note_launch());
+    (k_scan_top<<<1, 1024, 0, s>>>(tmp, ntiles, Out1{out}, cnt), note_launch());
+    if (ntiles > 0) (k_scan_down<<<ntiles, kScanThreads, 0, s>>>(In1{in}, Out1{out}, cnt, tmp), note_launch());
 }
 
-void scan_excl2(const int32_t *a, const int32_t *b, int32_t *oa, int32_t *ob, int64_t cnt, int32_t *tmp,
-                cudaStream_t s) {
-    if (cnt <= kScanSmall) {
-        (k_scan_one<Pair><<<1, 1024, 0, s>>>(In2{a, b}, Out2{oa, ob}, cnt), note_launch());
+void scan_pairs(const ScanPair *j, int jobs, int32_t *tmp, cudaStream_t s) {
+    PairJob J[2] = {};
+    int64_t most = 0;
+    int32_t tiles = 0;
+    for (int q = 0; q < jobs; q++) {
+        J[q] = PairJob{In2{j[q].a, j[q].b}, Out2{j[q].oa, j[q].ob}, j[q].cnt, reinterpret_cast<Pair *>(tmp),
+                       (int32_t)((j[q].cnt + kScanTile - 1) / kScanTile)};
+        tmp += scan_tmp_elems(j[q].cnt);
+        most = std::max(most, j[q].cnt);
+        tiles += J[q].tiles;
+    }
+    if (most <= kScanSmall) {
+        (k_pairs_one<<<jobs, 1024, 0, s>>>(J[0], J[1]), note_launch());
         return;
     }
-    const int32_t ntiles = (int32_t)((cnt + kScanTile - 1) / kScanTile);
-    Pair *t = reinterpret_cast<Pair *>(tmp);
-    if (ntiles > 0) (k_scan_reduce<Pair><<<ntiles, kScanThreads, 0, s>>>(In2{a, b}, cnt, t), note_launch());
-    (k_scan_top<Pair><<<1, 1024, 0, s>>>(t, ntiles, Out2{oa, ob}, cnt), note_launch());
-    if (ntiles > 0) (k_scan_down<Pair><<<ntiles, kScanThreads, 0, s>>>(In2{a, b}, Out2{oa, ob}, cnt, t), note_launch());
+    (k_pairs_reduce<<<tiles, kScanThreads, 0, s>>>(J[0], J[1]), note_launch());
+    (k_pairs_top<<<jobs, 1024, 0, s>>>(J[0], J[1]), note_launch());
+    (k_pairs_down<<<tiles, kScanThreads, 0, s>>>(J[0], J[1]), note_launch());
 }
 
 size_t sched_tile_hist_elems(int64_t cnt) {
@@ -645,16 +719,21 @@ size_t sched_tile_hist_elems(int64_t cnt) {
 
 int32_t sched_cap_long(int64_t nnz) { return (int32_t)std::max<int64_t>(1, nnz / kLongMin); }
 
-void build_schedule(const int32_t *ptr, const int32_t *cnt_dev, int32_t cnt_max, int64_t nnz_max,
-                    const SchedBufs &b, int32_t *cls_out, int32_t *nchunk_out, cudaStream_t s) {
-    // tiles cover cnt_max segments; tiles past the actual count hold zeros
-    const int32_t ntiles = std::max<int32_t>(1, (int32_t)((cnt_max + kScanTile - 1) / kScanTile));
-    cudaMemsetAsync(cls_out, 0, kNumClass * sizeof(int32_t), s);
-    (k_bin_count<<<ntiles, kScanThreads, 0, s>>>(ptr, cnt_dev, cls_out, b.tile_hist), note_launch());
-    (k_bin_fill<<<ntiles, kScanThreads, 0, s>>>(ptr, cnt_dev, cls_out, b.tile_hist, b.order), note_launch());
-    // chunks of the long segments: at most nnz / kLongMin of them
-    const int32_t cap_long = sched_cap_long(nnz_max);
-    (k_chunks<<<1, 1024, 0, s>>>(ptr, b.order, cls_out, cap_long, b.lfirst, b.chunks, nchunk_out), note_launch());
+void build_schedules(const SchedIn *in, int jobs, cudaStream_t s) {
+    SchedJob J[2] = {};
+    int32_t tiles = 0;
+    for (int q = 0; q < jobs; q++) {
+        // tiles cover cnt_max segments; tiles past the actual count hold zeros;
+        // at most nnz / kLongMin long segments
+        J[q] = SchedJob{in[q].ptr, in[q].cnt_dev, in[q].b, in[q].cls_out, in[q].nchunk_out,
+                        std::max<int32_t>(1, (int32_t)((in[q].cnt_max + kScanTile - 1) / kScanTile)),
+                        sched_cap_long(in[q].nnz_max)};
+        tiles += J[q].tiles;
+        cudaMemsetAsync(in[q].cls_out, 0, kNumClass * sizeof(int32_t), s);
+    }
+    (k_bin_count<<<tiles, kScanThreads, 0, s>>>(J[0], J[1]), note_launch());
+    (k_bin_fill<<<tiles, kScanThreads, 0, s>>>(J[0], J[1]), note_launch());
+    (k_chunks<<<jobs, 1024, 0, s>>>(J[0], J[1]), note_launch());
 }
 
 void segmat_from_counts(SegMat &M, const int32_t cls[kNumClass], int32_t nchunks) {

@@ -354,7 +354,7 @@ void Engine::setup(const lpp_opts &opts, int32_t nlp_, const std::vector<Member>
     const int64_t max_scan = std::max<int64_t>({nnz0 + 1, (int64_t)transpose_hist_elems(nnz0),
                                                 (int64_t)sched_tile_hist_elems(std::max(m0, n0)), m0 + 1, n0 + 1,
                                                 (int64_t)cap_long_a + 1});
-    scan_tmp = pool.alloc<int32_t>(scan_tmp_elems(max_scan));
+    scan_tmp = pool.alloc<int32_t>(std::max(scan_tmp_elems(max_scan), scan_tmp_elems(m0) + scan_tmp_elems(n0)));
     for (int w = 0; w < 2; w++) {
         SchedBufs &b = w == 0 ? sa : sb;
         const int32_t cnt = w == 0 ? m0 : n0;
@@ -744,8 +744,9 @@ void Engine::check_status() {
 // Launches the schedule builds of the current CSR and (cols) CSC; the segment
 // counts are read from st->m_new / st->n_new on the device (m, n bound them).
 void Engine::schedule_current(bool cols) {
-    build_schedule(m_rp, &st->m_new, m, nnz, sa, st->cls_r, &st->nchunk_r, s);
-    if (cols) build_schedule(tp[cur], &st->n_new, n, nnz, sb, st->cls_c, &st->nchunk_c, s);
+    const SchedIn in[2] = {{m_rp, &st->m_new, m, nnz, sa, st->cls_r, &st->nchunk_r},
+                           {tp[cur], &st->n_new, n, nnz, sb, st->cls_c, &st->nchunk_c}};
+    build_schedules(in, cols ? 2 : 1, s);
     LPP_CUDA(cudaGetLastError());
 }
 
@@ -936,8 +937,8 @@ void Engine::compact(int32_t round) {
     // columns in place: no column scan, no column vectors moved; the slots of
     // the columns that leave are marked (cinv) and dropped once, at the end
     tbegin(F_SCAN, 16.0 * (m + (in_place ? 0 : n)) * 2);
-    scan_excl2(K.r_keep, K.r_len, K.r_pos, K.r_off, m, scan_tmp, s);
-    if (!in_place) scan_excl2(K.c_keep, K.c_len, K.c_pos, K.c_off, n, scan_tmp, s);
+    const ScanPair pairs[2] = {{K.r_keep, K.r_len, K.r_pos, K.r_off, m}, {K.c_keep, K.c_len, K.c_pos, K.c_off, n}};
+    scan_pairs(pairs, in_place ? 1 : 2, scan_tmp, s);
     tend();
     // the objective constant of the columns that left: with the columns in
     // place each slot's contribution stays until one sum at the end

@@ -15,9 +15,14 @@ int64_t launch_count();
 // must hold scan_tmp_elems(cnt) int32 values.  in == out is allowed.
 size_t scan_tmp_elems(int64_t cnt);
 void scan_excl(const int32_t *in, int32_t *out, int64_t cnt, int32_t *tmp, cudaStream_t s);
-// two exclusive scans in one pass (oa[cnt], ob[cnt] = totals)
-void scan_excl2(const int32_t *a, const int32_t *b, int32_t *oa, int32_t *ob, int64_t cnt, int32_t *tmp,
-                cudaStream_t s);
+// two exclusive scans in one pass (oa[cnt], ob[cnt] = totals), for one or two
+// such pairs of arrays; tmp: scan_tmp_elems of each
+struct ScanPair {
+    const int32_t *a, *b;
+    int32_t *oa, *ob;
+    int64_t cnt;
+};
+void scan_pairs(const ScanPair *j, int jobs, int32_t *tmp, cudaStream_t s);
 
 // Schedule (class lists + chunks) of a segmented matrix with ptr[cnt+1].
 struct SchedBufs {
@@ -31,11 +36,17 @@ struct SchedBufs {
 size_t sched_tile_hist_elems(int64_t cnt);
 // most long segments a matrix with nnz entries can have (sizes lfirst, nch)
 int32_t sched_cap_long(int64_t nnz);
-// Builds the schedule and writes the class sizes to cls_out[7] and the chunk
-// count to *nchunk_out (device addresses inside DevStatus).  Chunks need at
-// most nnz / kChunk + cap_long entries.
-void build_schedule(const int32_t *ptr, const int32_t *cnt_dev, int32_t cnt_max, int64_t nnz_max,
-                    const SchedBufs &b, int32_t *cls_out, int32_t *nchunk_out, cudaStream_t s);
+// Builds the schedules of one or two matrices and writes the class sizes to
+// cls_out[7] and the chunk count to *nchunk_out (device addresses inside
+// DevStatus).  Chunks need at most nnz / kChunk + cap_long entries.
+struct SchedIn {
+    const int32_t *ptr, *cnt_dev;
+    int32_t cnt_max;
+    int64_t nnz_max;
+    SchedBufs b;
+    int32_t *cls_out, *nchunk_out;
+};
+void build_schedules(const SchedIn *in, int jobs, cudaStream_t s);
 // Fill the host-side part of a SegMat from class sizes read back.
 void segmat_from_counts(SegMat &M, const int32_t cls[kNumClass], int32_t nchunks);
 GroupGrid group_grid(const SegMat &M);
