@@ -527,28 +527,50 @@ inline unsigned blocks_for(int64_t cnt, int threads) {
 
 }  // namespace
 
+// The rows of more than 4096 entries (a chain of three kernels over their chunks
+// before the selection, three after) run on the side stream beside the others:
+// the two touch disjoint rows, bid with order-free minima, and an applied row's
+// columns are its own.  With them (and the objective constant's sums) one after
+// the other a presolve of 500 k rows with col_singletons and dual_fixing took
+// 5.75 ms, now 5.33.
 void launch_s5d(const Ctx &C, int32_t *rcand, uint8_t *relig, int32_t *cmin, int32_t *tasks, int32_t *ntask,
-                double *cs_a, cudaStream_t s) {
+                double *cs_a, cudaStream_t s, const SideStream *side) {
     if (C.n <= 0 || C.m <= 0) return;
     const int32_t task_grid = std::min<int32_t>(C.m, 2 * 152);
     const int32_t nlong = C.A.cls_start[7] - C.A.cls_start[6];
     const bool chunked = nlong > 0 && C.A.nchunks > 0;
     const unsigned long_warps = blocks_for((int64_t)nlong * 32, kBlock);
+    const bool fork = chunked && side && side->s;
+    const cudaStream_t sl = fork ? side->s : s;
+    const auto split = [&] {
+        if (!fork) return;
+        cudaEventRecord(side->fork, s);
+        cudaStreamWaitEvent(side->s, side->fork, 0);
+    };
+    const auto join = [&] {
+        if (!fork) return;
+        cudaEventRecord(side->join, side->s);
+        cudaStreamWaitEvent(s, side->join, 0);
+    };
     (k_s5d_detect<<<blocks_for(C.n, kBlock), kBlock, 0, s>>>(C, rcand), note_launch());
+    split();
+    if (chunked) {
+        (k_s5d_chunk_sums<<<C.A.nchunks, kTaskThreads, 0, sl>>>(C, rcand, cs_a), note_launch());
+        (k_s5d_chunk_elig<<<long_warps, kBlock, 0, sl>>>(C, rcand, cs_a, relig), note_launch());
+        (k_s5d_chunk_bid<<<C.A.nchunks, kTaskThreads, 0, sl>>>(C, rcand, relig, cmin), note_launch());
+    }
     (k_s5d_check<<<blocks_for(C.m, kBlock), kBlock, 0, s>>>(C, rcand, relig, cmin, tasks, ntask), note_launch());
     (k_s5d_check_long<<<task_grid, kTaskThreads, 0, s>>>(C, rcand, relig, cmin, tasks, ntask), note_launch());
+    join();  // every bid is in before a row is selected
+    split();
     if (chunked) {
-        (k_s5d_chunk_sums<<<C.A.nchunks, kTaskThreads, 0, s>>>(C, rcand, cs_a), note_launch());
-        (k_s5d_chunk_elig<<<long_warps, kBlock, 0, s>>>(C, rcand, cs_a, relig), note_launch());
-        (k_s5d_chunk_bid<<<C.A.nchunks, kTaskThreads, 0, s>>>(C, rcand, relig, cmin), note_launch());
+        (k_s5d_chunk_sel<<<C.A.nchunks, kTaskThreads, 0, sl>>>(C, rcand, relig, cmin), note_launch());
+        (k_s5d_chunk_row<<<long_warps, kBlock, 0, sl>>>(C, rcand, cs_a, relig), note_launch());
+        (k_s5d_chunk_apply<<<C.A.nchunks, kTaskThreads, 0, sl>>>(C, rcand, cs_a, relig), note_launch());
     }
     (k_s5d_apply<<<blocks_for(C.m, kBlock), kBlock, 0, s>>>(C, rcand, relig, cmin), note_launch());
     (k_s5d_apply_long<<<task_grid, kTaskThreads, 0, s>>>(C, rcand, relig, cmin, tasks, ntask), note_launch());
-    if (chunked) {
-        (k_s5d_chunk_sel<<<C.A.nchunks, kTaskThreads, 0, s>>>(C, rcand, relig, cmin), note_launch());
-        (k_s5d_chunk_row<<<long_warps, kBlock, 0, s>>>(C, rcand, cs_a, relig), note_launch());
-        (k_s5d_chunk_apply<<<C.A.nchunks, kTaskThreads, 0, s>>>(C, rcand, cs_a, relig), note_launch());
-    }
+    join();
 }
 
 }  // namespace lpp

@@ -942,10 +942,17 @@ void Engine::compact(int32_t round) {
     tend();
     // the objective constant of the columns that left: with the columns in
     // place each slot's contribution stays until one sum at the end
-    if (!in_place) launch_offset(C, K, s);
+    // (nothing else reads the contributions: beside the scatter)
+    if (!in_place) {
+        LPP_CUDA(cudaEventRecord(ev_fork, s));
+        LPP_CUDA(cudaStreamWaitEvent(s_long, ev_fork, 0));
+        launch_offset(C, K, s_long);
+        LPP_CUDA(cudaEventRecord(ev_join, s_long));
+    }
     tbegin(F_SCATTER, 24.0 * nnz * 2 + 48.0 * (m + n));
     launch_compact_scatter(C, K, (int32_t)nnz, s);
     tend();
+    if (!in_place) LPP_CUDA(cudaStreamWaitEvent(s, ev_join, 0));
     LPP_CUDA(cudaGetLastError());
     // the next buffers become current; sizes and schedules are read back at
     // the end of the round (one host sync per round)
@@ -1183,7 +1190,9 @@ void Engine::run_s5d(const Ctx &C) {
         fill_i32(cs_cmin, n, kNone, s);
         LPP_CUDA(cudaMemsetAsync(cs_relig, 0, (size_t)m, s));
         LPP_CUDA(cudaMemsetAsync(cs_ntask, 0, sizeof(int32_t), s));
-        launch_s5d(C, cs_rcand, cs_relig, cs_cmin, cs_tasks, cs_ntask, cs_a, s);
+        ensure_side_stream();
+        const SideStream side{s_long, ev_fork, ev_join};
+        launch_s5d(C, cs_rcand, cs_relig, cs_cmin, cs_tasks, cs_ntask, cs_a, s, &side);
         LPP_CUDA(cudaGetLastError());
     }
     tend();

@@ -151,8 +151,9 @@ void launch_s5c_groups(const Ctx &C, const uint32_t *slot, const int32_t *col, i
 // listed in tasks / *ntask, 0 before; longer rows by chunks, their candidate's
 // coefficient in cs_a per row), the first bidding row per column (cmin,
 // kNone before), then the substitutions
+struct SideStream;
 void launch_s5d(const Ctx &C, int32_t *rcand, uint8_t *relig, int32_t *cmin, int32_t *tasks, int32_t *ntask,
-                double *cs_a, cudaStream_t s);
+                double *cs_a, cudaStream_t s, const SideStream *side);
 
 // ------------------------------------------------------------- k_doubleton.cu
 // S5e work: per row the candidate's eliminated column (dk, -1 if none), the
