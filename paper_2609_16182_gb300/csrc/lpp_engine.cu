@@ -998,38 +998,57 @@ Engine::StepOut Engine::step(int32_t r, bool first_round, bool force) {
     launch_round_start(C, !first_round, s);
     tbegin(F_PROP, 0.0);  // bytes and ops set once the evaluated nonzeros are known
     const size_t prop_mark = marks.size();
-    // the long rows' chunk kernels on a second stream, beside the short
-    // rows' kernel, joined before S3'
-    const bool long_rows = prop_has_long(C);
-    if (long_rows) {
-        ensure_side_stream();
-        LPP_CUDA(cudaEventRecord(ev_fork, s));
-        LPP_CUDA(cudaStreamWaitEvent(s_long, ev_fork, 0));
-        launch_prop_long(C, s_long);
-        LPP_CUDA(cudaEventRecord(ev_join, s_long));
-    }
-    launch_prop_short(C, s);
-    if (long_rows) LPP_CUDA(cudaStreamWaitEvent(s, ev_join, 0));
-    tend();
-    tbegin(F_COLFIN, 33.0 * n);
-    if (o.dual_records) launch_bound_src(C, s);
-    launch_colfin(C, first_round, s);
-    if (!in_place) launch_mark_dirty(C, nnz, s);
-    tend();
-    LPP_CUDA(cudaGetLastError());
     // S5: leader passes.  Skipped when the last S5 resolved every key group
     // (no row left unmatched at the pass cap) and no row lost an entry since:
     // its survivors are pairwise not parallel, so it would remove nothing.
     const bool run_s5 = first_round || !s5_clean;
     int32_t tcap = std::min(tcap_max, pow2_at_least(2 * (int64_t)std::max(m, 1)));
-    tbegin(F_S5, run_s5 ? 16.0 * tcap + 12.0 * m : 0.0);
-    if (run_s5) {
-        launch_s5_init(C, tcap, s5_cnt, o.par_max_iter + 3, s);
-        C.tcap = tcap;
-        C.s5_out = s5_list[0];
-        C.s5_out_cnt = s5_cnt + 1;
-        launch_s5_pass(C, s);
+    // the second stream: the long rows' chunk kernels beside the short rows'
+    // kernel, joined before S3', and S5's first pass (rows: keys, coefficients,
+    // sides) beside S3', S4 and the marking (columns and flags; they share only
+    // counters and the changed flag), joined before the counters are read; its
+    // table is emptied meanwhile.  With S5 after S3' to the marking (as with
+    // `timing`, whose families are timed on one stream) 2 M rows take 1% longer
+    // (6.05 ms, now 5.98), 500 k rows with parallel_cols 2% (6.80, 6.65).
+    const bool long_rows = prop_has_long(C), s5_beside = run_s5 && !o.timing;
+    const bool side = long_rows || s5_beside;
+    if (side) {
+        ensure_side_stream();
+        LPP_CUDA(cudaEventRecord(ev_fork, s));
+        LPP_CUDA(cudaStreamWaitEvent(s_long, ev_fork, 0));
     }
+    if (long_rows) {
+        launch_prop_long(C, s_long);
+        LPP_CUDA(cudaEventRecord(ev_join, s_long));
+    }
+    if (s5_beside) launch_s5_init(C, tcap, s5_cnt, o.par_max_iter + 3, s_long);
+    launch_prop_short(C, s);
+    if (long_rows) LPP_CUDA(cudaStreamWaitEvent(s, ev_join, 0));
+    tend();
+    tbegin(F_COLFIN, 33.0 * n);
+    if (o.dual_records) launch_bound_src(C, s);
+    Ctx C5 = C;
+    C5.tcap = tcap;
+    C5.s5_out = s5_list[0];
+    C5.s5_out_cnt = s5_cnt + 1;
+    if (s5_beside) {
+        LPP_CUDA(cudaEventRecord(ev_fork, s));
+        LPP_CUDA(cudaStreamWaitEvent(s_long, ev_fork, 0));
+        launch_s5_pass(C5, s_long);
+        LPP_CUDA(cudaEventRecord(ev_join, s_long));
+    }
+    launch_colfin(C, first_round, s);
+    if (!in_place) launch_mark_dirty(C, nnz, s);
+    tend();
+    LPP_CUDA(cudaGetLastError());
+    tbegin(F_S5, run_s5 ? 16.0 * tcap + 12.0 * m : 0.0);
+    if (s5_beside) {
+        LPP_CUDA(cudaStreamWaitEvent(s, ev_join, 0));
+    } else if (run_s5) {
+        launch_s5_init(C5, tcap, s5_cnt, o.par_max_iter + 3, s);
+        launch_s5_pass(C5, s);
+    }
+    if (run_s5) C = C5;
     tend();
     LPP_CUDA(cudaGetLastError());
     read_status();
