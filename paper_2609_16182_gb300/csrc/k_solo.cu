@@ -8,8 +8,8 @@
 // decisions (which steps run, whether to compact, whether to stop) are taken
 // by every block alike from counters read after a barrier, as the host takes
 // them in Engine::step, so an LP gets the bits of the launched path.  A call on
-// 20 k rows (0.18 M entries, 13 rounds) takes 1.6 ms, 2.3 ms launched; on 200
-// rows (one block, its barriers block barriers) 0.83 ms, 1.16 ms launched.
+// 20 k rows (0.18 M entries, 13 rounds) takes 1.36 ms, 2.3 ms launched; on 200
+// rows 0.68 ms, 1.16 ms launched.
 //
 // The columns stay in place (Ctx::in_place); row vectors and matrix alternate
 // between two buffers as there.  Counters exist twice, by the round's parity:
