@@ -328,7 +328,7 @@ void Engine::setup(const lpp_opts &opts, int32_t nlp_, const std::vector<Member>
     st = reinterpret_cast<DevStatus *>(pool.alloc<unsigned char>(st_bytes));
     verdict = reinterpret_cast<int32_t *>(st + 1);
     lp_changed = reinterpret_cast<uint8_t *>(verdict + (size_t)nlp * V_SLOTS);
-    s5_left_h = static_cast<int32_t *>(pinned_get_sized(sizeof(int32_t)));
+    s5_left_h = static_cast<int32_t *>(pinned_get_sized(2 * sizeof(int32_t)));
     fetch_flag = static_cast<uint32_t *>(pinned_get_sized(sizeof(uint32_t)));
     *fetch_flag = fetch_seq = 0;
     const bool arena = nlp > 1;
@@ -1178,13 +1178,13 @@ void Engine::run_s5c(const Ctx &C0) {
     LPP_CUDA(cudaMemsetAsync(pc_cnt, 0, 4 * sizeof(int32_t), s));
     C.ctcap = std::min(ctcap_max, pow2_at_least(2 * (int64_t)std::max(n, 1)));
     launch_s5c_keys(C, s);
-    launch_s5c_members(C, pc_flags, pc_pos, pc_scan, pc_slot, pc_col, s);
+    launch_s5c_members(C, pc_flags, pc_pos, pc_scan, pc_slot, pc_col, pc_cnt + 2, s);
     LPP_CUDA(cudaGetLastError());
-    fetch({{s5_left_h, pc_pos + n, sizeof(int32_t)}});
+    fetch({{s5_left_h, pc_pos + n, sizeof(int32_t)}, {s5_left_h + 1, pc_cnt + 2, sizeof(int32_t)}});
     const int32_t F = n > 0 ? *s5_left_h : 0;
     if (F > 0) {
         int bits = 0;
-        while (((int64_t)1 << bits) < (int64_t)C.ctcap) bits++;
+        while (((int64_t)1 << bits) < (int64_t)s5_left_h[1]) bits++;  // the members' group numbers
         const uint32_t *ks = nullptr;
         const int32_t *vs = nullptr;
         sort_pairs(pc_slot, pc_col, F, bits, pc_sort, &ks, &vs, s);

@@ -132,17 +132,17 @@ void launch_s5_leader(const Ctx &C, cudaStream_t s);
 // column table (C.ctcap slots, empty before), which counts the columns per key
 void launch_s5c_keys(const Ctx &C, cudaStream_t s);
 // the columns of the groups that changed since their last S5c (a key or the
-// size) and have two or more columns, in column order: slot[p], col[p] for
-// p < pos[n] (flags, pos: n + 1 entries of scratch)
-void launch_s5c_members(const Ctx &C, int32_t *flags, int32_t *pos, int32_t *scan_tmp, uint32_t *slot, int32_t *col,
-                        cudaStream_t s);
+// size) and have two or more columns, in column order: group[p] (its number,
+// of *groups, zero before), col[p] for p < pos[n] (flags, pos: n + 1 entries of scratch)
+void launch_s5c_members(const Ctx &C, int32_t *flags, int32_t *pos, int32_t *scan_tmp, uint32_t *group, int32_t *col,
+                        int32_t *groups, cudaStream_t s);
 // bytes per grouped column of the launch_s5c_groups scratch `mem`
 size_t s5c_mem_bytes();
 // all leader passes of every group: F members sorted by slot (column order
 // within a slot), one warp per group of at most 256 columns, larger groups
 // listed in glist and run by thread blocks.  ctr[0]: groups left unresolved
 // at the pass cap, ctr[1]: large groups (both zero before).
-void launch_s5c_groups(const Ctx &C, const uint32_t *slot, const int32_t *col, int32_t F, void *mem, uint8_t *alive,
+void launch_s5c_groups(const Ctx &C, const uint32_t *group, const int32_t *col, int32_t F, void *mem, uint8_t *alive,
                        int2 *glist, int32_t *ctr, int32_t max_iter, cudaStream_t s);
 
 // --------------------------------------------------------------- k_colsing.cu
