@@ -1168,7 +1168,7 @@ Engine::StepOut Engine::step(int32_t r, bool first_round, bool force) {
 }
 
 // S5c: keys into the column table, the columns of the changed groups in
-// column order, sorted by slot, then every such group's passes on the
+// column order, sorted by group number, then every such group's passes on the
 // device.  Two host reads: the number of grouped columns (sizes the sort),
 // then the status.  Refreshes st_h, whose column count then includes the
 // merges.

@@ -138,7 +138,7 @@ void launch_s5c_members(const Ctx &C, int32_t *flags, int32_t *pos, int32_t *sca
                         int32_t *groups, cudaStream_t s);
 // bytes per grouped column of the launch_s5c_groups scratch `mem`
 size_t s5c_mem_bytes();
-// all leader passes of every group: F members sorted by slot (column order
+// all leader passes of every group: F members sorted by group number (column order
 // within a slot), one warp per group of at most 256 columns, larger groups
 // listed in glist and run by thread blocks.  ctr[0]: groups left unresolved
 // at the pass cap, ctr[1]: large groups (both zero before).
