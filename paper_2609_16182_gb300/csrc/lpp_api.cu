@@ -1150,8 +1150,8 @@ lpp_status lpp_postsolve_primal(const lpp_postsolve *Pc, const double *x_red, do
         const lpp_status st = guarded([&]() -> lpp_status {
             try {
                 return primal_on_device(P, x_red, x_orig);
-            } catch (const CudaError &e) {
-                if (e.code != cudaErrorMemoryAllocation) throw;
+            } catch (const StatusError &e) {  // what cuda_check makes of a refused allocation
+                if (e.st != LPP_ERR_OOM) throw;
                 cudaGetLastError();
                 room = false;  // the host form below needs none
                 return LPP_OK;

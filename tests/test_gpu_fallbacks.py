@@ -1,0 +1,65 @@
+"""Calls whose fast form the device cannot take: the other form has to answer.
+
+A device without room is a memory pool with a limit, made current for the
+calls under test; nothing is filled.
+"""
+import contextlib
+import ctypes as C
+
+import numpy as np
+import pytest
+
+from lpmake import INF
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+from paper_2609_16182_gb300 import lpp, synth  # noqa: E402
+
+
+class PoolProps(C.Structure):  # CUmemPoolProps
+    _fields_ = [("alloc_type", C.c_int), ("handle_types", C.c_int), ("loc_type", C.c_int), ("loc_id", C.c_int),
+                ("win32", C.c_void_p), ("max_size", C.c_size_t), ("usage", C.c_ushort), ("reserved", C.c_ubyte * 54)]
+
+
+@contextlib.contextmanager
+def pool_limit(max_bytes):
+    """Device 0's stream-ordered allocations come from a pool of max_bytes."""
+    cu = C.CDLL("libcuda.so.1")
+    old, pool = C.c_void_p(), C.c_void_p()
+    props = PoolProps(alloc_type=1, loc_type=1, loc_id=0, max_size=max_bytes)  # pinned, on device 0
+    assert cu.cuDeviceGetMemPool(C.byref(old), 0) == 0
+    assert cu.cuMemPoolCreate(C.byref(pool), C.byref(props)) == 0
+    try:
+        assert cu.cuDeviceSetMemPool(0, pool) == 0
+        yield
+    finally:
+        assert cu.cuDeviceSetMemPool(0, old) == 0
+        assert cu.cuMemPoolDestroy(pool) == 0
+
+
+def wide(n, m=64, seed=0):
+    """m rows of two entries each and n columns, most of them empty."""
+    r = np.random.default_rng(seed)
+    return synth.LP(m=m, n=n, row_ptr=np.arange(0, 2 * m + 1, 2, dtype=np.int32),
+                    col_idx=np.arange(2 * m, dtype=np.int32), val=r.choice([-1.0, 2.0], 2 * m),
+                    c=r.integers(-2, 3, n).astype(float), lhs=np.full(m, -INF), rhs=np.full(m, 3.0),
+                    lb=np.full(n, -5.0), ub=np.full(n, 5.0))
+
+
+def test_primal_postsolve_without_device_memory():
+    r = lpp.presolve(wide(9_000_001))  # two vectors: 72 MB or more
+    red = r.reduced()
+    assert red.n > 0
+    x = np.random.default_rng(1).standard_normal(red.n)
+    want = np.where(r.col_kind != 0, r.col_val, np.nan)
+    want[red.col_map] = x
+    # a second record, none of whose arrays is on the host yet
+    q = lpp.presolve(wide(9_000_001))
+    with pool_limit(1 << 22):
+        np.testing.assert_array_equal(q.postsolve_primal(x), want)
+    np.testing.assert_array_equal(q.postsolve_primal(x), want)
+    torch.cuda.synchronize()  # no error is left behind
