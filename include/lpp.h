@@ -31,7 +31,8 @@
  *       opts.dual_fixing every column no kept row locks in that direction
  *   S7  compaction of the CSR and CSC matrices and of all row/column vectors
  * The reduced LP has the same form (Sec. 3.3) and stays in device memory; the
- * postsolve record (Sec. 2.1, postsolver; Sec. 3.3) lives on the host.
+ * postsolve record (Sec. 2.1, postsolver; Sec. 3.3) keeps its arrays on the
+ * device until an accessor copies the ones it returns to the host.
  *
  * All floating point is IEEE binary64; all index work is exact int32/int64.
  *
@@ -161,7 +162,7 @@ typedef struct lpp_opts {
 } lpp_opts;
 
 typedef struct lpp_reduced lpp_reduced;     /* reduced LP, device resident */
-typedef struct lpp_postsolve lpp_postsolve; /* verdict, records, counters; host resident */
+typedef struct lpp_postsolve lpp_postsolve; /* verdict, records, counters (arrays on the device until asked for) */
 
 /* Summary of one presolve. */
 typedef struct lpp_info {
@@ -287,8 +288,11 @@ lpp_status lpp_result_kernels(const lpp_postsolve *rec, int32_t cap, lpp_kernel_
 lpp_status lpp_result_bound_sources(const lpp_postsolve *rec, int32_t *lsrc, int32_t *lrnd, int32_t *usrc,
                                     int32_t *urnd);
 
-/* Primal postsolve on the CPU (Sec. 2.1 postsolver; Sec. 3.3): x_red[n_red]
- * -> x_orig[n] (host arrays): kept columns take their reduced value, fixed
+/* Primal postsolve (Sec. 2.1 postsolver; Sec. 3.3): x_red[n_red]
+ * -> x_orig[n] (host arrays), on the CPU, or, where there are no merges and
+ * substitutions to undo, on the device for the first call on a record and for
+ * LPs of more than 65,536 columns (those on a stream that waits for no other;
+ * without device memory for the two vectors, on the CPU): kept columns take their reduced value, fixed
  * columns their recorded value.  Merges and substitutions are undone latest
  * first (round; in a round substitutions before merges; then index).  A
  * substitution sets x_j = (b - sum_k a_ik x_k) / a_ij.  A merge: with the

@@ -375,6 +375,11 @@ void materialize(lpp_postsolve *P, int want) {
 // column map): it runs where the records are, so that only the two solutions
 // cross the host link.  Copying the records to the host instead, twelve arrays
 // into fresh vectors, made a round trip on 200 k rows 6.0 ms instead of 3.4.
+// A record that is asked again: the columns' records are copied once and the
+// call is then a pass over host arrays, up to kPrimalHost columns, beyond which
+// the device is faster on every call.  Host / device, us: 300 columns 3 / 25,
+// 30 k 33 / 43, 300 k 339 / 234, 3 M 3450 / 1970.
+constexpr int32_t kPrimalHost = 1 << 16;
 __global__ void __launch_bounds__(256) k_post_values(const int32_t *kind, const double *val, int32_t n, double *x) {
     const int32_t j = blockIdx.x * 256 + threadIdx.x;
     if (j < n) x[j] = kind[j] != LPP_COL_KEPT ? val[j] : __longlong_as_double(0x7ff8000000000000LL);
@@ -410,17 +415,32 @@ lpp_status primal_on_device(const lpp_postsolve *P, const double *x_red, double 
         explicit Stage(size_t cnt) : p(static_cast<double *>(pinned_get_sized(8 * cnt))) {}
         ~Stage() { pinned_put(p); }
     } h((size_t)n + r + 1);
-    DevPool pool;  // on the legacy default stream, as the copies of the records are
+    // where every call comes here, on a stream of its own, which waits for no
+    // other work of the caller's (the records were complete when lpp_presolve
+    // returned); a first call of a small LP takes the legacy default stream, as
+    // the copies of the records do (10 us less of 50)
+    struct Stream {
+        cudaStream_t s = nullptr;
+        explicit Stream(bool own) {
+            if (own) LPP_CUDA(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
+        }
+        ~Stream() {
+            if (s) cudaStreamDestroy(s);
+        }
+    } own(n > kPrimalHost);
+    const cudaStream_t s = own.s;
+    DevPool pool;
+    pool.s = s;
     double *dx = pool.alloc<double>((size_t)n + r + 1), *dr = dx + n + 1;  // x, an error flag, the reduced x
     int32_t *bad = reinterpret_cast<int32_t *>(dx + n);
     h.p[n] = 0.0;
     if (r) std::memcpy(h.p + n + 1, x_red, 8 * (size_t)r);
-    LPP_CUDA(cudaMemcpyAsync(dx + n, h.p + n, 8 * ((size_t)r + 1), cudaMemcpyHostToDevice, 0));
-    (k_post_values<<<nblk(n), 256>>>(D.ck + P->c0, D.cv + P->c0, n, dx), note_launch());
-    if (r) (k_post_kept<<<nblk(r), 256>>>(D.cmap + P->cstart, dr, r, P->c0, n, dx, bad), note_launch());
+    LPP_CUDA(cudaMemcpyAsync(dx + n, h.p + n, 8 * ((size_t)r + 1), cudaMemcpyHostToDevice, s));
+    (k_post_values<<<nblk(n), 256, 0, s>>>(D.ck + P->c0, D.cv + P->c0, n, dx), note_launch());
+    if (r) (k_post_kept<<<nblk(r), 256, 0, s>>>(D.cmap + P->cstart, dr, r, P->c0, n, dx, bad), note_launch());
     LPP_CUDA(cudaGetLastError());
-    LPP_CUDA(cudaMemcpyAsync(h.p, dx, 8 * ((size_t)n + 1), cudaMemcpyDeviceToHost, 0));
-    LPP_CUDA(cudaStreamSynchronize(0));
+    LPP_CUDA(cudaMemcpyAsync(h.p, dx, 8 * ((size_t)n + 1), cudaMemcpyDeviceToHost, s));
+    LPP_CUDA(cudaStreamSynchronize(s));
     int32_t flag;
     std::memcpy(&flag, h.p + n, sizeof flag);
     if (flag) return set_err(LPP_ERR_INVALID, "corrupt column map");
@@ -1146,18 +1166,31 @@ lpp_status lpp_postsolve_primal(const lpp_postsolve *Pc, const double *x_red, do
     lpp_postsolve *P = const_cast<lpp_postsolve *>(Pc);
     if (!P->dev->ca && !P->dev->sb) {
         if (!x_red && P->info.n_red > 0) return set_err(LPP_ERR_INVALID, "NULL argument");
-        bool room = true;
-        const lpp_status st = guarded([&]() -> lpp_status {
-            try {
-                return primal_on_device(P, x_red, x_orig);
-            } catch (const StatusError &e) {  // what cuda_check makes of a refused allocation
-                if (e.st != LPP_ERR_OOM) throw;
-                cudaGetLastError();
-                room = false;  // the host form below needs none
-                return LPP_OK;
-            }
-        });
-        if (room) return st;
+        if (P->info.n > kPrimalHost || (!(P->host_have & REC_COLS) && !P->primal_asked)) {
+            P->primal_asked = true;
+            bool room = true;
+            const lpp_status st = guarded([&]() -> lpp_status {
+                try {
+                    return primal_on_device(P, x_red, x_orig);
+                } catch (const StatusError &e) {  // what cuda_check makes of a refused allocation
+                    if (e.st != LPP_ERR_OOM) throw;
+                    cudaGetLastError();
+                    room = false;  // the host form below needs none
+                    return LPP_OK;
+                }
+            });
+            if (room) return st;
+        }
+        const lpp_status st = guarded([&]() -> lpp_status { materialize(P, REC_COLS); return LPP_OK; });
+        if (st != LPP_OK) return st;
+        PostsolveRecords R = {};  // no rows: no step to undo
+        R.n = (int64_t)P->col_kind.size();
+        R.n_red = (int64_t)P->col_map.size();
+        R.col_kind = P->col_kind.data();
+        R.col_map = P->col_map.data();
+        R.col_val = P->col_val.data();
+        const char *err = postsolve_primal(R, x_red, x_orig);
+        return err ? set_err(LPP_ERR_INVALID, err) : LPP_OK;
     }
     const lpp_status st = guarded([&]() -> lpp_status { materialize(P, REC_ROWS | REC_COLS | REC_MERGES | REC_SUBST); return LPP_OK; });
     if (st != LPP_OK) return st;

@@ -348,6 +348,7 @@ struct lpp_postsolve {
     int32_t cstart = 0;              // first kept column of this LP in the final arena
     int32_t astart = 0, acnt = 0;    // this LP's rows in the last round's numbering
     int host_have = 0;               // record groups copied to the host (REC_* in lpp_api.cu)
+    bool primal_asked = false;       // lpp_postsolve_primal has run on the device
     std::vector<int32_t> row_kind, row_round, row_aux, col_kind, col_round, col_map, col_aux, col_pass;
     std::vector<double> row_val, col_val, col_lb, col_ub, act_min, act_max, col_mrg;
     std::vector<int64_t> sub_beg;                 // substitutions: per row, into sub_col / sub_val

@@ -63,3 +63,46 @@ def test_primal_postsolve_without_device_memory():
         np.testing.assert_array_equal(q.postsolve_primal(x), want)
     np.testing.assert_array_equal(q.postsolve_primal(x), want)
     torch.cuda.synchronize()  # no error is left behind
+
+
+def launches():
+    f = lpp.load()._ZN3lpp12launch_countEv  # kernels the library has launched
+    f.restype = C.c_int64
+    return f()
+
+
+# up to 65,536 columns
+@pytest.mark.parametrize("n", [300, 65_536])
+@pytest.mark.parametrize("first", ["postsolve", "records"])
+def test_a_repeated_primal_postsolve_is_host_work(n, first):
+    r = lpp.presolve(wide(n))
+    red = r.reduced()
+    r.info
+    x, y = np.random.default_rng(2).standard_normal((2, red.n))
+    if first == "records":
+        r.col_kind
+    a = r.postsolve_primal(x)
+    k = launches()
+    b = r.postsolve_primal(y)
+    np.testing.assert_array_equal(r.postsolve_primal(x), a)
+    assert launches() == k
+    for got, sol in ((a, x), (b, y)):
+        want = np.where(r.col_kind != 0, r.col_val, np.nan)
+        want[red.col_map] = sol
+        np.testing.assert_array_equal(got, want)
+
+
+def test_primal_postsolve_waits_for_no_other_stream():
+    lp = wide(65_537)
+    warm = lpp.presolve(lp)
+    x = np.random.default_rng(3).standard_normal(warm.info.n_red)
+    want = warm.postsolve_primal(x)
+    for r in (lpp.presolve(lp), warm):
+        r.info
+        torch.cuda._sleep(1_000_000_000)  # about half a second on the default stream
+        busy = torch.cuda.Event()
+        busy.record()
+        got = r.postsolve_primal(x)
+        assert not busy.query()
+        torch.cuda.synchronize()
+        np.testing.assert_array_equal(got, want)
