@@ -216,8 +216,7 @@ lpp_postsolve *make_postsolve(Engine &E, const std::shared_ptr<DeviceRecords> &D
             std::snprintf(ks[f].name, sizeof ks[f].name, "%s", fam_name(f));
         }
         for (auto &mk : E.marks) {
-            float ms = 0.f;
-            LPP_CUDA(cudaEventElapsedTime(&ms, mk.a, mk.b));
+            const float ms = elapsed_ms(mk.a, mk.b);
             ks[mk.fam].launches++;
             ks[mk.fam].ms += ms;
             ks[mk.fam].bytes += mk.bytes;
@@ -665,8 +664,7 @@ bool batch_fused(Engine &E, const std::vector<Member> &mem, int32_t count, lpp_r
     LPP_CUDA(cudaStreamSynchronize(s));
     for (auto &x : sts)
         if (x.err) throw StatusError(LPP_ERR_CUDA, "internal: S5 hash table overflow (batch)");
-    float ms = 0.f;
-    LPP_CUDA(cudaEventElapsedTime(&ms, e0, e1));
+    const float ms = elapsed_ms(e0, e1);
     g_tuner.record(key, cand, ms);
     E.loop_ms = ms;
     // per-LP verdicts and counters for the records

@@ -19,6 +19,13 @@ void cuda_check(cudaError_t e, const char *expr, const char *file, int line) {
     throw CudaError(e, buf);
 }
 
+float elapsed_ms(cudaEvent_t a, cudaEvent_t b) {
+    float ms = 0.f;
+    LPP_CUDA(cudaEventSynchronize(b));
+    LPP_CUDA(cudaEventElapsedTime(&ms, a, b));
+    return ms;
+}
+
 void DevPool::forget(void *p) {
     auto it = std::find(ptrs.begin(), ptrs.end(), p);
     if (it != ptrs.end()) {
@@ -1158,7 +1165,7 @@ Engine::StepOut Engine::step(int32_t r, bool first_round, bool force) {
         nnz = nnz_new;
         adopt_schedule(!in_place);
     }
-    LPP_CUDA(cudaEventElapsedTime(&out.ms, ev_round[0], ev_round[1]));
+    out.ms = elapsed_ms(ev_round[0], ev_round[1]);
     r_ms.push_back(out.ms);
     r_rows.push_back(rows_removed);
     r_cols.push_back(st_h->cols_fixed);
@@ -1457,11 +1464,8 @@ void Engine::run() {
         if (st_h->n_new < 0 || st_h->n_new > n) throw StatusError(LPP_ERR_CUDA, "internal: column compaction size");
         n = st_h->n_new;
     }
-    float lms = 0.f;
     LPP_CUDA(cudaEventRecord(eend, s));
-    LPP_CUDA(cudaEventSynchronize(eend));
-    LPP_CUDA(cudaEventElapsedTime(&lms, eloop, eend));
-    loop_ms = lms;
+    loop_ms = elapsed_ms(eloop, eend);
 }
 
 // The dependent-row step (Sec. 5, the hybrid design): the current CSR and

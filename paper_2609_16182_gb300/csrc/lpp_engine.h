@@ -31,6 +31,10 @@ struct StatusError : std::runtime_error {
 
 void cuda_check(cudaError_t e, const char *expr, const char *file, int line);
 #define LPP_CUDA(x) ::lpp::cuda_check((x), #x, __FILE__, __LINE__)
+// milliseconds between two recorded events, after a wait for the second (a
+// value that a later kernel stored in host memory, as Engine::fetch reads, does
+// not yet say that the runtime sees an earlier event as complete)
+float elapsed_ms(cudaEvent_t a, cudaEvent_t b);
 
 // A process-wide cache of device blocks that finished presolves released,
 // by device and exact size: a presolve makes some seventy allocations, and
