@@ -391,19 +391,11 @@ void launch_s5_tail_block(const Ctx &C, int32_t *l0, int32_t *l1, int32_t *cnt, 
 // device cannot take a cooperative launch (the caller then launches passes)
 bool launch_s5_tail_grid(const Ctx &C, int32_t *l0, int32_t *l1, int32_t *cnt, int32_t p0, int32_t max_iter,
                          int32_t rows, unsigned *bar, cudaStream_t s) {
-    static int per_sm = -1, sms = 0;
-    if (per_sm < 0) {
-        int dev = 0, coop = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        int nb = 0;
-        if (coop) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_s5_tail_grid, kBlock, 0);
-        per_sm = coop ? nb : 0;
-    }
-    if (per_sm <= 0 || sms <= 0) return false;
+    static CoopCache cache;
+    const int most = coop_blocks((const void *)k_s5_tail_grid, cache);
+    if (most <= 0) return false;
     const int64_t want = std::max<int64_t>(1, ((int64_t)rows + kBlock - 1) / kBlock);
-    const unsigned grid = (unsigned)std::min<int64_t>(want, (int64_t)per_sm * sms);
+    const unsigned grid = (unsigned)std::min<int64_t>(want, most);
     Ctx Cv = C;
     void *args[] = {&Cv, &l0, &l1, &cnt, &p0, &max_iter, &bar};
     if (cudaLaunchCooperativeKernel((const void *)k_s5_tail_grid, dim3(grid), dim3(kBlock), args, 0, s) != cudaSuccess)

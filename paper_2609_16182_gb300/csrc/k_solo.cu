@@ -799,27 +799,14 @@ __global__ void __launch_bounds__(kBlock) k_solo_finish(const __grid_constant__ 
 
 }  // namespace
 
-namespace {
-
-// blocks of `kernel` that the device holds at once, 0 if it takes no cooperative launch
-int coop_blocks(const void *kernel) {
-    int dev = 0, coop = 0, nb = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (coop) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, kBlock, 0);
-    return coop && nb > 0 && sms > 0 ? nb * sms : 0;
-}
-
-}  // namespace
-
 // blocks of a cooperative launch of k_solo for an LP of these sizes, 0 if the
-// device cannot take one: a block per 512 entries, which spreads the longer rows
+// current device cannot take it or that of k_solo_finish: a block per 512 entries, which spreads the longer rows
 // (a block or a warp each) over the SMs.  With 2048, 1024, 512 and 256 entries per
 // block a presolve takes, in us: 500 skewed rows 1401, 1036, 857, 801; 5,000 rows
 // 1047, 905, 850, 858; 20,000 rows 1299, 1162, 1163, 1165; 100,000 rows the same.
 int solo_blocks(int32_t m, int32_t n, int64_t nnz) {
-    static const int most = coop_blocks((const void *)k_solo);
+    static CoopCache cache;
+    const int most = solo_finish_blocks(n, nnz) > 0 ? coop_blocks((const void *)k_solo, cache) : 0;
     const int64_t want = std::max<int64_t>({1, ((int64_t)m + kBlock - 1) / kBlock, ((int64_t)n + 2 * kBlock - 1) / (2 * kBlock),
                                             (nnz + 2 * kBlock - 1) / (2 * kBlock)});
     return (int)std::min<int64_t>(want, most);
@@ -827,7 +814,9 @@ int solo_blocks(int32_t m, int32_t n, int64_t nnz) {
 // of k_solo_finish: a tile of entries or two of columns each, one per SM at
 // most (more read more tables of counts)
 int solo_finish_blocks(int32_t n, int64_t nnz) {
-    static const int most = std::min(coop_blocks((const void *)k_solo_finish), 152);
+    static CoopCache cache;
+    int sms = 0;
+    const int most = std::min(coop_blocks((const void *)k_solo_finish, cache, &sms), sms);
     const int64_t want = std::max<int64_t>({1, (nnz + kFinTile - 1) / kFinTile, ((int64_t)n + 2 * kBlock - 1) / (2 * kBlock)});
     return (int)std::min<int64_t>(want, most);
 }

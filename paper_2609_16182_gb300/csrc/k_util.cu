@@ -13,6 +13,28 @@ std::atomic<int64_t> g_launches{0};
 void note_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
 int64_t launch_count() { return g_launches.load(std::memory_order_relaxed); }
 
+int coop_blocks(const void *kernel, CoopCache &cache, int *sms_out) {
+    int dev = 0, nb = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return 0;
+    const bool kept = dev < CoopCache::kDevices;
+    if (kept && (nb = cache.blocks[dev].load(std::memory_order_acquire)) > 0) {
+        if (sms_out) *sms_out = cache.sms[dev].load(std::memory_order_relaxed);
+        return nb - 1;
+    }
+    int coop = 0;
+    nb = 0;
+    cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (coop) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, kBlock, 0);
+    const int blocks = coop && nb > 0 && sms > 0 ? nb * sms : 0;
+    if (kept) {
+        cache.sms[dev].store(sms, std::memory_order_relaxed);
+        cache.blocks[dev].store(blocks + 1, std::memory_order_release);
+    }
+    if (sms_out) *sms_out = sms;
+    return blocks;
+}
+
 namespace {
 
 constexpr int kScanThreads = 256;

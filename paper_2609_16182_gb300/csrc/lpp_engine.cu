@@ -730,10 +730,15 @@ void Engine::prepare() {
         for (int32_t k = 0; k < nlp; k++) offs[k] = mem[k].obj_offset;
         LPP_CUDA(cudaMemcpyAsync(K.offset, offs.data(), sizeof(double) * nlp, cudaMemcpyHostToDevice, s));
     }
-    // sizes for the schedules: k_init_work (none if a check failed, so that
-    // they read no unchecked pointer)
+    first_schedules();  // also keeps offs alive until its copy is done
+}
+
+// The input's schedules for the launched rounds, and the checks' verdict.
+// Sizes: k_init_work (none if a check failed, so that they read no unchecked pointer).
+void Engine::first_schedules() {
+    const bool want_t = !in_place || need_t;
     schedule_current(want_t);
-    read_status();  // also keeps offs alive until its copy is done
+    read_status();
     check_status();
     adopt_schedule(want_t);
 }
@@ -1316,7 +1321,10 @@ void Engine::run_rounds() {
 }
 
 // The rounds in one cooperative kernel: one launch, one read of its results.
-void Engine::run_solo() {
+// False, with nothing done, if the launch was refused (the caller's stream may
+// own fewer SMs than the device): the rounds are then launched.  The kernel of
+// the end fits where the first does: no more blocks, and more of them per SM.
+bool Engine::run_solo() {
     const int32_t R = o.max_rounds;
     const int blocks = solo_blocks(m0, n0, nnz0);
     const size_t ctl_bytes = sizeof(SoloCtl) + 6 * sizeof(int32_t) * (size_t)R;
@@ -1388,7 +1396,11 @@ void Engine::run_solo() {
     G.offset = K.offset;
     G.btot = pool.alloc<int32_t>((size_t)fblocks);
     G.hist = pool.alloc<int32_t>((size_t)fblocks * 256);
-    if (!launch_solo(F, blocks, s) || !launch_solo_finish(G, fblocks, s)) {
+    if (!launch_solo(F, blocks, s)) {
+        cudaGetLastError();
+        return false;
+    }
+    if (!launch_solo_finish(G, fblocks, s)) {
         cudaGetLastError();
         throw StatusError(LPP_ERR_CUDA, "internal: cooperative launch refused");
     }
@@ -1400,8 +1412,7 @@ void Engine::run_solo() {
     if (c.err & 4) throw StatusError(LPP_ERR_CUDA, "internal: round barrier timed out");
     if (c.err) throw StatusError(LPP_ERR_CUDA, "internal: S5 hash table overflow");
     const SoloOut &u = c.out;
-    if (u.rounds < 1 || u.rounds > R || u.m < 0 || u.m > m0 || u.nnz < 0 || u.nnz > nnz0 || u.n < 0 ||
-        u.n > n0)
+    if (u.rounds < 1 || u.rounds > R || u.m < 0 || u.m > m0 || u.nnz < 0 || u.nnz > nnz0 || u.n < 0 || u.n > n0)
         throw StatusError(LPP_ERR_CUDA, "internal: sizes of the rounds' kernel");
     for (int32_t r = 0; r < u.rounds; r++, q += 6) {
         r_nnz.push_back(q[0]);
@@ -1434,6 +1445,7 @@ void Engine::run_solo() {
     T.ptr = tp[cur];
     T.idx = ti[cur];
     T.val = tv[cur];
+    return true;
 }
 
 void Engine::run() {
@@ -1453,8 +1465,11 @@ void Engine::run() {
     spare_events.push_back(eloop);
     spare_events.push_back(eend);
     LPP_CUDA(cudaEventRecord(eloop, s));
-    if (solo) run_solo();
-    else run_rounds();
+    if (!solo || !run_solo()) {
+        if (solo) first_schedules();
+        solo = false;
+        run_rounds();
+    }
     if (o.dep_rows && nlp == 1 && lp_status[0] == LPP_OK) remove_dependent();
     if (in_place && !solo) {
         launch_offset(ctx(rounds), K, s);  // every slot's contribution, once, in column order

@@ -235,7 +235,8 @@ struct Engine {
     void prepare();  // after ingest: transpose, schedules, work init
     void run();      // the round loop
     bool solo = false;  // all rounds in one kernel (one LP of at most kSoloNnz entries, columns in place)
-    void run_solo();
+    bool run_solo();
+    void first_schedules();
     void run_rounds();
     struct StepOut {
         bool structural = false;

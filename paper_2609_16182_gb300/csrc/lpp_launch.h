@@ -2,6 +2,8 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <atomic>
+
 #include "lpp_dev.cuh"
 
 namespace lpp {
@@ -9,6 +11,15 @@ namespace lpp {
 // number of kernels the library has launched in this process (all threads)
 void note_launch();
 int64_t launch_count();
+// Blocks of kBlock threads of `kernel` that the current device holds at once, 0 if
+// it takes no cooperative launch; sms: its SMs.  Asked once per device and
+// kernel (cache).  A stream may own fewer SMs than the device, so such a launch
+// can be refused all the same, and its caller has another form.
+struct CoopCache {
+    static constexpr int kDevices = 64;
+    std::atomic<int> blocks[kDevices] = {}, sms[kDevices] = {};  // blocks + 1, 0: not asked
+};
+int coop_blocks(const void *kernel, CoopCache &cache, int *sms = nullptr);
 
 // ----------------------------------------------------------------- k_util.cu
 // Exclusive scan of in[0..cnt) into out[0..cnt], out[cnt] = total.  `tmp`
@@ -226,6 +237,7 @@ struct SoloArgs {
     int32_t m, n, nnz, tcap_max, max_rounds, par_max_iter;
 };
 int solo_blocks(int32_t m, int32_t n, int64_t nnz);
+// false: the launch was refused, nothing has run
 bool launch_solo(const SoloArgs &F, int blocks, cudaStream_t s);
 // The end of such a run: objective constant, the columns' one compaction and
 // the reduced LP's A^T.  Reads the sizes launch_solo left in ctl.

@@ -106,3 +106,45 @@ def test_primal_postsolve_waits_for_no_other_stream():
         assert not busy.query()
         torch.cuda.synchronize()
         np.testing.assert_array_equal(got, want)
+
+
+class SmResource(C.Structure):  # CUdevResource of streaming multiprocessors
+    _fields_ = [("type", C.c_int), ("pad", C.c_ubyte * 92), ("sms", C.c_uint), ("rest", C.c_ubyte * 44)]
+
+
+@contextlib.contextmanager
+def small_stream(sms):
+    """A stream that owns a part of the device of at least `sms` SMs (a green context's)."""
+    cu = C.CDLL("libcuda.so.1")
+    torch.cuda.current_stream()  # the device's primary context is there
+    every, part, count = SmResource(), SmResource(), C.c_uint(1)
+    desc, ctx, stream = C.c_void_p(), C.c_void_p(), C.c_void_p()
+    assert cu.cuDeviceGetDevResource(0, C.byref(every), 1) == 0
+    assert cu.cuDevSmResourceSplitByCount(C.byref(part), C.byref(count), C.byref(every), None, 0, sms) == 0
+    assert cu.cuDevResourceGenerateDesc(C.byref(desc), C.byref(part), 1) == 0
+    assert cu.cuGreenCtxCreate(C.byref(ctx), desc, 0, 1) == 0
+    try:
+        assert cu.cuGreenCtxStreamCreate(C.byref(stream), ctx, 1, 0) == 0  # non-blocking
+        yield stream.value, part.sms, every.sms
+        assert cu.cuStreamSynchronize(stream) == 0
+        assert cu.cuStreamDestroy(stream) == 0
+    finally:
+        assert cu.cuGreenCtxDestroy(ctx) == 0
+
+
+@pytest.mark.parametrize("m", [300, 30_000])
+def test_presolve_on_a_stream_with_few_sms(m):
+    """Its cooperative kernels hold two blocks per SM: the larger LP's are refused there."""
+    lp = synth.skewed(5, m=m, n=3 * m // 2, target_nnz=10 * m, row_cap=9000)
+    want = lpp.presolve(lp)
+    with small_stream(8) as (stream, sms, every):
+        assert sms <= every // 2
+        got = lpp.presolve(lp, stream=stream)
+        a, b = got.reduced(), want.reduced()
+        x = np.random.default_rng(4).standard_normal(b.n)
+        np.testing.assert_array_equal(got.postsolve_primal(x), want.postsolve_primal(x))
+        got.close()
+    assert want.rounds == got.rounds
+    for k in ("row_ptr", "col_idx", "val", "c", "lhs", "rhs", "lb", "ub", "obj_offset", "row_map", "col_map", "csc_ptr",
+              "csc_idx", "csc_val"):
+        np.testing.assert_array_equal(getattr(a, k), getattr(b, k))
