@@ -65,10 +65,11 @@ __device__ __forceinline__ bool gt0(double s) { return dbits(s) > 0; }
 // terms.  It replaces, for nearly every entry, a queue trip with two FP64
 // instructions and two gathers by a few single-precision ones.
 // High words (sign bit cleared) to single precision: above / below |x|, by
-// at least 2^-21 |x|; then the same for signed values.
+// at least 2^-21 |x|; then the same for signed values.  Above is infinity from
+// 2^128 (1 - 2^-20) on, where the sum below would run past infinity's bits.
 __device__ __forceinline__ float f32_above(uint32_t hi) {
     if (hi < (897u << 20)) return __uint_as_float(0x01000000u);  // |x| < 2^-126: 2^-125
-    if (hi >= (1151u << 20)) return __uint_as_float(0x7f800000u);
+    if (hi >= (1151u << 20) - 2u) return __uint_as_float(0x7f800000u);
     return __uint_as_float((hi << 3) - 0xc0000000u + 16u);
 }
 __device__ __forceinline__ float f32_below(uint32_t hi) {
@@ -150,7 +151,7 @@ __device__ __forceinline__ float entry_span(double a, double2 b) {
 }
 // below the slack hi - lo of a row side
 __device__ __forceinline__ float slack_below(double hi, double lo) { return __fsub_rd(f32_lo(hi), f32_hi(lo)); }
-// may the exact test pass (a NaN span or slack passes)
+// may the exact test pass (a NaN slack or span, 0 times infinity, passes)
 __device__ __forceinline__ bool span_passes(float slack, float span) { return !(slack >= span); }
 
 // one entry that passed the filter: the exact test of one of its sides.
