@@ -877,6 +877,7 @@ lpp_status lpp_presolve_batch(const lpp_lp *ins, int32_t count, const lpp_opts *
         auto E = std::make_unique<Engine>();
         E->lazy_req = true;  // no A^T during the rounds when no step reads it
         E->need_t = fused_options(o);  // the persistent kernel starts from it
+        E->many = true;
         E->setup(o, count, mem);
         E->ingest_batch(ins, count);
         E->prepare();

@@ -338,7 +338,7 @@ void Engine::setup(const lpp_opts &opts, int32_t nlp_, const std::vector<Member>
     s5_left_h = static_cast<int32_t *>(pinned_get_sized(2 * sizeof(int32_t)));
     fetch_flag = static_cast<uint32_t *>(pinned_get_sized(sizeof(uint32_t)));
     *fetch_flag = fetch_seq = 0;
-    const bool arena = nlp > 1;
+    const bool arena = nlp > 1 || many;
     for (int b = 0; b < 2; b++) {
         rp[b] = pool.alloc<int32_t>(m0 + 1);
         ci[b] = pool.alloc<int32_t>(nnz0);
@@ -382,7 +382,7 @@ void Engine::setup(const lpp_opts &opts, int32_t nlp_, const std::vector<Member>
     cchg = pool.alloc<uint8_t>(n0);
     in_place = lazy_req && !o.parallel_cols && !o.col_singletons && !o.dual_fixing && !o.doubletons;
     if (in_place) cinv = pool.alloc<int32_t>(n0);
-    solo = in_place && nlp == 1 && nnz0 <= kSoloNnz && !o.timing && !o.dep_rows && o.max_rounds > 0 &&
+    solo = in_place && !arena && nnz0 <= kSoloNnz && !o.timing && !o.dep_rows && o.max_rounds > 0 &&
            o.max_rounds <= 1024 && solo_blocks(m0, n0, nnz0) > 0;
     rkind = pool.alloc<uint8_t>(m0);
     rwork = pool.alloc<uint8_t>(m0);

@@ -87,6 +87,7 @@ struct Engine {
     bool own_stream = false;
     DevPool pool;
     int32_t nlp = 1;
+    bool many = false;  // an arena also of one LP: the LP of every row and column is kept (set before setup)
     std::vector<Member> mem;
     int32_t m0 = 0, n0 = 0;
     int64_t nnz0 = 0;
