@@ -517,9 +517,27 @@ void Engine::setup(const lpp_opts &opts, int32_t nlp_, const std::vector<Member>
     LPP_CUDA(cudaMemsetAsync(st, 0, sizeof(DevStatus), s));
 }
 
+// Can kernels on `device` load this input where it lies: every array in the
+// device's memory or managed (a peer's needs peer access) and on a boundary of
+// its elements.  Copies take any.
+static bool readable_in_place(const lpp_lp &in, int device) {
+    const auto ok = [&](const void *p, int64_t cnt, uintptr_t align) {
+        if (cnt == 0) return true;
+        cudaPointerAttributes a;
+        if (reinterpret_cast<uintptr_t>(p) % align) return false;
+        if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        return (a.type == cudaMemoryTypeDevice && a.device == device) || a.type == cudaMemoryTypeManaged;
+    };
+    return ok(in.row_ptr, (int64_t)in.m + 1, 4) && ok(in.col_idx, in.nnz, 4) && ok(in.val, in.nnz, 8) &&
+           ok(in.lhs, in.m, 8) && ok(in.rhs, in.m, 8) && ok(in.lb, in.n, 8) && ok(in.ub, in.n, 8) && ok(in.c, in.n, 8);
+}
+
 void Engine::ingest_plain(const lpp_lp &in) {
     set_matrix();
-    if (in.on_device && in_place && o.max_rounds > 0) {
+    if (in.on_device && in_place && o.max_rounds > 0 && readable_in_place(in, o.device)) {
         // read where they lie: the first round always compacts, into the
         // library's buffers
         m_rp = in.row_ptr;

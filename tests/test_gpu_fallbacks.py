@@ -148,3 +148,30 @@ def test_presolve_on_a_stream_with_few_sms(m):
     for k in ("row_ptr", "col_idx", "val", "c", "lhs", "rhs", "lb", "ub", "obj_offset", "row_map", "col_map", "csc_ptr",
               "csc_idx", "csc_val"):
         np.testing.assert_array_equal(getattr(a, k), getattr(b, k))
+
+
+def at(offset, a):
+    """The array on the device, `offset` bytes past a 256-byte boundary; keeps its memory."""
+    raw = torch.zeros(offset + a.nbytes + 8, dtype=torch.uint8, device="cuda")
+    raw[offset:offset + a.nbytes] = torch.from_numpy(a.view(np.uint8)).cuda()
+    return raw, raw.data_ptr() + offset
+
+
+@pytest.mark.parametrize("timing", [0, 1])
+@pytest.mark.parametrize("shift", [0, 4, 8, 12, 1, 6])
+def test_device_inputs_off_the_boundaries(shift, timing):
+    """Device arrays that start off a boundary of their elements are copied, as host arrays are."""
+    lp = synth.skewed(6, m=3000, n=4500, target_nnz=30000, row_cap=2000)
+    keep, s = [], lpp.LpStruct(lp.m, lp.n, lp.val.size, on_device=1)
+    for k, v in lp.arrays().items():
+        raw, p = at(shift, np.ascontiguousarray(v, np.int32 if k in ("row_ptr", "col_idx") else np.float64))
+        keep.append(raw)
+        setattr(s, k, p)
+    torch.cuda.synchronize()
+    red, rec = C.c_void_p(), C.c_void_p()
+    o = lpp.opts(timing=timing)
+    assert lpp.load().lpp_presolve(C.byref(s), C.byref(o), C.byref(red), C.byref(rec)) == 0
+    a, b = lpp.Result(red.value, rec.value).reduced(), lpp.presolve(lp, timing=timing).reduced()
+    for k in ("row_ptr", "col_idx", "val", "c", "lhs", "rhs", "lb", "ub", "row_map", "col_map", "csc_ptr", "csc_idx",
+              "csc_val"):
+        np.testing.assert_array_equal(getattr(a, k), getattr(b, k))
