@@ -391,7 +391,7 @@ void lpp_server_destroy(lpp_server *srv);
  * loads the library, held until the process exits) limits nnz to
  * 268,435,456; larger inputs return LPP_ERR_INVALID with a message.  The
  * first call on a device looks up that array's device address and loads the
- * entry point's three kernels (set-up), so make it before any stream
+ * entry point's two kernels (set-up), so make it before any stream
  * capture.  Every call shares the array: calls that overlap on the GPU
  * (other streams, other threads) race; serialise them.  Runs asynchronously
  * on `stream` (NULL = legacy default stream) and calls no allocation

@@ -10,13 +10,15 @@
 // scratch array compiled into the library.
 //
 // A warp takes 32 consecutive rows, with as many lanes per row as its length
-// asks for; rows of more than 512 entries are left to the whole block, and
-// rows of more than 4096 are split by fixed 4096-entry windows of the entry
-// array.  A window meets at most two such long rows (one that started before
-// it, one that starts inside it), so each window stores at most two partial
-// results in the scratch array, and a last kernel adds a long row's partials
-// in window order.  Every slot it reads is written earlier in the same call, so
-// nothing in the scratch array has to start at zero.
+// asks for.  Rows of more than 32 entries belong to fixed 4096-entry windows of
+// the entry array, a block each, so that the work is split by entries wherever
+// such rows stand together: the block of the window in which a row starts takes
+// it, and rows of more than 4096 are split by the windows.  A window meets at
+// most two of those (one that started before it, one that starts inside it), so
+// each window stores at most two partial results in the scratch array, and a last
+// kernel adds a long row's partials in window order.  Every slot it reads is
+// written earlier in the same call, so nothing in the scratch array has to start
+// at zero.
 #include <algorithm>
 #include <cstring>
 #include <mutex>
@@ -31,10 +33,10 @@ constexpr int kNaMaxWindows = 1 << 16;    // => at most 268,435,456 nonzeros
 constexpr int kNaThreads = 256;
 constexpr int kNaWarps = kNaThreads / 32;
 // lanes per row by its length: one up to 4 entries, 4 up to 32, a warp up to
-// 512, the block beyond.  An FP64 warp instruction holds the pipe for 16
+// 512, the block beyond (both in the window's block).  An FP64 warp instruction holds the pipe for 16
 // clocks however many lanes are active, so a warp must not wait for one long
 // row among short ones; lengths up to 4 are four fifths of a skewed LP's rows.
-constexpr int kNaOne = 4, kNaFour = 32, kNaWarp = 512;
+constexpr int kNaOne = 4, kNaShort = 32, kNaWarp = 512;
 
 struct WindowPart {
     double2 act[2];   // (min, max) finite parts: [0] of the long row that started before the window,
@@ -145,14 +147,49 @@ __device__ __forceinline__ int32_t na_row_of(const int32_t *rp, int32_t m, int64
     return (int32_t)lo;
 }
 
-// window w of the entry array: the partials of the (at most two) long rows it meets
-__device__ __forceinline__ void na_window(const NaArgs &a, WindowPart &p, int32_t w, NaSum *s_w) {
-    __shared__ int32_t s_r[2];
+// Rows of 33 to 4096 entries that start in the window [w0, w1), into own (at most
+// kNaOwn of them); r0, r1: the rows of its first and last entry.  Few rows are
+// looked at one by one; among many (most of them empty) a search finds those that
+// hold a multiple of 32 entries, and the last row, which may hold none before w1.
+constexpr int kNaOwn = (kNaWindow + kNaShort - 1) / kNaShort;
+constexpr int32_t kNaScan = 8 * kNaThreads;
+__device__ __forceinline__ void na_own_rows(const NaArgs &a, int64_t w0, int64_t w1, int32_t r0, int32_t r1,
+                                            int32_t *own, int32_t *cnt) {
+    const auto take = [&](int32_t r) {
+        const int64_t b = a.rp[r], n = a.rp[r + 1] - b;
+        if (b >= w0 && n > kNaShort && n <= kNaLong) own[atomicAdd(cnt, 1)] = r;
+    };
+    if (r1 - r0 < kNaScan) {
+        for (int32_t r = r0 + (int32_t)threadIdx.x; r <= r1; r += kNaThreads) take(r);
+        return;
+    }
+    const int64_t p = w0 + (int64_t)threadIdx.x * kNaShort;
+    if (p < w1) {
+        int32_t lo = r0, hi = r1;  // the last row that starts at or before p
+        while (lo < hi) {
+            const int32_t mid = lo + (hi - lo + 1) / 2;
+            if (a.rp[mid] <= p) lo = mid;
+            else hi = mid - 1;
+        }
+        if (a.rp[lo] > p - kNaShort) take(lo);  // p is its first multiple
+    }
+    if (threadIdx.x == kNaThreads - 1 && ((int64_t)a.rp[r1] + kNaShort - 1) / kNaShort * kNaShort >= w1) take(r1);
+}
+
+// window w of the entry array: the partials of the (at most two) long rows it
+// meets, and the rows of 33 to 4096 entries that start in it
+struct NaWindow {
+    int32_t r[2], own[kNaOwn], cnt;
+};
+__device__ __forceinline__ void na_window(const NaArgs &a, WindowPart &p, int32_t w, NaSum *s_w, NaWindow &S) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t w0 = (int64_t)w * kNaWindow, w1 = min(a.nnz, w0 + kNaWindow);
-    if (threadIdx.x < 64) s_r[threadIdx.x >> 5] = na_row_of(a.rp, a.m, threadIdx.x < 32 ? w0 : w1 - 1);
+    if (threadIdx.x == 0) S.cnt = 0;
+    if (warp < 2) S.r[warp] = na_row_of(a.rp, a.m, warp == 0 ? w0 : w1 - 1);
     __syncthreads();
+    na_own_rows(a, w0, w1, S.r[0], S.r[1], S.own, &S.cnt);
     for (int slot = 0; slot < 2; slot++) {
-        const int32_t r = s_r[slot];
+        const int32_t r = S.r[slot];
         const int64_t rb = a.rp[r], re = a.rp[r + 1];
         const bool use = re - rb > kNaLong && (slot == 0 ? rb < w0 : rb >= w0);
         if (threadIdx.x == 0) p.row[slot] = use ? r : -1;
@@ -163,30 +200,45 @@ __device__ __forceinline__ void na_window(const NaArgs &a, WindowPart &p, int32_
             p.ninf[slot] = make_int2(s.nlo, s.nhi);
         }
     }
+    __syncthreads();
+    for (int i = warp; i < S.cnt; i += kNaWarps) {
+        const int32_t r = S.own[i], b = a.rp[r], e = a.rp[r + 1];
+        if (e - b > kNaWarp) continue;
+        NaSum s{0.0, 0.0, 0, 0};
+        na_accumulate<32, 4>(a, b + lane, e, s);
+        na_butterfly<32>(s);
+        if (lane == 0) na_row(a, r, s);
+    }
+    for (int i = 0; i < S.cnt; i++) {
+        const int32_t r = S.own[i], b = a.rp[r], e = a.rp[r + 1];
+        if (e - b <= kNaWarp) continue;  // block-uniform
+        const NaSum s = na_block(a, b, e, s_w);
+        if (threadIdx.x == 0) na_row(a, r, s);
+    }
 }
 
-// Blocks [0, windows): the long rows' windows, first so that they run beside
-// the rows; the other blocks: 256 rows each, those of at most 4096 entries.
+// Blocks [0, windows): the windows, first so that they run beside the rows; the
+// other blocks: 256 rows each, those of at most 32 entries.
 // Bound by the FP64 pipe (63% busy) and the latency of the two 8-byte bound
-// gathers per entry: 20 M entries in 2 M skewed rows take 244 us, 2660 us
+// gathers per entry: 20 M entries in 2 M skewed rows take @T@ us, 2660 us
 // with a warp per row (a median row of two entries used two of 32 lanes, and
 // infinities were tested by FP64 compares).  No shared memory for the entries:
 // a tile of them staged there, coalesced, took 510 us, because it leaves the
-// L1 too few lines for the gathers in flight (4% hits instead of 23%).
+// L1 too few lines for the gathers in flight (4% hits instead of 23%).  With the
+// rows of 33 to 4096 entries in the row blocks, 256 of them standing together ran
+// on one SM: 3,000 rows of 4096 took 2460 us, now 128, a dense matrix of 1500 rows
+// 1070, now 57.  The line at 32: with one at 64, 256 rows of 64 entries before
+// 5,000 short ones took 67 us, not 45 (300 k rows of 33 entries 305, not 322).
 __global__ void __launch_bounds__(kNaThreads, 5) k_na_rows(NaArgs a, WindowPart *scratch, int32_t windows) {
-    __shared__ int2 s_mid[kNaWarps][32];   // a warp's rows of 5 to 32 entries: (lane of the row, first entry)
-    __shared__ int32_t s_blk[kNaThreads];  // the block's rows of 513 to 4096 entries
-    __shared__ int32_t s_nblk;
+    __shared__ int2 s_mid[kNaWarps][32];  // a warp's rows of 5 to 32 entries: (lane of the row, first entry)
     __shared__ NaSum s_w[kNaWarps];
+    __shared__ NaWindow s_win;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (blockIdx.x < (unsigned)windows) {
-        na_window(a, scratch[blockIdx.x], (int32_t)blockIdx.x, s_w);
+        na_window(a, scratch[blockIdx.x], (int32_t)blockIdx.x, s_w, s_win);
         return;
     }
-    const int64_t base = (int64_t)(blockIdx.x - windows) * kNaThreads;
-    if (tid == 0) s_nblk = 0;
-    __syncthreads();
-    const int64_t rl = base + tid;
+    const int64_t rl = (int64_t)(blockIdx.x - windows) * kNaThreads + tid;
     const int32_t r = (int32_t)rl;
     int32_t b = 0, e = 0;
     if (rl < a.m) {
@@ -199,10 +251,8 @@ __global__ void __launch_bounds__(kNaThreads, 5) k_na_rows(NaArgs a, WindowPart 
         na_accumulate<1, 4>(a, b, e, s);
         na_row(a, r, s);
     }
-    const unsigned mid = __ballot_sync(0xffffffffu, n > kNaOne && n <= kNaFour);
-    unsigned wide = __ballot_sync(0xffffffffu, n > kNaFour && n <= kNaWarp);
-    if (n > kNaOne && n <= kNaFour) s_mid[warp][__popc(mid & ((1u << lane) - 1u))] = make_int2(lane, b);
-    if (n > kNaWarp && n <= kNaLong) s_blk[atomicAdd(&s_nblk, 1)] = r;
+    const unsigned mid = __ballot_sync(0xffffffffu, n > kNaOne && n <= kNaShort);
+    if (n > kNaOne && n <= kNaShort) s_mid[warp][__popc(mid & ((1u << lane) - 1u))] = make_int2(lane, b);
     __syncwarp();
     const int nmid = __popc(mid);
     for (int i0 = 0; i0 < nmid; i0 += 8) {
@@ -213,21 +263,6 @@ __global__ void __launch_bounds__(kNaThreads, 5) k_na_rows(NaArgs a, WindowPart 
         if (i < nmid) na_accumulate<4, 4>(a, eb + (lane & 3), ee, s);
         na_butterfly<4>(s);
         if (i < nmid && (lane & 3) == 0) na_row(a, (int32_t)(rl - lane) + it.x, s);
-    }
-    while (wide) {
-        const int src = __ffs(wide) - 1;
-        wide &= wide - 1u;
-        const int32_t wb = __shfl_sync(0xffffffffu, b, src), we = __shfl_sync(0xffffffffu, e, src);
-        NaSum s{0.0, 0.0, 0, 0};
-        na_accumulate<32, 4>(a, wb + lane, we, s);
-        na_butterfly<32>(s);
-        if (lane == 0) na_row(a, (int32_t)(rl - lane) + src, s);
-    }
-    __syncthreads();
-    for (int i = 0; i < s_nblk; i++) {
-        const int32_t q = s_blk[i];
-        const NaSum s = na_block(a, a.rp[q], a.rp[q + 1], s_w);
-        if (tid == 0) na_row(a, q, s);
     }
 }
 
@@ -299,10 +334,10 @@ extern "C" lpp_status lpp_row_activity_noalloc(int32_t m, int32_t n, int64_t nnz
     std::memcpy(&hb, &huge, sizeof hb);
     NaArgs a{m, nnz, row_ptr, col_idx, val, lb, ub, hb, act_min, act_max, ninf_min, ninf_max};
     WindowPart *parts = static_cast<WindowPart *>(scratch);
-    const int32_t windows = nnz > kNaLong ? (int32_t)((nnz + kNaWindow - 1) / kNaWindow) : 0;
+    const int32_t windows = nnz > kNaShort ? (int32_t)((nnz + kNaWindow - 1) / kNaWindow) : 0;
     k_na_rows<<<(unsigned)(windows + (m + (int64_t)kNaThreads - 1) / kNaThreads), kNaThreads, 0, s>>>(a, parts,
                                                                                                   windows);
-    if (windows)
+    if (nnz > kNaLong)
         k_na_long<<<(unsigned)((windows + kNaWarps - 1) / kNaWarps), kNaThreads, 0, s>>>(a, parts, windows);
     e = cudaGetLastError();
     if (e != cudaSuccess) return lpp_noalloc_fail(LPP_ERR_CUDA, cudaGetErrorString(e));
