@@ -432,6 +432,14 @@ __device__ __forceinline__ T lanes_sum(T v, int W, unsigned mask) {
     return v;
 }
 
+// bits 4 c + e to c + 4 e, in both halves
+__device__ __forceinline__ unsigned transpose_4x4(unsigned x) {
+    unsigned t = (x ^ (x >> 3)) & 0x0a0a0a0au;
+    x ^= t ^ (t << 3);
+    t = (x ^ (x >> 6)) & 0x00cc00ccu;
+    return x ^ t ^ (t << 6);
+}
+
 // S1-S3 of row i by W lanes.  LONG: a warp (W = 32) per row of any length, S3
 // walks the row again.  Else W = 1, 2 or 4 with at most 16 entries per lane,
 // whose spans stay in registers for S3, so that S3 reads only the entries that
@@ -459,23 +467,29 @@ __device__ __forceinline__ void prop_row(const Ctx &C, int32_t i, bool valid, in
     // The lane's entries in steps of four, the tail of a step predicated: the
     // four bound gathers of a step overlap, and a warp whose lanes hold rows of
     // different lengths runs no separate remainder loop (which would issue
-    // its FP64 work a second time for the lanes still in it).  The sums take
-    // the entries in the same order as a plain loop.
+    // its FP64 work a second time for the lanes still in it).  A lone lane's sums
+    // take the entries in the same order as a plain loop.
+    // A lane of several (W = 2, 4) takes, in step c, the entries of residue class
+    // lane + c W modulo 4 W, a chain each, added as a butterfly over 4 W lanes
+    // adds them: the bits, and so the error, of 8 and 16 lanes per row.  (One
+    // chain of a lane's 16 entries had up to 18 roundings where this has 7 or 8,
+    // and a mean error 3 to 20% larger.)
+    const int32_t es = !LONG && W > 1 ? 4 * W : W, cs = !LONG && W > 1 ? W : 4 * W;
     auto step = [&](int32_t k0, int c4) {
         int32_t jq[4];
         double aq[4];
         double2 bq[4];
 #pragma unroll
         for (int e = 0; e < 4; e++) {
-            const int32_t k = k0 + e * W;
+            const int32_t k = k0 + e * es;
             jq[e] = k < end ? C.A.idx[k] : 0;
             aq[e] = k < end ? C.A.val[k] : 0.0;
         }
 #pragma unroll
-        for (int e = 0; e < 4; e++) bq[e] = act && k0 + e * W < end ? C.lu[jq[e]] : make_double2(0.0, 0.0);
+        for (int e = 0; e < 4; e++) bq[e] = act && k0 + e * es < end ? C.lu[jq[e]] : make_double2(0.0, 0.0);
 #pragma unroll
         for (int e = 0; e < 4; e++) {
-            if (k0 + e * W >= end) break;
+            if (k0 + e * es >= end) break;
             const double a = aq[e];
             const double2 b = bq[e];
             const bool neg = is_neg(a);
@@ -496,9 +510,28 @@ __device__ __forceinline__ void prop_row(const Ctx &C, int32_t i, bool valid, in
     if constexpr (LONG) {
         for (int32_t k0 = beg + lane; k0 < end; k0 += 4 * W) step(k0, 0);
     } else {
+        double t0 = 0.0, t1 = 0.0, u0 = 0.0, u1 = 0.0;
 #pragma unroll
-        for (int c = 0; c < 4; c++)
-            if (beg + lane + 4 * c * W < end) step(beg + lane + 4 * c * W, 4 * c);
+        for (int c = 0; c < 4; c++) {
+            if (beg + lane + c * cs < end) step(beg + lane + c * cs, 4 * c);
+            if (W > 1) {  // the same W in the whole warp
+                if (c == 0) {
+                    t0 = smin;
+                    t1 = smax;
+                } else if (c == 1) {
+                    u0 = smin;
+                    u1 = smax;
+                } else if (c == 2) {
+                    t0 += smin;
+                    t1 += smax;
+                }
+                if (c < 3) smin = smax = 0.0;
+            }
+        }
+        if (W > 1) {
+            smin = t0 + (u0 + smin);
+            smax = t1 + (u1 + smax);
+        }
     }
     if (W > 1) {  // the same W in the whole warp
         smin = lanes_sum(smin, W, mask);
@@ -535,20 +568,27 @@ __device__ __forceinline__ void prop_row(const Ctx &C, int32_t i, bool valid, in
     if constexpr (!LONG) {
         // a x_j <= U - (min activity of the others): every entry when no term
         // is infinite, the one infinite term alone when there is one
+        // Bit 4 c + e: the entry of step c; with several lanes it is the lane's
+        // (c + 4 e)th, and a transposition of the 4 x 4 bits puts them in order.
         const int nq = lane < len ? (len - lane + W - 1) / W : 0;
-        const unsigned all = (1u << nq) - 1u;
+        const unsigned all = W > 1 ? transpose_4x4((1u << nq) - 1u) : (1u << nq) - 1u;
         const unsigned q1 = up_row ? (nmin == 0 ? all : imin) : 0u, q2 = lo_row ? (nmax == 0 ? all : imax) : 0u;
         tested += __popc(q1) + __popc(q2);
         unsigned todo = 0;
         if (q1 | q2) {
 #pragma unroll
             for (int c = 0; c < 4; c++) {
-                if (nq <= 4 * c) break;
+                if (nq <= (W > 1 ? c : 4 * c)) break;
 #pragma unroll
                 for (int e = 4 * c; e < 4 * c + 4; e++)
                     todo |= (unsigned)span_passes(fU, span[e]) << e | (unsigned)span_passes(fL, span[e]) << (16 + e);
             }
             todo &= q1 | (q2 << 16);
+        }
+        if (W > 1 && todo) {
+            todo = transpose_4x4(todo);
+            imin = transpose_4x4(imin);
+            imax = transpose_4x4(imax);
         }
         // a singleton row L <= a x_j <= U becomes the bounds L/a and U/a, always
         // applied (no threshold)
@@ -566,7 +606,9 @@ __device__ __forceinline__ void prop_row(const Ctx &C, int32_t i, bool valid, in
 // Lanes per row in S1-S3: a lane holds up to 16 entries (rows up to 16, 32 and
 // 64 entries: 1, 2, 4 lanes), longer rows take a warp.  Fewer lanes per row
 // cost fewer butterfly steps, each two FP64 instructions: 8 lanes for 17 to
-// 32 entries cost 3.5 FP64 warp instructions a row, 2 lanes 2.1.
+// 32 entries cost 3.5 FP64 warp instructions a row, 2 lanes with four chains
+// each 2.5 (one chain each 2.1, but off by more: the relaxation of 500 k rows
+// takes 5.55 ms for 5.42).
 __host__ __device__ __forceinline__ int prop_lanes(int c) { return c <= 2 ? 1 : (c == 5 ? 32 : 1 << (c - 2)); }
 
 // ------------------------------------------------- S3' finalise + S4 fixing
