@@ -194,9 +194,9 @@ __global__ void __launch_bounds__(kBlock, 2) k_solo(const __grid_constant__ Solo
     int32_t status = LPP_OK, where = LPP_WHERE_NONE, vindex = -1, vround = 0;
     // every block takes the same branches, so each passes the same barriers
     unsigned gen = 0;
-#define GRID_SYNC()                                            \
-    do {                                                       \
-        if (!grid_barrier(ctl->bar, &ctl->err, gen)) goto out; \
+#define GRID_SYNC()                                                            \
+    do {                                                                       \
+        if (!grid_barrier(ctl->bar, &ctl->err, gen, &ctl->progress)) goto out; \
     } while (0)
 
     // the input's rows by class
@@ -375,7 +375,7 @@ __global__ void __launch_bounds__(kBlock, 2) k_solo(const __grid_constant__ Solo
                 }
                 GRID_SYNC();
                 if (!s5_later_passes(C, F.s5l[0], F.s5l[1], F.s5_cnt, 1, F.par_max_iter, left, removed, ctl->bar,
-                                     &ctl->err, gen))
+                                     &ctl->err, gen, &ctl->progress))
                     goto out;
                 __syncwarp();
                 warp_add(removed, &N.merged);

@@ -212,7 +212,7 @@ struct SoloOut {
 struct SoloCtl {  // zero before the launch
     SoloOut out;
     unsigned bar[2];  // arrivals at the barriers of the rounds, of the finish
-    int32_t err, pad;
+    int32_t err, progress;  // S5's later passes on one block, as they go
     SoloCnt c[2];  // by the round's parity
 };
 struct SoloArgs {

@@ -442,10 +442,12 @@ __device__ __forceinline__ void match_long(const Ctx &C, int32_t t, int32_t *out
 // last one: no counter to reset, no second word to publish.  With those, a call
 // on 20 k rows (110 barriers of 176 blocks) took 8% longer, 1.59 ms, not 1.47
 // to 1.54.  One block: a block barrier.
-// A wait that takes too long (it cannot, with every block resident) sets *err
-// bit 4 and returns false, as do then all later waits.
+// A wait that takes too long (with every block resident: longer than any work
+// between two barriers) sets *err bit 4 and returns false, as do then all later
+// waits.  Work that may take longer changes *progress (if given) as it goes, and
+// the waits count anew.
 constexpr int32_t kBarSpins = 1 << 22;
-__device__ bool grid_barrier(unsigned *bar, int32_t *err, unsigned &gen) {
+__device__ bool grid_barrier(unsigned *bar, int32_t *err, unsigned &gen, const int32_t *progress = nullptr) {
     __shared__ int s_ok;
     __syncthreads();
     if (gridDim.x == 1) return true;
@@ -453,12 +455,19 @@ __device__ bool grid_barrier(unsigned *bar, int32_t *err, unsigned &gen) {
     if (threadIdx.x == 0) {
         const unsigned want = gen * gridDim.x;
         int ok = 1;
+        int32_t seen = 0;
         asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
         for (int32_t spins = 0;; spins++) {
             unsigned v;
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
             if ((int)(v - want) >= 0) break;
-            if (spins > kBarSpins || ((spins & 255) == 255 && (*(volatile int32_t *)err & 4))) {
+            if ((spins & 255) != 255) continue;
+            if (progress) {
+                const int32_t p = *(const volatile int32_t *)progress;
+                if (p != seen) spins = 0;
+                seen = p;
+            }
+            if (spins > kBarSpins || (*(volatile int32_t *)err & 4)) {
                 atomicOr(err, 4);
                 ok = 0;
                 break;
@@ -478,13 +487,15 @@ __device__ bool grid_barrier(unsigned *bar, int32_t *err, unsigned &gen) {
 // emptied for pass p + 1, so a pass has two barriers, not three; a list too long
 // for half the table (the first passes, if at all: lists shrink) empties the
 // slots it used behind a barrier of its own.  From kTailAlone rows on block 0
-// goes on alone (its barriers are block barriers); n and removed are its then.
+// goes on alone (its barriers are block barriers); n and removed are its then,
+// and it counts its passes in *progress (if given): there are up to as many as
+// rows, of rows of any length.
 // On 2 M rows the tail took 326 us with three barriers a pass of the
 // former kind, now 244; on 500 k rows 184, now 110.
 constexpr int32_t kTailAlone = 2 * kBlock;
 __device__ __forceinline__ bool s5_later_passes(const Ctx &C, int32_t *l0, int32_t *l1, int32_t *cnt, int32_t p0,
                                                 int32_t max_iter, int32_t &n, int32_t &removed, unsigned *bar,
-                                                int32_t *err, unsigned &gen) {
+                                                int32_t *err, unsigned &gen, int32_t *progress = nullptr) {
     const int32_t gt = blockIdx.x * kBlock + threadIdx.x;
     bool one = gridDim.x == 1;
     uint32_t prev_off = 0, prev_cap = 0, own = 0;
@@ -539,6 +550,7 @@ __device__ __forceinline__ bool s5_later_passes(const Ctx &C, int32_t *l0, int32
         prev_off = off;
         prev_cap = turns ? cap : 0;
         n = __ldcg(cnt + p);
+        if (one && progress && threadIdx.x == 0) *(volatile int32_t *)progress = p;
     }
     return true;
 }
