@@ -1,5 +1,6 @@
 // lpp_engine.cu -- device state and the round loop (S0 .. S8) of the presolve.
 #include <algorithm>
+#include <atomic>
 #include <cstdio>
 #include <cstring>
 #include <map>
@@ -1339,12 +1340,13 @@ void Engine::run_rounds() {
 }
 
 // The rounds in one cooperative kernel: one launch, one read of its results.
+// share: presolves in flight on the device, which its blocks are shared with.
 // False, with nothing done, if the launch was refused (the caller's stream may
 // own fewer SMs than the device): the rounds are then launched.  The kernel of
 // the end fits where the first does: no more blocks, and more of them per SM.
-bool Engine::run_solo() {
+bool Engine::run_solo(int share) {
     const int32_t R = o.max_rounds;
-    const int blocks = solo_blocks(m0, n0, nnz0);
+    const int blocks = solo_blocks(m0, n0, nnz0, share);
     const size_t ctl_bytes = sizeof(SoloCtl) + 6 * sizeof(int32_t) * (size_t)R;
     SoloArgs F;
     std::memset(&F, 0, sizeof F);
@@ -1388,7 +1390,7 @@ bool Engine::run_solo() {
     F.par_max_iter = o.par_max_iter;
     SoloFinish G;
     std::memset(&G, 0, sizeof G);
-    const int fblocks = solo_finish_blocks(n0, nnz0);
+    const int fblocks = solo_finish_blocks(n0, nnz0, share);
     G.ctl = F.ctl;
     G.err_in = F.err_in;
     G.n = n0;
@@ -1483,7 +1485,15 @@ void Engine::run() {
     spare_events.push_back(eloop);
     spare_events.push_back(eend);
     LPP_CUDA(cudaEventRecord(eloop, s));
-    if (!solo || !run_solo()) {
+    // presolves in flight on the device, from any thread, this one included
+    static std::atomic<int> in_flight[CoopCache::kDevices];
+    struct Share {
+        std::atomic<int> &c;
+        const int n;
+        explicit Share(std::atomic<int> &x) : c(x), n(x.fetch_add(1) + 1) {}
+        ~Share() { c.fetch_sub(1); }
+    } share(in_flight[o.device % CoopCache::kDevices]);
+    if (!solo || (share.n > 1 && nnz0 > kSoloShared) || !run_solo(share.n)) {
         if (solo) first_schedules();
         solo = false;
         run_rounds();

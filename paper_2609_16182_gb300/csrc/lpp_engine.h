@@ -70,6 +70,11 @@ struct DevPool {
 // blocks per SM at 128 registers hold fewer gathers in flight than the launched
 // kernels).
 constexpr int64_t kSoloNnz = 5 << 19;
+// The same while other presolves are in flight on the device, whose launched
+// rounds fill the gaps of each other: ms a call with eight and sixteen threads,
+// launched / in one kernel: 0.18 M entries 0.57, 0.57 / 0.24, 0.26; 0.43 M 0.64,
+// 0.59 / 0.44, 0.55; 0.9 M 0.78, 0.67 / 0.72, 0.96; 1.9 M 0.98, 0.82 / 1.22, 1.70.
+constexpr int64_t kSoloShared = 1 << 19;
 
 // per-LP description of an arena member
 struct Member {
@@ -236,7 +241,7 @@ struct Engine {
     void prepare();  // after ingest: transpose, schedules, work init
     void run();      // the round loop
     bool solo = false;  // all rounds in one kernel (one LP of at most kSoloNnz entries, columns in place)
-    bool run_solo();
+    bool run_solo(int share);
     void first_schedules();
     void run_rounds();
     struct StepOut {

@@ -236,7 +236,8 @@ struct SoloArgs {
     int32_t *rstat;            // six per round: nonzeros, rows removed, columns fixed, bounds changed, ns
     int32_t m, n, nnz, tcap_max, max_rounds, par_max_iter;
 };
-int solo_blocks(int32_t m, int32_t n, int64_t nnz);
+// blocks of the launches below, where `share` such presolves share the device
+int solo_blocks(int32_t m, int32_t n, int64_t nnz, int share = 1);
 // false: the launch was refused, nothing has run
 bool launch_solo(const SoloArgs &F, int blocks, cudaStream_t s);
 // The end of such a run: objective constant, the columns' one compaction and
@@ -260,7 +261,7 @@ struct SoloFinish {
     double *contrib, *part, *offset;
     int32_t *btot, *hist;            // one / 256 per block
 };
-int solo_finish_blocks(int32_t n, int64_t nnz);
+int solo_finish_blocks(int32_t n, int64_t nnz, int share = 1);
 bool launch_solo_finish(const SoloFinish &F, int blocks, cudaStream_t s);
 
 // ---------------------------------------------------------------- k_batch.cu
