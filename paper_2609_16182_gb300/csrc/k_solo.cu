@@ -804,13 +804,18 @@ __global__ void __launch_bounds__(kBlock) k_solo_finish(const __grid_constant__ 
 // (a block or a warp each) over the SMs.  With 2048, 1024, 512 and 256 entries per
 // block a presolve takes, in us: 500 skewed rows 1401, 1036, 857, 801; 5,000 rows
 // 1047, 905, 850, 858; 20,000 rows 1299, 1162, 1163, 1165; 100,000 rows the same.
+// One slot in 32 stays free: two of these blocks hold all registers of an SM, and
+// no other stream's kernels or copies ran until a grid that held every SM twice
+// had ended.  A server's submissions then waited for the request being presolved,
+// its queue stayed short, and 80 requests of 0.55 M entries were presolved one by
+// one: 108 ms, batched 60.  An LP of 1.9 M entries alone takes 1.80 ms for 1.78.
 // Presolves in flight at once (share) get a part of the slots each: a grid that
 // fills the device waits for all of it, and they would run one after the other.
 // 20,000 rows from eight threads took 0.91 ms a call, now 0.24.
 int solo_blocks(int32_t m, int32_t n, int64_t nnz, int share) {
     static CoopCache cache;
     int most = solo_finish_blocks(n, nnz) > 0 ? coop_blocks((const void *)k_solo, cache) : 0;
-    if (most > 0) most = std::max(1, most / share);
+    if (most > 0) most = std::max(1, (most - most / 32) / share);
     const int64_t want = std::max<int64_t>({1, ((int64_t)m + kBlock - 1) / kBlock, ((int64_t)n + 2 * kBlock - 1) / (2 * kBlock),
                                             (nnz + 2 * kBlock - 1) / (2 * kBlock)});
     return (int)std::min<int64_t>(want, most);
