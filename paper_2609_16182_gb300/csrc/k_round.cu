@@ -77,13 +77,13 @@ __global__ void __launch_bounds__(kBlock) k_prop_long_combine(Ctx C) {
     int32_t removed = 0, evaluated = 0;
     prop_long_row(C, (int32_t)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5), removed, evaluated);
     warp_add(removed, &C.st->rows_removed);
-    warp_add(evaluated, &C.st->nnz_eval);
+    if (C.count_work) warp_add(evaluated, &C.st->nnz_eval);
 }
 
 __global__ void __launch_bounds__(kBlock) k_prop_long_tighten(Ctx C) {
     int32_t tested = 0;
     prop_long_tighten(C, blockIdx.x, tested);
-    warp_add(tested, &C.st->sides_tested);
+    if (C.count_work) warp_add(tested, &C.st->sides_tested);
 }
 
 __global__ void __launch_bounds__(kBlock) k_bsrc_groups(Ctx C, RowGrid R) { bsrc_block(C, R, blockIdx.x); }

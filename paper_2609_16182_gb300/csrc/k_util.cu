@@ -678,17 +678,6 @@ __global__ void k_colptr_from_keys(const uint32_t *key, int64_t nnz, int32_t n, 
     for (int32_t j = kq + 1; j <= kp; j++) tptr[j] = (int32_t)p;
 }
 
-// segment lengths from a pointer array
-__global__ void k_ptr_diff(const int32_t *ptr, int32_t cnt, int32_t *out) {
-    const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < cnt) out[i] = ptr[i + 1] - ptr[i];
-}
-
-__global__ void k_iota(int32_t *a, int32_t cnt, int32_t base) {
-    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < cnt) a[k] = base + (int32_t)k;
-}
-
 __global__ void k_fill_u64(unsigned long long *a, int64_t cnt, unsigned long long v) {
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (k < cnt) a[k] = v;
@@ -778,8 +767,7 @@ GroupGrid group_grid(const SegMat &M) {
 }
 
 void check_csr(const int32_t *ptr, const int32_t *idx, const double *val, int32_t m, int32_t n, int64_t nnz,
-               int32_t *row_of, int32_t *tmp, int32_t *err, cudaStream_t s) {
-    (void)tmp;
+               int32_t *row_of, int32_t *err, cudaStream_t s) {
     (k_check_ptr<<<blocks_for((int64_t)m + 1, 256), 256, 0, s>>>(ptr, m, nnz, err), note_launch());
     // row_of[0] is unused (callers read row_of + 1)
     if (nnz > 0 && m > 0)
@@ -857,14 +845,6 @@ void sort_pairs(const uint32_t *keys, const int32_t *vals, int64_t cnt, int bits
     }
     *kout = kin;
     *vout = vin;
-}
-
-void ptr_diff(const int32_t *ptr, int32_t cnt, int32_t *out, cudaStream_t s) {
-    if (cnt > 0) (k_ptr_diff<<<blocks_for(cnt, 256), 256, 0, s>>>(ptr, cnt, out), note_launch());
-}
-
-void iota(int32_t *a, int32_t cnt, int32_t base, cudaStream_t s) {
-    if (cnt > 0) (k_iota<<<blocks_for(cnt, 256), 256, 0, s>>>(a, cnt, base), note_launch());
 }
 
 void fill_u64(unsigned long long *a, int64_t cnt, unsigned long long v, cudaStream_t s) {

@@ -660,7 +660,7 @@ void Engine::prepare() {
     // S0: checks, then A^T by a stable transpose where it is needed
     const bool want_t = !in_place || need_t;
     int32_t *row_of = want_t ? pool.alloc<int32_t>(nnz0 + 1) : nullptr;
-    check_csr(m_rp, m_ci, m_rv, m0, n0, nnz0, row_of, scan_tmp, &st->err, s);
+    check_csr(m_rp, m_ci, m_rv, m0, n0, nnz0, row_of, &st->err, s);
     t_hist = pool.alloc<int32_t>(transpose_hist_elems(nnz0));  // S5e and the result's A^T transpose with it too
     LPP_CUDA(cudaGetLastError());
     if (want_t) {
@@ -1087,7 +1087,6 @@ Engine::StepOut Engine::step(int32_t r, bool first_round, bool force) {
     tend();
     LPP_CUDA(cudaGetLastError());
     read_status();
-    r_eval.push_back(st_h->nnz_eval);
     if (o.timing && prop_mark > 0) {
         // S1-S3 algorithmic work: per evaluated nonzero its 12 bytes and two
         // FMAs (activities), per tested entry side two FMAs (the residual and

@@ -229,7 +229,6 @@ struct Engine {
         cudaEvent_t a, b;
         double bytes, ops;
     };
-    std::vector<int64_t> r_eval;  // nonzeros S1 evaluated per round
     std::vector<Tmark> marks;
     std::vector<cudaEvent_t> spare_events;
 

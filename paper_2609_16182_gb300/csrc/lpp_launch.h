@@ -65,7 +65,7 @@ GroupGrid group_grid(const SegMat &M);
 // Input checks: returns error bits in *err (device).  row_of (unless NULL)
 // gets the row of each entry from row_of[1] on.
 void check_csr(const int32_t *ptr, const int32_t *idx, const double *val, int32_t m, int32_t n, int64_t nnz,
-               int32_t *row_of, int32_t *tmp, int32_t *err, cudaStream_t s);
+               int32_t *row_of, int32_t *err, cudaStream_t s);
 // Vectors: normalise |v| >= huge to +-inf, check NaN / wrong-signed infinity,
 // interleave (lb, ub) into lu.
 void ingest_vectors(const double *lhs, const double *rhs, const double *lb, const double *ub, const double *c,
@@ -90,8 +90,6 @@ void transpose(const int32_t *ptr, const int32_t *idx, const double *val, const 
 // themselves when cnt == 0).  b.hist needs transpose_hist_elems(cnt) entries.
 void sort_pairs(const uint32_t *keys, const int32_t *vals, int64_t cnt, int bits, const TransposeBufs &b,
                 const uint32_t **kout, const int32_t **vout, cudaStream_t s);
-void iota(int32_t *a, int32_t cnt, int32_t base, cudaStream_t s);
-void ptr_diff(const int32_t *ptr, int32_t cnt, int32_t *out, cudaStream_t s);  // out[i] = ptr[i+1] - ptr[i]
 void fill_u64(unsigned long long *a, int64_t cnt, unsigned long long v, cudaStream_t s);
 void fill_i32(int32_t *a, int64_t cnt, int32_t v, cudaStream_t s);
 // device words to pinned host memory, then seq to *flag (pinned)
@@ -132,7 +130,7 @@ void launch_s5_tail_block(const Ctx &C, int32_t *l0, int32_t *l1, int32_t *cnt, 
                           cudaStream_t s);
 constexpr int32_t kTailBlockRows = 4096;  // longest list the one-block form takes
 // all remaining later S5 passes of a longer list in one cooperative launch
-// with grid barriers (bar: two zeroed words kept by the caller); false if
+// with grid barriers (bar: a zeroed word kept by the caller); false if
 // the launch is not possible
 bool launch_s5_tail_grid(const Ctx &C, int32_t *l0, int32_t *l1, int32_t *cnt, int32_t p0, int32_t max_iter,
                          int32_t rows, unsigned *bar, cudaStream_t s);

@@ -234,7 +234,7 @@ void Engine::append(int32_t slot, const lpp_lp &in, int32_t rbase, int32_t cbase
     LPP_CUDA(cudaMemsetAsync(&st->err, 0, sizeof(int32_t), s));
     int32_t *row_of = tmp.alloc<int32_t>((size_t)zl + 1);
     int32_t *stmp = tmp.alloc<int32_t>(scan_tmp_elems(std::max<int64_t>({(int64_t)zl + 1, (int64_t)nl + 1, (int64_t)transpose_hist_elems(zl)})));
-    check_csr(rp_in, ci_in, rv_in, ml, nl, zl, row_of, stmp, &st->err, s);
+    check_csr(rp_in, ci_in, rv_in, ml, nl, zl, row_of, &st->err, s);
     ingest_vectors(lhs, rhs, lb, ub, cc, ml, nl, o.huge, L[cur] + m, U[cur] + m, lu[cur] + n, c[cur] + n, &st->err,
                    s);
     LPP_CUDA(cudaGetLastError());
