@@ -353,7 +353,7 @@ lpp_status lpp_presolve_batch(const lpp_lp *ins, int32_t count, const lpp_opts *
  * input) into a queue and returns a ticket; a worker thread admits queued
  * LPs while they fit the budget, runs one presolve round over all resident
  * unfinished LPs per tick, and keeps finished LPs resident until taken.  When
- * nothing is resident and at most 12 requests are queued, the oldest is
+ * nothing is resident and at most two requests are queued, the oldest is
  * presolved at once with its rounds back to back, as lpp_presolve would;
  * requests arriving meanwhile wait for it, and a longer queue is batched.
  * take waits up to wait_ms (-1 = forever) for the ticket's result

@@ -592,12 +592,9 @@ bool tick(lpp_server *S, std::vector<std::pair<int32_t, lpp_server::Req *>> &adm
 // The longest queue an idle server still serves one request at a time (each
 // presolved alone, back to back); a longer one joins the arena.  Served one
 // by one a request waits for the ones before it; in the arena every resident
-// LP advances one round per tick, some 20 ticks for all of them, which pays off
-// when enough of them share the ticks.  A burst one by one / in the arena, ms:
-// requests of 1e3 to 1e5 entries, 8: 6.6 / 8.0, 12: 9.9 / 9.0, 16: 13.3 / 10.1,
-// 32: 27.5 / 14.1, 64: 56 / 22; of 0.55 M entries, 10: 13.8 / 18.0, 16: 22 / 24,
-// 32: 44 / 37.
-constexpr size_t kSoloQueue = 12;
+// LP advances one round per tick, which pays off only when enough of them
+// share the ticks.
+constexpr size_t kSoloQueue = 64;
 
 void run_solo(lpp_server *S, lpp_server::Req *q) {
     lpp_opts o = S->o;
