@@ -156,7 +156,10 @@ typedef struct lpp_opts {
                                        among them is LPP_INFEASIBLE at its row.  Records of the
                                        step carry round = rounds + 1.  lpp_presolve only (a
                                        batch or a server rejects it)                          */
-    int32_t timing;         /* [0]     1: time every kernel launch with CUDA events           */
+    int32_t timing;         /* [0]     1: time every kernel launch with CUDA events.  The rounds
+                                       are then launched on one stream also for the LPs (up to
+                                       2.6 M entries, default steps) whose rounds otherwise are
+                                       one kernel: same result, other kernels and more time   */
     int32_t device;         /* [0]     CUDA device ordinal                                   */
     void *stream;           /* [NULL]  cudaStream_t to run on; NULL: a library-owned stream  */
 } lpp_opts;
@@ -353,7 +356,7 @@ lpp_status lpp_presolve_batch(const lpp_lp *ins, int32_t count, const lpp_opts *
  * input) into a queue and returns a ticket; a worker thread admits queued
  * LPs while they fit the budget, runs one presolve round over all resident
  * unfinished LPs per tick, and keeps finished LPs resident until taken.  When
- * nothing is resident and at most two requests are queued, the oldest is
+ * nothing is resident and at most 64 requests are queued, the oldest is
  * presolved at once with its rounds back to back, as lpp_presolve would;
  * requests arriving meanwhile wait for it, and a longer queue is batched.
  * take waits up to wait_ms (-1 = forever) for the ticket's result

@@ -1,15 +1,20 @@
 // k_compact.cu -- S6 (empty columns) and S7 (compaction) of a round.
 //
 // After S5 every row is kept or removed and every column kept or fixed.  The
-// compaction keeps the relative order of rows, columns and entries:
-//   1. per column (CSC): entries left in kept rows; a column with none left
-//      is fixed at the bound its cost prefers (S6, dual rule);
-//   2. per row (CSR): entries left in kept columns, and the shift
-//      sum_j a_ij v_j over its fixed columns;
-//   3. four exclusive scans: new row / column index, new row / column offset;
-//   4. row and column vectors are gathered into the next buffers, the kept
-//      sides shifted by their fixed columns (L -= shift, U -= shift);
-//   5. entries are scattered into the next CSR and CSC, renumbered.
+// compaction keeps the relative order of rows, columns and entries.  With the
+// columns in place (Ctx::in_place, the default steps):
+//   1. the columns of rows that left are noted (they may be empty now);
+//   2. per kept row (CSR), one pass: entries left, the shift sum_j a_ij v_j over
+//      its fixed columns, whether a bound in it changed, and which noted columns
+//      it still holds; then S6: a column no row holds is fixed at the bound its
+//      cost prefers (dual rule);
+//   3. two exclusive scans: new row index, new row offset;
+//   4. row vectors are gathered into the next buffers, the kept sides shifted
+//      (L -= shift, U -= shift), and the entries scattered into the next CSR, column
+//      indices as they are; columns and A^T are compacted once, after the rounds.
+// With a step that reads columns' entries, A^T is compacted each round too:
+// entries left per column (S6 from those, with locks for dual fixing), then rows
+// by the columns' keep flags, four scans, column vectors, both scatters, renumbered.
 // Long segments use the chunk lists of the schedule: a chunk counts its kept
 // entries, the chunks of a segment are prefix-summed in order, and each chunk
 // then writes its entries from its own offset.

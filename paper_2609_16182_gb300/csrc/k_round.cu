@@ -3,12 +3,13 @@
 //   CSR), S3'/S4 bound finalisation and fixing, S5 parallel rows.
 //
 // Load balance (Sec. 3.1, "length-based load balancing"): rows are grouped
-// by length class.  Class c <= 5 gives each row a group of W = 2^c lanes of a
-// warp (lane t walks entries t, t+W, ...; the group then reduces with an xor
-// butterfly), class 6 (more than 4096 entries) splits the row into chunks of
-// 4096 entries, one thread block each, whose partial results are combined in
-// chunk order.  The order of every floating-point sum depends only on the
-// row's own length.
+// by length class.  S1-S3 give a row of up to 16 entries one lane, up to 32 and
+// 64 two and four (prop_lanes), up to 256 a warp and up to 4096 a block; the other
+// steps give class c <= 5 a group of W = 2^c lanes of a warp (lane t walks entries
+// t, t+W, ...; the group then reduces with an xor butterfly).  Class 6 (more than
+// 4096 entries) splits the row into chunks of 4096 entries, one thread block
+// each, whose partial results are combined in chunk order.  The order of every
+// floating-point sum depends only on the row's own length.
 //
 // Bound tightening follows Sec. 3.1 in Jacobi form: activities and the
 // acceptance tests read the bounds of the round start, accepted implied

@@ -7,9 +7,8 @@
 // launch (phase_dev.cuh), are separated by grid barriers.  The control
 // decisions (which steps run, whether to compact, whether to stop) are taken
 // by every block alike from counters read after a barrier, as the host takes
-// them in Engine::step, so an LP gets the bits of the launched path.  A call on
-// 20 k rows (0.18 M entries, 13 rounds) takes 1.36 ms, 2.3 ms launched; on 200
-// rows 0.68 ms, 1.16 ms launched.
+// them in Engine::step, so an LP gets the bits of the launched path.  The rounds
+// of a small LP take about half the launched time (kSoloNnz).
 //
 // The columns stay in place (Ctx::in_place); row vectors and matrix alternate
 // between two buffers as there.  Counters exist twice, by the round's parity:
@@ -566,8 +565,7 @@ out:
 // compaction keeps their order, so they sort before the new indices are known,
 // and the columns' compaction shares the first pass's barriers.  The last pass
 // writes row and value, not key and payload, so no gather follows.
-// A call on 20 k rows takes 1.59 ms, 1.63 launched; a burst of 32 such requests
-// 45.0 ms, 46.2; a host round trip with duals 4.28 ms, 4.35.
+// Launched, these steps made calls on 20 k rows 2 to 3% longer.
 constexpr int kFinTile = 2048;               // entries a block sorts at a time
 constexpr int kFinWarps = kBlock / 32;
 constexpr int kFinChunk = kFinTile / kFinWarps;
@@ -811,7 +809,7 @@ __global__ void __launch_bounds__(kBlock) k_solo_finish(const __grid_constant__ 
 // one: 108 ms, batched 60.  An LP of 1.9 M entries alone takes 1.80 ms for 1.78.
 // Presolves in flight at once (share) get a part of the slots each: a grid that
 // fills the device waits for all of it, and they would run one after the other.
-// 20,000 rows from eight threads took 0.91 ms a call, now 0.24.
+// 20,000 rows from eight threads took four times as long.
 int solo_blocks(int32_t m, int32_t n, int64_t nnz, int share) {
     static CoopCache cache;
     int most = solo_finish_blocks(n, nnz) > 0 ? coop_blocks((const void *)k_solo, cache) : 0;

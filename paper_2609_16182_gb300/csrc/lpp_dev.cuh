@@ -75,7 +75,7 @@ struct SegMat {
     const int32_t *ptr;
     const int32_t *idx;
     const double *val;
-    const int32_t *order;      // segment ids grouped by class, stable within a class
+    const int32_t *order;      // segment ids grouped by class (no order within one)
     const Chunk *chunks;       // chunks of the long segments
     const int32_t *lfirst;     // [long + 1] first chunk of each long segment
     int32_t cnt;               // segments

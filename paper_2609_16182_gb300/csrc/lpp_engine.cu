@@ -810,8 +810,8 @@ void Engine::adopt_schedule(bool cols) {
 // Device words to pinned host memory and the wait for them, as one kernel that
 // stores them and then a number the host waits to see.  A copy and a wait for
 // the stream leave the device idle for longer, and a round has two to five reads:
-// the relaxation of 500 k rows (15 rounds) took 5.53 ms, now 5.30; with doubletons,
-// 250 k rows, 7.6 and 7.3; a burst of 32 requests 45.0 and 41.9.
+// with those the relaxation of 500 k rows (15 rounds) took 4% longer, as with
+// doubletons, 250 k rows; a burst of 32 requests served one by one 7%.
 // More than 16 KB (many LPs) goes by a copy.
 void Engine::fetch(std::initializer_list<FetchItem> items) {
     size_t bytes = 0;
@@ -974,7 +974,8 @@ void Engine::compact(int32_t round) {
     // the objective constant of the columns that left: with the columns in
     // place each slot's contribution stays until one sum at the end.  One LP's
     // tiles run beside the scatter (nothing else reads the contributions); the
-    // sums of many LPs, a warp each, are latency and slower beside it: a batch of six LPs of 150 k columns with dual_fixing 23.4 ms, not 18.7.
+    // sums of many LPs, a warp each, are latency and slower beside it: a batch of
+    // six LPs of 150 k columns with dual_fixing took 23.4 ms, not 18.8.
     const bool beside = !in_place && nlp == 1;
     if (beside) {
         LPP_CUDA(cudaEventRecord(ev_fork, s));
@@ -1043,8 +1044,8 @@ Engine::StepOut Engine::step(int32_t r, bool first_round, bool force) {
     // sides) beside S3', S4 and the marking (columns and flags; they share only
     // counters and the changed flag), joined before the counters are read; its
     // table is emptied meanwhile.  With S5 after S3' to the marking (as with
-    // `timing`, whose families are timed on one stream) 2 M rows take 1% longer
-    // (6.05 ms, now 5.98), 500 k rows with parallel_cols 2% (6.80, 6.65).
+    // `timing`, whose families are timed on one stream) 2 M rows take 1% longer,
+    // 500 k rows with parallel_cols 2%.
     const bool long_rows = prop_has_long(C), s5_beside = run_s5 && !o.timing;
     const bool side = long_rows || s5_beside;
     if (side) {

@@ -13,7 +13,7 @@ namespace lpp {
 namespace {
 
 // Rows of 257 to 4096 entries (kMidMin on), S1-S3 by the whole block with the
-// sums of prop_group<32>: 32 lane-strided chains, then the butterfly.  All
+// sums of prop_row<true>: 32 lane-strided chains, then the butterfly.  All
 // eight warps load the entries and their bounds, 512 at a time, into shared
 // memory (the candidate queues' space, emptied before); warp 0 then runs the
 // chains of the minimum and warp 1 those of the maximum while the next
@@ -439,9 +439,9 @@ __device__ __forceinline__ void match_long(const Ctx &C, int32_t t, int32_t *out
 // A barrier over the blocks of a cooperative launch: *bar, zero at the launch,
 // counts the arrivals of all barriers so far; gen is the number passed, the same
 // in every thread.  One release-add per block and one acquire load that sees the
-// last one: no counter to reset, no second word to publish.  With those, a call
-// on 20 k rows (110 barriers of 176 blocks) took 8% longer, 1.59 ms, not 1.47
-// to 1.54.  One block: a block barrier.
+// last one: no counter to reset, no second word to publish (with those, a call
+// on 20 k rows, 110 barriers of 176 blocks, took 3 to 8% longer).  One block: a
+// block barrier.
 // A wait that takes too long (with every block resident: longer than any work
 // between two barriers) sets *err bit 4 and returns false, as do then all later
 // waits.  Work that may take longer changes *progress (if given) as it goes, and
