@@ -317,7 +317,7 @@ __device__ __forceinline__ void prop_long_tighten(const Ctx &C, int32_t b, int32
 __device__ __forceinline__ void bsrc_offer(const Ctx &C, int32_t j, double x, double a, bool upper, bool capped,
                                            unsigned long long el, unsigned long long eu, int32_t o) {
     if (capped && gt0(fma(-C.max_implied, fabs(a), fabs(x)))) return;
-    const double v = x / a;
+    const double v = bound_value(x, a);
     if (!is_fin(v)) return;
     const unsigned long long e = enc_dbl(v);
     if (upper) {

@@ -121,6 +121,13 @@ __device__ __forceinline__ bool pass_lower(const Ctx &C, unsigned long long e, d
     return is_neg(a) ? lt0(s) : gt0(s);
 }
 
+// The bound x / a, with one zero: of two candidates -0 and +0 the second does not
+// improve on the first and is dropped, so their order would decide the sign.
+__device__ __forceinline__ double bound_value(double x, double a) {
+    const double v = x / a;
+    return (dbits(v) & 0x7fffffffffffffffLL) == 0 ? 0.0 : v;
+}
+
 // candidate kinds: implied bounds (capped) and singleton-row bounds (not)
 enum : int32_t { CQ_UPPER = 0, CQ_LOWER = 1, CQ_SING_UPPER = 2, CQ_SING_LOWER = 3 };  // bit 0: a lower bound
 
@@ -133,7 +140,7 @@ __device__ __forceinline__ void apply_cand(const Ctx &C, int32_t j, double x, do
         const float cap = __fmul_rd(f32_below(hi_word(C.max_implied)), f32_below(hi_word(a) & 0x7fffffffu));
         if (!(f32_mag(x) <= cap) && gt0(fma(-C.max_implied, fabs(a), fabs(x)))) return;
     }
-    const double v = x / a;
+    const double v = bound_value(x, a);
     if (!is_fin(v)) return;
     const unsigned long long e = enc_dbl(v);
     if (kind == CQ_UPPER || kind == CQ_SING_UPPER) {
