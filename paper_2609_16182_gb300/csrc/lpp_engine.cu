@@ -80,8 +80,12 @@ void dev_cache_put(void *p, size_t bytes, cudaStream_t s) {
 
 // Pinned host buffers (status mirrors, host copies of reduced LPs) are reused
 // across presolves: pinning memory costs far more than the rounds of a small LP.
+// Beyond kPinCacheMax of free ones, a buffer given back is unpinned: a caller
+// whose LPs grow would otherwise leave one of every size behind.
 static std::mutex g_pin_mu;
 static std::vector<std::pair<size_t, void *>> g_pin_free;
+static size_t g_pin_free_bytes = 0;
+constexpr size_t kPinCacheMax = size_t(4) << 30;
 
 // best fit among the free buffers, and none more than 4x (+ 1 MiB) the
 // request: a status mirror must not take the block a reduced LP needs next
@@ -98,6 +102,7 @@ static void *pinned_get(size_t bytes) {
         }
         if (best < g_pin_free.size()) {
             void *p = g_pin_free[best].second;
+            g_pin_free_bytes -= g_pin_free[best].first;
             g_pin_free.erase(g_pin_free.begin() + (long)best);
             return p;
         }
@@ -131,8 +136,24 @@ void pinned_put(void *p) {
         for (auto &e : g_pin_cap)
             if (e.first == p) cap = e.second;
     }
-    std::lock_guard<std::mutex> g(g_pin_mu);
-    g_pin_free.emplace_back(cap, p);
+    {
+        std::lock_guard<std::mutex> g(g_pin_mu);
+        if (g_pin_free_bytes + cap <= kPinCacheMax) {
+            g_pin_free.emplace_back(cap, p);
+            g_pin_free_bytes += cap;
+            return;
+        }
+    }
+    {  // forgotten before the address can come back from another thread's allocation
+        std::lock_guard<std::mutex> g(g_cap_mu);
+        for (size_t k = 0; k < g_pin_cap.size(); k++)
+            if (g_pin_cap[k].first == p) {
+                g_pin_cap[k] = g_pin_cap.back();
+                g_pin_cap.pop_back();
+                break;
+            }
+    }
+    cudaFreeHost(p);
 }
 
 namespace {

@@ -175,3 +175,26 @@ def test_device_inputs_off_the_boundaries(shift, timing):
     for k in ("row_ptr", "col_idx", "val", "c", "lhs", "rhs", "lb", "ub", "row_map", "col_map", "csc_ptr", "csc_idx",
               "csc_val"):
         np.testing.assert_array_equal(getattr(a, k), getattr(b, k))
+
+
+def test_free_pinned_buffers_are_bounded():
+    """Of five buffers of 1 GiB given back, at most the cache's 4 GiB stay pinned; one of them serves
+    the next request of their size."""
+    L, cu = lpp.load(), C.CDLL("libcuda.so.1")
+    get, put = L._ZN3lpp16pinned_get_sizedEm, L._ZN3lpp10pinned_putEPv
+    get.restype, get.argtypes, put.restype, put.argtypes = C.c_void_p, [C.c_size_t], None, [C.c_void_p]
+    torch.cuda.synchronize()
+
+    def pinned(p):
+        kind = C.c_uint(0)
+        return cu.cuPointerGetAttribute(C.byref(kind), 2, C.c_uint64(p)) == 0  # memory type
+
+    ps = [get(1 << 30) for _ in range(5)]
+    assert len(set(ps)) == 5 and all(pinned(p) for p in ps)
+    for p in ps:
+        put(p)
+    left = [p for p in ps if pinned(p)]
+    assert 1 <= len(left) <= 4
+    q = get(1 << 30)
+    assert q in left
+    put(q)
